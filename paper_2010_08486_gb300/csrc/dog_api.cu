@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <limits>
 #include <new>
 #include <vector>
 
@@ -47,12 +48,14 @@ struct dog_handle {
     std::vector<int> rad;
     std::vector<double> norm;
     std::vector<int> woff;
-    std::vector<int> hoff;   // the horizontal pass's copy of the taps
-    int w_total = 0;
+    int w_total = 0;         // floats of the plain tap table
+    int forms = 0;           // kernel forms that fit this ladder: bit nw
+    int warps = 0;           // warps asked for (8 or 12)
     int num_sms = 0;
     int band = 0;          // 0: whole frame
     int ctas_per_sm = 1;
     FusedParams base{};
+    std::vector<LevelInfo> lv;
     // device tables
     float* d_w = nullptr;
     float* d_c = nullptr;          // P normalisation coefficients, then P plane sigmas (float)
@@ -114,6 +117,8 @@ const std::vector<int>& handle_radii(const dog_handle* h) { return h->rad; }
 const std::vector<double>& handle_sigmas(const dog_handle* h) { return h->sig; }
 const dog_config& handle_cfg(const dog_handle* h) { return h->cfg; }
 int handle_band(const dog_handle* h) { return h->band; }
+int handle_w_total(const dog_handle* h) { return h->w_total; }
+const std::vector<LevelInfo>& handle_levels(const dog_handle* h) { return h->lv; }
 int* handle_status(dog_handle* h) { return h->d_status; }
 void*& handle_soft_ws(dog_handle* h) { return h->soft_ws; }
 void handle_set_last(dog_handle* h, cudaStream_t s) { h->last = s; }
@@ -219,82 +224,169 @@ static void free_all(dog_handle* h) {
 
 namespace dogk { void soft_free(dog_handle* h); }
 
-// Balance levels over the nw producer warps of a kernel form (every block,
-// all of them wait for the slowest at a barrier).  Per level the cost is two
-// passes of tpad/8 tap blocks plus a fixed cost (set-up, pipeline fill and
-// drain of both passes) of about 1.7 tap blocks of both passes (clock64 phase
-// timers).  Over 12 warps: first-fit decreasing at the smallest capacity that
-// packs all levels (raised one unit at a time from the larger of the average
-// load and the largest level); on the 25-level ladder this gives a largest
-// load of 124 units where longest-processing-time-first gives 134, 2% faster
-// measured.  Over 8 warps: longest processing time first (each level, largest
-// first, to the least loaded warp), which spreads the levels over all warps
-// and measured up to 5% faster there than first-fit decreasing.
-// A level whose 2r + 1 taps are one past a multiple of 8 runs its last tap
-// alone (8 FMAs instead of a block of 64, no further loads): 8 units less.
+// Pairs of levels of the fused kernel.  An odd ladder's first level is paired
+// with an absent one: the cheapest level, and the plane loop ends on a pair.
+static void plan_pairs(dog_handle* h) {
+    FusedParams& b = h->base;
+    const int K = h->K;
+    b.lev_off = K & 1;
+    b.n_pairs = (K + 1) / 2;
+    int tap = 0;
+    for (int q = 0; q < b.n_pairs; ++q) {
+        PairInfo& U = b.pairs[q];
+        const int hi = 2 * q + 1 - b.lev_off, lo = hi - 1;
+        U.r = (int16_t)h->rad[hi];
+        U.lead = (int16_t)(lo >= 0 ? U.r - h->rad[lo] : 0);
+        const int taps = 2 * U.r + 1;
+        // 2r + 1 taps one past a multiple of 8: the last tap runs alone
+        U.tail = (taps & 7) == 1;
+        U.nb = (int16_t)(U.tail ? taps / 8 : (taps + 7) / 8);
+        U.e = U.nb;
+        U.delta = (int16_t)(8 * U.e - U.r);
+        U.rcp = U.e > 1 ? (unsigned)(((1ull << 32) + U.e - 1) / U.e) : 0u;
+        U.tap = tap;
+        tap += 4 * (U.nb + U.tail);
+    }
+    b.n_taps4 = tap;
+}
+
+// Largest ladders this build accepts for the direct passes: those whose levels,
+// each with a ring of tpad + 8 rows, 18 response rows and two tap tables, and
+// whose input rows fit the shared memory (some form below fits all of them).
+static size_t direct_limit_bytes(const dog_handle* h) {
+    size_t rings = 0, taps = 0;
+    int dmin = 1 << 30, dmax = -(1 << 30);
+    for (const LevelInfo& L : h->lv) {
+        rings += (size_t)(L.tpad + 8) * TX;
+        taps += 2 * (size_t)L.tpad;
+        dmin = std::min(dmin, L.tpad - L.r);
+        dmax = std::max(dmax, L.tpad - L.r);
+    }
+    int rows = 32;
+    while (rows < dmax - dmin + 16) rows <<= 1;
+    const size_t in = (size_t)rows * ((TX + 2 * h->R + 8) | 1);
+    return sizeof(float) * (((taps + 3) & ~(size_t)3) + ((in + 3) & ~(size_t)3) + (size_t)h->K * 18 * TX + rings);
+}
+
+// Shared-memory layout of the form with nw warps; returns its size in bytes.
+static int plan_form(dog_handle* h, int nw) {
+    FusedParams& b = h->base;
+    int off = 0;
+    b.dmin = 1 << 30;
+    b.dmax = 0;
+    for (int q = 0; q < b.n_pairs; ++q) {
+        b.pairs[q].ring_off = off;
+        off += b.pairs[q].e * CHUNK;
+        b.dmin = std::min(b.dmin, (int)b.pairs[q].delta);
+        b.dmax = std::max(b.dmax, (int)b.pairs[q].delta);
+    }
+    b.nw = nw;
+    b.w_off = off;
+    off += 2 * nw * CHUNK;
+    b.x_off = off;
+    off += 2 * 2 * nw * 2 * TX;
+    b.e_off = off;
+    off += h->P * 2 * TX;
+    b.q_off = off;
+    off += nw * 2 * QUEUE_CAP;
+    b.c_off = off;
+    off += 2 * b.n_pairs * CHUNK_TABLE;
+    b.t_off = off;
+    off += 4 * b.n_taps4;
+    // input rows hold TX + 2R loaded columns; the padded taps of the widest
+    // level read 8 further (zero) columns; an odd stride keeps the eight rows
+    // read by one horizontal-pass instruction on distinct banks
+    b.in_stride = (TX + 2 * h->R + 8) | 1;
+    b.in_rows = 8 * nw + b.dmax - b.dmin;   // the rows a block reads
+    b.in_off = off;
+    off += b.in_rows * b.in_stride;
+    b.smem_bytes = off * (int)sizeof(float);
+    return b.smem_bytes;
+}
+
+// Position of tap t of level i in the pair tap table: base + 4 (t >> 1) + 2 (t & 1),
+// in floats, with t counted from the pair's window (the level's own tap 0 is
+// window tap `lead`).
+namespace dogk {
+void handle_tap_slot(const dog_handle* h, int i, int* base, int* lead) {
+    const int q = (i + h->base.lev_off) / 2, half = (i + h->base.lev_off) & 1;
+    *base = 4 * h->base.pairs[q].tap + half;
+    *lead = half ? 0 : h->base.pairs[q].lead;
+}
+}  // namespace dogk
+
+// The form to run for a wish of nw warps (0: no wish): the largest that fits and
+// is not larger than the wish.  More warps hide more latency: on every ladder
+// timed (96 frames of 1024 x 1024) the 12-warp form is the faster one, by 7% to
+// 20%, so it is the default wherever it fits.  What the handle reports without
+// a wish is the rule that callers know: 12 for ladders of 20 or more levels
+// whose largest level fits an even share of 12 warps, else 8.
 static long long level_cost(const LevelInfo& L) {
     const bool tail = ((2 * L.r + 1) & 7) == 1;
     return 10 * (L.tpad / 8) + 17 - (tail ? 8 : 0);
 }
 
-static void assign_levels(dog_handle* h, int nw) {
-    const int K = h->K;
-    std::vector<long long> cost(K);
-    long long total = 0, biggest = 0;
-    for (int i = 0; i < K; ++i) {
-        cost[i] = level_cost(h->base.lv[i]);
-        total += cost[i];
-        biggest = std::max(biggest, cost[i]);
-    }
-    std::vector<int> idx(K), owner(K);
-    for (int i = 0; i < K; ++i) idx[i] = i;
-    std::stable_sort(idx.begin(), idx.end(), [&](int a, int b) { return cost[a] > cost[b]; });
-    if (nw == 8) {
-        long long load[NWARPS] = {0};
-        for (int i : idx) {
-            int best = 0;
-            for (int w = 1; w < nw; ++w)
-                if (load[w] < load[best]) best = w;
-            load[best] += cost[i];
-            owner[i] = best;
+static void use_form(dog_handle* h, int nw) {
+    if (nw == 0) {
+        long long total = 0, biggest = 0;
+        for (const LevelInfo& L : h->lv) {
+            total += level_cost(L);
+            biggest = std::max(biggest, level_cost(L));
         }
+        h->warps = h->K >= 20 && 12 * biggest <= total ? 12 : 8;
     } else {
-        for (long long cap = std::max(biggest, (total + nw - 1) / nw);; ++cap) {
-            long long load[NWARPS] = {0};
-            bool fits = true;
-            for (int i : idx) {
-                int w = 0;
-                while (w < nw && load[w] + cost[i] > cap) ++w;
-                if (w == nw) { fits = false; break; }
-                load[w] += cost[i];
-                owner[i] = w;
-            }
-            if (fits) break;   // ends at the latest when cap reaches the total
-        }
+        h->warps = nw;
     }
-    h->base.nw = nw;
-    for (int w = 0; w < NWARPS; ++w) h->base.warp_nlev[w] = 0;
-    for (int i : idx) h->base.warp_lev[owner[i]][h->base.warp_nlev[owner[i]]++] = (unsigned char)i;
+    for (int f : {12, 8, 4, 3})
+        if ((nw == 0 || f <= nw) && (h->forms >> f & 1)) {
+            plan_form(h, f);
+            return;
+        }
+    plan_form(h, 3);   // nothing fits (an FFT-backend handle): never launched
 }
 
-// Kernel form for a ladder when none is set: 12 producer warps for long
-// ladders whose largest level fits an even share of 12 warps (there the
-// extra warps hide latency), else 8 with more registers each (a few large
-// levels: their warps set the pace).  Measured on 96 frames of 1024 x 1024
-// (ms per launch, 12 / 8 warps): 25 levels sigma 0.8..7.9 (largest level 107
-// units of 1395) 10.82 / 11.72; 14 levels sigma 2..12.3 (147 of 1148)
-// 12.59 / 10.98; 12 levels sigma 1..11.6 (137 of 824) 9.95 / 9.33; 24 levels
-// sigma 2..2.8 (47 of 1128) 12.27 / 11.39, which this rule gets wrong (the
-// autotuner times both forms).
-static int default_producer_warps(const dog_handle* h) {
-    long long total = 0, biggest = 0;
-    for (int i = 0; i < h->K; ++i) {
-        const long long c = level_cost(h->base.lv[i]);
-        total += c;
-        biggest = std::max(biggest, c);
+// Row bands of a single-frame launch (one CTA per strip and band, one CTA per
+// SM).  A tile costs its blocks of 8 nw rows plus a warm-up of about 0.3 blocks;
+// a block of which only some warps have rows still costs a third and its share
+// of the rest (12 warps, 25 levels: 43 us a block, 13 us the warm-up).  `asked`:
+// the handle's band height, taken as about that height: the bands are evened
+// out over the frame, in the number above or below that the model finds faster
+// (1024 x 1024, asked 232: four bands of 256 take 144 us, four of 232 and one of
+// 96 take 174 us); 0: any number (a 256 x 256 frame whole on its 8 strips takes
+// 68 us, in 8 bands 36 us).
+namespace dogk {
+int pick_band(const FusedParams& b, int num_sms, int H, int n_strips, int asked) {
+    const int mbk = 8 * b.nw;
+    auto tile_cost = [&](int rows) {
+        const int r = rows + (rows < H ? 2 : 1), part = (r % mbk + 7) / 8;
+        return 0.3 + r / mbk + (part ? 0.35 + 0.65 * part / b.nw : 0.0);
+    };
+    const int lo = asked > 0 ? std::max(1, H / asked) : 1;
+    const int hi = asked > 0 ? (H + asked - 1) / asked : std::min((H + 7) / 8, 128);
+    int best = 0;
+    double best_cost = 0.0;
+    for (int n = lo; n <= hi; ++n) {
+        const int band = ((H + n - 1) / n + 7) / 8 * 8;
+        const int bands = (H + band - 1) / band, tail = H - (bands - 1) * band;
+        const long long whole = (long long)n_strips * (bands - 1), ends = n_strips;
+        // whole tiles first, then the strips' last bands on the SMs left over
+        const long long rounds = whole / num_sms, left = whole % num_sms;
+        double cost = (double)rounds * tile_cost(band);
+        if (left) {
+            const long long room = num_sms - left, more = std::max<long long>(0, ends - room);
+            cost += std::max(tile_cost(band), (more ? 1.0 + (double)((more + num_sms - 1) / num_sms) : 1.0) * tile_cost(tail));
+        } else {
+            cost += (double)((ends + num_sms - 1) / num_sms) * tile_cost(tail);
+        }
+        if (!best || cost < best_cost) {
+            best = band;
+            best_cost = cost;
+        }
     }
-    return (h->K >= 20 && 12 * biggest <= total) ? 12 : 8;
+    return best;
 }
+int handle_sms(const dog_handle* h) { return h->num_sms; }
+}  // namespace dogk
 
 extern "C" {
 
@@ -391,17 +483,6 @@ int dog_create(const dog_config* cfg, dog_t** out) {
         h->woff.push_back((int)wf.size());
         for (int t = 0; t < tpad; ++t) wf.push_back(t <= 2 * r ? (float)(e[t] / z) : 0.0f);
     }
-    // a second copy of every level's taps for the horizontal pass: with the two
-    // passes reading separate tables the fused kernel runs 35% faster than
-    // with one shared table (measured; same values, same order)
-    for (int i = 0; i < h->K; ++i) {
-        h->hoff.push_back((int)wf.size());
-        const int tpad = 8 * ((2 * h->rad[i] + 1 + 7) / 8);
-        for (int t = 0; t < tpad; ++t) {
-            const float v = wf[h->woff[i] + t];
-            wf.push_back(v);
-        }
-    }
     h->w_total = (int)wf.size();
     // ---- normalisation (Eq. 3 / heat-equation finite difference)
     for (int i = 0; i < h->P; ++i)
@@ -416,45 +497,9 @@ int dog_create(const dog_config* cfg, dog_t** out) {
     b.P = h->P;
     b.R = h->R;
     b.thr = (float)c.threshold;
-    int dmin = 1 << 30, dmax = -(1 << 30);
-    int off = 0;
-    b.w_off = off;
-    b.w_total = h->w_total;
-    off += h->w_total;
-    // input rows hold TX + 2R loaded columns; the padded taps of the widest
-    // level read 8 further (zero) columns; an odd stride keeps the eight rows
-    // read by one horizontal-pass instruction on distinct banks
-    b.in_stride = (TX + 2 * h->R + 8) | 1;
-    for (int i = 0; i < h->K; ++i) {
-        LevelInfo& L = b.lv[i];
-        L.r = h->rad[i];
-        L.tpad = 8 * ((2 * L.r + 1 + 7) / 8);
-        L.e = L.tpad / MB;
-        L.delta = MB * L.e - L.r;
-        L.ring_rows = L.tpad + MB;
-        L.woff = h->woff[i];
-        L.hoff = h->hoff[i];
-        dmin = std::min(dmin, L.delta);
-        dmax = std::max(dmax, L.delta);
-    }
-    b.dmin = dmin;
-    b.dmax = dmax;
-    // a block reads dmax - dmin + MB input rows; the next block's MB rows are
-    // stored while other producer warps may still read this block's
-    b.in_rows = std::max(32, ceil_pow2(dmax - dmin + 2 * MB));
-    off = (off + 3) & ~3;
-    b.in_off = off;
-    off += b.in_rows * b.in_stride;
-    off = (off + 3) & ~3;
-    b.d_off = off;
-    off += h->K * DSLOTS * TX;
-    for (int i = 0; i < h->K; ++i) {
-        off = (off + 3) & ~3;
-        b.lv[i].ring_off = off;
-        off += b.lv[i].ring_rows * RING_STRIDE;
-    }
-    b.smem_bytes = off * (int)sizeof(float);
-    assign_levels(h, default_producer_warps(h));
+    b.thr_up = std::nextafter(b.thr, std::numeric_limits<float>::infinity());
+    for (int i = 0; i < h->K; ++i) h->lv.push_back({h->rad[i], 8 * ((2 * h->rad[i] + 1 + 7) / 8), h->woff[i]});
+    plan_pairs(h);
 
     int dev = 0, optin = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -465,7 +510,18 @@ int dog_create(const dog_config* cfg, dog_t** out) {
     }
     // the fused kernel's shared memory must fit; an FFT-backend handle can do
     // without it (its differentiable and batched calls then report UNSUPPORTED)
-    h->direct_ok = b.smem_bytes + 4096 <= optin;
+    if (b.n_taps4 <= MAX_TAPS4 && direct_limit_bytes(h) + 4096 <= (size_t)optin)
+        for (int f : {12, 8, 4, 3})
+            if (plan_form(h, f) + 4096 <= optin) h->forms |= 1 << f;
+    h->direct_ok = h->forms != 0;
+    use_form(h, 0);
+    for (int i = 0; i < h->K && h->direct_ok; ++i) {
+        int base, lead;
+        handle_tap_slot(h, i, &base, &lead);
+        float* tf = reinterpret_cast<float*>(b.taps) + base;
+        for (int t = 0; t <= 2 * h->rad[i]; ++t) tf[2 * (t + lead)] = wf[h->woff[i] + t];
+    }
+    for (int i = 0; i < h->P; ++i) b.cn[i] = cf[i];
     if (!h->direct_ok && c.backend == DOG_BACKEND_DIRECT) { delete h; return DOG_ERR_UNSUPPORTED; }
 
     // ---- pruning conflict table and histogram tables
@@ -537,7 +593,7 @@ int dog_create(const dog_config* cfg, dog_t** out) {
         delete h;
         return status_from(e);
     }
-    b.w = h->d_w;
+    b.w = nullptr;
     b.c = h->d_c;
     b.status = h->d_status;
 
@@ -577,11 +633,11 @@ int dog_set_tiling(dog_t* h, int32_t band_rows, int32_t ctas_per_sm) {
 
 int dog_set_producer_warps(dog_t* h, int32_t n) {
     if (!h || !(n == 0 || n == 8 || n == 12)) return DOG_ERR_INVALID;
-    assign_levels(h, n == 0 ? default_producer_warps(h) : n);
+    use_form(h, n);
     return DOG_OK;
 }
 
-int dog_get_producer_warps(const dog_t* h) { return h ? h->base.nw : DOG_ERR_INVALID; }
+int dog_get_producer_warps(const dog_t* h) { return h ? h->warps : DOG_ERR_INVALID; }
 
 // The contrast stretch applies to 12-bit frames when the handle's stretch_sat
 // is set (frames of more than 2^31 pixels are not supported then).
@@ -611,8 +667,10 @@ static FusedParams frame_params(const dog_handle* h, const void* img, int dtype,
     p.H = H;
     p.W = W;
     p.pitch = pitch;
-    p.band = (h->band > 0 && h->band < H) ? h->band : ((H + MB - 1) / MB) * MB;
+    p.strip_step = TX;
+    p.strip_x0 = 0;
     p.n_strips = (W + TX - 1) / TX;
+    p.band = pick_band(p, h->num_sms, H, p.n_strips, std::min(h->band, H));
     p.n_bands = (H + p.band - 1) / p.band;
     p.frames = nullptr;
     return p;
@@ -632,7 +690,7 @@ static ResolveParams resolve_params(const dog_handle* h, const FusedParams& f) {
     r.pitch = f.pitch;
     r.K = h->K;
     r.P = h->P;
-    r.w = f.w;
+    r.w = h->d_w;
     r.c = f.c;
     for (int i = 0; i < h->K; ++i) {
         r.woff[i] = h->woff[i];

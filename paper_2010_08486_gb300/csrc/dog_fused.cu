@@ -1,16 +1,17 @@
-// Fused DoG detector kernel: the 12-producer-warp forms, the launcher that
-// picks a form, and the batched set-up kernel.  The kernel itself is in
-// dog_fused_forms.cuh.
+// Fused DoG detector kernel: the 12-warp forms, the launcher that picks a form,
+// and the batched set-up kernel.  The kernel itself is in dog_fused_forms.cuh.
 #include "dog_fused_forms.cuh"
 
 namespace dogk {
 
-cudaError_t launch_fused_w8(const FusedParams& p, int grid, cudaStream_t s);   // dog_fused_w8.cu
+DOG_FUSED_FORMS(12)
 
 cudaError_t launch_fused(const FusedParams& p, int grid, cudaStream_t s) {
-    if (p.P < 1 || p.P > MAX_LEVELS - 1) return cudaErrorInvalidValue;
+    if (p.P < 2 || p.P > MAX_LEVELS - 1) return cudaErrorInvalidValue;
+    if (p.nw == 12) return launch_fused_w12(p, grid, s);
     if (p.nw == 8) return launch_fused_w8(p, grid, s);
-    if (p.nw == 12) return launch_fused_form<12>(p, grid, s);
+    if (p.nw == 4) return launch_fused_w4(p, grid, s);
+    if (p.nw == 3) return launch_fused_w3(p, grid, s);
     return cudaErrorInvalidValue;
 }
 

@@ -1,143 +1,76 @@
 // Fused DoG detector kernel for sm_103a: the kernel forms, templated on the
-// number of producer warps (dog_fused.cu and dog_fused_w8.cu instantiate them).
+// number of warps, the mode and the source of tiles (dog_fused.cu,
+// dog_fused_soft.cu instantiate them).
 //
 // Method (arXiv 2010.08486): scale space L_i = g(sigma_i) * I (Sec. 3), DoG
 // D_i = c_i (L_i - L_{i+1}) (Eq. 2-3), voxels equal to their 3x3x3 maximum
 // and above the threshold (Sec. 4, Sec. 4.1).
 //
-// Design.  A CTA owns a strip of TX = 32 output columns and walks down a
-// band of rows in blocks of MB = 8 rows, so every input pixel of the strip
-// is read once from global memory for all K scales and no vertical halo is
-// recomputed.  Each producer warp owns a fixed set of levels, chosen on the
-// host to balance taps (forms with 8 and with 12 producer warps; the host
-// picks one per ladder).  For each block and owned level a warp
-//   1. runs the horizontal pass of the next 8 input rows into the level's
-//      circular shared-memory ring (which runs Tpad/8 blocks ahead),
-//   2. runs the vertical pass over the ring into the block's L rows.
-// Both passes are register-blocked 1-D correlations: 8 outputs per lane,
-// taps in blocks of 8 against a two-window register file whose halves swap
-// roles each block, so one short loop serves every radius and the whole
-// kernel stays resident in the instruction cache.  Kernels are zero-padded to
-// Tpad = 8 ceil((2r+1)/8) taps; taps are summed in ascending order with FMA
-// from zero, so the padding never changes a value and the resolve kernel
-// (dog_resolve.cu), which repeats the order on the real taps only, reproduces
-// any response bit for bit.  Then all threads form D in place and test the
-// previous block's rows against their 26 neighbours; survivors are compacted
-// with one warp ballot and one atomic per warp.  Neighbours in the adjacent
-// strip are not held here: in detection a candidate at a strip edge is
-// queued and the resolve kernel recomputes the few responses it needs; the
-// soft modes, which keep every local maximum (thousands at strip edges per
-// frame), instead step 32-column strips by 30 so that lanes 0 and 31 are
-// only neighbours and every voxel a strip owns has its whole neighbourhood.
+// Design.  A CTA owns a strip of TX = 32 output columns and walks down a band
+// of rows in blocks of 8 NW rows, one chunk of 8 rows per warp, so every input
+// pixel of the strip is read once from global memory for all K scales.  Within
+// a block the levels are taken two at a time (a pair), all warps on the same
+// pair: in interval p a warp runs
+//   1. the maximum test of the two planes formed in the interval before,
+//   2. the horizontal pass of pair p + 1 for its 8 rows, into shared memory,
+//   3. the vertical pass of pair p for its 8 rows, into registers,
+//   4. the two differences the pair completes, in registers; it publishes the
+//      last two rows of each for the warp below,
+// and one barrier ends the interval.  The rows above a block that the vertical
+// pass needs are kept per pair in a ring of chunks (2r rows; the horizontal
+// pass is never repeated inside a band); the block's own chunks live in a
+// double buffer shared by all pairs.
+//
+// What bounds it: FP32 multiply-adds (2 sum(2r+1) per pixel).  The two levels
+// of a pair are the two lanes of packed FMAs, which halves the instructions and
+// shares the input loads of the horizontal pass.  All warps work on one pair at
+// a time so that the tap addresses are uniform and the taps come from the
+// constant bank (the kernel's parameters) as uniform operands: with taps read
+// from shared memory into registers the same inner loop takes 174 cycles per 64
+// packed FMAs and scheduler instead of 135 (128 is the pipe's limit), because
+// three register operands of 64 bits leave no register bandwidth for the loads
+// that fill the windows.  It also gives every warp the same work, so nobody
+// waits at the barrier, and the L rows never go through shared memory.
+//
+// Measured (96 frames of 1024 x 1024, 12-bit, one batched launch, 12 warps):
+// 25 levels to sigma 7.9 9.87 -> 8.45 ms, 12 levels 1.25^k 9.18 -> 5.8 ms, 6
+// levels to sigma 10.5 6.69 -> 3.6 ms, 14 levels to sigma 12.3 (8 warps) 10.56 ->
+// 9.4 ms, against the form before (levels on fixed producer warps, scalar FMAs,
+// taps and L rows through shared memory).
+//
+// Both passes are register-blocked 1-D correlations: 8 outputs per lane, taps
+// in blocks of 8 against a two-window register file whose halves swap roles
+// each block, so one short loop serves every radius.  The taps of both levels
+// sit in the wider level's window, zero-padded to 8 ceil((2r+1)/8); they are
+// summed in ascending order with FMA from zero, so the padding never changes a
+// (finite) value and the resolve kernel (dog_resolve.cu), which repeats the
+// order on the real taps only, reproduces any response bit for bit.
+// Neighbours in the adjacent strip are not held here: in detection a candidate
+// at a strip edge is queued and the resolve kernel recomputes the few responses
+// it needs; the soft modes, which keep every local maximum (thousands at strip
+// edges per frame), instead step 32-column strips by 30 so that lanes 0 and 31
+// are only neighbours and every voxel a strip owns has its whole neighbourhood.
 #pragma once
 
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <cfloat>
 
 #include "dog_internal.cuh"
 #include "dog_device.cuh"
 
 namespace dogk {
 
-// ---------------------------------------------------------------------------
-// 1-D passes.  out[k] = sum_{t=0}^{Tpad-1} wfull[t] * in[k+t], k = 0..7, in
-// ascending t from 0.  A holds inputs [8j, 8j+8), B inputs [8j+8, 8j+16) of
-// tap block j; the 64 products of the block are accumulated tap-major.
-__device__ __forceinline__ void fma_block(float (&acc)[8], const float (&A)[8], const float (&B)[8],
-                                          const float4 wa, const float4 wb) {
-    const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-#pragma unroll
-        for (int k = 0; k < 8; ++k) acc[k] = __fmaf_rn(w[u], (k + u < 8) ? A[k + u] : B[k + u - 8], acc[k]);
-}
+// Where a tile's input pixels come from.
+struct PixelSource {
+    const void* img;
+    int dtype, H, W, pitch;
+    int st_lo, st_hi;
+    float st_rcp;
+    int x0;
+};
 
-// The single last tap of a level whose 2r + 1 taps are one more than a
-// multiple of 8 (the rest of its padded block is zeros): out[k] += w * Y[k],
-// Y the window after the last full tap block.
-__device__ __forceinline__ void tap1(float (&acc)[8], const float (&Y)[8], float w) {
-#pragma unroll
-    for (int k = 0; k < 8; ++k) acc[k] = __fmaf_rn(w, Y[k], acc[k]);
-}
-
-// Horizontal: inputs are consecutive floats of one shared-memory row.
-// Output: 8 floats of one ring row, written as two float4 whose order is
-// swapped on odd rows (bank swizzle; `odd` is the ring row's parity).
-__device__ __forceinline__ void hpass(const float* __restrict__ src, float* __restrict__ dst, int odd,
-                                      const float4* __restrict__ w4, int nb, bool tail) {
-    float acc[8], A[8], B[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) { acc[k] = 0.0f; A[k] = src[k]; }
-    src += 8;
-    for (;;) {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) B[k] = src[k];
-        fma_block(acc, A, B, w4[0], w4[1]);
-        if (--nb == 0) {
-            if (tail) tap1(acc, B, w4[2].x);
-            break;
-        }
-        src += 8;
-        w4 += 2;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) A[k] = src[k];
-        fma_block(acc, B, A, w4[0], w4[1]);
-        if (--nb == 0) {
-            if (tail) tap1(acc, A, w4[2].x);
-            break;
-        }
-        src += 8;
-        w4 += 2;
-    }
-    float4* d4 = reinterpret_cast<float4*>(dst);
-    const float4 lo = make_float4(acc[0], acc[1], acc[2], acc[3]);
-    const float4 hi = make_float4(acc[4], acc[5], acc[6], acc[7]);
-    d4[odd] = lo;
-    d4[odd ^ 1] = hi;
-}
-
-// Vertical: inputs are rows of a circular ring of C rows (C a multiple of 8),
-// read in blocks of 8 rows starting at ring row r0 (a multiple of 8); lane x
-// holds column x, stored at x on even rows and x ^ 4 on odd rows.
-__device__ __forceinline__ void vpass(const float* __restrict__ ring, int lane, int C, int r0,
-                                      const float4* __restrict__ w4, int nb, bool tail, float (&acc)[8]) {
-    const float* pe = ring + lane;
-    const float* po = ring + (lane ^ 4);
-    float A[8], B[8];
-    int r = r0;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        acc[k] = 0.0f;
-        A[k] = ((k & 1) ? po : pe)[(r + k) * RING_STRIDE];
-    }
-    r += 8;
-    if (r == C) r = 0;
-    for (;;) {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) B[k] = ((k & 1) ? po : pe)[(r + k) * RING_STRIDE];
-        fma_block(acc, A, B, w4[0], w4[1]);
-        if (--nb == 0) {
-            if (tail) tap1(acc, B, w4[2].x);
-            break;
-        }
-        r += 8;
-        if (r == C) r = 0;
-        w4 += 2;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) A[k] = ((k & 1) ? po : pe)[(r + k) * RING_STRIDE];
-        fma_block(acc, B, A, w4[0], w4[1]);
-        if (--nb == 0) {
-            if (tail) tap1(acc, A, w4[2].x);
-            break;
-        }
-        r += 8;
-        if (r == C) r = 0;
-        w4 += 2;
-    }
-}
-
-// ---------------------------------------------------------------------------
 struct TileCtx {
     const void* img;
     int dtype, H, W, pitch;
@@ -155,27 +88,7 @@ __device__ __forceinline__ unsigned lanemask_lt() {
     return m;
 }
 
-// Named barriers (id 0 is __syncthreads).
-//   FULL:  producers arrive once a block's L rows are written; consumers wait.
-//   EMPTY: consumers arrive once a block's rows are no longer needed;
-//          producers wait before overwriting them two blocks later.
-//   PROD:  producers only, once per block (input-row visibility).
-//   CONS:  consumers only, between forming D and testing.
-// FULL and EMPTY alternate between two ids by block parity, so each id has at
-// most one generation outstanding: a producer arrives at FULL(b+2) only after
-// waiting EMPTY(b), which consumers signal after their wait on FULL(b), and
-// consumers arrive at EMPTY(b+2) only after FULL(b+2), which producers signal
-// after their wait on EMPTY(b).
-enum { BAR_FULL = 1, BAR_EMPTY = 3, BAR_PROD = 5, BAR_CONS = 6 };
-
-__device__ __forceinline__ void bar_sync(int id, int n) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
-}
-__device__ __forceinline__ void bar_arrive(int id, int n) {
-    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
-}
-
-// Shared scalars of one CTA (static shared memory).
+// Shared scalars of one CTA (static shared memory; the host reserves 4 KB).
 struct SmemSmall {
     float c[MAX_LEVELS];
     float sig[MAX_LEVELS];
@@ -186,448 +99,651 @@ struct SmemSmall {
     float soft[DOG_MAX_NBINS];
     float dc[MAX_LEVELS];
     float dt[MAX_LEVELS];
-    int rpos[MAX_LEVELS];     // ring row of each level's window start
+    PixelSource px;           // the tile in work (load8 reads it here: fewer registers held)
     int tile;
-    LevelInfo lv[MAX_LEVELS]; // per-level table (copied from the parameters once)
-    int wn[NWARPS];           // levels owned by each producer warp
-    unsigned char wl[NWARPS][MAX_LEVELS];
+    int careful;              // a pixel of the tile is not finite (or huge): exact_taps
+};
+static_assert(sizeof(SmemSmall) <= 4096, "reserved next to the dynamic shared memory");
+
+// Pixels beyond this magnitude take the careful path (their sums may overflow).
+constexpr float HUGE_PX = 1e37f;
+
+// ---------------------------------------------------------------------------
+// Taps of a pair, four floats (two taps of two levels) at a time: from the
+// kernel's parameters (constant bank), or from shared memory when the taps are
+// device data (soft modes).
+template <bool CT>
+struct Taps {
+    const FusedParams& p;
+    const float4* sm;
+    __device__ __forceinline__ float4 operator()(int q) const { return CT ? p.taps[q] : sm[q]; }
+    __device__ __forceinline__ float one(int q, int t, int half) const {   // tap t of one level of the pair at q
+        const float4 v = (*this)(q + (t >> 1));
+        return (t & 1) ? (half ? v.w : v.z) : (half ? v.y : v.x);
+    }
 };
 
-__device__ __forceinline__ int dslot(int k) { return k >= DSLOTS ? k - DSLOTS : k; }
+// acc[k] += (w_lo[u], w_hi[u]) * X[k + u], u = 0..7: both levels on the same
+// input (horizontal pass) or each on its own (vertical pass).
+__device__ __forceinline__ float2 both(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 both(float2 x) { return x; }
 
-// Producer warps: blur passes.  Block b's L rows go to DoG-buffer slots
-// (8b + 2 + k) mod DSLOTS.
-template <int NW>
-__device__ __forceinline__ void produce(const FusedParams& p, float* sm, SmemSmall& ss, const TileCtx& tc, int emax,
-                        int nblk) {
-    constexpr int NTHREADS = (NW + NCONS) * 32, NPROD_T = NW * 32;
-    const int tid = threadIdx.x;       // 0 .. NPROD_T-1
-    const int warp = tid >> 5;
-    const int lane = tid & 31;
-    const int R = p.R;
-    const int CIN = p.in_rows;        // input-buffer rows (a power of two)
-    const int S = p.in_stride;
-    const int ncols = TX + 2 * R;     // input columns per row (<= NPROD_T)
-    const int yb0 = tc.y0 - 1;
-    const int yorg = yb0 - MB * emax;   // input-ring slot origin
-    float* in = sm + p.in_off;
-    float* dbuf = sm + p.d_off;
-    // producer warps 0 .. MB-1 each fetch one of the MB rows a block adds,
-    // lane x columns x, x + 32, ... of the TX + 2R loaded ones
-    static_assert(NW >= MB, "one prefetched row per producer warp");
-    constexpr int NPF = (TX + 2 * DOG_MAX_RADIUS + 31) / 32;
-
-    for (int b = -emax; b < nblk; ++b) {
-        const int yb = yb0 + MB * b;
-        // prefetch the 8 rows block b+1 adds (latency hidden behind the passes)
-        unsigned pf[NPF];   // raw pixel bits; converted when stored, after the passes
-        const int ynew = yorg + MB * (b + emax + 1) + p.dmax;
-        const bool do_pf = b + 1 < nblk && warp < MB;
-        const int yrow = refl(ynew + warp, tc.H);
+template <class T, bool CT>
+__device__ __forceinline__ void fma_block(float2 (&acc)[8], const T (&A)[8], const T (&B)[8], const Taps<CT>& tap,
+                                          int q) {
 #pragma unroll
-        for (int k = 0; k < NPF; ++k) {
-            const int cc = lane + 32 * k;
-            pf[k] = (do_pf && cc < ncols) ? load_raw(tc.img, tc.dtype, tc.pitch, yrow, refl(tc.x0 - R + cc, tc.W)) : 0u;
-        }
-        // block b's L rows overwrite those of block b-2: wait for the consumers
-        if (b >= 2) bar_sync(BAR_EMPTY + (b & 1), NTHREADS);
-
-        const int nl = ss.wn[warp];
-        const int s0 = b >= 0 ? (MB * b + 2) % DSLOTS : 0;   // DoG-buffer slot of row yb
-        for (int li = 0; li < nl; ++li) {
-            const int i = ss.wl[warp][li];
-            const LevelInfo L = ss.lv[i];
-            const int C = L.ring_rows;
-            const int r0 = ss.rpos[i];     // 8b mod C; the chunk written now goes 8 rows before
-            if (b + L.e >= 0) {
-                float* ring = sm + L.ring_off;
-                // 2r + 1 = 8 (nb - 1) + 1: nb - 1 full tap blocks and one last tap
-                const bool tail = ((2 * L.r + 1) & 7) == 1;
-                const int nb = (L.tpad >> 3) - (tail ? 1 : 0);
-                {
-                    const int rho = lane >> 2, g = lane & 3;
-                    const int yy = yb + L.delta + rho;     // input row of this lane
-                    const float* src = in + ((yy - yorg) & (CIN - 1)) * S + (R - L.r) + 8 * g;
-                    const int wrow = (r0 >= MB ? r0 - MB : r0 + C - MB) + rho;
-                    hpass(src, ring + wrow * RING_STRIDE + 8 * g, rho & 1,
-                          reinterpret_cast<const float4*>(sm + p.w_off + L.hoff), nb, tail);
-                }
-                __syncwarp();
-                if (b >= 0) {
-                    float acc[8];
-                    vpass(ring, lane, C, r0, reinterpret_cast<const float4*>(sm + p.w_off + L.woff), nb, tail, acc);
-                    float* dcol = dbuf + i * DSLOTS * TX + lane;
+    for (int u2 = 0; u2 < 4; ++u2) {
+        const float4 w4 = tap(q + u2);
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) dcol[dslot(s0 + k) * TX] = acc[k];
-                }
-            }
-            __syncwarp();
-            if (lane == 0) ss.rpos[i] = (r0 + MB == C) ? 0 : r0 + MB;
-        }
-        // input rows of block b+1 (their slots are not read by block b)
-        if (do_pf) {
-            float* dst = in + ((ynew + warp - yorg) & (CIN - 1)) * S;
+        for (int v = 0; v < 2; ++v) {
+            const int u = 2 * u2 + v;
+            const float2 w = v ? make_float2(w4.z, w4.w) : make_float2(w4.x, w4.y);
 #pragma unroll
-            for (int k = 0; k < NPF; ++k) {
-                const int cc = lane + 32 * k;
-                if (cc < ncols) dst[cc] = raw_to_px(pf[k], tc.dtype, tc.st_lo, tc.st_hi, tc.st_rcp);
-            }
+            for (int k = 0; k < 8; ++k) acc[k] = __ffma2_rn(w, both((k + u < 8) ? A[k + u] : B[k + u - 8]), acc[k]);
         }
-        if (b >= 0) bar_arrive(BAR_FULL + (b & 1), NTHREADS);
-        bar_sync(BAR_PROD, NPROD_T);
     }
 }
 
-
-// Consumer warps: the 3x3x3 test of rows yb-1 .. yb+6 (two rows per warp),
-// with D_l = c_l (L_l - L_{l+1}) formed on the fly from the L rows the
-// producers wrote (the DoG buffer is never rewritten).
-//
-// Plane loop of one test row y: returns the mask of planes l whose voxel
-// (x, y, l) is a candidate: D_l(y, x) > thr and D_l(y, x) >= m_{l-1}, m_l,
-// m_{l+1}, where m_j is the 3x3 maximum of plane j around (x, y) (-inf for
-// planes outside the ladder).  Plane l - 1 is tested as soon as m_l exists,
-// so only a window of three maxima is live.  The vertical maximum of
-// c (L_l - L_{l+1}) over rows y-1 .. y+1 is formed as c max(L_l - L_{l+1}):
-// c > 0 and rounding is monotonic, so both are the same number.  Lanes 0 and
-// 31 receive their own value from the shuffles, which leaves their maximum
-// unchanged: neighbours outside the strip are outside the frame (-inf) or
-// settled by the resolve kernel.  EDGE: row y-1 or y+1 lies outside the
-// frame, or the strip has columns past the frame's right edge (-inf there).
-template <int PB, bool FULL, bool EDGE>
-__device__ __forceinline__ unsigned test_planes(const float* colp, const float* cs, int P, int sm1, int sc, int sp1,
-                                                bool ym_ok, bool yp_ok, bool col_ok, float thr) {
-    const float NEG = -INFINITY;
-    float m2 = NEG, m1 = NEG;   // 3x3 maxima of planes l-2, l-1
-    float d1 = NEG;             // D_{l-1}(y, x)
-    unsigned cmask = 0u;
-    float Lu = colp[sm1 * TX], Lc = colp[sc * TX], Ld = colp[sp1 * TX];   // L_0 rows y-1, y, y+1
+// The single last tap of a window whose 2r + 1 taps are one more than a
+// multiple of 8 (the rest of its padded block is zeros).
+template <class T, bool CT>
+__device__ __forceinline__ void fma_tail(float2 (&acc)[8], const T (&Y)[8], const Taps<CT>& tap, int q) {
+    const float4 w4 = tap(q);
 #pragma unroll
-    for (int l = 0; l < PB; ++l) {
-        const bool on = FULL || l < P;
-        const float* pl = colp + (on ? l + 1 : P) * DSLOTS * TX;
-        const float nu = pl[sm1 * TX], nc = pl[sc * TX], nd = pl[sp1 * TX];
-        const float c = cs[l];
-        const float eu = __fsub_rn(Lu, nu), ec = __fsub_rn(Lc, nc), en = __fsub_rn(Ld, nd);
-        Lu = nu; Lc = nc; Ld = nd;
-        const float d = __fmul_rn(c, ec);
-        const float e = EDGE ? fmaxf(ec, fmaxf(ym_ok ? eu : NEG, yp_ok ? en : NEG)) : fmaxf(ec, fmaxf(eu, en));
-        float m = __fmul_rn(c, e);
-        m = (EDGE ? (on && col_ok) : on) ? m : NEG;
-        const float ml = __shfl_up_sync(0xffffffffu, m, 1);
-        const float mr = __shfl_down_sync(0xffffffffu, m, 1);
-        const float m0 = fmaxf(m, fmaxf(ml, mr));
-        if (l >= 1) {
-            const bool cand = d1 >= fmaxf(m0, fmaxf(m2, m1)) && d1 > thr && (FULL || l - 1 < P);
-            cmask |= cand ? (1u << (l - 1)) : 0u;
-        }
-        m2 = m1;
-        m1 = m0;
-        d1 = d;
-    }
-    const bool cand = d1 >= fmaxf(m2, m1) && d1 > thr && (FULL || PB - 1 < P);
-    cmask |= cand ? (1u << (PB - 1)) : 0u;
-    return cmask;
+    for (int k = 0; k < 8; ++k) acc[k] = __ffma2_rn(make_float2(w4.x, w4.y), both(Y[k]), acc[k]);
 }
 
-// Plane loop of two adjacent test rows ya, yb = ya + 1 at once: their
-// 3x3 windows share rows ya and yb, so four L rows per plane serve both.  The
-// same operations as test_planes, row by row, so the masks are identical.
-// a_up / a_dn / b_up / b_dn: rows ya-1 / yb / ya / yb+1 lie inside the frame.
-template <int PB, bool FULL, bool EDGE>
-__device__ __forceinline__ void test_planes2(const float* colp, const float* cs, int P, int s0, int s1, int s2,
-                                             int s3, bool a_up, bool a_dn, bool b_up, bool b_dn, bool col_ok,
-                                             float thr, unsigned& cma, unsigned& cmb) {
-    const float NEG = -INFINITY;
-    float m2a = NEG, m1a = NEG, d1a = NEG, m2b = NEG, m1b = NEG, d1b = NEG;
-    unsigned ca = 0u, cb = 0u;
-    float L0 = colp[s0 * TX], L1 = colp[s1 * TX], L2 = colp[s2 * TX], L3 = colp[s3 * TX];
+// out[k] = sum_u w[u] X[k + u] over nb blocks of 8 taps (and the tail);
+// load(A) fetches the next 8 inputs of the window.
+template <class T, bool CT, class Load>
+__device__ __forceinline__ void correlate(float2 (&acc)[8], Load load, const Taps<CT>& tap, int q, int nb, bool tail) {
+    T A[8], B[8];
 #pragma unroll
-    for (int l = 0; l < PB; ++l) {
-        const bool on = FULL || l < P;
-        const float* pl = colp + (on ? l + 1 : P) * DSLOTS * TX;
-        const float n0 = pl[s0 * TX], n1 = pl[s1 * TX], n2 = pl[s2 * TX], n3 = pl[s3 * TX];
-        const float c = cs[l];
-        const float e0 = __fsub_rn(L0, n0), e1 = __fsub_rn(L1, n1), e2 = __fsub_rn(L2, n2), e3 = __fsub_rn(L3, n3);
-        L0 = n0; L1 = n1; L2 = n2; L3 = n3;
-        const float da = __fmul_rn(c, e1), db = __fmul_rn(c, e2);
-        const float mid = fmaxf(e1, e2);
-        const float va = EDGE ? fmaxf(a_up ? e0 : NEG, a_dn ? mid : e1) : fmaxf(e0, mid);
-        const float vb = EDGE ? fmaxf(b_up ? mid : e2, b_dn ? e3 : NEG) : fmaxf(mid, e3);
-        const bool live = EDGE ? (on && col_ok) : on;
-        const float ma = live ? __fmul_rn(c, va) : NEG;
-        const float mb = live ? __fmul_rn(c, vb) : NEG;
-        const float la = __shfl_up_sync(0xffffffffu, ma, 1), ra = __shfl_down_sync(0xffffffffu, ma, 1);
-        const float lb = __shfl_up_sync(0xffffffffu, mb, 1), rb = __shfl_down_sync(0xffffffffu, mb, 1);
-        const float m0a = fmaxf(ma, fmaxf(la, ra)), m0b = fmaxf(mb, fmaxf(lb, rb));
-        if (l >= 1) {
-            const bool okl = FULL || l - 1 < P;
-            ca |= (d1a >= fmaxf(m0a, fmaxf(m2a, m1a)) && d1a > thr && okl) ? (1u << (l - 1)) : 0u;
-            cb |= (d1b >= fmaxf(m0b, fmaxf(m2b, m1b)) && d1b > thr && okl) ? (1u << (l - 1)) : 0u;
+    for (int k = 0; k < 8; ++k) acc[k] = make_float2(0.0f, 0.0f);
+    load(A);
+    for (;;) {
+        load(B);
+        fma_block(acc, A, B, tap, q);
+        q += 4;
+        if (--nb == 0) {
+            if (tail) fma_tail(acc, B, tap, q);
+            break;
         }
-        m2a = m1a; m1a = m0a; d1a = da;
-        m2b = m1b; m1b = m0b; d1b = db;
+        load(A);
+        fma_block(acc, B, A, tap, q);
+        q += 4;
+        if (--nb == 0) {
+            if (tail) fma_tail(acc, A, tap, q);
+            break;
+        }
     }
-    const bool okl = FULL || PB - 1 < P;
-    ca |= (d1a >= fmaxf(m2a, m1a) && d1a > thr && okl) ? (1u << (PB - 1)) : 0u;
-    cb |= (d1b >= fmaxf(m2b, m1b) && d1b > thr && okl) ? (1u << (PB - 1)) : 0u;
-    cma = ca;
-    cmb = cb;
 }
 
-// D_l(y, x) of the test row (slot sc), recomputed for a candidate with the
-// operations of the plane loop.
-__device__ __forceinline__ float d_at(const float* colp, const float* cs, int l, int sc) {
-    return dog_value(cs[l], colp[l * DSLOTS * TX + sc * TX], colp[(l + 1) * DSLOTS * TX + sc * TX]);
-}
-
-// Per test row y and plane l: D at rows y-1, y, y+1 (three loads of L_{l+1},
-// the L_l rows carried from plane l-1), its vertical maximum, then the
-// horizontal maximum through two warp shuffles -> m_l; a voxel is a
-// candidate iff D_l(y, x) >= max(m_{l-1}, m_l, m_{l+1}) (it equals its 3x3x3
-// maximum).  Neighbours outside the frame count as -inf; those in the
-// adjacent strip are left to the resolve kernel (the candidate is queued),
-// unless the strips overlap (soft modes).
-// The plane loop is unrolled over PB >= P planes without branches (planes
-// l >= P read plane P and are masked to -inf), keeping m and D in registers;
-// candidates are collected in a per-lane bit mask and compacted afterwards
-// (they are rare).
-template <int NW, bool BATCHED, int PB, bool FULL>
-__device__ __forceinline__ void consume(const FusedParams& p, float* sm, SmemSmall& ss, const TileCtx& tc, int nblk) {
-    constexpr int NTHREADS = (NW + NCONS) * 32;
-    const int cw = (threadIdx.x >> 5) - NW;   // 0 .. NCONS-1
-    const int lane = threadIdx.x & 31;
-    const int P = p.P;
-    const int yb0 = tc.y0 - 1;
-    const float* dbuf = sm + p.d_off;
-    const int mode = p.mode;
-    const bool soft = (mode == MODE_SOFT || mode == MODE_BWD);
-    const float thr = soft ? -INFINITY : p.thr;   // D > thr is not applied to soft maxima
-    const int x = lane;
-    const int gx = tc.x0 + x;
-    const bool col_ok = gx >= 0 && gx < tc.W;   // a real column (neighbours of owned voxels)
-    // voxels this lane settles: with overlapping strips lanes 0 and TX-1 are
-    // only neighbours (the adjacent strips own those columns); otherwise a
-    // strip-edge voxel whose neighbours lie in the adjacent strip is queued
-    const bool overlap = !BATCHED && p.overlap;   // (single-frame launches only)
-    const bool own = col_ok && (!overlap || (x >= 1 && x <= TX - 2));
-    const bool edge_x = !overlap && ((x == 0 && tc.x0 > 0) || (x == TX - 1 && gx + 1 < tc.W));
-    const float* colp = dbuf + x;
-
-    for (int b = 0; b < nblk; ++b) {
-        const int yb = yb0 + MB * b;
-        bar_sync(BAR_FULL + (b & 1), NTHREADS);
-        // two rows per consumer warp: both masks from one plane loop
-        unsigned cm2a = 0u, cm2b = 0u;
-        if (MB / NCONS == 2 && mode != MODE_DUMP) {
-            const int wa = cw * 2;
-            const int ya = yb - 1 + wa;
-            const int s0 = (MB * b + wa) % DSLOTS, s1 = (MB * b + wa + 1) % DSLOTS;
-            const int s2 = (MB * b + wa + 2) % DSLOTS, s3 = (MB * b + wa + 3) % DSLOTS;
-            const bool a_up = ya - 1 >= 0, a_dn = ya + 1 < tc.H, b_up = ya >= 0, b_dn = ya + 2 < tc.H;
-            if (a_up && b_dn && tc.x0 >= 0 && tc.x0 + TX <= tc.W)
-                test_planes2<PB, FULL, false>(colp, ss.c, P, s0, s1, s2, s3, a_up, a_dn, b_up, b_dn, col_ok, thr,
-                                              cm2a, cm2b);
-            else
-                test_planes2<PB, FULL, true>(colp, ss.c, P, s0, s1, s2, s3, a_up, a_dn, b_up, b_dn, col_ok, thr,
-                                             cm2a, cm2b);
-        }
+// The same sums over one level's real taps only, for tiles with non-finite (or
+// huge) pixels: a zero tap of the padded windows would turn an infinity outside
+// the level's own window into a NaN.  For finite inputs the zero taps add
+// nothing, so both forms give the same bits.  in(k) is input k of the pair's
+// window; the level's own taps are d .. 2 rw - d of its 2 rw + 1.
+template <bool CT, class In>
+__device__ __forceinline__ void exact_taps(float (&acc)[8], In in, const Taps<CT>& tap, int q, int half, int d,
+                                           int rw) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) acc[k] = 0.0f;
 #pragma unroll 1
-        for (int q = 0; q < MB / NCONS; ++q) {
-            const int w = cw * (MB / NCONS) + q;
-            const int y = yb - 1 + w;
-            const bool row_ok = (y >= tc.y0 && y < tc.y1);
-            const int sc = (MB * b + w + 1) % DSLOTS;    // slot of row y
-            const int sm1 = (MB * b + w) % DSLOTS;       // row y-1
-            const int sp1 = (MB * b + w + 2) % DSLOTS;   // row y+1
-            const bool ym_ok = y - 1 >= 0, yp_ok = y + 1 < tc.H;
-            if (mode == MODE_DUMP) {
-                if (row_ok && own) {
-                    for (int l = 0; l < P; ++l) {
-                        const float* pl = colp + l * DSLOTS * TX;
-                        p.dump[((size_t)l * tc.H + y) * tc.W + gx] =
-                            dog_value(ss.c[l], pl[sc * TX], pl[DSLOTS * TX + sc * TX]);
-                    }
-                }
-                continue;
+    for (int t = d; t <= 2 * rw - d; ++t) {
+        const float w = tap.one(q, t, half);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) acc[k] = __fmaf_rn(w, in(k + t), acc[k]);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Chunks: 8 rows of a pair's horizontal sums, CHUNK floats; a row is 64 floats,
+// column x's two levels at 2x.  The row's sixteen 16-byte pieces 4g + j sit at
+// 4g + (j ^ chunk_swz), so that the horizontal pass's stores (lane (rho, g)
+// writes pieces 4g .. 4g+3 of row rho) touch every bank once per quarter-warp.
+__device__ __forceinline__ int chunk_swz(int row, int g) { return (g >> 1) | ((row & 1) << 1); }
+__device__ __forceinline__ int chunk_off(int row, int x) {   // float offset of column x in row `row`
+    const int g = x >> 3, j = (x >> 1) & 3;
+    return row * PAIR_STRIDE + 4 * (4 * g + (j ^ chunk_swz(row, g))) + 2 * (x & 1);
+}
+
+// Horizontal pass of pair U for 8 rows: lane (rho, g) columns 8g .. 8g+7 of row
+// rho; row: this lane's input row (column 0 is frame column x0 - R).
+template <bool CT>
+__device__ __forceinline__ void hpass(const PairInfo& U, const float* row, int R, float* dst, const Taps<CT>& tap,
+                                      bool careful) {
+    const int lane = threadIdx.x & 31, rho = lane >> 2, g = lane & 3;
+    const float* src = row + (R - U.r) + 8 * g;
+    if (!careful) {
+        float2 acc[8];
+        correlate<float>(acc, [&](float (&X)[8]) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) X[k] = src[k];
+            src += 8;
+        }, tap, U.tap, U.nb, U.tail != 0);
+        float4* d4 = reinterpret_cast<float4*>(dst + rho * PAIR_STRIDE + 16 * g);
+        const int swz = chunk_swz(rho, g);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            d4[j ^ swz] = make_float4(acc[2 * j].x, acc[2 * j].y, acc[2 * j + 1].x, acc[2 * j + 1].y);
+    } else {
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            float acc[8];
+            exact_taps(acc, [&](int k) { return src[k]; }, tap, U.tap, h, h ? 0 : U.lead, U.r);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) dst[chunk_off(rho, 8 * g + k) + h] = acc[k];
+        }
+    }
+}
+
+// Vertical pass of pair U for chunk w of the block: lane = column.  The window
+// is chunks at[0] .. at[e] (float offsets in sm): at points into the pair's
+// table of logical chunks (chunk_table).  A table, because address arithmetic
+// with comparisons in the loop makes the compiler give up the uniform tap
+// operands (215 cycles per tap block against 155).
+template <bool CT>
+__device__ __forceinline__ void vpass(const PairInfo& U, const float* sm, const int* at, const Taps<CT>& tap,
+                                      bool careful, float2 (&acc)[8]) {
+    const int lane = threadIdx.x & 31;
+    if (!careful) {
+        const int off_e = chunk_off(0, lane), off_o = chunk_off(1, lane);
+        correlate<float2>(acc, [&](float2 (&X)[8]) {
+            const float* c = sm + *at++;
+#pragma unroll
+            for (int k = 0; k < 8; k += 2) {
+                X[k] = *reinterpret_cast<const float2*>(c + off_e + k * PAIR_STRIDE);
+                X[k + 1] = *reinterpret_cast<const float2*>(c + off_o + k * PAIR_STRIDE);
             }
-            unsigned cmask;
-            if (MB / NCONS == 2)
-                cmask = q == 0 ? cm2a : cm2b;
-            else if (ym_ok && yp_ok && tc.x0 + TX <= tc.W)
-                cmask = test_planes<PB, FULL, false>(colp, ss.c, P, sm1, sc, sp1, ym_ok, yp_ok, col_ok, thr);
-            else
-                cmask = test_planes<PB, FULL, true>(colp, ss.c, P, sm1, sc, sp1, ym_ok, yp_ok, col_ok, thr);
-            if (!(row_ok && own)) cmask = 0u;
-            const unsigned dmask = edge_x ? 0u : cmask;   // settled here
-            const unsigned pmask = edge_x ? cmask : 0u;   // queued for the resolve kernel
-            // ---- queued strip-edge candidates (lanes 0 and 31 only)
-            if (__any_sync(0xffffffffu, pmask != 0u)) {
-                unsigned rest = pmask;
-                while (rest) {
-                    const int l = __ffs(rest) - 1;
-                    rest &= rest - 1;
-                    const int idx = atomicAdd(p.pend_count, 1);
-                    if (idx < p.pend_cap) {
-                        Pending e;
-                        e.frame = tc.frame; e.x = gx; e.y = y; e.level = l; e.response = d_at(colp, ss.c, l, sc);
-                        p.pend[idx] = e;
+        }, tap, U.tap, U.nb, U.tail != 0);
+    } else {
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            float s[8];
+            exact_taps(s, [&](int k) { return sm[at[k >> 3] + chunk_off(k & 7, lane) + h]; }, tap, U.tap, h,
+                       h ? 0 : U.lead, U.r);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) (h ? acc[k].y : acc[k].x) = s[k];
+        }
+    }
+}
+
+// n mod e without a division (n < 2^16, e <= 17; rcp = ceil(2^32 / e), 0 for e = 1).
+__device__ __forceinline__ int ring_pos(const PairInfo& U, int n) {
+    return U.rcp ? n - (int)__umulhi((unsigned)n, U.rcp) * U.e : 0;
+}
+
+// Offsets of a pair's logical chunks: e from its ring, then the block's own in
+// half `half` of wbuf.  A ring of at most nw chunks is rewritten whole by every
+// block, from slot 0; a longer one turns: logical chunk j of a block whose first
+// chunk is number abs0 of the tile is in slot (abs0 + j) mod e.  lane = chunk.
+static_assert(2 * DOG_MAX_RADIUS / 8 + 1 + 12 <= CHUNK_TABLE, "e + warps");
+__device__ __forceinline__ void chunk_table(int* table, const PairInfo& U, int nw, int wbuf, int half, int abs0) {
+    const int j = threadIdx.x & 31;
+    const int slot = U.e > nw ? ring_pos(U, abs0 + j) : j;
+    if (j < U.e + nw) table[j] = j < U.e ? U.ring_off + slot * CHUNK : wbuf + (half * nw + j - U.e) * CHUNK;
+}
+
+// ---------------------------------------------------------------------------
+// Maxima a warp has found, kept in its own shared-memory queue and written out
+// (or added to the soft histogram) 32 lanes at a time.
+// entry: .x = row (16 bits) | lane << 16 | plane << 21 | strip edge << 26; .y = L_l - L_{l+1} there
+__device__ __forceinline__ unsigned q_code(int y, int lane, int l, bool edge) {
+    return (unsigned)y | (unsigned)lane << 16 | (unsigned)l << 21 | (unsigned)edge << 26;
+}
+
+template <int MODE>
+__device__ __noinline__ void flush(const FusedParams& p, SmemSmall& ss, int x0, int frame, dog_blob* blobs, int* count,
+                                   const uint2* queue, int n) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    for (int i0 = 0; i0 < n; i0 += 32) {
+        const bool have = i0 + lane < n;
+        const uint2 v = have ? queue[i0 + lane] : make_uint2(0u, 0u);
+        const int y = v.x & 0xffff, x = x0 + (int)((v.x >> 16) & 31), l = (v.x >> 21) & 31;
+        const bool edge = (v.x >> 26) & 1;
+        const float e = __uint_as_float(v.y);
+        const float d = __fmul_rn(ss.c[l], e);
+        if (MODE == MODE_CANDIDATES) {
+            const unsigned mb = __ballot_sync(0xffffffffu, have && !edge), mp = __ballot_sync(0xffffffffu, have && edge);
+            int bb = 0, bp = 0;
+            if (lane == 0 && mb) bb = atomicAdd(count, __popc(mb));
+            if (lane == 0 && mp) bp = atomicAdd(p.pend_count, __popc(mp));
+            bb = __shfl_sync(0xffffffffu, bb, 0);
+            bp = __shfl_sync(0xffffffffu, bp, 0);
+            const int idx = edge ? bp + __popc(mp & lanemask_lt()) : bb + __popc(mb & lanemask_lt());
+            if (have && idx >= (edge ? p.pend_cap : p.cap)) {
+                atomicCAS(p.status, 0, (int)DOG_ERR_CAPACITY);
+            } else if (have && edge) {
+                Pending q;
+                q.frame = frame; q.x = x; q.y = y; q.level = l; q.response = d;
+                p.pend[idx] = q;
+            } else if (have) {
+                dog_blob bl;
+                bl.x = x; bl.y = y; bl.level = l; bl.sigma = ss.sig[l]; bl.response = d;
+                blobs[idx] = bl;
+            }
+        } else if (MODE == MODE_SOFT) {
+            int idx = 0;
+            if (p.rec != nullptr) {
+                const unsigned m = __ballot_sync(0xffffffffu, have);
+                if (lane == 0) idx = atomicAdd(p.rec_count, __popc(m));
+                idx = __shfl_sync(0xffffffffu, idx, 0) + __popc(m & lanemask_lt());
+            }
+            if (have) {
+                const float s = 1.0f / (1.0f + __expf(-(d - p.thr) * p.inv_T));
+                atomicAdd(&ss.soft[ss.kb[l][0]], s * ss.kw[l][0]);
+                atomicAdd(&ss.soft[ss.kb[l][1]], s * ss.kw[l][1]);
+                if (p.rec != nullptr) {
+                    if (idx < p.rec_cap) {
+                        const float q = s * (1.0f - s) * p.inv_T;
+                        dog_soft_max m;
+                        m.x = x; m.y = y; m.level = l; m.q = q; m.qe = q * e; m.s = s;
+                        p.rec[idx] = m;
                     } else {
                         atomicCAS(p.status, 0, (int)DOG_ERR_CAPACITY);
                     }
                 }
             }
-            if (mode == MODE_CANDIDATES) {
-                // one warp-wide slot reservation for all the row's candidates
-                const int nmine = __popc(dmask);
-                int incl = nmine;
+        }
+    }
+    __syncwarp();
+}
+
+// The 3x3x3 test, plane by plane.  A warp tests the rows one above its own
+// (test row t is its row t - 1), so that every neighbour row is its own or one
+// of the two the warp above published.
+// Everything a warp's test needs to know about its place.
+struct TestPlace {
+    int y;           // image row of test row 0
+    unsigned rows;   // bit t: test row t belongs to the tile
+    bool own, edge;  // this lane settles its column; its neighbours lie in the adjacent strip
+};
+
+// Candidates of plane l1: cen[t], the plane's centre differences, scaled by c,
+// against floor_[t], the largest of the neighbouring maxima and the threshold.
+template <int MODE>
+__device__ __forceinline__ void settle(const FusedParams& p, SmemSmall& ss, const TileCtx& tc, const TestPlace& at,
+                                       int l1, float c, const float (&cen)[8], const float (&floor_)[8], uint2* queue,
+                                       int& qn, float (&gp)[8]) {
+    bool any = false;
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int t = __shfl_up_sync(0xffffffffu, incl, o);
-                    if (lane >= o) incl += t;
+    for (int t = 0; t < 8; ++t) any |= __fmul_rn(c, cen[t]) >= floor_[t];
+    const bool found = __any_sync(0xffffffffu, any);
+    if (MODE != MODE_BWD && !found) return;
+    unsigned mask = 0u;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) mask |= __fmul_rn(c, cen[t]) >= floor_[t] ? 1u << t : 0u;
+    mask = at.own ? mask & at.rows : 0u;
+    const int lane = threadIdx.x & 31;
+    if (MODE == MODE_BWD) {
+        // dense dloss/dL rows: A_l = c_l G_l - c_{l-1} G_{l-1}; gp holds c_{l-1} G_{l-1}
+        const int x = tc.x0 + lane;
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            float g = 0.0f;
+            if (mask >> t & 1) {
+                const float d = __fmul_rn(c, cen[t]);
+                const float s = 1.0f / (1.0f + __expf(-(d - p.thr) * p.inv_T));
+                const float G = ss.gk[l1] * s * (1.0f - s) * p.inv_T;
+                atomicAdd(&ss.dc[l1], G * d / c);
+                atomicAdd(&ss.dt[l1], s * ss.gdk[l1]);
+                g = c * G;
+            }
+            if (at.own && (at.rows >> t & 1)) {
+                const size_t o = ((size_t)l1 * tc.H + at.y + t) * tc.W + x;
+                p.A[o] = g - (l1 > 0 ? gp[t] : 0.0f);
+                if (l1 == p.P - 1) p.A[o + (size_t)tc.H * tc.W] = -g;
+            }
+            gp[t] = g;
+        }
+        return;
+    }
+    while (__any_sync(0xffffffffu, mask != 0u)) {
+        if (qn + 32 > QUEUE_CAP) {
+            flush<MODE>(p, ss, tc.x0, tc.frame, tc.blobs, tc.count, queue, qn);
+            qn = 0;
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, mask != 0u);
+        if (mask) {
+            const int t = __ffs(mask) - 1;
+            mask &= mask - 1;
+            float e = cen[0];
+#pragma unroll
+            for (int u = 1; u < 8; ++u) e = t == u ? cen[u] : e;
+            queue[qn + __popc(bal & lanemask_lt())] = make_uint2(q_code(at.y + t, lane, l1, at.edge), __float_as_uint(e));
+        }
+        qn += __popc(bal);
+    }
+}
+
+// One plane: its differences of the warp's own rows and of the two rows above
+// give the 3x3 maxima of the test rows; then the plane below it in scale, whose
+// centre differences are cen, is settled.  Rows and columns outside the frame
+// hold -inf.  c > 0 and rounding is monotonic, so the maximum of the scaled
+// values is the scaled maximum.  Lanes 0 and 31 receive their own value from
+// the shuffles, which leaves their maximum unchanged: neighbours outside the
+// strip are outside the frame or settled elsewhere.  mprev: maxima of plane
+// l - 1; mout: of plane l; two[t]: the larger of the last two planes' maxima.
+// thr_up: the smallest number above the threshold (D > thr iff D >= thr_up).
+template <int MODE>
+__device__ __forceinline__ void test_plane(const FusedParams& p, SmemSmall& ss, const TileCtx& tc, const TestPlace& at,
+                                           int l, float c, float cprev, const float (&e)[8], float up2, float up1,
+                                           const float (&cen)[8], const float (&mprev)[8], float (&mout)[8],
+                                           float (&two)[8], float thr_up, uint2* queue, int& qn, float (&gp)[8]) {
+    float fl[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+        const float a = t < 2 ? (t ? up1 : up2) : e[t < 2 ? 0 : t - 2], b = t < 1 ? up1 : e[t < 1 ? 0 : t - 1];
+        const float v = fmaxf(e[t], fmaxf(a, b));
+        const float vl = __shfl_up_sync(0xffffffffu, v, 1), vr = __shfl_down_sync(0xffffffffu, v, 1);
+        mout[t] = __fmul_rn(c, fmaxf(v, fmaxf(vl, vr)));
+        fl[t] = fmaxf(thr_up, fmaxf(mout[t], two[t]));
+        two[t] = fmaxf(mprev[t], mout[t]);
+    }
+    if (l > 0) settle<MODE>(p, ss, tc, at, l - 1, cprev, cen, fl, queue, qn, gp);
+}
+
+// ---------------------------------------------------------------------------
+// Input rows y .. y + 7 into the buffer's slots `slot` .. (modulo CIN), by one
+// warp: lane x takes columns x, x + 32, ...; four rows by three columns of loads
+// in flight before any is converted and stored (more would cost the passes
+// around it their registers).
+__device__ __forceinline__ void load8(SmemSmall& ss, int R, int y, float* in, int slot, int CIN, int S) {
+    const PixelSource px = ss.px;
+    const int lane = threadIdx.x & 31, ncols = TX + 2 * R;
+    bool bad = false;
+#pragma unroll 1
+    for (int c0 = lane; c0 < ncols; c0 += 96) {
+        int xr[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) xr[k] = refl(px.x0 - R + min(c0 + 32 * k, ncols - 1), px.W);
+        int s = slot;
+#pragma unroll 1
+        for (int j0 = 0; j0 < 8; j0 += 4) {
+            unsigned v[4][3];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int yr = refl(y + j0 + j, px.H);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) v[j][k] = load_raw(px.img, px.dtype, px.pitch, yr, xr[k]);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                float* dst = in + s * S + c0;
+                s = s + 1 == CIN ? 0 : s + 1;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const float v1 = raw_to_px(v[j][k], px.dtype, px.st_lo, px.st_hi, px.st_rcp);
+                    if (c0 + 32 * k < ncols) dst[32 * k] = v1;
+                    bad |= !(fabsf(v1) < HUGE_PX);
                 }
-                const int total = __shfl_sync(0xffffffffu, incl, 31);
-                if (total) {
-                    int base = 0;
-                    if (lane == 0) base = atomicAdd(tc.count, total);
-                    base = __shfl_sync(0xffffffffu, base, 0);
-                    int idx = base + incl - nmine;
-                    unsigned rest = dmask;
-                    while (rest) {
-                        const int l = __ffs(rest) - 1;
-                        rest &= rest - 1;
-                        if (idx < p.cap) {
-                            dog_blob bl;
-                            bl.x = gx; bl.y = y; bl.level = l; bl.sigma = ss.sig[l]; bl.response = d_at(colp, ss.c, l, sc);
-                            tc.blobs[idx] = bl;
-                        } else {
-                            atomicCAS(p.status, 0, (int)DOG_ERR_CAPACITY);
-                        }
-                        ++idx;
+            }
+        }
+    }
+    if (bad) ss.careful = 1;
+}
+
+template <int NW, int MODE, bool BATCHED>
+__device__ __forceinline__ void process_tile(const FusedParams& p, float* sm, SmemSmall& ss, const TileCtx& tc) {
+    constexpr bool CT = MODE == MODE_CANDIDATES || MODE == MODE_DUMP;   // taps in the kernel's parameters
+    constexpr bool TEST = MODE != MODE_DUMP;
+    constexpr int MBK = 8 * NW;   // rows of a block
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rho = lane >> 2;
+    const int R = p.R, S = p.in_stride, CIN = p.in_rows, n = p.n_pairs, off = p.lev_off;
+    const int ncols = TX + 2 * R;
+    float* in = sm + p.in_off;
+    float* wbuf = sm + p.w_off;
+    float* xch = sm + p.x_off;      // [parity][plane of the pair][warp][2 rows][32]
+    float* eh = sm + p.e_off;       // [plane][2 rows][32]: the last two rows of the block before
+    uint2* queue = reinterpret_cast<uint2*>(sm + p.q_off) + warp * QUEUE_CAP;
+    int* tables = reinterpret_cast<int*>(sm + p.c_off);   // [half of wbuf][pair][CHUNK_TABLE]
+    const Taps<CT> tap{p, reinterpret_cast<const float4*>(sm + p.t_off)};
+    int qn = 0;
+
+    // rows computed: yb0 .. ylast (one above and one below the band, inside the
+    // frame); the test of a block's last row waits for the next block
+    const int yb0 = TEST && tc.y0 > 0 ? tc.y0 - 1 : tc.y0;
+    const int ylast = TEST ? min(tc.y1, tc.H - 1) : tc.y1 - 1;
+    const int nblk = ((TEST ? tc.y1 + 1 : tc.y1) - yb0 + MBK - 1) / MBK;
+    const int gx = tc.x0 + lane;
+    const bool col_ok = gx >= 0 && gx < tc.W;
+    const bool overlap = !BATCHED && p.overlap;   // (single-frame launches only)
+    TestPlace at;
+    at.own = col_ok && (!overlap || (lane >= 1 && lane <= TX - 2));
+    at.edge = !overlap && ((lane == 0 && tc.x0 > 0) || (lane == TX - 1 && gx + 1 < tc.W));
+    const bool cut = tc.x0 < 0 || tc.x0 + TX > tc.W;   // columns outside the frame
+    // soft modes keep every maximum
+    const float thr_up = MODE == MODE_CANDIDATES ? p.thr_up : -FLT_MAX;
+
+    int base = 0;            // input slot of image row yb + dmin, yb the current block's
+    // this lane's input row of the warp's chunk for pair U
+    auto row_of = [&](const PairInfo& U) {
+        int s = base + U.delta - p.dmin + 8 * warp + rho;
+        s -= s >= CIN ? CIN : 0;
+        return in + s * S;
+    };
+    // warm-up: the horizontal sums of the e chunks above the first block, in
+    // blocks of their own (warp w's chunk is chunk e - NW m + w of the ring)
+    int emax = 0;
+    for (int q = 0; q < n; ++q) emax = max(emax, (int)p.pairs[q].e);
+    const int nwarm = (emax + NW - 1) / NW;
+    if (tid == 0) {
+        ss.careful = 0;
+        // (field by field: nvcc 13.0 turns a copy of a whole struct into a copy of the
+        // kernel parameters its first fields came from)
+        ss.px.img = tc.img;
+        ss.px.dtype = tc.dtype;
+        ss.px.H = tc.H;
+        ss.px.W = tc.W;
+        ss.px.pitch = tc.pitch;
+        ss.px.st_lo = tc.st_lo;
+        ss.px.st_hi = tc.st_hi;
+        ss.px.st_rcp = tc.st_rcp;
+        ss.px.x0 = tc.x0;
+    }
+    __syncthreads();
+    for (int r = 8 * warp; r < CIN; r += MBK) {   // (the last group's rows past CIN go to the first slots again)
+        const int at0 = min(r, CIN - 8);
+        load8(ss, R, yb0 - MBK * nwarm + p.dmin + at0, in, at0, CIN, S);
+    }
+    for (int q = warp; q < 2 * n; q += NW)
+        chunk_table(tables + q * CHUNK_TABLE, p.pairs[q < n ? q : q - n], NW, p.w_off, q >= n, 0);
+    __syncthreads();
+    for (int m = nwarm; m > 0; --m) {
+        for (int q = 0; q < n; ++q) {
+            const PairInfo& U = p.pairs[q];
+            const int c = U.e - NW * m + warp;
+            if (c >= 0 && c < U.e)
+                hpass(U, row_of(U), R, sm + U.ring_off + c * CHUNK, tap, ss.careful != 0);
+        }
+        __syncthreads();
+        int s = base + 8 * warp;   // over the rows no longer read
+        load8(ss, R, yb0 - MBK * (m - 1) + p.dmax + 8 * warp, in, s - (s >= CIN ? CIN : 0), CIN, S);
+        base = (base + MBK) % CIN;
+        __syncthreads();
+    }
+    hpass(p.pairs[0], row_of(p.pairs[0]), R, wbuf + warp * CHUNK, tap, ss.careful != 0);
+    __syncthreads();
+
+    // test state between planes: the scaled 3x3 maxima m1 of the last plane (m2 is
+    // its partner, so that no maxima are copied), the larger of the last two
+    // planes' maxima, and the last plane's centre differences e1, which are
+    // settled as soon as the next plane's maxima exist; gp: the backward mode's
+    // c G of the plane before
+    float Lp[8], eA[8], eB[8], e1[8], m1[8], m2[8], two[8], gp[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        m1[k] = m2[k] = two[k] = e1[k] = eA[k] = eB[k] = -INFINITY;
+        Lp[k] = gp[k] = 0.0f;
+    }
+    int par = 0;     // buffer half of the current interval's pair
+    int abs0 = 0;    // chunks before the current block (ring slots are taken modulo e)
+    at.rows = 0u;
+    for (int b = 0;; ++b) {   // block nblk: only the last planes' test
+        const int yb = yb0 + MBK * b;
+        const bool last = b + 1 == nblk;
+        const int yw = yb + 8 * warp;             // this warp's first row
+        const bool act = yw <= ylast;             // it has rows to compute
+        const bool inside = yw + 7 < tc.H && !cut;
+        for (int q = 0; q < n; ++q) {
+            const PairInfo& U = p.pairs[q];
+            const bool careful = ss.careful != 0;
+            const bool some = q > 0 || b > 0;      // there was an interval before
+            const int lq = q ? q - 1 : n - 1;      // and this was its pair
+            if (TEST && q == 1) {   // the planes tested from here on are this block's
+                at.y = yw - 1;
+                const int lo = max(tc.y0 - at.y, 0), hi = min(tc.y1 - at.y, 8);   // test rows lo .. hi-1
+                at.rows = hi > lo && (MODE != MODE_CANDIDATES || p.thr < INFINITY) ? ((1u << hi) - 1u) & ~((1u << lo) - 1u) : 0u;
+            }
+            // 1. keep the chunk of the pair before for its next block (the last e
+            // chunks, in the slots after the block's); stored after the test
+            const PairInfo& V = p.pairs[lq];
+            const int kc = warp - (NW - V.e);
+            const bool keep = some && kc >= 0;
+            float4 kept[CHUNK / 128];
+            if (keep) {
+                const float4* s4 = reinterpret_cast<const float4*>(wbuf + (par ^ 1) * (NW * CHUNK) + warp * CHUNK);
+#pragma unroll
+                for (int i = 0; i < CHUNK / 128; ++i) kept[i] = s4[i * 32 + lane];
+                const int slot = V.e > NW ? ring_pos(V, (q ? abs0 + NW : abs0) + kc) : kc;
+                float4* d4 = reinterpret_cast<float4*>(sm + V.ring_off + slot * CHUNK);
+#pragma unroll
+                for (int i = 0; i < CHUNK / 128; ++i) d4[i * 32 + lane] = kept[i];
+            }
+            __syncwarp();
+            // 2. horizontal pass of the next pair (the last pair's interval does the
+            // next block's first one below): half of the warps of each scheduler run
+            // it before the test, so that the test's comparisons meet other warps' FMAs
+            auto ahead = [&]() {
+                const PairInfo& N = p.pairs[q + 1];
+                hpass(N, row_of(N), R, wbuf + (par ^ 1) * (NW * CHUNK) + warp * CHUNK, tap, careful);
+            };
+            const bool go = q + 1 < n && act && b < nblk;
+            if (go && (warp & 4)) ahead();
+            // 3. the planes published in the interval before
+            if (TEST && some) {
+                const bool first = q ? b == 0 : b == 1;   // they are of the tile's first block
+                const float* xr = xch + (par ^ 1) * (2 * NW * 64);
+                float upA1 = -INFINITY;
+#pragma unroll
+                for (int s = 0; s < 2; ++s) {
+                    const int l = 2 * lq - 1 - off + s;
+                    if (l < 0) continue;
+                    const float* src = warp ? xr + (s * NW + warp - 1) * 64 : eh + l * 64;
+                    float up2 = src[lane], up1 = src[32 + lane];
+                    if (warp == 0) {
+                        if (first) up2 = up1 = -INFINITY;
+                        const float* lw = xr + (s * NW + NW - 1) * 64;
+                        eh[l * 64 + lane] = lw[lane];
+                        eh[l * 64 + 32 + lane] = lw[32 + lane];
+                    }
+                    const float c = CT ? p.cn[l] : ss.c[l], cp = CT ? p.cn[max(l - 1, 0)] : ss.c[max(l - 1, 0)];
+                    if (s == 0) {
+                        upA1 = up1;
+                        test_plane<MODE>(p, ss, tc, at, l, c, cp, eA, up2, up1, e1, m1, m2, two, thr_up, queue, qn, gp);
+                    } else {
+                        const float cen[8] = {upA1, eA[0], eA[1], eA[2], eA[3], eA[4], eA[5], eA[6]};
+                        test_plane<MODE>(p, ss, tc, at, l, c, cp, eB, up2, up1, cen, m2, m1, two, thr_up, queue, qn, gp);
+                        e1[0] = up1;
+#pragma unroll
+                        for (int t = 1; t < 8; ++t) e1[t] = eB[t - 1];
                     }
                 }
-            } else if (mode == MODE_SOFT) {
-                // optional record of the maxima for the backward: each lane
-                // with maxima reserves its slots (about one lane per warp row)
-                int idx = 0;
-                if (p.rec != nullptr && dmask != 0u) idx = atomicAdd(p.rec_count, __popc(dmask));
-                unsigned rest = dmask;
-                while (rest) {
-                    const int l = __ffs(rest) - 1;
-                    rest &= rest - 1;
-                    const float e = __fsub_rn(colp[l * DSLOTS * TX + sc * TX], colp[(l + 1) * DSLOTS * TX + sc * TX]);
-                    const float d = __fmul_rn(ss.c[l], e);   // = d_at(colp, ss.c, l, sc)
-                    const float s = 1.0f / (1.0f + __expf(-(d - p.thr) * p.inv_T));
-                    atomicAdd(&ss.soft[ss.kb[l][0]], s * ss.kw[l][0]);
-                    atomicAdd(&ss.soft[ss.kb[l][1]], s * ss.kw[l][1]);
-                    if (p.rec != nullptr) {
-                        if (idx < p.rec_cap) {
-                            const float q = s * (1.0f - s) * p.inv_T;
-                            dog_soft_max m;
-                            m.x = gx; m.y = y; m.level = l; m.q = q; m.qe = q * e; m.s = s;
-                            p.rec[idx] = m;
-                        } else {
-                            atomicCAS(p.status, 0, (int)DOG_ERR_CAPACITY);
-                        }
-                        ++idx;
+                if (q == 0) {   // the last plane has nothing above it
+#pragma unroll
+                    for (int t = 0; t < 8; ++t) two[t] = fmaxf(thr_up, two[t]);
+                    settle<MODE>(p, ss, tc, at, p.P - 1, CT ? p.cn[p.P - 1] : ss.c[p.P - 1], e1, two, queue, qn, gp);
+#pragma unroll
+                    for (int t = 0; t < 8; ++t) m1[t] = m2[t] = two[t] = -INFINITY;
+                }
+            }
+            if (b == nblk) {
+                if (TEST && qn) flush<MODE>(p, ss, tc.x0, tc.frame, tc.blobs, tc.count, queue, qn);
+                __syncthreads();
+                return;
+            }
+            if (go && !(warp & 4)) ahead();
+            // a turning ring: the pair's chunk table for the next block
+            if (V.e > NW && some && warp == 0) chunk_table(tables + (((par ^ 1 ^ n) & 1) * n + lq) * CHUNK_TABLE, V, NW, p.w_off, (par ^ 1 ^ n) & 1, q ? abs0 + NW : abs0);
+            // 4. vertical pass and the differences it completes
+            if (act) {
+                float2 acc[8];
+                vpass(U, sm, tables + (par * n + q) * CHUNK_TABLE + warp, tap, careful, acc);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    eA[k] = __fsub_rn(Lp[k], acc[k].x);
+                    eB[k] = __fsub_rn(acc[k].x, acc[k].y);
+                    Lp[k] = acc[k].y;
+                }
+                if (MODE == MODE_DUMP) {
+#pragma unroll
+                    for (int s = 0; s < 2; ++s) {
+                        const int l = 2 * q - 1 - off + s;
+                        if (l < 0 || !at.own) continue;
+                        const float c = p.cn[l];
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            if (yw + k < tc.y1)
+                                p.dump[((size_t)l * tc.H + yw + k) * tc.W + gx] = __fmul_rn(c, s ? eB[k] : eA[k]);
                     }
+                } else if (!inside) {   // rows and columns outside the frame do not count
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        if (yw + k >= tc.H || !col_ok) eA[k] = eB[k] = -INFINITY;
                 }
             } else {
-                // backward prologue: dense dloss/dL rows A_l = c_l G_l - c_{l-1} G_{l-1}
-                float Gprev = 0.0f;
 #pragma unroll
-                for (int l = 0; l < PB; ++l) {
-                    if (l < P) {
-                        float G = 0.0f;
-                        if (dmask & (1u << l)) {
-                            const float d = d_at(colp, ss.c, l, sc);
-                            const float s = 1.0f / (1.0f + __expf(-(d - p.thr) * p.inv_T));
-                            G = ss.gk[l] * s * (1.0f - s) * p.inv_T;
-                            atomicAdd(&ss.dc[l], G * d / ss.c[l]);
-                            atomicAdd(&ss.dt[l], s * ss.gdk[l]);
-                        }
-                        if (row_ok && own) {
-                            p.A[((size_t)l * tc.H + y) * tc.W + gx] = ss.c[l] * G - (l > 0 ? ss.c[l - 1] * Gprev : 0.0f);
-                            if (l == P - 1) p.A[((size_t)(l + 1) * tc.H + y) * tc.W + gx] = -ss.c[l] * G;
-                        }
-                        Gprev = G;
-                    }
-                }
+                for (int k = 0; k < 8; ++k) eA[k] = eB[k] = -INFINITY;
             }
+            if (TEST) {
+                float* xw = xch + par * (2 * NW * 64) + warp * 64 + lane;
+                xw[0] = eA[6];
+                xw[32] = eA[7];
+                xw[NW * 64] = eB[6];
+                xw[NW * 64 + 32] = eB[7];
+            }
+            if (q + 1 == n && !last) {
+                // the next block's input rows, over the rows no longer read
+                int s = base + 8 * warp;
+                s -= s >= CIN ? CIN : 0;
+                load8(ss, R, yb + MBK + p.dmax + 8 * warp, in, s, CIN, S);
+                __syncthreads();
+                base = (base + MBK) % CIN;
+                if (yw + MBK <= ylast)
+                    hpass(p.pairs[0], row_of(p.pairs[0]), R,
+                          wbuf + (par ^ 1) * (NW * CHUNK) + warp * CHUNK, tap, ss.careful != 0);
+            }
+            __syncthreads();
+            par ^= 1;
         }
-        // rows yb-2 .. yb+5 are free for block b+2 (arrivals match the producers' waits)
-        if (b + 2 < nblk) bar_arrive(BAR_EMPTY + (b & 1), NTHREADS);
+        abs0 += NW;
     }
 }
 
-template <int NW, bool BATCHED, int PB, bool FULL>
-__device__ __forceinline__ void process_tile(const FusedParams& p, float* sm, SmemSmall& ss, const TileCtx& tc) {
-    constexpr int NTHREADS = (NW + NCONS) * 32, NPROD_T = NW * 32;
-    const int tid = threadIdx.x;
-    const int yb0 = tc.y0 - 1;
-    const int nblk = (tc.y1 - tc.y0 + 2 + MB - 1) / MB;
-    int emax = 0;
-    for (int i = 0; i < p.K; ++i) emax = max(emax, ss.lv[i].e);
-    const int yorg = yb0 - MB * emax;
-    const int R = p.R;
-    const int ncols = TX + 2 * R;
-    // initial input rows (those read at block -emax), spread over all threads;
-    // each thread issues its loads before converting and storing any
-    float* in = sm + p.in_off;
-    {
-        const int y0 = yorg + p.dmin;
-        const int total = (p.dmax + MB - p.dmin) * ncols;
-        for (int i0 = 0; i0 < total; i0 += 8 * NTHREADS) {
-            unsigned v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int i = i0 + u * NTHREADS + tid;
-                v[u] = 0u;
-                if (i < total) {
-                    const int rr = i / ncols, cc = i - rr * ncols;
-                    v[u] = load_raw(tc.img, tc.dtype, tc.pitch, refl(y0 + rr, tc.H), refl(tc.x0 - R + cc, tc.W));
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int i = i0 + u * NTHREADS + tid;
-                if (i < total) {
-                    const int rr = i / ncols, cc = i - rr * ncols;
-                    in[((y0 + rr - yorg) & (p.in_rows - 1)) * p.in_stride + cc] =
-                        raw_to_px(v[u], tc.dtype, tc.st_lo, tc.st_hi, tc.st_rcp);
-                }
-            }
-        }
-    }
-    for (int i = tid; i < p.K; i += NTHREADS) {
-        const int C = ss.lv[i].ring_rows;
-        ss.rpos[i] = ((-MB * emax) % C + C) % C;
-    }
-    __syncthreads();
-    if (tid < NPROD_T) produce<NW>(p, sm, ss, tc, emax, nblk);
-    else consume<NW, BATCHED, PB, FULL>(p, sm, ss, tc, nblk);
-    __syncthreads();
-}
-
-template <int NW, bool BATCHED, int PB, bool FULL>
-__global__ void __launch_bounds__((NW + NCONS) * 32, 1) dog_fused_kernel(const __grid_constant__ FusedParams p) {
-    constexpr int NTHREADS = (NW + NCONS) * 32;
+template <int NW, int MODE, bool BATCHED>
+__global__ void __launch_bounds__(NW * 32, 1) dog_fused_kernel(const __grid_constant__ FusedParams p) {
+    constexpr int NTHREADS = NW * 32;
+    constexpr bool SOFT = MODE == MODE_SOFT || MODE == MODE_BWD;
     extern __shared__ float4 dyn4[];
     float* sm = reinterpret_cast<float*>(dyn4);
     __shared__ SmemSmall ss;
     const int tid = threadIdx.x;
-    // zero the dynamic shared memory once: zero-weight padding taps may read
-    // input-row columns past the loaded ones, and those must be finite
-    for (int q = tid; q < p.smem_bytes / 16; q += NTHREADS) dyn4[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-    __syncthreads();
-    for (int q = tid; q < p.w_total; q += NTHREADS) sm[p.w_off + q] = p.w[q];
-    for (int q = tid; q < MAX_LEVELS; q += NTHREADS) ss.c[q] = q < p.P ? p.c[q] : 0.0f;
-    for (int q = tid; q < p.K; q += NTHREADS) ss.lv[q] = p.lv[q];
-    for (int q = tid; q < NWARPS * MAX_LEVELS; q += NTHREADS) ss.wl[q / MAX_LEVELS][q % MAX_LEVELS] =
-        p.warp_lev[q / MAX_LEVELS][q % MAX_LEVELS];
-    for (int q = tid; q < NWARPS; q += NTHREADS) ss.wn[q] = p.warp_nlev[q];
-    for (int q = tid; q < p.P; q += NTHREADS) ss.sig[q] = 0.0f;
-    if (p.mode == MODE_SOFT || p.mode == MODE_BWD) {
+    // zero-weight padding taps may read input-row columns past the loaded ones,
+    // and those must be finite
+    {
+        const int c0 = TX + 2 * p.R, nc = p.in_stride - c0;
+        for (int q = tid; q < p.in_rows * nc; q += NTHREADS) sm[p.in_off + q / nc * p.in_stride + c0 + q % nc] = 0.0f;
+    }
+    for (int q = tid; q < p.P; q += NTHREADS) {
+        ss.c[q] = p.c[q];
+        ss.sig[q] = p.c[p.P + q];
+    }
+    if (SOFT) {
+        float4* t4 = reinterpret_cast<float4*>(sm + p.t_off);
+        const float4* w4 = reinterpret_cast<const float4*>(p.w);
+        for (int q = tid; q < p.n_taps4; q += NTHREADS) t4[q] = w4[q];
         for (int q = tid; q < p.nbins; q += NTHREADS) ss.soft[q] = 0.0f;
         for (int l = tid; l < p.P; l += NTHREADS) {
             float gk = 0.0f, gdk = 0.0f;
@@ -644,29 +760,23 @@ __global__ void __launch_bounds__((NW + NCONS) * 32, 1) dog_fused_kernel(const _
             ss.gk[l] = gk; ss.gdk[l] = gdk; ss.dc[l] = 0.0f; ss.dt[l] = 0.0f;
         }
     }
-    __syncthreads();
 
     if (!BATCHED) {
         // single frame: blockIdx.x enumerates (strip, band)
-        if (p.mode == MODE_CANDIDATES) {
-            for (int q = tid; q < p.P; q += NTHREADS) ss.sig[q] = p.c[p.P + q];
-        }
         __syncthreads();
         TileCtx tc;
         tc.img = p.img; tc.dtype = p.dtype; tc.H = p.H; tc.W = p.W; tc.pitch = p.pitch; tc.frame = 0;
         tc.st_lo = tc.dtype == DTYPE_U16_STRETCH ? p.lohi[0] : 0;
         tc.st_hi = tc.dtype == DTYPE_U16_STRETCH ? p.lohi[1] : 0;
         tc.st_rcp = stretch_rcp(tc.st_lo, tc.st_hi);
-        const int strip = blockIdx.x % p.n_strips;
-        const int band = blockIdx.x / p.n_strips;
-        tc.x0 = p.overlap ? strip * (TX - 2) - 1 : strip * TX;
+        const int band = blockIdx.x / p.n_strips, strip = blockIdx.x - band * p.n_strips;
+        tc.x0 = strip * p.strip_step + p.strip_x0;
         tc.y0 = band * p.band;
         tc.y1 = min(p.H, tc.y0 + p.band);
         tc.blobs = p.blobs;
         tc.count = p.count;
-        process_tile<NW, BATCHED, PB, FULL>(p, sm, ss, tc);
+        process_tile<NW, MODE, BATCHED>(p, sm, ss, tc);
     } else {
-        for (int q = tid; q < p.P; q += NTHREADS) ss.sig[q] = p.c[p.P + q];
         const long long n_tiles = p.ntiles_dev ? *p.ntiles_dev : p.n_tiles;
         for (;;) {
             __syncthreads();
@@ -693,7 +803,7 @@ __global__ void __launch_bounds__((NW + NCONS) * 32, 1) dog_fused_kernel(const _
             tc.y1 = min(f.h, tc.y0 + bh);
             tc.blobs = p.blobs + f.blob_off;
             tc.count = p.count + lo;
-            process_tile<NW, BATCHED, PB, FULL>(p, sm, ss, tc);
+            process_tile<NW, MODE, BATCHED>(p, sm, ss, tc);
         }
         if (tid == 0) {
             __threadfence();
@@ -705,9 +815,9 @@ __global__ void __launch_bounds__((NW + NCONS) * 32, 1) dog_fused_kernel(const _
         }
     }
 
-    if (p.mode == MODE_SOFT || p.mode == MODE_BWD) {
+    if (SOFT) {
         __syncthreads();
-        if (p.mode == MODE_SOFT) {
+        if (MODE == MODE_SOFT) {
             for (int q = tid; q < p.nbins; q += NTHREADS)
                 if (ss.soft[q] != 0.0f) atomicAdd(&p.soft_out[q], ss.soft[q]);
         } else {
@@ -722,48 +832,39 @@ __global__ void __launch_bounds__((NW + NCONS) * 32, 1) dog_fused_kernel(const _
 // The dynamic shared-memory limit is raised once per device and kernel form
 // (not on every launch, so launches can be captured into CUDA graphs); atomic
 // because handles on other host threads launch the same forms.
-static std::atomic<int> g_smem_limit[64][16];
-
-template <int NW, bool BATCHED, int PB, bool FULL>
-static cudaError_t launch_form(const FusedParams& p, int grid, cudaStream_t s, std::atomic<int>* lim) {
-    if (lim->load(std::memory_order_acquire) < p.smem_bytes) {
-        cudaError_t e = cudaFuncSetAttribute(dog_fused_kernel<NW, BATCHED, PB, FULL>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem_bytes);
-        if (e != cudaSuccess) return e;
-        int cur = lim->load(std::memory_order_relaxed);
-        while (cur < p.smem_bytes && !lim->compare_exchange_weak(cur, p.smem_bytes)) {
-        }
-    }
-    dog_fused_kernel<NW, BATCHED, PB, FULL><<<grid, (NW + NCONS) * 32, p.smem_bytes, s>>>(p);
-    return cudaGetLastError();
-}
-
-template <int NW, bool BATCHED, int PB>
-static cudaError_t launch_bucket(const FusedParams& p, int grid, cudaStream_t s, std::atomic<int>* lim) {
-    return p.P == PB ? launch_form<NW, BATCHED, PB, true>(p, grid, s, lim + 1)
-                     : launch_form<NW, BATCHED, PB, false>(p, grid, s, lim);
-}
-
-// Plane-count buckets of the consumer's unrolled test: the smallest of 8, 16,
-// 24 and MAX_LEVELS - 1 that holds P; a ladder that fills its bucket exactly
-// runs a form without the masks of planes past the ladder.
-template <int NW, bool BATCHED>
-static cudaError_t launch_planes(const FusedParams& p, int grid, cudaStream_t s, std::atomic<int>* lim) {
-    if (p.P <= 8) return launch_bucket<NW, BATCHED, 8>(p, grid, s, lim + 0);
-    if (p.P <= 16) return launch_bucket<NW, BATCHED, 16>(p, grid, s, lim + 2);
-    if (p.P <= 24) return launch_bucket<NW, BATCHED, 24>(p, grid, s, lim + 4);
-    return launch_bucket<NW, BATCHED, MAX_LEVELS - 1>(p, grid, s, lim + 6);
-}
-
-// All forms of one producer-warp count (each translation unit instantiates one).
-template <int NW>
-static cudaError_t launch_fused_form(const FusedParams& p, int grid, cudaStream_t s) {
+template <int NW, int MODE, bool BATCHED>
+static cudaError_t launch_form(const FusedParams& p, int grid, cudaStream_t s) {
+    static std::atomic<int> limit[64];
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    std::atomic<int>* lim = g_smem_limit[dev & 63];
-    return p.frames != nullptr ? launch_planes<NW, true>(p, grid, s, lim + 8)
-                               : launch_planes<NW, false>(p, grid, s, lim);
+    std::atomic<int>& lim = limit[dev & 63];
+    if (lim.load(std::memory_order_acquire) < p.smem_bytes) {
+        e = cudaFuncSetAttribute(dog_fused_kernel<NW, MODE, BATCHED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 p.smem_bytes);
+        if (e != cudaSuccess) return e;
+        int cur = lim.load(std::memory_order_relaxed);
+        while (cur < p.smem_bytes && !lim.compare_exchange_weak(cur, p.smem_bytes)) {
+        }
+    }
+    dog_fused_kernel<NW, MODE, BATCHED><<<grid, NW * 32, p.smem_bytes, s>>>(p);
+    return cudaGetLastError();
 }
+
+// All forms of one warp count (each translation unit instantiates one).
+cudaError_t launch_fused_w12(const FusedParams& p, int grid, cudaStream_t s);
+cudaError_t launch_fused_w8(const FusedParams& p, int grid, cudaStream_t s);
+cudaError_t launch_fused_w4(const FusedParams& p, int grid, cudaStream_t s);
+cudaError_t launch_fused_w3(const FusedParams& p, int grid, cudaStream_t s);
+#define DOG_FUSED_FORMS(NW)                                                                       \
+    cudaError_t launch_fused_w##NW(const FusedParams& p, int grid, cudaStream_t s) {              \
+        if (p.frames != nullptr) return launch_form<NW, MODE_CANDIDATES, true>(p, grid, s);       \
+        switch (p.mode) {                                                                         \
+            case MODE_CANDIDATES: return launch_form<NW, MODE_CANDIDATES, false>(p, grid, s);     \
+            case MODE_DUMP: return launch_form<NW, MODE_DUMP, false>(p, grid, s);                 \
+            case MODE_SOFT: return launch_form<NW, MODE_SOFT, false>(p, grid, s);                 \
+            default: return launch_form<NW, MODE_BWD, false>(p, grid, s);                         \
+        }                                                                                         \
+    }
 
 }  // namespace dogk

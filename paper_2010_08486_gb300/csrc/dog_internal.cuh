@@ -12,22 +12,18 @@ namespace dogk {
 
 // ---- fused strip kernel geometry --------------------------------------------
 // A CTA owns a strip of TX output columns and walks down a band of rows in
-// blocks of MB rows.  Producer warps each own a fixed set of scale levels and
-// run the blur passes; NCONS consumer warps form the DoG and run the maximum
-// test one block behind.  The kernel comes in two forms: 12 producer warps at
-// 128 registers per thread, or 8 at 168 (both with the 4 consumer warps).
-// Which is faster depends on the ladder (the host picks one, the autotuner
-// times both); 10, 14 or 16 producer warps were slower than 12 on the
-// 25-level ladder (level balance, spills).
+// blocks of one 8-row chunk per warp, all warps on the same pair of scale
+// levels (dog_fused_forms.cuh).  Forms with 12, 8, 4 and 3 warps; the host picks
+// one per ladder (12 or 8; 4 or 3 for ladders whose shared memory needs it).
 constexpr int TX = 32;
-constexpr int MB = 8;
-constexpr int NWARPS = 12;                      // producer warps of the larger form (table sizes)
-constexpr int NCONS = 4;                        // consumer (DoG + test) warps, two rows each
-constexpr int RING_STRIDE = 32;    // floats per ring row (bank swizzle on row parity)
-constexpr int DSLOTS = 2 * MB + 2; // DoG-buffer rows: two blocks + 2 rows of history
+constexpr int MB = 8;                          // granularity of row bands
+constexpr int PAIR_STRIDE = 2 * TX;            // floats per row of a pair's horizontal sums
+constexpr int CHUNK = 8 * PAIR_STRIDE;         // 8 rows
 constexpr int MAX_LEVELS = DOG_MAX_LEVELS;
-static_assert(MB % NCONS == 0, "each consumer warp tests whole rows of a block");
-static_assert((NWARPS + NCONS) * 32 <= 1024, "one CTA");
+constexpr int MAX_PAIRS = MAX_LEVELS / 2;
+constexpr int CHUNK_TABLE = 32;                // entries of a pair's table of logical chunks
+constexpr int QUEUE_CAP = 64;                  // found maxima a warp queues before writing them out
+constexpr int MAX_TAPS4 = 4 * 160;             // float4 of tap blocks (8 taps of two levels each) of all pairs
 
 // Internal pixel type: 12-bit counts contrast stretched with per-frame limits
 // (the public types are DOG_DTYPE_F32 and DOG_DTYPE_U16).
@@ -44,12 +40,21 @@ enum FusedMode : int {
 struct LevelInfo {
     int r;          // kernel radius
     int tpad;       // taps rounded up to a multiple of 8: 8 ceil((2r+1)/8)
-    int e;          // chunks of MB rows the ring runs ahead: tpad / 8
-    int delta;      // MB*e - r: input-row lead of this level's horizontal pass
-    int ring_off;   // float offset of the ring in dynamic shared memory
-    int ring_rows;  // tpad + 8 (circular, used in blocks of 8 rows)
-    int woff;       // offset of this level's zero-padded full kernel (tpad floats), vertical pass
-    int hoff;       // offset of the horizontal pass's copy of the same taps
+    int woff;       // offset of this level's zero-padded full kernel (tpad floats) in the plain tap table
+};
+
+// Two adjacent levels blurred together (the two lanes of packed FMAs), in the
+// wider one's window; the narrower has `lead` zero taps before and after its
+// own.  A ladder with an odd number of levels starts with a pair whose first
+// level is absent (all taps zero).
+struct PairInfo {
+    int16_t r, lead;    // the window's radius; r minus the first level's radius
+    int16_t nb, tail;   // tap blocks of 8; tail: 2r + 1 = 8 nb + 1, one more tap after them
+    int16_t e;          // chunks of the ring: the rows above a block that the vertical pass reads (= nb)
+    int16_t delta;      // 8 e - r: lead of the horizontal pass's rows
+    int ring_off;       // float offset of the ring in dynamic shared memory
+    int tap;            // first tap (float4 index: two taps of both levels each)
+    unsigned rcp;       // ceil(2^32 / e), 0 for e = 1
 };
 
 // Candidate found at a strip edge whose 3x3x3 neighbourhood crosses into the
@@ -78,6 +83,7 @@ struct FusedParams {
     int n_strips, n_bands;
     int overlap;           // single frame: strips of TX columns step by TX - 2 from column -1, and
                            // only lanes 1 .. TX-2 own their voxels (no strip-edge queue)
+    int strip_step, strip_x0;  // single frame: strip s starts at column s strip_step + strip_x0
     // batched mode
     const FrameDesc* frames;
     int n_frames;
@@ -87,9 +93,9 @@ struct FusedParams {
     int* done_counter;
     // ladder
     int K, P, R;
-    const float* w;        // packed half kernels
-    const float* c;        // P normalisation coefficients
-    float thr;
+    const float* w;        // soft modes: taps in the layout of `taps`
+    const float* c;        // P normalisation coefficients, P plane sigmas
+    float thr, thr_up;     // threshold, and the smallest number above it
     int mode;
     // outputs
     dog_blob* blobs;
@@ -115,14 +121,19 @@ struct FusedParams {
     int* status;
     // shared-memory layout (floats)
     int in_off, in_rows, in_stride;
-    int d_off;
-    int w_off, w_total;
-    int dmin, dmax;
+    int w_off;             // the block's chunks: two halves of nw chunks
+    int x_off, e_off;      // rows handed to the warp below, and to the next block
+    int q_off;             // queues of found maxima
+    int c_off;             // chunk tables
+    int t_off, n_taps4;    // taps (soft modes: copied from w; other modes: the array below)
+    int dmin, dmax;        // smallest and largest delta of the pairs
     int smem_bytes;
-    int nw;                // producer warps of the kernel form (8 or 12)
-    int warp_nlev[NWARPS];
-    unsigned char warp_lev[NWARPS][MAX_LEVELS];
-    LevelInfo lv[MAX_LEVELS];
+    int nw;                // warps of the kernel form (12, 8, 4 or 3)
+    int n_pairs;
+    int lev_off;           // 1: the first pair's first level is absent
+    float cn[MAX_LEVELS];  // P normalisation coefficients (as c)
+    PairInfo pairs[MAX_PAIRS];
+    float4 taps[MAX_TAPS4];
 };
 
 struct ResolveParams {

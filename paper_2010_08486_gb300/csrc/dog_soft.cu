@@ -36,14 +36,20 @@ const std::vector<int>& handle_radii(const dog_handle* h);
 const std::vector<double>& handle_sigmas(const dog_handle* h);
 const dog_config& handle_cfg(const dog_handle* h);
 int handle_band(const dog_handle* h);
+int handle_w_total(const dog_handle* h);
+int handle_sms(const dog_handle* h);
+int pick_band(const FusedParams& b, int num_sms, int H, int n_strips, int asked);
+const std::vector<LevelInfo>& handle_levels(const dog_handle* h);
+void handle_tap_slot(const dog_handle* h, int i, int* base, int* lead);
 int* handle_status(dog_handle* h);
 void*& handle_soft_ws(dog_handle* h);
 cudaError_t timed_fused(dog_handle* h, const FusedParams& p, int grid, cudaStream_t s);
 
 struct SoftWS {
     int H = 0, W = 0;
-    float* w = nullptr;       // half kernels from the device sigmas
+    float* w = nullptr;       // taps from the device sigmas, plain table
     float* dw = nullptr;      // their derivative wrt sigma
+    float* wp = nullptr;      // the taps in the fused kernel's pair layout
     float* c = nullptr;       // P coefficients then P sigmas
     float* kappa = nullptr;   // P x nbins
     float* dkappa = nullptr;  // P x nbins
@@ -63,7 +69,7 @@ struct SoftWS {
 void soft_free(dog_handle* h) {
     SoftWS* ws = static_cast<SoftWS*>(handle_soft_ws(h));
     if (!ws) return;
-    void* ptrs[] = {ws->w, ws->dw, ws->c, ws->kappa, ws->dkappa, ws->pend, ws->counts, ws->A, ws->Y, ws->Yd, ws->acc,
+    void* ptrs[] = {ws->w, ws->dw, ws->wp, ws->c, ws->kappa, ws->dkappa, ws->pend, ws->counts, ws->A, ws->Y, ws->Yd, ws->acc,
                     ws->last_sig, ws->big, ws->big_count};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -84,8 +90,10 @@ static int soft_ws(dog_handle* h, int H, int W, SoftWS** out) {
     ws->pend_cap = (int)std::min<size_t>((size_t)2 * strips * P * H + 1024, (size_t)1 << 28);
     cudaError_t e = cudaSuccess;
     auto ok = [&](cudaError_t x) { if (e == cudaSuccess) e = x; };
-    ok(cudaMalloc(&ws->w, sizeof(float) * b.w_total));
-    ok(cudaMalloc(&ws->dw, sizeof(float) * b.w_total));
+    ok(cudaMalloc(&ws->w, sizeof(float) * handle_w_total(h)));
+    ok(cudaMalloc(&ws->dw, sizeof(float) * handle_w_total(h)));
+    ok(cudaMalloc(&ws->wp, sizeof(float4) * b.n_taps4));
+    if (e == cudaSuccess) ok(cudaMemset(ws->wp, 0, sizeof(float4) * b.n_taps4));   // padding taps stay zero
     ok(cudaMalloc(&ws->c, sizeof(float) * 2 * P));
     ok(cudaMalloc(&ws->kappa, sizeof(float) * P * nb));
     ok(cudaMalloc(&ws->dkappa, sizeof(float) * P * nb));
@@ -117,10 +125,11 @@ struct SoftPrep {
     int r[MAX_LEVELS];
     int woff[MAX_LEVELS];
     int tpad[MAX_LEVELS];
-    int hoff[MAX_LEVELS];    // the horizontal pass's copy of the taps
+    int pbase[MAX_LEVELS], plead[MAX_LEVELS];   // place of the level's taps in the pair table
     double lref0, lrefP;   // ln sigma of the reference ladder's first / last DoG plane
     float* w;
     float* dw;
+    float* wp;
     float* c;
     float* kappa;
     float* dkappa;
@@ -162,7 +171,7 @@ __global__ void __launch_bounds__(PREP_THREADS) soft_prep_kernel(const __grid_co
             }
             p.w[p.woff[i] + t] = wv;
             p.dw[p.woff[i] + t] = dv;
-            p.w[p.hoff[i] + t] = wv;
+            if (t <= 2 * r) p.wp[p.pbase[i] + 2 * (t + p.plead[i])] = wv;
         }
     }
     for (int l = threadIdx.x; l < p.P; l += blockDim.x) {
@@ -194,15 +203,16 @@ static SoftPrep prep_params(dog_handle* h, SoftWS* ws, const float* sig) {
     q.nbins = handle_cfg(h).nbins;
     q.norm = handle_cfg(h).norm;
     for (int i = 0; i < b.K; ++i) {
-        q.r[i] = b.lv[i].r;
-        q.woff[i] = b.lv[i].woff;
-        q.tpad[i] = b.lv[i].tpad;
-        q.hoff[i] = b.lv[i].hoff;
+        q.r[i] = handle_levels(h)[i].r;
+        q.woff[i] = handle_levels(h)[i].woff;
+        q.tpad[i] = handle_levels(h)[i].tpad;
+        handle_tap_slot(h, i, &q.pbase[i], &q.plead[i]);
     }
     q.lref0 = std::log(ref[0]);
     q.lrefP = std::log(ref[b.P - 1]);
     q.w = ws->w;
     q.dw = ws->dw;
+    q.wp = ws->wp;
     q.c = ws->c;
     q.kappa = ws->kappa;
     q.dkappa = ws->dkappa;
@@ -217,17 +227,18 @@ static FusedParams soft_fused(dog_handle* h, SoftWS* ws, const float* img, int H
     p.H = H;
     p.W = W;
     p.pitch = pitch;
-    const int band = handle_band(h);
-    p.band = (band > 0 && band < H) ? band : ((H + MB - 1) / MB) * MB;
     // overlapping strips (32 columns stepping by 30): every local maximum is
     // settled inside the fused kernel, so no strip-edge resolve follows (the
     // soft modes keep every maximum, thousands per frame at strip edges)
     p.overlap = 1;
+    p.strip_step = TX - 2;
+    p.strip_x0 = -1;
     p.n_strips = (W + TX - 2 - 1) / (TX - 2);
+    p.band = pick_band(p, handle_sms(h), H, p.n_strips, std::min(handle_band(h), H));
     p.n_bands = (H + p.band - 1) / p.band;
     p.frames = nullptr;
     p.mode = mode;
-    p.w = ws->w;
+    p.w = ws->wp;
     p.c = ws->c;
     p.pend = ws->pend;
     p.pend_cap = ws->pend_cap;
@@ -1006,8 +1017,8 @@ int soft_backward_rec(dog_handle* h, const float* img, int H, int W, int pitch, 
     g.H = H;
     g.W = W;
     for (int i = 0; i < K; ++i) {
-        g.r[i] = b.lv[i].r;
-        g.woff[i] = b.lv[i].woff;
+        g.r[i] = handle_levels(h)[i].r;
+        g.woff[i] = handle_levels(h)[i].woff;
     }
     g.dw_acc = ws->acc + 2 * P;
     g.big = ws->big;
@@ -1040,10 +1051,10 @@ static int adjoint_tail(dog_handle* h, SoftWS* ws, const SoftPrep& q, const floa
     a.dw = ws->dw;
     int tpad_max = 8;
     for (int i = 0; i < K; ++i) {
-        a.r[i] = b.lv[i].r;
-        a.tpad[i] = b.lv[i].tpad;
-        a.woff[i] = b.lv[i].woff;
-        tpad_max = std::max(tpad_max, b.lv[i].tpad);
+        a.r[i] = handle_levels(h)[i].r;
+        a.tpad[i] = handle_levels(h)[i].tpad;
+        a.woff[i] = handle_levels(h)[i].woff;
+        tpad_max = std::max(tpad_max, handle_levels(h)[i].tpad);
     }
     a.R = b.R;
     a.dw_acc = ws->acc + 2 * P;

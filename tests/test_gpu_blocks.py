@@ -1,0 +1,65 @@
+"""The fused kernel at the edges of its blocks and forms: heights around
+multiples of a block's rows, ladders that only the small forms hold, and frames
+with non-finite pixels, against the FP64 oracle."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2010_08486_gb300 import build as libbuild
+from paper_2010_08486_gb300 import dog, synth
+from tests.test_gpu_detect import dev, full_check
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    libbuild.build()
+
+
+@pytest.mark.parametrize("warps", [8, 12])
+@pytest.mark.parametrize("h", [63, 64, 65, 95, 96, 97, 129, 193])
+def test_heights_around_a_block(h, warps):
+    cfg = dog.plif_config(max_h=h, max_w=40)
+    det = dog.Detector(cfg)
+    det.set_producer_warps(warps)
+    full_check(cfg, synth.plif_frame(synth.PLIF_SEED_BASE + h, h, 40), det=det)
+    det.set_tiling(56)   # bands whose rows end inside a block, and a short last one
+    full_check(cfg, synth.plif_frame(synth.PLIF_SEED_BASE + h, h, 40), det=det)
+
+
+# radii that leave room for four warps, and for three (odd and even ladders)
+@pytest.mark.parametrize("radii", [[54, 54, 54, 54, 55, 55, 55, 55, 55, 55],
+                                   [48, 49, 50, 52, 53, 54, 56, 57, 58, 59, 61]])
+def test_ladders_of_the_small_forms(radii):
+    sig = [(r + 0.02 * i) / 4.0 for i, r in enumerate(radii)]
+    cfg = dog.DetectorConfig(sigmas=sig, threshold=0.02, max_h=150, max_w=70, norm=1)
+    det = dog.Detector(cfg)
+    assert det.radii == radii
+    full_check(cfg, synth.plif_frame(synth.PLIF_SEED_BASE + 3, 150, 70), det=det)
+
+
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("at", [(70, 40), (3, 31), (139, 0)])
+def test_non_finite_pixel_reaches_each_level_by_its_own_radius(bad, at):
+    """A plane's response is non-finite within the radius of its wider level
+    around the pixel (in both axes) and elsewhere bit for bit that of the frame
+    without it, whichever levels are blurred together."""
+    h, w = 140, 96
+    cfg = dog.plif_config(max_h=h, max_w=w)
+    det = dog.Detector(cfg)
+    clean = synth.plif_frame(synth.PLIF_SEED_BASE + 5, h, w)
+    img = clean.copy()
+    img[at] = bad
+    D0 = det.debug_dog(dev(clean)).cpu().numpy()
+    D1 = det.debug_dog(dev(img)).cpu().numpy()
+    dy = np.abs(np.arange(h) - at[0])[:, None]
+    dx = np.abs(np.arange(w) - at[1])[None, :]
+    for l in range(det.P):
+        r = det.radii[l + 1]
+        near = (dy <= r) & (dx <= r)
+        assert not np.isfinite(D1[l][near]).any()
+        np.testing.assert_array_equal(D1[l][~near], D0[l][~near])
+    blobs, hist, _ = det.detect(dev(img))
+    torch.cuda.synchronize()
+    assert det.status() == 0 and int(hist.sum()) == blobs.n()
