@@ -21,6 +21,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <climits>
 
 #include "dog_internal.cuh"
 
@@ -30,9 +31,10 @@ namespace dogk {
 // plane's single-precision sigma takes its plane's precomputed bin; another
 // sigma (a coalesced mean) is binned by log volume (LOGV) or by the nearest
 // ladder radius in log space (LADDER).
-__device__ __forceinline__ int hist_bin(const dog_blob& b, const HistParams& p) {
+__device__ __forceinline__ int hist_bin(const dog_blob& b, const HistParams& p, const float* sig_f,
+                                        const int* level_bin) {
     const int l = min(max(b.level, 0), p.P - 1);
-    if (b.sigma == p.sig_f[l]) return p.level_bin[l];
+    if (b.sigma == sig_f[l]) return level_bin[l];
     if (p.mode == DOG_HIST_LADDER) {
         const double ls = log((double)b.sigma);
         int best = 0;
@@ -44,6 +46,16 @@ __device__ __forceinline__ int hist_bin(const dog_blob& b, const HistParams& p) 
         return best;
     }
     const double span = p.log_hi - p.log_lo;
+    // single precision decides away from the bin edges: |ln sigma| of a positive
+    // float is below 104, logf is off by less than 1e-6 of it and so are the
+    // subtraction and the product, so t32 is within `off` of the position in
+    // double precision (whose logarithm is for the few blobs next to an edge)
+    if (p.P >= 2 && span > 0.0 && b.sigma > 0.0f && b.sigma < INFINITY) {
+        const float inv = (float)((double)p.nbins / span), lo = (float)p.log_lo;
+        const float t32 = (logf(b.sigma) - lo) * inv, off = 1e-5f * (104.0f + fabsf(lo)) * inv;
+        const float fl = floorf(t32);
+        if (t32 - fl > off && fl + 1.0f - t32 > off) return (int)fminf(fmaxf(fl, 0.0f), (float)(p.nbins - 1));
+    }
     const double t = (p.P >= 2 && span > 0.0) ? (log((double)b.sigma) - p.log_lo) / span : 0.0;
     double fb = floor((double)p.nbins * t);
     fb = fmin(fmax(fb, 0.0), (double)(p.nbins - 1));
@@ -74,9 +86,10 @@ __device__ __forceinline__ unsigned bucket_of(int cx, int cy) {
 }
 
 struct PruneSmem {
-    int bcount[NBUCKET];
-    int boff[NBUCKET + 1];
+    alignas(16) int bcount[NBUCKET];
+    alignas(16) int boff[NBUCKET + 1];
     int d2[MAX_LEVELS * MAX_LEVELS];
+    int wsum[32];
     int changed;
     int scan_carry;
 };
@@ -107,7 +120,7 @@ __device__ void frame_hist(const PruneParams& p, PruneSmem& s, const dog_blob* o
     const int nout = min(p.out_count[f], p.cap_out);
     for (int i = tid; i < nout; i += PRUNE_THREADS) {
         const dog_blob b = out[i];
-        const int bin = hist_bin(b, hp);
+        const int bin = hist_bin(b, hp, hp.sig_f, hp.level_bin);
         atomicAdd(&hc[bin], 1u);
         if (hp.vol) atomicAdd(&hv[bin], blob_volume(b.sigma));
     }
@@ -118,11 +131,290 @@ __device__ void frame_hist(const PruneParams& p, PruneSmem& s, const dog_blob* o
     }
 }
 
-// Frames with at most PRUNE_SMEM_CAND candidates run every pass on
-// shared-memory copies of the candidates and the per-candidate arrays
-// (dynamic shared memory, PRUNE_DYN_BYTES); larger ones work in global memory.
+// Exclusive scan of the NBUCKET counts in s.bcount into s.boff (s.boff[NBUCKET]
+// the total): four buckets per thread.
+static_assert(NBUCKET == 4 * PRUNE_THREADS, "four buckets per thread");
+__device__ __forceinline__ void scan_buckets(PruneSmem& s) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int4 c = reinterpret_cast<const int4*>(s.bcount)[tid];
+    const int v = c.x + c.y + c.z + c.w;
+    int x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) s.wsum[warp] = x;
+    __syncthreads();
+    if (warp == 0) {
+        int t = s.wsum[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, t, o);
+            if (lane >= o) t += y;
+        }
+        s.wsum[lane] = t;
+    }
+    __syncthreads();
+    const int e = x - v + (warp > 0 ? s.wsum[warp - 1] : 0);
+    reinterpret_cast<int4*>(s.boff)[tid] = make_int4(e, e + c.x, e + c.x + c.y, e + c.x + c.y + c.z);
+    if (tid == PRUNE_THREADS - 1) s.boff[NBUCKET] = e + v;
+}
+
+// Frames with at most PRUNE_SMEM_CAND candidates run in shared memory; larger
+// ones work in global memory.
 constexpr int PRUNE_SMEM_CAND = 4096;
-constexpr int PRUNE_DYN_BYTES = PRUNE_SMEM_CAND * ((int)sizeof(dog_blob) + 3 * (int)sizeof(int));
+constexpr int EDGE_WARP = 640;   // conflicts one warp may list
+
+// Shared memory of the frames that fit: the candidates in the order of a grid
+// of cells, so that a row of three cells is one contiguous range.
+struct CellSmem {
+    double hv[DOG_MAX_NBINS], sig[MAX_LEVELS];
+    float sig_f[MAX_LEVELS];
+    int level_bin[MAX_LEVELS];
+    int x[PRUNE_SMEM_CAND], y[PRUNE_SMEM_CAND], level[PRUNE_SMEM_CAND];
+    float resp[PRUNE_SMEM_CAND];
+    int target[PRUNE_SMEM_CAND];
+    unsigned hc[DOG_MAX_NBINS];
+    unsigned char state[PRUNE_SMEM_CAND], in[PRUNE_SMEM_CAND], und[PRUNE_SMEM_CAND];
+    union {   // the edges are gone when the members come
+        unsigned edge[PRUNE_THREADS / 32 * EDGE_WARP];
+        unsigned short member[PRUNE_SMEM_CAND];
+    };
+    int box[4];   // smallest and largest x and y
+
+    __device__ __forceinline__ bool before(int a, int b) const {   // higher(), by place
+        if (resp[a] != resp[b]) return resp[a] > resp[b];
+        if (level[a] != level[b]) return level[a] < level[b];
+        if (y[a] != y[b]) return y[a] < y[b];
+        return x[a] < x[b];
+    }
+};
+constexpr int PRUNE_OLD_BYTES = PRUNE_SMEM_CAND * ((int)sizeof(dog_blob) + 3 * (int)sizeof(int));
+constexpr int PRUNE_DYN_BYTES = (int)sizeof(CellSmem) > PRUNE_OLD_BYTES ? (int)sizeof(CellSmem) : PRUNE_OLD_BYTES;
+static_assert(PRUNE_DYN_BYTES + (int)sizeof(PruneSmem) <= 226 * 1024, "shared memory of one CTA");
+
+// Pruning and histogram of one frame in shared memory.  One thread per
+// candidate walking its nine hashed cells, once a round and once per group
+// member, is a chain of dependent loads as long as the fullest cell among 32
+// lanes, and the histogram's passes over global memory come on top (69 us for
+// the 1,700 candidates of a 1024 x 1024 frame).  Here the candidates are copied
+// in the order of a plain grid, the conflicts (few: 2 to 5% of the candidates on
+// PLIF frames) are listed once as edges (candidate, higher-priority neighbour),
+// the rounds, targets and members run over the edges, and the accepted blobs are
+// binned as they are written.  (Sorting by priority instead, so that it becomes
+// an integer comparison, took 17 us for the sort alone.)  Returns false, having
+// written nothing, when a warp finds more than EDGE_WARP conflicts.
+__device__ __forceinline__ bool prune_cells(const PruneParams& p, PruneSmem& s, CellSmem& r, const dog_blob* cand,
+                                            int n, dog_blob* out, int f) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    const HistParams& hp = p.hist;
+    const int nbo = hp.hist ? (hp.mode == DOG_HIST_LADDER ? hp.P : hp.nbins) : 0;
+    for (int q = tid; q < NBUCKET; q += PRUNE_THREADS) s.bcount[q] = 0;
+    for (int q = tid; q < p.P * p.P; q += PRUNE_THREADS) s.d2[q] = p.d2thr[q];
+    for (int q = tid; q < p.P; q += PRUNE_THREADS) {
+        r.sig[q] = p.sig[q];
+        r.sig_f[q] = hp.hist ? hp.sig_f[q] : 0.0f;
+        r.level_bin[q] = hp.hist ? hp.level_bin[q] : 0;
+    }
+    for (int q = tid; q < nbo; q += PRUNE_THREADS) { r.hc[q] = 0u; r.hv[q] = 0.0; }
+    if (tid < 4) r.box[tid] = tid & 1 ? INT_MIN : INT_MAX;
+    // this thread's candidates: tid, tid + 1024, ...
+    constexpr int PER = PRUNE_SMEM_CAND / PRUNE_THREADS;
+    dog_blob mine[PER];
+    int bk[PER];
+    int x0 = INT_MAX, x1 = INT_MIN, y0 = INT_MAX, y1 = INT_MIN;
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        const int i = tid + u * PRUNE_THREADS;
+        if (i < n) {
+            mine[u] = cand[i];
+            x0 = min(x0, mine[u].x); x1 = max(x1, mine[u].x);
+            y0 = min(y0, mine[u].y); y1 = max(y1, mine[u].y);
+        }
+    }
+    x0 = __reduce_min_sync(0xffffffffu, x0); x1 = __reduce_max_sync(0xffffffffu, x1);
+    y0 = __reduce_min_sync(0xffffffffu, y0); y1 = __reduce_max_sync(0xffffffffu, y1);
+    __syncthreads();
+    if (lane == 0) {
+        atomicMin(&r.box[0], x0); atomicMax(&r.box[1], x1);
+        atomicMin(&r.box[2], y0); atomicMax(&r.box[3], y1);
+    }
+    __syncthreads();
+    // the grid: cells of at least the largest conflict distance, at most NBUCKET
+    // of them with a margin of one column on either side
+    const long long ox = r.box[0], oy = r.box[2];
+    const long long wx = n ? r.box[1] - ox : 0, wy = n ? r.box[3] - oy : 0;
+    long long cell = p.cell;
+    while ((wx / cell + 3) * (wy / cell + 1) > NBUCKET) cell *= 2;
+    const int nx = (int)(wx / cell) + 3, ny = (int)(wy / cell) + 1;
+    const unsigned uc = (unsigned)cell;   // (at most the extent, below 2^32)
+#pragma unroll
+    for (int u = 0; u < PER; ++u)
+        if (tid + u * PRUNE_THREADS < n) {
+            bk[u] = (int)((unsigned)(mine[u].y - oy) / uc) * nx + (int)((unsigned)(mine[u].x - ox) / uc) + 1;
+            atomicAdd(&s.bcount[bk[u]], 1);
+        }
+    __syncthreads();
+    scan_buckets(s);
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < PER; ++u)
+        if (tid + u * PRUNE_THREADS < n) {
+            const int at = s.boff[bk[u]] + atomicSub(&s.bcount[bk[u]], 1) - 1;
+            r.x[at] = mine[u].x;
+            r.y[at] = mine[u].y;
+            r.level[at] = mine[u].level;
+            r.resp[at] = mine[u].response;
+            r.target[at] = -1;
+            r.state[at] = ST_UND;
+            r.in[at] = 0;
+            r.und[at] = 0;
+        }
+    __syncthreads();
+    // edges: candidate i and row of cells dy per thread; every warp fills and
+    // later reads its own part of the list (hits are rare, so they may diverge)
+    unsigned* edge = r.edge + (tid >> 5) * EDGE_WARP;
+    int* n_edge = &s.wsum[tid >> 5];
+    if (lane == 0) *n_edge = 0;
+    __syncwarp();
+    const int reach = p.cell < 46340 ? p.cell * p.cell : INT_MAX;   // no smaller than any conflict distance squared
+    for (int t = tid; t < 3 * n; t += PRUNE_THREADS) {
+        const int i = t / 3, cy0 = t - 3 * i - 1;
+        const int xi = r.x[i], yi = r.y[i];
+        const int cy = (int)((unsigned)(yi - oy) / uc) + cy0, cx = (int)((unsigned)(xi - ox) / uc) + 1;
+        if (cy < 0 || cy >= ny) continue;
+        const int end = s.boff[cy * nx + cx + 2];
+        for (int k = s.boff[cy * nx + cx - 1]; k < end; ++k) {
+            const int ex = r.x[k] - xi, ey = r.y[k] - yi, d = ex * ex + ey * ey;
+            if (d >= reach || k == i) continue;
+            const int li = min(max(r.level[i], 0), p.P - 1), lk = min(max(r.level[k], 0), p.P - 1);
+            if (d >= s.d2[li * p.P + lk] || !r.before(k, i)) continue;
+            const int e = atomicAdd(n_edge, 1);
+            if (e < EDGE_WARP) edge[e] = (unsigned)i << 16 | (unsigned)k;
+        }
+    }
+    __syncwarp();
+    const int ne = *n_edge;
+    if (__syncthreads_or(ne > EDGE_WARP)) return false;
+    // rounds of the independent-set rule
+    for (;;) {
+        for (int e = lane; e < ne; e += 32) {
+            const int i = edge[e] >> 16;
+            if (r.state[i] != ST_UND) continue;
+            const int st = r.state[edge[e] & 0xffffu];
+            if (st == ST_IN) r.in[i] = 1;
+            else if (st == ST_UND) r.und[i] = 1;
+        }
+        __syncthreads();
+        bool wait = false;
+        for (int i = tid; i < n; i += PRUNE_THREADS) {
+            if (r.state[i] != ST_UND) continue;
+            if (r.in[i] || !r.und[i]) r.state[i] = r.in[i] ? ST_OUT : ST_IN;
+            else wait = true;
+            r.und[i] = 0;
+        }
+        if (!__syncthreads_or(wait)) break;   // (each round settles the first undecided)
+    }
+    // every rejected candidate joins its highest-priority accepted neighbour
+    bool any = false;
+    for (int e = lane; e < ne; e += 32) {
+        const int i = edge[e] >> 16, j = edge[e] & 0xffffu;
+        if (r.state[i] != ST_OUT || r.state[j] != ST_IN) continue;
+        any = true;
+        int seen = r.target[i];
+        while (seen < 0 || r.before(j, seen)) {
+            const int now = atomicCAS(&r.target[i], seen, j);
+            if (now == seen) break;
+            seen = now;
+        }
+    }
+    // members of every accepted candidate (the edges are no longer needed)
+    const bool groups = __syncthreads_or(any) && p.mode == DOG_PRUNE_COALESCE;
+    if (groups) {
+        for (int q = tid; q < NBUCKET; q += PRUNE_THREADS) s.bcount[q] = 0;
+        __syncthreads();
+        for (int i = tid; i < n; i += PRUNE_THREADS)
+            if (r.state[i] == ST_OUT) atomicAdd(&s.bcount[r.target[i]], 1);
+        __syncthreads();
+        scan_buckets(s);
+        __syncthreads();
+        for (int i = tid; i < n; i += PRUNE_THREADS)
+            if (r.state[i] == ST_OUT) {
+                const int t = r.target[i];
+                r.member[s.boff[t] + atomicSub(&s.bcount[t], 1) - 1] = (unsigned short)i;
+            }
+    }
+    if (tid == 0) s.scan_carry = s.changed = 0;
+    __syncthreads();
+    // accepted blobs: compaction and bin
+    auto emit = [&](int a, int idx, float sigma) {
+        dog_blob o;
+        o.x = r.x[a];
+        o.y = r.y[a];
+        o.level = r.level[a];
+        o.sigma = sigma;
+        o.response = r.resp[a];
+        if (idx < p.cap_out) {
+            out[idx] = o;
+            if (nbo) {
+                const int bin = hist_bin(o, hp, r.sig_f, r.level_bin);
+                atomicAdd(&r.hc[bin], 1u);
+                if (hp.vol) atomicAdd(&r.hv[bin], blob_volume(sigma));
+            }
+        } else {
+            atomicCAS(p.status, 0, (int)DOG_ERR_CAPACITY);
+        }
+    };
+    for (int a0 = tid & ~31; a0 < n; a0 += PRUNE_THREADS) {
+        const int a = a0 + lane;
+        const bool acc = a < n && r.state[a] == ST_IN;
+        const bool alone = acc && !(groups && s.boff[a + 1] > s.boff[a]);
+        const unsigned m = __ballot_sync(0xffffffffu, alone), g = __ballot_sync(0xffffffffu, acc && !alone);
+        int idx = 0, gi = 0;
+        if (lane == 0 && m) idx = atomicAdd(&s.scan_carry, __popc(m));
+        if (lane == 0 && g) gi = atomicAdd(&s.changed, __popc(g));
+        idx = __shfl_sync(0xffffffffu, idx, 0) + __popc(m & ((1u << lane) - 1u));
+        gi = __shfl_sync(0xffffffffu, gi, 0) + __popc(g & ((1u << lane) - 1u));
+        if (alone) emit(a, idx, (float)r.sig[min(max(r.level[a], 0), p.P - 1)]);
+        else if (acc) r.target[gi] = a;   // (targets are in the member lists now)
+    }
+    if (groups) {
+        // groups: mean sigma summed in visiting order.  Gathered in a list, so that
+        // the double-precision instructions (two lanes a cycle and SM) run in few
+        // full warps and not in every warp that has a group
+        __syncthreads();
+        const int ng = s.changed, first = s.scan_carry;
+        for (int q = tid; q < ng; q += PRUNE_THREADS) {
+            const int a = r.target[q];
+            const int m0 = s.boff[a], m1 = s.boff[a + 1];
+            for (int u = m0 + 1; u < m1; ++u) {   // by priority (few members)
+                const unsigned short v = r.member[u];
+                int w = u;
+                for (; w > m0 && r.before(v, r.member[w - 1]); --w) r.member[w] = r.member[w - 1];
+                r.member[w] = v;
+            }
+            const int la = min(max(r.level[a], 0), p.P - 1);
+            double sum = r.sig[la];
+            bool mixed = false;
+            for (int u = m0; u < m1; ++u) {
+                const int lv = r.level[r.member[u]];
+                sum += r.sig[min(max(lv, 0), p.P - 1)];
+                mixed |= lv != r.level[a];
+            }
+            emit(a, first + q, mixed ? (float)(sum / (double)(1 + m1 - m0)) : (float)r.sig[la]);
+        }
+        __syncthreads();
+        if (tid == 0) s.scan_carry += ng;
+    }
+    __syncthreads();
+    if (tid == 0) p.out_count[f] = s.scan_carry;
+    for (int q = tid; q < nbo; q += PRUNE_THREADS) {
+        hp.hist[(size_t)f * nbo + q] = r.hc[q];
+        if (hp.vol) hp.vol[(size_t)f * nbo + q] = r.hv[q];
+    }
+    return true;
+}
 
 __global__ void __launch_bounds__(PRUNE_THREADS) dog_prune_kernel(const __grid_constant__ PruneParams p) {
     __shared__ PruneSmem s;
@@ -138,6 +430,8 @@ __global__ void __launch_bounds__(PRUNE_THREADS) dog_prune_kernel(const __grid_c
     dog_blob* out = p.out + ooff;
     const int n = min(p.cand_count[f], p.cap_in);
     if (n <= PRUNE_SMEM_CAND && p.mode != DOG_PRUNE_OFF) {
+        if (prune_cells(p, s, *reinterpret_cast<CellSmem*>(prune_dyn), cand, n, out, f)) return;
+        __syncthreads();
         dog_blob* sc = reinterpret_cast<dog_blob*>(prune_dyn);
         int* si = reinterpret_cast<int*>(sc + PRUNE_SMEM_CAND);
         for (int i = tid; i < n; i += PRUNE_THREADS) sc[i] = cand[i];
@@ -162,7 +456,7 @@ __global__ void __launch_bounds__(PRUNE_THREADS) dog_prune_kernel(const __grid_c
 
     for (int q = tid; q < NBUCKET; q += PRUNE_THREADS) s.bcount[q] = 0;
     for (int q = tid; q < p.P * p.P; q += PRUNE_THREADS) s.d2[q] = p.d2thr[q];
-    if (tid == 0) { s.scan_carry = 0; p.out_count[f] = 0; }
+    if (tid == 0) p.out_count[f] = 0;
     __syncthreads();
     const int cell = p.cell;
 
@@ -175,37 +469,8 @@ __global__ void __launch_bounds__(PRUNE_THREADS) dog_prune_kernel(const __grid_c
         state[i] = ST_UND;
     }
     __syncthreads();
-    // exclusive scan of the bucket counts (4 per thread, sequential carry across chunks)
-    for (int base = 0; base < NBUCKET; base += PRUNE_THREADS) {
-        const int v = s.bcount[base + tid];
-        int x = v;
-        // warp inclusive scan
-        const int lane = tid & 31, warp = tid >> 5;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        __shared__ int wsum[32];
-        if (lane == 31) wsum[warp] = x;
-        __syncthreads();
-        if (warp == 0) {
-            int t = wsum[lane];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, t, o);
-                if (lane >= o) t += y;
-            }
-            wsum[lane] = t;
-        }
-        __syncthreads();
-        const int incl = x + (warp > 0 ? wsum[warp - 1] : 0);
-        s.boff[base + tid] = s.scan_carry + incl - v;
-        __syncthreads();
-        if (tid == PRUNE_THREADS - 1) s.scan_carry += incl;
-        __syncthreads();
-    }
-    if (tid == 0) s.boff[NBUCKET] = s.scan_carry;
+    scan_buckets(s);
+    __syncthreads();
     for (int q = tid; q < NBUCKET; q += PRUNE_THREADS) s.bcount[q] = 0;
     __syncthreads();
     for (int i = tid; i < n; i += PRUNE_THREADS) {
@@ -349,7 +614,7 @@ __global__ void __launch_bounds__(256) dog_hist_kernel(const __grid_constant__ H
     const int n = min(p.count[f], p.cap);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const dog_blob b = p.blobs[off + i];
-        const int bin = hist_bin(b, p);
+        const int bin = hist_bin(b, p, p.sig_f, p.level_bin);
         atomicAdd(&hc[bin], 1u);
         if (p.vol) atomicAdd(&hv[bin], blob_volume(b.sigma));
     }

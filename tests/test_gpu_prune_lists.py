@@ -1,0 +1,42 @@
+"""Pruning of given candidate lists against the oracle's greedy pruning: list
+lengths around the shared-memory limit, sparse lists, lists so dense that the
+conflict list overflows, and equal responses."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2010_08486_gb300 import _lib, build as libbuild, dog
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    libbuild.build()
+
+
+@pytest.mark.parametrize("mode", [_lib.PRUNE_COALESCE, _lib.PRUNE_SUPPRESS])
+@pytest.mark.parametrize("n,size", [(0, 9), (1, 9), (33, 40), (900, 24), (1500, 300), (3000, 150), (4095, 2000),
+                                    (4096, 900), (4097, 900)])
+def test_prune_of_a_list(n, size, mode):
+    rng = np.random.default_rng(1000 * n + size)
+    cfg = dog.plif_config(max_h=2048, max_w=2048, blob_cap=8192, prune=mode)
+    det = dog.Detector(cfg)
+    # distinct (x, y, level), in any order; responses in few values, so that ties are many
+    cells = rng.choice(size * size * det.P, size=n, replace=False)
+    level, pos = cells % det.P, cells // det.P
+    x, y = pos % size, pos // size
+    resp = (rng.integers(1, 40, n) / 64.0).astype(np.float32)
+    sig = np.asarray(det.sigmas, np.float32)[level]
+    raw = np.zeros((8192, 5), np.int32)
+    raw[:n, 0], raw[:n, 1], raw[:n, 2] = x, y, level
+    raw[:n, 3], raw[:n, 4] = sig.view(np.int32), resp.view(np.int32)
+    cand = dog.BlobList(torch.from_numpy(raw).cuda(), torch.tensor(n, dtype=torch.int32, device="cuda"))
+    out = det.prune(cand, 2048, 2048)
+    torch.cuda.synchronize()
+    want = oracle.prune(parity.blobs_to_oracle(x, y, level, sig, resp), parity.oracle_params(cfg))
+    want.sigma = want.sigma.astype(np.float32).astype(np.float64)
+    assert parity.same_blob_sets(parity.blobs_to_oracle(*out.to_numpy()), want)
+    assert det.status() == 0
