@@ -1,0 +1,33 @@
+"""Rendered counts where single precision cannot decide them, and tiles cut at
+every side, against the CPU restatement bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2010_08486_gb300 import build as libbuild
+from paper_2010_08486_gb300 import dog, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    libbuild.build()
+
+
+@pytest.mark.parametrize("h,w,n,bg,gain,rn", [
+    (31, 33, 9, 0.05, 2000.0, 4.0), (32, 15, 3, 0.05, 2000.0, 4.0), (1, 65, 5, 0.1, 3.7, 0.0),
+    (34, 17, 400, 0.02, 900.0, 4.0),          # more spheres than one scan of the table
+    (64, 64, 0, 0.0, 4096.0, 0.0),            # every value exactly on an edge (0.5 above a whole number)
+    (64, 64, 0, 0.25, 1.0e-3, 0.0), (64, 64, 0, 1.0, 4000.5, 1.0e-6), (64, 64, 4, 0.5, 1.0e30, 2.0),
+    (64, 64, 0, 0.5, 5.0, 3000.0),            # clipped at both ends
+])
+def test_counts_at_rounding_edges(h, w, n, bg, gain, rn):
+    table = synth.sphere_table(synth.SPHERE_SEED_BASE + h * w, n=n, h=h, w=w, r_range=(1.0, 9.0))
+    counts, inten = dog.render_spheres(torch.from_numpy(table).cuda(), h, w, ss=4, background=bg, gain=gain,
+                                       read_noise=rn, seed=h + w, with_intensity=True)
+    torch.cuda.synchronize()
+    want_i, want_c = oracle.render_spheres(table, h, w, ss=4, background=bg, gain=gain, read_noise=rn, seed=h + w)
+    assert np.array_equal(inten.cpu().numpy().view(np.uint32), want_i.view(np.uint32))
+    assert np.array_equal(counts.cpu().numpy().view(np.uint16), want_c)
