@@ -337,13 +337,28 @@ int dog_soft_hist_rec(dog_t* h, const float* d_img, int32_t img_h, int32_t img_w
                       int32_t* d_count, void* stream);
 
 /* Backward of dog_soft_hist_rec from its list of maxima (same frame, same
- * d_sigmas): the dloss/dL planes are scattered from the list and no blur level
- * is recomputed; then the same adjoint blurs as dog_backward.  Outputs as in
- * dog_backward.  An incomplete list (*d_count > cap) sets DOG_ERR_CAPACITY and
+ * d_sigmas): dloss/dI is gathered from the maxima whose windows reach a pixel and
+ * the sigma gradient is summed over the maxima; no blur level is recomputed (a
+ * frame too dense in maxima for that is blurred from its dloss/dL planes, in the
+ * same call).  Outputs as in dog_backward.  An incomplete list (*d_count > cap) sets DOG_ERR_CAPACITY and
  * uses the first cap entries. */
 int dog_backward_rec(dog_t* h, const float* d_img, int32_t img_h, int32_t img_w, int32_t pitch,
                      const float* d_sigmas, const dog_soft_max* d_max, const int32_t* d_count, int32_t cap,
                      const float* d_grad_hist, float* d_grad_img, float* d_grad_sigmas, void* stream);
+
+/* The two calls above for n frames of one size in device memory, frame_stride
+ * floats from one to the next (>= pitch * (img_h - 1) + img_w), the same sigmas
+ * and loss for all: one launch works on every frame.  d_max is n x cap and
+ * d_counts n (both NULL: nothing is recorded); the histogram is the sum over the
+ * frames, d_grad_img is n x img_h x img_w, and d_grad_sigmas receives the sum.
+ * n = 0 does nothing. */
+int dog_soft_hist_batched(dog_t* h, const float* d_img, int32_t n, int64_t frame_stride, int32_t img_h,
+                          int32_t img_w, int32_t pitch, const float* d_sigmas, float* d_soft_hist,
+                          dog_soft_max* d_max, int32_t cap, int32_t* d_counts, void* stream);
+int dog_backward_rec_batched(dog_t* h, const float* d_img, int32_t n, int64_t frame_stride, int32_t img_h,
+                             int32_t img_w, int32_t pitch, const float* d_sigmas, const dog_soft_max* d_max,
+                             const int32_t* d_counts, int32_t cap, const float* d_grad_hist, float* d_grad_img,
+                             float* d_grad_sigmas, void* stream);
 
 /* Debug/parity: write the DoG cube D (K-1 x img_h x img_w floats, row-major
  * planes) computed by the same fused kernel as dog_candidates. */

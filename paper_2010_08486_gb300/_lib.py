@@ -33,7 +33,7 @@ NOALLOC_MAX_CAND = 65536
 EXPORTS = (
     "dog_config_default", "dog_create", "dog_destroy", "dog_ladder", "dog_candidates", "dog_prune",
     "dog_prune_noalloc", "dog_stretch_limits", "dog_stretch", "dog_render_spheres", "dog_volume_hist", "dog_detect", "dog_detect_batched", "dog_set_tiling", "dog_set_producer_warps", "dog_get_producer_warps", "dog_soft_hist",
-    "dog_backward", "dog_soft_hist_rec", "dog_backward_rec", "dog_debug_dog", "dog_ring_hist_push", "dog_ring_hist_push_batched",
+    "dog_backward", "dog_soft_hist_rec", "dog_backward_rec", "dog_soft_hist_batched", "dog_backward_rec_batched", "dog_debug_dog", "dog_ring_hist_push", "dog_ring_hist_push_batched",
     "dog_profile_enable", "dog_profile_read", "dog_fma_peak",
     "dog_get_status", "dog_test_fail_alloc", "dog_status_string",
 )
@@ -130,6 +130,8 @@ def load(path: str | None = None):
         lib.dog_get_producer_warps.argtypes = [vp]
         lib.dog_soft_hist.argtypes = [vp, vp, i32, i32, i32, vp, vp, vp]
         lib.dog_backward.argtypes = [vp, vp, i32, i32, i32, vp, vp, vp, vp, vp]
+        lib.dog_soft_hist_batched.argtypes = [vp, vp, i32, ctypes.c_int64, i32, i32, i32, vp, vp, vp, i32, vp, vp]
+        lib.dog_backward_rec_batched.argtypes = [vp, vp, i32, ctypes.c_int64, i32, i32, i32, vp, vp, vp, i32, vp, vp, vp, vp]
         lib.dog_soft_hist_rec.argtypes = [vp, vp, i32, i32, i32, vp, vp, vp, i32, vp, vp]
         lib.dog_backward_rec.argtypes = [vp, vp, i32, i32, i32, vp, vp, vp, i32, vp, vp, vp, vp]
         lib.dog_debug_dog.argtypes = [vp, vp, i32, i32, i32, i32, vp, vp]

@@ -328,19 +328,29 @@ __device__ __noinline__ void flush(const FusedParams& p, SmemSmall& ss, int x0, 
             int idx = 0;
             if (p.rec != nullptr) {
                 const unsigned m = __ballot_sync(0xffffffffu, have);
-                if (lane == 0) idx = atomicAdd(p.rec_count, __popc(m));
+                if (lane == 0) idx = atomicAdd(p.rec_count + frame, __popc(m));
                 idx = __shfl_sync(0xffffffffu, idx, 0) + __popc(m & lanemask_lt());
             }
+            const float s = have ? 1.0f / (1.0f + __expf(-(d - p.thr) * p.inv_T)) : 0.0f;
+            // one addition per plane and bin: nearly all maxima are of the finest
+            // plane, and 32 lanes adding to one word of shared memory take turns
+            // (16 frames of 1024 x 1024 with 12 levels: 1657 -> 1549 us)
+            for (unsigned left = __ballot_sync(0xffffffffu, have); left;) {
+                const int lv = __shfl_sync(0xffffffffu, l, __ffs(left) - 1);
+                const bool same = have && l == lv;
+                left &= ~__ballot_sync(0xffffffffu, same);
+                float t = same ? s : 0.0f;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+                if (lane < 2) atomicAdd(&ss.soft[ss.kb[lv][lane]], t * ss.kw[lv][lane]);
+            }
             if (have) {
-                const float s = 1.0f / (1.0f + __expf(-(d - p.thr) * p.inv_T));
-                atomicAdd(&ss.soft[ss.kb[l][0]], s * ss.kw[l][0]);
-                atomicAdd(&ss.soft[ss.kb[l][1]], s * ss.kw[l][1]);
                 if (p.rec != nullptr) {
                     if (idx < p.rec_cap) {
                         const float q = s * (1.0f - s) * p.inv_T;
                         dog_soft_max m;
                         m.x = x; m.y = y; m.level = l; m.q = q; m.qe = q * e; m.s = s;
-                        p.rec[idx] = m;
+                        p.rec[(size_t)frame * p.rec_cap + idx] = m;
                     } else {
                         atomicCAS(p.status, 0, (int)DOG_ERR_CAPACITY);
                     }
@@ -765,11 +775,17 @@ __global__ void __launch_bounds__(NW * 32, 1) dog_fused_kernel(const __grid_cons
         // single frame: blockIdx.x enumerates (strip, band)
         __syncthreads();
         TileCtx tc;
-        tc.img = p.img; tc.dtype = p.dtype; tc.H = p.H; tc.W = p.W; tc.pitch = p.pitch; tc.frame = 0;
+        int tile = blockIdx.x, frame = 0;
+        if (MODE == MODE_SOFT) {   // of a batch of equal frames, frame after frame
+            frame = tile / (p.n_strips * p.n_bands);
+            tile -= frame * (p.n_strips * p.n_bands);
+        }
+        tc.img = MODE == MODE_SOFT ? static_cast<const float*>(p.img) + frame * p.frame_stride : p.img;
+        tc.dtype = p.dtype; tc.H = p.H; tc.W = p.W; tc.pitch = p.pitch; tc.frame = frame;
         tc.st_lo = tc.dtype == DTYPE_U16_STRETCH ? p.lohi[0] : 0;
         tc.st_hi = tc.dtype == DTYPE_U16_STRETCH ? p.lohi[1] : 0;
         tc.st_rcp = stretch_rcp(tc.st_lo, tc.st_hi);
-        const int band = blockIdx.x / p.n_strips, strip = blockIdx.x - band * p.n_strips;
+        const int band = tile / p.n_strips, strip = tile - band * p.n_strips;
         tc.x0 = strip * p.strip_step + p.strip_x0;
         tc.y0 = band * p.band;
         tc.y1 = min(p.H, tc.y0 + p.band);

@@ -84,6 +84,7 @@ struct FusedParams {
     int overlap;           // single frame: strips of TX columns step by TX - 2 from column -1, and
                            // only lanes 1 .. TX-2 own their voxels (no strip-edge queue)
     int strip_step, strip_x0;  // single frame: strip s starts at column s strip_step + strip_x0
+    long long frame_stride;    // MODE_SOFT: n_frames frames of one size, pixels from one to the next
     // batched mode
     const FrameDesc* frames;
     int n_frames;

@@ -12,13 +12,15 @@
 //   dloss/dI = sum_i B_i^T A_i,     B_i = row blur o column blur (reflect)
 //   dloss/dsigma_i = <B_y^T A_i, B_x' I> + <B_y'^T A_i, B_x I>  (kernel shape)
 //                  + dloss/dc terms + dloss/dt terms.
+// Every B_i is symmetric: its kernel is even and the boundary reflects about
+// the half sample, so B_i^T A is the blur of A itself with the same boundary.
 // Two backward paths.  From a record of the forward's maxima (soft forward
-// with `rec`): A is scattered from the list, and the kernel-shape term is
-// evaluated at the maxima as sum_v A_i(v) dL_i/dsigma_i(v) (the same sum,
-// since A_i vanishes elsewhere); no blur level is formed.  Without a record:
-// the fused kernel (MODE_BWD) recomputes the L_i and writes A densely, and
-// the kernel-shape term is the two inner products above.  Both then run the
-// adjoint blurs, which gather through the reflect fold-back.
+// with `rec`): A is zero outside the maxima's voxels, so dloss/dI is gathered
+// tile by tile from the maxima whose windows reach it, and the kernel-shape
+// term is evaluated at the maxima as sum_v A_i(v) dL_i/dsigma_i(v); no plane of
+// A and no blur level is formed.  Without a record: the fused kernel (MODE_BWD)
+// recomputes the L_i and writes A densely, two passes blur it, and the
+// kernel-shape term is the two inner products above.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -53,28 +55,83 @@ struct SoftWS {
     float* c = nullptr;       // P coefficients then P sigmas
     float* kappa = nullptr;   // P x nbins
     float* dkappa = nullptr;  // P x nbins
+    float* gk = nullptr;      // P sums gH . kappa_l, then P sums gH . dkappa_l
+    float* wpad = nullptr;    // the taps with TAP_PAD zeros around each level's
+    float4* wt = nullptr;     // per plane and window offset: taps and their derivatives of both its levels
     Pending* pend = nullptr;
     int pend_cap = 0;
     int* counts = nullptr;
     float* A = nullptr;       // K x H x W
+    void* lists = nullptr;    // the record path's lists (see Lists) of n_lists frames
+    int n_lists = 0;
+    int* flags = nullptr;     // per listed frame: dense form wanted, entries linked; then the grid barrier's counter
+    int dense_grid = 0;       // co-resident CTAs of the dense record kernel (0: not asked yet)
     float* Y = nullptr;       // K x H x W
     float* Yd = nullptr;      // K x H x W
-    double* acc = nullptr;    // dc (P), dt (P), dw (K)
+    double* acc = nullptr;    // dc (P), dt (P), dw (K), ACC_COPIES times
     float* last_sig = nullptr;   // the sigmas the tables were last built from (NaN: none)
-    int* big = nullptr;          // wide-window maxima queued by the sigma kernel
-    int* big_count = nullptr;
-    int big_cap = 0;
 };
 
 void soft_free(dog_handle* h) {
     SoftWS* ws = static_cast<SoftWS*>(handle_soft_ws(h));
     if (!ws) return;
-    void* ptrs[] = {ws->w, ws->dw, ws->wp, ws->c, ws->kappa, ws->dkappa, ws->pend, ws->counts, ws->A, ws->Y, ws->Yd, ws->acc,
-                    ws->last_sig, ws->big, ws->big_count};
+    void* ptrs[] = {ws->w, ws->dw, ws->wp, ws->c, ws->kappa, ws->dkappa, ws->gk, ws->wpad, ws->wt, ws->pend, ws->counts, ws->A,
+                    ws->lists, ws->flags, ws->Y, ws->Yd, ws->acc, ws->last_sig};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete ws;
     handle_soft_ws(h) = nullptr;
+}
+
+// CTAs of the record pass spread their atomics over copies of the sums.
+constexpr int ACC_COPIES = 16;
+
+// The record path lists the maxima by cells of CELL x CELL pixels.  A cell has
+// CELL_SLOTS places for the maxima of narrow planes (nearly all; two to a cell in
+// a dense frame), which a reader fetches side by side; those of wider planes,
+// and what does not fit, are linked.  A frame that overflows the entries or links
+// more than CHAIN_MAX to a cell takes the dense form.
+constexpr int CELL_SHIFT = 3, CELL_SLOTS = 8, CHAIN_MAX = 64, NARROW_R = 7;
+__host__ __device__ static inline int cells(int n) { return (n + (1 << CELL_SHIFT) - 1) >> CELL_SHIFT; }
+
+struct Lists {
+    int4* slots;      // cells x CELL_SLOTS: x, y * 32 + plane, A_l there
+    int4* ent;        // ent_cap: the same, and the next entry
+    int* count;       // cells: maxima of narrow planes
+    int* linked;      // cells: entries linked
+    int* head;        // cells: first of them, -1 for none
+    int n_cells, ent_cap;
+    long long ints;   // ints of a frame
+};
+constexpr int LIST_FRAMES = 64;                      // frames of a batch listed at a time, at most,
+constexpr size_t LIST_BYTES = (size_t)256 << 20;     // and the lists' size (one frame's always fit)
+
+// Frame f's lists (all of a frame's arrays lie together).
+__host__ __device__ static inline Lists frame_lists(void* base, int H, int W, int f) {
+    Lists a;
+    a.n_cells = cells(H) * cells(W);
+    a.ent_cap = (int)((long long)H * W / 16) + 4096;
+    a.ints = 4LL * a.n_cells * CELL_SLOTS + 4LL * a.ent_cap + ((3LL * a.n_cells + 3) & ~3LL);
+    int* b = static_cast<int*>(base) + f * a.ints;
+    a.slots = reinterpret_cast<int4*>(b);
+    a.ent = a.slots + (long long)a.n_cells * CELL_SLOTS;
+    a.count = reinterpret_cast<int*>(a.ent + a.ent_cap);
+    a.linked = a.count + a.n_cells;
+    a.head = a.linked + a.n_cells;
+    return a;
+}
+
+// Plane l's window holds the kernels of both its levels; offset of its taps.
+static int plane_radius(const dog_handle* h, int l) {
+    return std::max(handle_levels(h)[l].r, handle_levels(h)[l + 1].r);
+}
+
+// Place of level i's taps among the padded ones (i = K: their number).
+constexpr int TAP_PAD = 32;
+static int pad_offset(const dog_handle* h, int i) {
+    int n = TAP_PAD;   // neighbours share the zeros between them
+    for (int k = 0; k < i; ++k) n += 2 * handle_levels(h)[k].r + 1 + TAP_PAD;
+    return n;
 }
 
 static int soft_ws(dog_handle* h, int H, int W, SoftWS** out) {
@@ -99,14 +156,20 @@ static int soft_ws(dog_handle* h, int H, int W, SoftWS** out) {
     ok(cudaMalloc(&ws->dkappa, sizeof(float) * P * nb));
     ok(cudaMalloc(&ws->pend, sizeof(Pending) * ws->pend_cap));
     ok(cudaMalloc(&ws->counts, sizeof(int) * 4));
+    int n_wt = 0;
+    for (int l = 0; l < P; ++l) n_wt += 2 * plane_radius(h, l) + 1;
+    ok(cudaMalloc(&ws->wt, sizeof(float4) * n_wt));
+    ok(cudaMalloc(&ws->gk, sizeof(float) * 2 * P));
+    ok(cudaMalloc(&ws->wpad, sizeof(float) * pad_offset(h, K)));
+    if (e == cudaSuccess) ok(cudaMemset(ws->wpad, 0, sizeof(float) * pad_offset(h, K)));
     ok(cudaMalloc(&ws->A, sizeof(float) * plane * K));
+    ok(cudaMalloc(&ws->lists, sizeof(int) * frame_lists(nullptr, H, W, 0).ints));
+    ws->n_lists = 1;
+    ok(cudaMalloc(&ws->flags, sizeof(int) * (2 * LIST_FRAMES + 1)));
     ok(cudaMalloc(&ws->Y, sizeof(float) * plane * K));
     ok(cudaMalloc(&ws->Yd, sizeof(float) * plane * K));
-    ok(cudaMalloc(&ws->acc, sizeof(double) * (2 * P + K)));
+    ok(cudaMalloc(&ws->acc, sizeof(double) * ACC_COPIES * (2 * P + K)));
     ok(cudaMalloc(&ws->last_sig, sizeof(float) * K));
-    ws->big_cap = 1 << 16;
-    ok(cudaMalloc(&ws->big, sizeof(int) * ws->big_cap));
-    ok(cudaMalloc(&ws->big_count, sizeof(int)));
     if (e == cudaSuccess) ok(cudaMemset(ws->last_sig, 0xff, sizeof(float) * K));   // NaN: tables not built
     if (e != cudaSuccess) {
         soft_free(h);
@@ -126,6 +189,7 @@ struct SoftPrep {
     int woff[MAX_LEVELS];
     int tpad[MAX_LEVELS];
     int pbase[MAX_LEVELS], plead[MAX_LEVELS];   // place of the level's taps in the pair table
+    int wtoff[MAX_LEVELS];                      // place of plane l's taps in wt
     double lref0, lrefP;   // ln sigma of the reference ladder's first / last DoG plane
     float* w;
     float* dw;
@@ -134,16 +198,22 @@ struct SoftPrep {
     float* kappa;
     float* dkappa;
     float* last_sig;
+    float4* wt;
+    float* wpad;
+    int padoff[MAX_LEVELS];
+    const float* gH;   // backward: dloss/dH (nullptr in the forward)
+    float* gk;
+    int* zero[2];      // counters to clear (nullptr: none), n_zero[k] ints each
+    int n_zero[2];
+    double* acc;       // sums to clear
+    int n_acc;
+    void* lists;       // lists of n_lists frames of H x W to empty
+    int n_lists, H, W;
 };
 
-// Tap, coefficient and bin-weight tables of the device sigmas.  Skipped when
-// the sigmas equal those the tables were last built from (a batch of frames
-// at one ladder builds them once); last_sig is NaN after allocation.
-constexpr int PREP_THREADS = 512;
-__global__ void __launch_bounds__(PREP_THREADS) soft_prep_kernel(const __grid_constant__ SoftPrep p) {
-    bool changed = false;
-    for (int i = threadIdx.x; i < p.K; i += blockDim.x) changed |= !(p.sig[i] == p.last_sig[i]);
-    if (!__syncthreads_or(changed)) return;
+constexpr int PREP_THREADS = 512, PREP_CELLS = 8 * PREP_THREADS;
+
+__device__ void soft_tables(const SoftPrep& p) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int i = warp; i < p.K; i += PREP_THREADS / 32) {
         const double s = (double)p.sig[i];
@@ -171,7 +241,10 @@ __global__ void __launch_bounds__(PREP_THREADS) soft_prep_kernel(const __grid_co
             }
             p.w[p.woff[i] + t] = wv;
             p.dw[p.woff[i] + t] = dv;
-            if (t <= 2 * r) p.wp[p.pbase[i] + 2 * (t + p.plead[i])] = wv;
+            if (t <= 2 * r) {
+                p.wp[p.pbase[i] + 2 * (t + p.plead[i])] = wv;
+                p.wpad[p.padoff[i] + t] = wv;
+            }
         }
     }
     for (int l = threadIdx.x; l < p.P; l += blockDim.x) {
@@ -190,9 +263,50 @@ __global__ void __launch_bounds__(PREP_THREADS) soft_prep_kernel(const __grid_co
             p.dkappa[l * p.nbins + b] = (a < 1.0 && !clamped) ? (float)(-(double)p.nbins * sg) : 0.0f;
         }
     }
-    for (int i = threadIdx.x; i < p.K; i += blockDim.x) p.last_sig[i] = p.sig[i];
+    for (int i = threadIdx.x; i < p.K; i += blockDim.x) p.last_sig[i] = p.sig[i];    __syncthreads();
+    for (int l = warp; l < p.P; l += PREP_THREADS / 32) {
+        const int ra = p.r[l], rb = p.r[l + 1], R2 = max(ra, rb);
+        for (int t = lane; t <= 2 * R2; t += 32) {
+            const int ta = t - R2 + ra, tb = t - R2 + rb;
+            const bool ia = ta >= 0 && ta <= 2 * ra, ib = tb >= 0 && tb <= 2 * rb;
+            p.wt[p.wtoff[l] + t] = make_float4(ia ? p.w[p.woff[l] + ta] : 0.0f, ia ? p.dw[p.woff[l] + ta] : 0.0f,
+                                               ib ? p.w[p.woff[l + 1] + tb] : 0.0f,
+                                               ib ? p.dw[p.woff[l + 1] + tb] : 0.0f);
+        }
+    }
 }
 
+// What a soft call starts from, in one launch: block 0 clears the counters and
+// sums, builds the tap, coefficient and bin-weight tables of the device sigmas
+// (skipped when the sigmas equal those the tables were last built from: a batch
+// of frames at one ladder builds them once; last_sig is NaN after allocation)
+// and folds dloss/dH into one weight per plane; the other blocks empty the
+// record path's lists.
+__global__ void __launch_bounds__(PREP_THREADS) soft_prep_kernel(const __grid_constant__ SoftPrep p) {
+    if (blockIdx.x > 0) {
+        const Lists a = frame_lists(p.lists, p.H, p.W, blockIdx.y);
+        const int h0 = (blockIdx.x - 1) * PREP_CELLS;
+        for (int i = h0 + threadIdx.x; i < min(h0 + PREP_CELLS, 3 * a.n_cells); i += PREP_THREADS)
+            a.count[i] = i < 2 * a.n_cells ? 0 : -1;   // count, linked; head
+        return;
+    }
+    if (blockIdx.y > 0) return;
+    for (int k = 0; k < 2; ++k)
+        for (int i = threadIdx.x; i < p.n_zero[k]; i += PREP_THREADS) p.zero[k][i] = 0;
+    for (int i = threadIdx.x; i < p.n_acc; i += PREP_THREADS) p.acc[i] = 0.0;
+    bool changed = false;
+    for (int i = threadIdx.x; i < p.K; i += blockDim.x) changed |= !(p.sig[i] == p.last_sig[i]);
+    if (__syncthreads_or(changed)) soft_tables(p);
+    if (p.gH == nullptr) return;
+    __syncthreads();
+    for (int l = threadIdx.x; l < 2 * p.P; l += PREP_THREADS) {
+        const float* kap = l < p.P ? p.kappa + l * p.nbins : p.dkappa + (l - p.P) * p.nbins;
+        float a = 0.0f;
+#pragma unroll 8
+        for (int k = 0; k < p.nbins; ++k) a += p.gH[k] * kap[k];
+        p.gk[l] = a;
+    }
+}
 static SoftPrep prep_params(dog_handle* h, SoftWS* ws, const float* sig) {
     const FusedParams& b = handle_base(h);
     const std::vector<double>& ref = handle_sigmas(h);
@@ -207,6 +321,7 @@ static SoftPrep prep_params(dog_handle* h, SoftWS* ws, const float* sig) {
         q.woff[i] = handle_levels(h)[i].woff;
         q.tpad[i] = handle_levels(h)[i].tpad;
         handle_tap_slot(h, i, &q.pbase[i], &q.plead[i]);
+        q.padoff[i] = pad_offset(h, i);
     }
     q.lref0 = std::log(ref[0]);
     q.lrefP = std::log(ref[b.P - 1]);
@@ -217,10 +332,18 @@ static SoftPrep prep_params(dog_handle* h, SoftWS* ws, const float* sig) {
     q.kappa = ws->kappa;
     q.dkappa = ws->dkappa;
     q.last_sig = ws->last_sig;
+    q.wt = ws->wt;
+    q.wpad = ws->wpad;
+    q.gk = ws->gk;
+    for (int l = 0, n = 0; l < b.P; ++l) {
+        q.wtoff[l] = n;
+        n += 2 * plane_radius(h, l) + 1;
+    }
     return q;
 }
 
-static FusedParams soft_fused(dog_handle* h, SoftWS* ws, const float* img, int H, int W, int pitch, int mode) {
+static FusedParams soft_fused(dog_handle* h, SoftWS* ws, const float* img, int n, long long stride, int H, int W,
+                              int pitch, int mode) {
     FusedParams p = handle_base(h);
     p.img = img;
     p.dtype = DOG_DTYPE_F32;
@@ -234,9 +357,11 @@ static FusedParams soft_fused(dog_handle* h, SoftWS* ws, const float* img, int H
     p.strip_step = TX - 2;
     p.strip_x0 = -1;
     p.n_strips = (W + TX - 2 - 1) / (TX - 2);
-    p.band = pick_band(p, handle_sms(h), H, p.n_strips, std::min(handle_band(h), H));
+    p.band = pick_band(p, handle_sms(h), H, n * p.n_strips, std::min(handle_band(h), H));
     p.n_bands = (H + p.band - 1) / p.band;
     p.frames = nullptr;
+    p.n_frames = n;
+    p.frame_stride = stride;
     p.mode = mode;
     p.w = ws->wp;
     p.c = ws->c;
@@ -251,63 +376,58 @@ static FusedParams soft_fused(dog_handle* h, SoftWS* ws, const float* img, int H
     return p;
 }
 
+// Frames of a batch whose lists the workspace holds: grown to the batch unless
+// the stream is being captured (then the batch goes in several passes).
+static int list_frames(SoftWS* ws, int n, cudaStream_t s) {
+    const size_t one = sizeof(int) * (size_t)frame_lists(nullptr, ws->H, ws->W, 0).ints;
+    const int want = (int)std::max<size_t>(1, std::min({(size_t)n, (size_t)LIST_FRAMES, LIST_BYTES / one}));
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+    if (want > ws->n_lists && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+        void* more = nullptr;
+        if (cudaMalloc(&more, want * one) == cudaSuccess) {
+            cudaDeviceSynchronize();
+            cudaFree(ws->lists);
+            ws->lists = more;
+            ws->n_lists = want;
+        } else {
+            cudaGetLastError();
+        }
+    }
+    return std::min(n, ws->n_lists);
+}
+
 #define SOFT_CUDA(x)                                                                  \
     do {                                                                              \
         cudaError_t e_ = (x);                                                         \
         if (e_ != cudaSuccess) return e_ == cudaErrorMemoryAllocation ? DOG_ERR_NOMEM : DOG_ERR_CUDA; \
     } while (0)
 
-int soft_forward(dog_handle* h, const float* img, int H, int W, int pitch, const float* sig, float* out,
-                 dog_soft_max* rec, int rec_cap, int* rec_count, cudaStream_t s) {
+int soft_forward(dog_handle* h, const float* img, int n, long long stride, int H, int W, int pitch, const float* sig,
+                 float* out, dog_soft_max* rec, int rec_cap, int* rec_count, cudaStream_t s) {
     SoftWS* ws = nullptr;
     int st = soft_ws(h, H, W, &ws);
     if (st != DOG_OK) return st;
     SoftPrep q = prep_params(h, ws, sig);
+    q.zero[0] = ws->counts;
+    q.n_zero[0] = 4;
+    if (rec != nullptr) {
+        q.zero[1] = rec_count;
+        q.n_zero[1] = n;
+    }
     soft_prep_kernel<<<1, PREP_THREADS, 0, s>>>(q);
     SOFT_CUDA(cudaGetLastError());
-    SOFT_CUDA(cudaMemsetAsync(ws->counts, 0, sizeof(int) * 4, s));
-    FusedParams p = soft_fused(h, ws, img, H, W, pitch, MODE_SOFT);
+    FusedParams p = soft_fused(h, ws, img, n, stride, H, W, pitch, MODE_SOFT);
     p.soft_out = out;
     if (rec != nullptr) {
-        SOFT_CUDA(cudaMemsetAsync(rec_count, 0, sizeof(int), s));
         p.rec = rec;
         p.rec_cap = rec_cap;
         p.rec_count = rec_count;
     }
-    SOFT_CUDA(timed_fused(h, p, p.n_strips * p.n_bands, s));
+    SOFT_CUDA(timed_fused(h, p, n * p.n_strips * p.n_bands, s));
     return DOG_OK;
 }
 
 // ---------------------------------------------------------------------------
-// Reflected part of the 1-D adjoint of a reflect-boundary correlation with the
-// symmetric full kernel w[0..2r] (w[r + d] weighs offset d), at index m of a
-// line of length N with stride `st`.  The adjoint at m sums, over the
-// preimages q of m under the reflection that lie within r of the line,
-// sum_n w[|q-n|] a[n]; the zero-padded correlation gives the term q = m, and
-// this function the others (the reflected copies q = -1-m, 2N-1-m, ...).
-__device__ __forceinline__ float adj1d_mirror(const float* __restrict__ a, size_t st, int N, int m,
-                                              const float* __restrict__ w, int r) {
-    float acc = 0.0f;
-    const int per = 2 * N;
-    const int fam[2] = {m, per - 1 - m};
-#pragma unroll
-    for (int f = 0; f < 2; ++f) {
-        int q = fam[f];
-        const int k = (-r - q) > 0 ? ((-r - q) + per - 1) / per : -((q + r) / per);
-        for (q = q + k * per; q <= N - 1 + r; q += per) {
-            if (q == m) continue;
-            const int nlo = max(0, q - r), nhi = min(N - 1, q + r);
-            for (int n = nlo; n <= nhi; ++n) acc = __fmaf_rn(__ldg(w + r + (q - n)), __ldg(a + (size_t)n * st), acc);
-        }
-    }
-    return acc;
-}
-
-// Outputs of a line of length N that a reflected preimage reaches (those
-// within r of an end): count, and the j-th of them.
-__host__ __device__ inline int fold_count(int N, int r) { return N <= 2 * r ? N : 2 * r; }
-__host__ __device__ inline int fold_index(int N, int r, int j) { return (N <= 2 * r || j < r) ? j : N - 2 * r + j; }
-
 __device__ __forceinline__ int refl_i(int i, int n) {
     if (i >= 0 && i < n) return i;   // inside: no modulo
     int p = 2 * n;
@@ -317,7 +437,7 @@ __device__ __forceinline__ int refl_i(int i, int n) {
 }
 
 struct AdjParams {
-    const float* A;
+    float* A;
     float* Y;
     float* Yd;
     const float* img;
@@ -332,14 +452,12 @@ struct AdjParams {
     double* dw_acc;
 };
 
-// Tiled adjoints.  Both kernels of a level, w(t) and dw/dsigma(t), are even
-// in t, so away from the frame's edges the adjoint of a blur is the same
-// correlation: out(m) = sum_{u < Tpad} k[u] X(m - r + u) over zero-padded taps.
-// Eight consecutive outputs per thread are accumulated against a two-window
-// register file (8 inputs per block of 8 taps), for two tap sets at once.
-// Outputs within r of an edge, where the reflect boundary folds the sums, get
-// the reflected preimages' part added afterwards by the fold kernels, one
-// thread per such output (adj1d_mirror).
+// Dense adjoints.  Both kernels of a level, w(t) and dw/dsigma(t), are even in t
+// and the boundary reflects about the half sample, so the adjoint of a blur is
+// the same blur: out(m) = sum_{u < Tpad} k[u] X(refl(m - r + u)) over zero-padded
+// taps (cells that only padding taps reach are zero).  Eight consecutive outputs
+// per thread are accumulated against a two-window register file (8 inputs per
+// block of 8 taps), for two tap sets at once.
 __device__ __forceinline__ void tap_block2(float (&o)[8], float (&od)[8], const float (&A)[8], const float (&B)[8],
                                            const float* __restrict__ w, const float* __restrict__ dw) {
 #pragma unroll
@@ -405,42 +523,38 @@ __device__ __forceinline__ void corr8(const float* __restrict__ X, int st, const
     }
 }
 
-constexpr int ADJ_TM = 64;     // output rows per CTA of the column adjoint
-
-__host__ __device__ inline int adj_y_smem_floats(int tpad_max) { return (ADJ_TM + tpad_max + 8) * 32 + 2 * tpad_max; }
-
-// Column adjoint of level blockIdx.z: Y_i = B_y^T A_i (kernel w_i) and, when
-// SIG, Yd_i (dw_i) for the dense sigma gradient; a 32-column x 64-row tile per
-// CTA, warp g on rows 8g .. 8g+7, lane = column.
-template <bool SIG>
-__global__ void __launch_bounds__(256) adj_y_kernel(const __grid_constant__ AdjParams p) {
-    extern __shared__ float ysm[];
-    const int i = blockIdx.z;
+// Column adjoint of level i, columns x0 .. x0 + 31 and rows m0 .. m0 + 8 WARPS - 1:
+// Y_i = B_y^T A_i (kernel w_i) and, when SIG, Yd_i (dw_i) for the sigma
+// gradient; warp g on rows 8g .. 8g+7, lane = column.
+__host__ __device__ inline int adj_y_smem_floats(int warps, int tpad_max) {
+    return (8 * warps + tpad_max + 8) * 32 + 2 * tpad_max;
+}
+template <bool SIG, int WARPS>
+__device__ __forceinline__ void adj_y_tile(const AdjParams& p, float* ysm, int x0, int m0, int i) {
     const int r = p.r[i], tpad = p.tpad[i], nb = tpad >> 3;
-    const int x0 = blockIdx.x * 32, m0 = blockIdx.y * ADJ_TM;
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
-    const int rows = ADJ_TM + tpad + 8;
-    float* X = ysm;                  // rows x 32: A rows m0 - r + j, zero outside the frame
+    const int rows = 8 * WARPS + tpad + 8;
+    float* X = ysm;                  // rows x 32: A rows m0 - r + j, reflected
     float* ws = ysm + rows * 32;     // tpad
     float* wd = ws + tpad;           // tpad
     const size_t plane = (size_t)p.H * p.W;
     const float* A = p.A + plane * i;
-    for (int t = threadIdx.x; t < tpad; t += blockDim.x) {
+    for (int t = threadIdx.x; t < tpad; t += 32 * WARPS) {
         ws[t] = p.w[p.woff[i] + t];
         wd[t] = p.dw[p.woff[i] + t];
     }
     const int x = x0 + lane;
-    // warp g stages rows g, g + 8, ...; eight loads in flight before the stores
-    for (int j0 = g; j0 < rows; j0 += 64) {
+    // warp g stages rows g, g + WARPS, ...; eight loads in flight before the stores
+    for (int j0 = g; j0 < rows; j0 += 8 * WARPS) {
         float v[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            const int j = j0 + 8 * u, n = m0 - r + j;
-            v[u] = (j < rows && n >= 0 && n < p.H && x < p.W) ? A[(size_t)n * p.W + x] : 0.0f;
+            const int j = j0 + WARPS * u, n = m0 - r + j;
+            v[u] = (j < rows && n >= -r && n < p.H + r && x < p.W) ? __ldcg(A + (size_t)refl_i(n, p.H) * p.W + x) : 0.0f;
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-            if (j0 + 8 * u < rows) X[(j0 + 8 * u) * 32 + lane] = v[u];
+            if (j0 + WARPS * u < rows) X[(j0 + WARPS * u) * 32 + lane] = v[u];
     }
     __syncthreads();
     float o[8], od[8];
@@ -458,85 +572,10 @@ __global__ void __launch_bounds__(256) adj_y_kernel(const __grid_constant__ AdjP
     }
 }
 
-// Reflect fold of the column adjoint: rows within r_i of the top or bottom
-// edge (blockIdx.y-th of them) of level blockIdx.z, one thread per column.
-template <bool SIG>
-__global__ void __launch_bounds__(128) adj_y_fold_kernel(const __grid_constant__ AdjParams p) {
-    const int i = blockIdx.z, r = p.r[i];
-    const int j = blockIdx.y;
-    if (j >= fold_count(p.H, r)) return;
-    const int m = fold_index(p.H, r, j);
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= p.W) return;
-    const size_t plane = (size_t)p.H * p.W;
-    const float* A = p.A + plane * i + x;
-    const size_t o = plane * i + (size_t)m * p.W + x;
-    p.Y[o] += adj1d_mirror(A, p.W, p.H, m, p.w + p.woff[i], r);
-    if (SIG) p.Yd[o] += adj1d_mirror(A, p.W, p.H, m, p.dw + p.woff[i], r);
-}
-
-// Reflect fold of the row adjoint: one warp per row y, its lanes on the
-// columns within R of the left or right edge; sums the reflected preimages'
-// part over every level whose radius reaches the column.  When the frame is
-// wider than 2R, a level's reflected terms read only the first and last r_i
-// values of the row, which the warp first stages in shared memory (one round
-// of coalesced loads per level instead of a serial chain of global loads).
-constexpr int FOLD_ROWS = 4;   // warps (rows) per CTA
-__global__ void __launch_bounds__(32 * FOLD_ROWS) adj_x_fold_kernel(const __grid_constant__ AdjParams p) {
-    __shared__ float edge[FOLD_ROWS][2][DOG_MAX_RADIUS];
-    const int wq = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int y = blockIdx.x * FOLD_ROWS + wq;
-    if (y >= p.H) return;
-    const size_t plane = (size_t)p.H * p.W;
-    const int nf = fold_count(p.W, p.R);
-    if (p.W <= 2 * p.R) {   // narrow frame: several reflections, gather from global memory
-        for (int j = lane; j < nf; j += 32) {
-            const int x = fold_index(p.W, p.R, j);
-            float v = 0.0f;
-            for (int i = 0; i < p.K; ++i) {
-                const int r = p.r[i];
-                if (x >= r && x <= p.W - 1 - r) continue;
-                v += adj1d_mirror(p.Y + plane * i + (size_t)y * p.W, 1, p.W, x, p.w + p.woff[i], r);
-            }
-            p.gimg[(size_t)y * p.W + x] += v;
-        }
-        return;
-    }
-    float* sl = edge[wq][0];   // Y_i(y, 0 .. r-1)
-    float* sr = edge[wq][1];   // Y_i(y, W-r .. W-1)
-    float v[(2 * DOG_MAX_RADIUS + 31) / 32];
-#pragma unroll
-    for (int k = 0; k < (2 * DOG_MAX_RADIUS + 31) / 32; ++k) v[k] = 0.0f;
-    for (int i = 0; i < p.K; ++i) {
-        const int r = p.r[i];
-        const float* row = p.Y + plane * i + (size_t)y * p.W;
-        __syncwarp();
-        for (int n = lane; n < r; n += 32) {
-            sl[n] = row[n];
-            sr[n] = row[p.W - r + n];
-        }
-        __syncwarp();
-        const float* w = p.w + p.woff[i];   // w[r + d] weighs offset d
-#pragma unroll
-        for (int k = 0; k < (2 * DOG_MAX_RADIUS + 31) / 32; ++k) {
-            const int j = lane + 32 * k;
-            if (j >= nf) break;
-            const int x = fold_index(p.W, p.R, j);
-            float acc = 0.0f;
-            if (x < r) {   // reflected copy q = -1 - x: sum_{n=0}^{r-1-x} w[r + q - n] Y(n)
-                for (int n = 0; n <= r - 1 - x; ++n) acc = __fmaf_rn(__ldg(w + r - 1 - x - n), sl[n], acc);
-            } else if (x > p.W - 1 - r) {   // q = 2W - 1 - x: sum_{n=q-r}^{W-1} w[r + q - n] Y(n)
-                const int q = 2 * p.W - 1 - x;
-                for (int n = q - r; n <= p.W - 1; ++n) acc = __fmaf_rn(__ldg(w + r + q - n), sr[n - (p.W - r)], acc);
-            }
-            v[k] += acc;
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < (2 * DOG_MAX_RADIUS + 31) / 32; ++k) {
-        const int j = lane + 32 * k;
-        if (j < nf) p.gimg[(size_t)y * p.W + fold_index(p.W, p.R, j)] += v[k];
-    }
+constexpr int ADJ_WARPS = 8;
+__global__ void __launch_bounds__(32 * ADJ_WARPS) adj_y_kernel(const __grid_constant__ AdjParams p) {
+    extern __shared__ float ysm[];
+    adj_y_tile<true, ADJ_WARPS>(p, ysm, blockIdx.x * 32, blockIdx.y * 8 * ADJ_WARPS, blockIdx.z);
 }
 
 constexpr int ADJ_XR = 32;     // output rows per CTA of the row adjoint (4 warps x 8)
@@ -547,20 +586,18 @@ __host__ __device__ inline int adj_x_smem_floats(int tpad_max, int R, bool sig) 
     return ADJ_XR * (adj_x_stride_y(tpad_max) + (sig ? adj_x_stride_i(R) : 0)) + 2 * tpad_max;
 }
 
-// Row adjoint summed over levels into dloss/dI, and the kernel-shape part of
-// dloss/dsigma_i = <Y_i, B_x' I> + <Yd_i, B_x I>.  A CTA covers 32 columns x 32
+// Row adjoint summed over levels into dloss/dI and, when SIG, the kernel-shape part of
+// dloss/dsigma_i = <Y_i, B_x' I> + <Yd_i, B_x I>.  128 threads cover 32 columns x 32
 // rows; lane (rho, g) of warp q owns row 8q + rho, columns 8g .. 8g+7.
 template <bool SIG>
-__global__ void __launch_bounds__(128) adj_x_kernel(const __grid_constant__ AdjParams p, int tpad_max) {
-    extern __shared__ float xsm[];
-    __shared__ double red[4][MAX_LEVELS];
+__device__ __forceinline__ void adj_x_tile(const AdjParams& p, float* xsm, double (*red)[MAX_LEVELS], int tpad_max,
+                                           int x0, int y0) {
     const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
     const int rho = lane >> 2, g4 = lane & 3;
-    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * ADJ_XR;
     const int row = 8 * q + rho;                 // 0 .. 31
     const int y = y0 + row;
     const int SY = adj_x_stride_y(tpad_max), SI = adj_x_stride_i(p.R);
-    float* Yt = xsm;                              // ADJ_XR x SY: Y_i rows, columns x0 - r + c, zero outside
+    float* Yt = xsm;                              // ADJ_XR x SY: Y_i rows, columns x0 - r + c, reflected
     float* It = Yt + ADJ_XR * SY;                 // ADJ_XR x SI: image rows, columns x0 - R + c, reflected
     float* ws = SIG ? It + ADJ_XR * SI : It;      // tpad_max (no image tile without SIG)
     float* wd = ws + tpad_max;                    // tpad_max
@@ -600,7 +637,7 @@ __global__ void __launch_bounds__(128) adj_x_kernel(const __grid_constant__ AdjP
             wd[t] = p.dw[p.woff[i] + t];
         }
         const int wt = 32 + tpad + 8;
-        // Y_i rows y0 .. y0+31, columns x0-r .. x0-r+wt-1 (zero outside the frame)
+        // Y_i rows y0 .. y0+31, columns x0-r .. x0-r+wt-1 (reflected)
         const int xs = x0 - r;
         const int xa = xs >= 0 ? xs & ~3 : -((3 - xs) & ~3);   // xs rounded down to a multiple of 4
         const int off = xs - xa, n4 = (wt + off + 3) >> 2;     // float4 columns per row
@@ -616,7 +653,7 @@ __global__ void __launch_bounds__(128) adj_x_kernel(const __grid_constant__ AdjP
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         const int rr = min(rb + u * rpp, ADJ_XR - 1);
-                        v[u] = __ldg(src + (size_t)rr * row4);
+                        v[u] = __ldcg(src + (size_t)rr * row4);
                     }
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
@@ -634,15 +671,16 @@ __global__ void __launch_bounds__(128) adj_x_kernel(const __grid_constant__ AdjP
         } else {
             const int c0 = threadIdx.x, c1 = threadIdx.x + 128;
             const int xx0 = xs + c0, xx1 = xs + c1;
-            const bool ok0 = c0 < wt && xx0 >= 0 && xx0 < p.W, ok1 = c1 < wt && xx1 >= 0 && xx1 < p.W;
+            const bool ok0 = c0 < wt && xx0 < p.W + r, ok1 = c1 < wt && xx1 < p.W + r;
+            const int xr0 = refl_i(xx0, p.W), xr1 = refl_i(xx1, p.W);
             for (int rr0 = 0; rr0 < ADJ_XR; rr0 += 8) {   // 16 loads in flight before the stores
                 float v0[8], v1[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     const int yy = y0 + rr0 + u;
                     const float* src = Yi + (size_t)yy * p.W;
-                    v0[u] = (ok0 && yy < p.H) ? src[xx0] : 0.0f;
-                    v1[u] = (ok1 && yy < p.H) ? src[xx1] : 0.0f;
+                    v0[u] = (ok0 && yy < p.H) ? __ldcg(src + xr0) : 0.0f;
+                    v1[u] = (ok1 && yy < p.H) ? __ldcg(src + xr1) : 0.0f;
                 }
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
@@ -693,350 +731,557 @@ __global__ void __launch_bounds__(128) adj_x_kernel(const __grid_constant__ AdjP
     }
 }
 
+__global__ void __launch_bounds__(128) adj_x_kernel(const __grid_constant__ AdjParams p, int tpad_max) {
+    extern __shared__ float xsm[];
+    __shared__ double red[4][MAX_LEVELS];
+    adj_x_tile<true>(p, xsm, red, tpad_max, blockIdx.x * 32, blockIdx.y * ADJ_XR);
+}
+
 struct FinParams {
     const float* sig;
     int K, P, norm;
     double lref0, lrefP;
-    const double* acc;   // dc (P), dt (P), dw (K)
+    const double* acc;   // dc (P), dt (P), dw (K), ACC_COPIES times
     float* gsig;
 };
 
-__global__ void soft_finalize_kernel(const __grid_constant__ FinParams p) {
-    const int i = threadIdx.x;
+// dloss/dsigma_i from the sums (accumulated into gsig); thread i on level i.
+__device__ __forceinline__ void soft_finalize(const FinParams& p, int i) {
     if (i >= p.K) return;
-    const double* dc = p.acc;
-    const double* dt = p.acc + p.P;
-    const double* dwt = p.acc + 2 * p.P;
-    double g = dwt[i];
+    double g = 0.0, dc = 0.0, dt = 0.0, dcl = 0.0;   // dw_i, dc_i, dt_i, dc_{i-1}
+#pragma unroll
+    for (int c = 0; c < ACC_COPIES; ++c) {
+        const double* a = p.acc + c * (2 * p.P + p.K);
+        g += a[2 * p.P + i];
+        if (i < p.P) {
+            dc += a[i];
+            dt += a[p.P + i];
+        }
+        if (i > 0) dcl += a[i - 1];
+    }
     const double si = (double)p.sig[i];
     if (p.norm == DOG_NORM_PAPER) {
-        if (i < p.P) g += dc[i];
+        if (i < p.P) g += dc;
     } else {
         if (i < p.P) {
             const double d = (double)p.sig[i + 1] - si;
-            g += dc[i] * (double)p.sig[i + 1] / (d * d);
+            g += dc * (double)p.sig[i + 1] / (d * d);
         }
         if (i > 0) {
             const double d = si - (double)p.sig[i - 1];
-            g -= dc[i - 1] * (double)p.sig[i - 1] / (d * d);
+            g -= dcl * (double)p.sig[i - 1] / (d * d);
         }
     }
-    if (i < p.P) g += dt[i] / (si * (p.lrefP - p.lref0));
+    if (i < p.P) g += dt / (si * (p.lrefP - p.lref0));
     p.gsig[i] += (float)g;
 }
 
-// dloss/dL planes from a recorded list of maxima: A_l += c_l G_v and
-// A_{l+1} -= c_l G_v for a maximum v in plane l, G_v = gk_l q_v with
-// gk_l = sum_b gH_b kappa_b(t_l); dloss/dc_l += gk_l qe_v, dloss/dt_l +=
-// s_v sum_b gH_b dkappa_b(t_l).  A must be zero beforehand.
-struct ScatterParams {
+__global__ void soft_finalize_kernel(const __grid_constant__ FinParams p) { soft_finalize(p, threadIdx.x); }
+
+// ---- backward from a recorded list of maxima --------------------------------
+// A maximum v in plane l has G_v = gk_l q_v, gk_l = sum_b gH_b kappa_b(t_l), and
+//   A_l(v) += c_l G_v,  A_{l+1}(v) -= c_l G_v;
+//   dloss/dc_l += gk_l qe_v,  dloss/dt_l += s_v sum_b gH_b dkappa_b(t_l);
+//   dloss/dsigma_m += A_m(v) (sum (w'_j w_t + w_j w'_t) I(y + j, x + t))
+// for m = l, l + 1, over |j|, |t| <= r_m of the reflected image.
+//
+// One pass over the record, a chunk of records per CTA at a time:
+//  A  a thread per record links it into its cell's list for the gather below;
+//  B  the window sums of both levels, with lanes on columns: sum_j w_j I and
+//     sum_j w'_j I down the column (four FMAs per pixel for both levels), the
+//     column's own weights once at the end.  Windows up to 2 NARROW_R + 1 wide
+//     (nearly all: the finest planes) take eight lanes of two columns, wider
+//     ones a warp, and those wider than a warp (few: the coarse planes) all the
+//     CTA's warps, so that none runs a long serial window;
+//  C  the products with G_v, gk and gdk in FP64, lane = record, summed over the
+//     lanes of a level (the FP64 pipe takes a warp at two lanes a clock: one
+//     record per instruction would bound the kernel).
+// A CTA's records are gridDim apart, which evens out the planes.
+//
+// 16 frames of 1024 x 1024 with 35,000 maxima each, 12 levels, in us: this pass
+// 276 (latency of the small windows' loads and the meetings between A, B and C),
+// where a warp per maximum with all taps formed per pixel took 830, and its
+// scatter into zeroed planes 470.
+struct RecParams {
     const dog_soft_max* rec;
     const int* count;
     int cap;
-    const float* gH;
-    const float* kappa;
-    const float* dkappa;
+    const float* gk;        // P, then P of dkappa
     const float* c;
-    int P, nbins, H, W;
-    float* A;
-    double* dc_acc;
-    double* dt_acc;
+    const float4* wt;
+    const float* img;
+    long long img_stride, rec_stride;   // from a frame to the next
+    int pitch;
+    int P, K, H, W;
+    int r[MAX_LEVELS];
+    int wtoff[MAX_LEVELS];
+    double* acc;            // dc (P), dt (P), dw (K), ACC_COPIES times
+    void* lists;
+    int* flags;             // per frame: the dense form wanted; entries linked
     int* status;
 };
 
-__global__ void __launch_bounds__(256) soft_scatter_kernel(const __grid_constant__ ScatterParams p) {
-    __shared__ float gk[MAX_LEVELS], gdk[MAX_LEVELS], cl[MAX_LEVELS], dc[MAX_LEVELS], dt[MAX_LEVELS];
-    for (int l = threadIdx.x; l < p.P; l += blockDim.x) {
-        float a = 0.0f, b = 0.0f;
-        for (int k = 0; k < p.nbins; ++k) {
-            a += p.gH[k] * p.kappa[l * p.nbins + k];
-            b += p.gH[k] * p.dkappa[l * p.nbins + k];
-        }
-        gk[l] = a;
-        gdk[l] = b;
-        cl[l] = p.c[l];
-        dc[l] = 0.0f;
-        dt[l] = 0.0f;
-    }
-    __syncthreads();
-    const int n = *p.count;
-    if (n > p.cap && blockIdx.x == 0 && threadIdx.x == 0) atomicCAS(p.status, 0, (int)DOG_ERR_CAPACITY);
-    const int m = min(n, p.cap);
-    const size_t plane = (size_t)p.H * p.W;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
-        const dog_soft_max v = p.rec[i];
-        const int l = v.level;
-        if (v.x < 0 || v.x >= p.W || v.y < 0 || v.y >= p.H || l < 0 || l >= p.P) {   // not this frame's record
-            atomicCAS(p.status, 0, (int)DOG_ERR_INVALID);
-            continue;
-        }
-        const float G = gk[l] * v.q;
-        const size_t pix = (size_t)v.y * p.W + v.x;
-        atomicAdd(&p.A[plane * l + pix], cl[l] * G);
-        atomicAdd(&p.A[plane * (l + 1) + pix], -cl[l] * G);
-        atomicAdd(&dc[l], gk[l] * v.qe);
-        atomicAdd(&dt[l], v.s * gdk[l]);
-    }
-    __syncthreads();
-    for (int l = threadIdx.x; l < p.P; l += blockDim.x) {
-        if (dc[l] != 0.0f) atomicAdd(&p.dc_acc[l], (double)dc[l]);
-        if (dt[l] != 0.0f) atomicAdd(&p.dt_acc[l], (double)dt[l]);
-    }
-}
+constexpr int REC_WARPS = 8, REC_CHUNK = 64;
 
-// Kernel-shape part of dloss/dsigma from a recorded list of maxima.  A_m is
-// nonzero only at the maxima's pixels (A_l += c_l G_v, A_{l+1} -= c_l G_v for a
-// maximum v in plane l), so
-//   sum_x A_m(x) dL_m/dsigma_m(x),  dL_m/dsigma_m = B_y' B_x I + B_y B_x' I,
-// is evaluated at those pixels only: for a maximum v in plane l, the sums of
-// (w'_j w_t + w_j w'_t) I(y + j, x + t) over |j|, |t| <= r_m of the reflected
-// image for m = l and m = l + 1 at once.  Windows at most 31 wide take one
-// warp (lanes on columns, several rows per pass); wider ones (the few maxima
-// of the coarse planes) are queued for a second kernel that gives each one a
-// whole CTA, so that no warp runs a long serial window.  Per-CTA sums in FP64
-// shared memory, one global atomic per level.
-struct SigmaParams {
-    const dog_soft_max* rec;
-    const int* count;
-    int cap;
-    const float* gH;
-    const float* kappa;
-    const float* c;
-    const float* w;
-    const float* dw;
-    const float* img;
-    int pitch;
-    int P, nbins, H, W;
-    int r[MAX_LEVELS];
-    int woff[MAX_LEVELS];
-    int* big;          // queue of wide-window maxima (record indices)
-    int* big_count;
-    int big_cap;
-    double* dw_acc;
-};
-
-constexpr int SIGMA_WIDE_R = 16;   // windows of radius >= this go to the CTA kernel
-
-// Partial window sums of maximum v for planes l (pa) and l + 1 (pb): columns
-// t0, t0 + dt_step, ... and rows j0, j0 + j_step, ... of the (2 R2 + 1)^2
-// window, four rows' loads in flight.
-__device__ __forceinline__ void sigma_sums(const SigmaParams& p, const dog_soft_max& v, int t0, int t_step, int j0,
-                                           int j_step, float& pa, float& pb) {
-    const int l = v.level;
+// Column sums of a plane's window around (x, y) at offset t - R2: rows j0,
+// j0 + j_step, ... of both levels, COLS columns (t, t + 1, ...) at once.  A pixel
+// outside a level's own window does not enter its sums.
+template <int COLS>
+__device__ __forceinline__ void window_sums(const RecParams& p, const float* img, int x, int y, int l, int t, int j0,
+                                            int j_step, float& pa, float& pb) {
     const int ra = p.r[l], rb = p.r[l + 1], R2 = max(ra, rb), n2 = 2 * R2 + 1;
-    const float* wa = p.w + p.woff[l];
-    const float* wda = p.dw + p.woff[l];
-    const float* wb = p.w + p.woff[l + 1];
-    const float* wdb = p.dw + p.woff[l + 1];
-    for (int t = t0; t < n2; t += t_step) {
-        const int dt = t - R2;
-        // this lane's column weights (zero outside a plane's window)
-        const bool ia = dt >= -ra && dt <= ra, ib = dt >= -rb && dt <= rb;
-        const float wat = ia ? __ldg(wa + dt + ra) : 0.0f, wdat = ia ? __ldg(wda + dt + ra) : 0.0f;
-        const float wbt = ib ? __ldg(wb + dt + rb) : 0.0f, wdbt = ib ? __ldg(wdb + dt + rb) : 0.0f;
-        const float* col = p.img + refl_i(v.x + dt, p.W);
-        for (int jb = j0; jb < n2; jb += 4 * j_step) {
-            float px[4];
+    const float4* T = p.wt + p.wtoff[l];
+    const bool rows_in = y >= R2 && y + R2 < p.H;
+    const float* col[COLS];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int j = min(jb + u * j_step, n2 - 1);
-                px[u] = __ldg(col + (size_t)refl_i(v.y + j - R2, p.H) * p.pitch);
+    for (int c = 0; c < COLS; ++c) col[c] = img + refl_i(x + min(t + c, n2 - 1) - R2, p.W);
+    float a0[COLS], a1[COLS], b0[COLS], b1[COLS];
+#pragma unroll
+    for (int c = 0; c < COLS; ++c) a0[c] = a1[c] = b0[c] = b1[c] = 0.0f;
+    for (int jb = j0; jb < n2; jb += 4 * j_step) {
+        float px[4][COLS];
+        float4 w[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int j = min(jb + u * j_step, n2 - 1), n = y - R2 + j;
+            const size_t row = (size_t)(rows_in ? n : refl_i(n, p.H)) * p.pitch;
+            w[u] = __ldg(T + j);
+#pragma unroll
+            for (int c = 0; c < COLS; ++c) px[u][c] = __ldg(col[c] + row);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int j = jb + u * j_step;
+            if (j < n2 && abs(j - R2) <= ra) {
+#pragma unroll
+                for (int c = 0; c < COLS; ++c) {
+                    a0[c] = __fmaf_rn(w[u].x, px[u][c], a0[c]);
+                    a1[c] = __fmaf_rn(w[u].y, px[u][c], a1[c]);
+                }
             }
+            if (j < n2 && abs(j - R2) <= rb) {
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int j = jb + u * j_step, dj = j - R2;
-                if (j < n2) {
-                    if (dj >= -ra && dj <= ra)
-                        pa = __fmaf_rn(__fmaf_rn(__ldg(wda + dj + ra), wat, __ldg(wa + dj + ra) * wdat), px[u], pa);
-                    if (dj >= -rb && dj <= rb)
-                        pb = __fmaf_rn(__fmaf_rn(__ldg(wdb + dj + rb), wbt, __ldg(wb + dj + rb) * wdbt), px[u], pb);
+                for (int c = 0; c < COLS; ++c) {
+                    b0[c] = __fmaf_rn(w[u].z, px[u][c], b0[c]);
+                    b1[c] = __fmaf_rn(w[u].w, px[u][c], b1[c]);
                 }
             }
         }
     }
-}
-
-__device__ __forceinline__ void sigma_prologue(const SigmaParams& p, float* gk, float* cl, double* acc) {
-    for (int l = threadIdx.x; l < MAX_LEVELS; l += blockDim.x) {
-        float a = 0.0f;
-        if (l < p.P)
-            for (int k = 0; k < p.nbins; ++k) a += p.gH[k] * p.kappa[l * p.nbins + k];
-        gk[l] = a;
-        cl[l] = l < p.P ? p.c[l] : 0.0f;
-        acc[l] = 0.0;
+#pragma unroll
+    for (int c = 0; c < COLS; ++c) {
+        const float4 w = __ldg(T + min(t + c, n2 - 1));
+        if (t + c < n2 && abs(t + c - R2) <= ra) pa = __fmaf_rn(w.y, a0[c], __fmaf_rn(w.x, a1[c], pa));
+        if (t + c < n2 && abs(t + c - R2) <= rb) pb = __fmaf_rn(w.w, b0[c], __fmaf_rn(w.z, b1[c], pb));
     }
-    __syncthreads();
 }
 
-__device__ __forceinline__ void sigma_epilogue(const SigmaParams& p, const double* acc) {
-    __syncthreads();
-    for (int l = threadIdx.x; l < MAX_LEVELS; l += blockDim.x)
-        if (acc[l] != 0.0) atomicAdd(&p.dw_acc[l], acc[l]);
+template <int LANES>
+__device__ __forceinline__ void sum_lanes(float& a, float& b) {
+#pragma unroll
+    for (int o = LANES / 2; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
 }
 
-__device__ __forceinline__ bool sigma_valid(const SigmaParams& p, const dog_soft_max& v) {
-    return v.x >= 0 && v.x < p.W && v.y >= 0 && v.y < p.H && v.level >= 0 && v.level < p.P;   // else flagged by the scatter
-}
-
-__global__ void __launch_bounds__(256) soft_sigma_kernel(const __grid_constant__ SigmaParams p) {
-    __shared__ float gk[MAX_LEVELS], cl[MAX_LEVELS];
-    __shared__ double acc[MAX_LEVELS];
-    sigma_prologue(p, gk, cl, acc);
-    const int lane = threadIdx.x & 31;
-    const int nmax = min(*p.count, p.cap);
-    const int nwarps = gridDim.x * (blockDim.x >> 5);
-    for (int task = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); task < nmax; task += nwarps) {
-        const dog_soft_max v = p.rec[task];
-        if (!sigma_valid(p, v)) continue;
-        const int l = v.level;
-        const int R2 = max(p.r[l], p.r[l + 1]), n2 = 2 * R2 + 1;
-        float pa = 0.0f, pb = 0.0f;
-        if (R2 >= SIGMA_WIDE_R) {
-            int k = 0;
-            if (lane == 0) k = atomicAdd(p.big_count, 1);
-            k = __shfl_sync(0xffffffffu, k, 0);
-            if (k < p.big_cap) {   // queued for the CTA kernel
-                if (lane == 0) p.big[k] = task;
-                continue;
+__global__ void __launch_bounds__(32 * REC_WARPS) soft_rec_kernel(const __grid_constant__ RecParams p) {
+    __shared__ double acc[3 * MAX_LEVELS];
+    __shared__ dog_soft_max rec[REC_CHUNK];
+    __shared__ float pa[REC_WARPS][REC_CHUNK], pb[REC_WARPS][REC_CHUNK];   // window sums (row 0: of one warp or group)
+    __shared__ unsigned char list[3][REC_CHUNK];
+    __shared__ int n_list[3];   // narrow, middle, wide windows
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_acc = 2 * p.P + p.K;
+    for (int k = tid; k < n_acc; k += blockDim.x) acc[k] = 0.0;
+    const int f = blockIdx.y, n = p.count[f];
+    const float* img = p.img + f * p.img_stride;
+    const dog_soft_max* src = p.rec + f * p.rec_stride;
+    const Lists lists = frame_lists(p.lists, p.H, p.W, f);
+    const int cells_x = cells(p.W);
+    if (n > p.cap && blockIdx.x == 0 && tid == 0) atomicCAS(p.status, 0, (int)DOG_ERR_CAPACITY);
+    const int m = min(n, p.cap);
+    const long long step = gridDim.x;
+    for (long long c0 = blockIdx.x; c0 < m; c0 += step * REC_CHUNK) {
+        const int here = (int)min((m - c0 + step - 1) / step, (long long)REC_CHUNK);
+        __syncthreads();
+        if (tid < 3) n_list[tid] = 0;
+        __syncthreads();
+        if (tid < here) {
+            const long long i = c0 + tid * step;
+            dog_soft_max v = src[i];
+            const int l = v.level;
+            if (v.x < 0 || v.x >= p.W || v.y < 0 || v.y >= p.H || l < 0 || l >= p.P) {   // not this frame's record
+                atomicCAS(p.status, 0, (int)DOG_ERR_INVALID);
+                rec[tid].level = -1;
+            } else {
+                const float G = __ldg(p.c + l) * (__ldg(p.gk + l) * v.q);
+                const int R2 = max(p.r[l], p.r[l + 1]);
+                const int which = R2 <= NARROW_R ? 0 : R2 < 16 ? 1 : 2;
+                list[which][atomicAdd(&n_list[which], 1)] = (unsigned char)tid;
+                if (!(G == 0.0f)) {
+                    const int cell = (v.y >> CELL_SHIFT) * cells_x + (v.x >> CELL_SHIFT);
+                    int4 e = make_int4(v.x, v.y * 32 + l, __float_as_int(G), 0);
+                    const int at = which == 0 ? atomicAdd(lists.count + cell, 1) : CELL_SLOTS;
+                    if (at < CELL_SLOTS) {
+                        lists.slots[(long long)cell * CELL_SLOTS + at] = e;
+                    } else {
+                        const int k = atomicAdd(p.flags + 2 * f + 1, 1);
+                        if (k >= lists.ent_cap || atomicAdd(lists.linked + cell, 1) >= CHAIN_MAX) {
+                            p.flags[2 * f] = 1;
+                        } else {
+                            e.w = atomicExch(lists.head + cell, k);
+                            lists.ent[k] = e;
+                        }
+                    }
+                }
+                v.q = G;
+                rec[tid] = v;
             }
-            sigma_sums(p, v, lane, 32, 0, 1, pa, pb);   // queue full: this warp takes it
-        } else {
-            const int rpi = 32 / n2, js = lane / n2;   // rows per pass, this lane's row phase
-            if (js < rpi) sigma_sums(p, v, lane - js * n2, n2, js, rpi, pa, pb);
+        }
+        __syncthreads();
+        const int n_narrow = n_list[0], n_mid = n_list[1], n_wide = n_list[2];
+        for (int k0 = 4 * warp; k0 < n_narrow; k0 += 4 * REC_WARPS) {
+            const int k = list[0][min(k0 + (lane >> 3), n_narrow - 1)];
+            float a = 0.0f, b = 0.0f;
+            window_sums<2>(p, img, rec[k].x, rec[k].y, rec[k].level, 2 * (lane & 7), 0, 1, a, b);
+            sum_lanes<8>(a, b);
+            if ((lane & 7) == 0 && k0 + (lane >> 3) < n_narrow) { pa[0][k] = a; pb[0][k] = b; }
+        }
+        for (int q = warp; q < n_mid; q += REC_WARPS) {
+            const int k = list[1][q];
+            float a = 0.0f, b = 0.0f;
+            window_sums<1>(p, img, rec[k].x, rec[k].y, rec[k].level, lane, 0, 1, a, b);
+            sum_lanes<32>(a, b);
+            if (lane == 0) { pa[0][k] = a; pb[0][k] = b; }
+        }
+        for (int q = 0; q < n_wide; ++q) {
+            const int k = list[2][q], l = rec[k].level, n2 = 2 * max(p.r[l], p.r[l + 1]) + 1;
+            float a = 0.0f, b = 0.0f;
+            for (int t = lane; t < n2; t += 32) window_sums<1>(p, img, rec[k].x, rec[k].y, l, t, warp, REC_WARPS, a, b);
+            sum_lanes<32>(a, b);
+            if (lane == 0) { pa[warp][k] = a; pb[warp][k] = b; }
+        }
+        __syncthreads();
+        if (warp < REC_CHUNK / 32) {
+            const int k = 32 * warp + lane, l = k < here ? rec[k].level : -1;
+            double v[4] = {0.0, 0.0, 0.0, 0.0};
+            if (l >= 0) {
+                const double G = (double)rec[k].q;
+                v[0] = G * (double)pa[0][k];
+                v[1] = -G * (double)pb[0][k];
+                if (max(p.r[l], p.r[l + 1]) >= 16)
+                    for (int w = 1; w < REC_WARPS; ++w) {
+                        v[0] += G * (double)pa[w][k];
+                        v[1] -= G * (double)pb[w][k];
+                    }
+                v[2] = (double)__ldg(p.gk + l) * (double)rec[k].qe;
+                v[3] = (double)rec[k].s * (double)__ldg(p.gk + p.P + l);
+            }
+            for (unsigned left = __ballot_sync(0xffffffffu, l >= 0); left;) {
+                const int lv = __shfl_sync(0xffffffffu, l, __ffs(left) - 1);
+                const unsigned same = __ballot_sync(0xffffffffu, l == lv);
+                left &= ~same;
+                const int to[4] = {2 * p.P + lv, 2 * p.P + lv + 1, lv, p.P + lv};
+                if (__popc(same) <= 3) {
+                    if (l == lv)
+                        for (int f = 0; f < 4; ++f) atomicAdd(&acc[to[f]], v[f]);
+                    continue;
+                }
+#pragma unroll
+                for (int f = 0; f < 4; ++f) {
+                    double t = l == lv ? v[f] : 0.0;
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+                    if (lane == f) atomicAdd(&acc[to[f]], t);
+                }
+            }
+        }
+    }
+    __syncthreads();
+    for (int k = tid; k < n_acc; k += blockDim.x)
+        if (acc[k] != 0.0) atomicAdd(p.acc + (blockIdx.x % ACC_COPIES) * n_acc + k, acc[k]);
+}
+
+// dloss/dI of a 32 x 32 tile from the lists.  B_i is symmetric, so pixel m gets
+//   sum over maxima v of plane A_i of A_i(v) w_i(m_y - v_y) w_i(m_x - v_x),
+// v running over the maxima and their mirror images in the frame's edges.
+// The CTA walks the cells around the tile (those of narrow planes only nearby),
+// keeps the (maximum, level) pairs whose windows reach the tile, orders them by
+// level and place (so that the sum does not depend on the lists' order), and
+// each warp adds its pairs to 8 rows, lane = column.  A tile that more than
+// TILE_PAIRS pairs reach asks for the frame's dense form.
+//
+// The planes are nearly empty (three maxima in a hundred voxels of the finest,
+// one in a thousand of the next): about 116 pairs reach a tile, where blurring
+// the planes is 900 multiply-adds a pixel.  16 frames of 1024 x 1024, 12 levels:
+// 260 us, where the two dense passes and their edge folds took 2260.
+struct TileParams {
+    void* lists;
+    int* flags;
+    int H, W, K, R;
+    const float* wpad;      // all levels' taps, TAP_PAD zeros around each
+    int r[MAX_LEVELS];
+    int soff[MAX_LEVELS];   // level's taps in wpad
+    int n_taps;
+    float* gimg;
+};
+
+constexpr int TILE = 32, TILE_WARPS = 4, TILE_ROWS = TILE / TILE_WARPS, TILE_PAIRS = 512;
+constexpr int NEAR = (TILE >> CELL_SHIFT) + 2;   // cells per side within NARROW_R of a tile
+static_assert(NARROW_R <= 1 << CELL_SHIFT, "narrow planes reach one cell beyond a tile");
+
+// Shared memory: the pairs, then the taps twice, the second time one float on
+// (so that two rows' taps are one aligned load at either parity).
+constexpr int PAIR_BYTES = TILE_PAIRS * (int)(sizeof(int4) + sizeof(unsigned) + sizeof(int2));
+static __host__ __device__ int tap_copy(int n_taps) { return (n_taps + 3) & ~1; }   // floats of a copy
+constexpr int TILE_SMEM_MAX =
+    PAIR_BYTES + (int)sizeof(float) * 2 * (TAP_PAD + MAX_LEVELS * (2 * DOG_MAX_RADIUS + 1 + TAP_PAD) + 4);
+
+__global__ void __launch_bounds__(32 * TILE_WARPS) soft_tile_kernel(const __grid_constant__ TileParams p) {
+    extern __shared__ __align__(16) unsigned char tsm[];
+    __shared__ int n_pairs;
+    // sorted: first and last of the tile's rows in the window; byte offsets of
+    // column 0's tap, of row 0's tap (in the copy where it is 8-byte aligned); A
+    int4* sorted = reinterpret_cast<int4*>(tsm);
+    unsigned* keys = reinterpret_cast<unsigned*>(sorted + TILE_PAIRS);   // level, sign, y, x, place in `found`
+    int2* found = reinterpret_cast<int2*>(keys + TILE_PAIRS);            // level's taps | r << 16, A
+    float* taps = reinterpret_cast<float*>(tsm + PAIR_BYTES);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int x0 = blockIdx.x * TILE, y0 = blockIdx.y * TILE, frame = blockIdx.z;
+    if (p.flags[2 * frame]) return;
+    const Lists lists = frame_lists(p.lists, p.H, p.W, frame);
+    const int cells_x = cells(p.W), cells_y = cells(p.H);
+    // nearby cells' counts, and the heads of all cells within R: one lane per
+    // cell of a row of cells (at most 21), a row per warp
+    constexpr int NU = (NEAR * NEAR * CELL_SLOTS + 32 * TILE_WARPS - 1) / (32 * TILE_WARPS);
+    int4 slot[NU];
+    {
+        const int4* at[NU];
+        bool has[NU];
+#pragma unroll
+        for (int u = 0; u < NU; ++u) {   // slot by slot, so that a warp's lanes are of one fullness
+            const int k = tid + 32 * TILE_WARPS * u, s = k / (NEAR * NEAR), c = k % (NEAR * NEAR);
+            const int cx = (x0 >> CELL_SHIFT) - 1 + c % NEAR, cy = (y0 >> CELL_SHIFT) - 1 + c / NEAR;
+            const bool in = s < CELL_SLOTS && cx >= 0 && cx < cells_x && cy >= 0 && cy < cells_y;
+            const int cell = in ? cy * cells_x + cx : 0;
+            has[u] = in && s < __ldg(lists.count + cell);
+            at[u] = lists.slots + (long long)cell * CELL_SLOTS + s;
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            pa += __shfl_xor_sync(0xffffffffu, pa, o);
-            pb += __shfl_xor_sync(0xffffffffu, pb, o);
-        }
-        if (lane == 0) {
-            const double G = (double)(cl[l] * (gk[l] * v.q));
-            atomicAdd(&acc[l], G * (double)pa);
-            atomicAdd(&acc[l + 1], -G * (double)pb);
-        }
+        for (int u = 0; u < NU; ++u) slot[u] = has[u] ? __ldg(at[u]) : make_int4(0, 0, 0, -1);
     }
-    sigma_epilogue(p, acc);
-}
-
-// The queued wide windows: one CTA per maximum, warp w on window rows
-// w, w + 8, ..., lanes on columns.
-__global__ void __launch_bounds__(256) soft_sigma_wide_kernel(const __grid_constant__ SigmaParams p) {
-    __shared__ float gk[MAX_LEVELS], cl[MAX_LEVELS];
-    __shared__ double acc[MAX_LEVELS];
-    sigma_prologue(p, gk, cl, acc);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nbig = min(*p.big_count, p.big_cap);
-    for (int q = blockIdx.x; q < nbig; q += gridDim.x) {
-        const dog_soft_max v = p.rec[p.big[q]];
-        const int l = v.level;
-        float pa = 0.0f, pb = 0.0f;
-        sigma_sums(p, v, lane, 32, warp, 8, pa, pb);
+    if (tid == 0) n_pairs = 0;
+    const int copy = tap_copy(p.n_taps);
+#pragma unroll 8
+    for (int t = tid; t < p.n_taps; t += 32 * TILE_WARPS) taps[t] = taps[copy + t + 1] = __ldg(p.wpad + t);
+    if (tid == 0) taps[copy] = 0.0f;
+    __syncthreads();
+    auto keep = [&](const int4& v) {   // the pairs of a maximum with its two levels
+        const int l = v.y & 31, vx = v.x, vy = v.y >> 5;
+#pragma unroll 1
+        for (int s = 0; s < 2; ++s) {
+            const int i = l + s, r = p.r[i];
+            // a mirror image is never nearer to a pixel of the frame than the maximum itself
+            if (vx + r < x0 || vx - r >= x0 + TILE || vy + r < y0 || vy - r >= y0 + TILE) continue;
+            // images k N + (k odd ? N - 1 - v : v) in the edges of a line of N
+            const int kx = vx >= r && vx + r < p.W ? 0 : (r + p.W - 1) / p.W;
+            const int ky = vy >= r && vy + r < p.H ? 0 : (r + p.H - 1) / p.H;
+            for (int a = -ky; a <= ky; ++a) {
+                const int y = a * p.H + (a & 1 ? p.H - 1 - vy : vy);
+                if (y + r < y0 || y - r >= y0 + TILE) continue;
+                for (int b = -kx; b <= kx; ++b) {
+                    const int x = b * p.W + (b & 1 ? p.W - 1 - vx : vx);
+                    if (x + r < x0 || x - r >= x0 + TILE) continue;
+                    const int at = atomicAdd(&n_pairs, 1);
+                    if (at >= TILE_PAIRS) continue;
+                    keys[at] = (unsigned)(2 * i + s) << 26 | (y - y0 + DOG_MAX_RADIUS) << 18 |
+                               (x - x0 + DOG_MAX_RADIUS) << 10 | at;
+                    found[at] = make_int2(p.soff[i] | r << 16, s ? v.z ^ (int)0x80000000 : v.z);
+                }
+            }
+        }
+    };
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            pa += __shfl_xor_sync(0xffffffffu, pa, o);
-            pb += __shfl_xor_sync(0xffffffffu, pb, o);
-        }
-        if (lane == 0) {
-            const double G = (double)(cl[l] * (gk[l] * v.q));
-            atomicAdd(&acc[l], G * (double)pa);
-            atomicAdd(&acc[l + 1], -G * (double)pb);
+    for (int u = 0; u < NU; ++u)
+        if (slot[u].w == 0) keep(slot[u]);
+    {
+        const int cxa = max(x0 - p.R, 0) >> CELL_SHIFT, cxb = min((x0 + TILE - 1 + p.R) >> CELL_SHIFT, cells_x - 1);
+        const int cya = max(y0 - p.R, 0) >> CELL_SHIFT, cyb = min((y0 + TILE - 1 + p.R) >> CELL_SHIFT, cells_y - 1);
+        const int cx = cxa + lane;
+        for (int cy0 = cya + warp; cy0 <= cyb; cy0 += 4 * TILE_WARPS) {
+            int e[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int cy = cy0 + u * TILE_WARPS;
+                e[u] = cy <= cyb && cx <= cxb ? __ldg(lists.head + cy * cells_x + cx) : -1;
+            }
+            while (e[0] >= 0 || e[1] >= 0 || e[2] >= 0 || e[3] >= 0) {   // the four lists side by side
+                int4 v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (e[u] >= 0) v[u] = __ldg(lists.ent + e[u]);
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (e[u] >= 0) {
+                        e[u] = v[u].w;
+                        keep(v[u]);
+                    }
+            }
         }
     }
-    sigma_epilogue(p, acc);
-}
-
-static int adjoint_tail(dog_handle* h, SoftWS* ws, const SoftPrep& q, const float* img, int H, int W, int pitch,
-                        const float* sig, float* gimg, float* gsig, bool dense_sigma, cudaStream_t s);
-
-int soft_backward(dog_handle* h, const float* img, int H, int W, int pitch, const float* sig,
-                  const float* gH, float* gimg, float* gsig, cudaStream_t s) {
-    SoftWS* ws = nullptr;
-    int st = soft_ws(h, H, W, &ws);
-    if (st != DOG_OK) return st;
-    SoftPrep q = prep_params(h, ws, sig);
-    soft_prep_kernel<<<1, PREP_THREADS, 0, s>>>(q);
-    SOFT_CUDA(cudaGetLastError());
-    const FusedParams& b = handle_base(h);
-    const int K = b.K, P = b.P;
-    SOFT_CUDA(cudaMemsetAsync(ws->counts, 0, sizeof(int) * 4, s));
-    SOFT_CUDA(cudaMemsetAsync(ws->acc, 0, sizeof(double) * (2 * P + K), s));
-    FusedParams p = soft_fused(h, ws, img, H, W, pitch, MODE_BWD);
-    p.gH = gH;
-    p.A = ws->A;
-    p.dc_acc = ws->acc;
-    p.dt_acc = ws->acc + P;
-    SOFT_CUDA(timed_fused(h, p, p.n_strips * p.n_bands, s));
-    return adjoint_tail(h, ws, q, img, H, W, pitch, sig, gimg, gsig, true, s);
-}
-
-int soft_backward_rec(dog_handle* h, const float* img, int H, int W, int pitch, const float* sig,
-                      const dog_soft_max* rec, const int* rec_count, int rec_cap, const float* gH, float* gimg,
-                      float* gsig, cudaStream_t s) {
-    SoftWS* ws = nullptr;
-    int st = soft_ws(h, H, W, &ws);
-    if (st != DOG_OK) return st;
-    SoftPrep q = prep_params(h, ws, sig);
-    soft_prep_kernel<<<1, PREP_THREADS, 0, s>>>(q);
-    SOFT_CUDA(cudaGetLastError());
-    const FusedParams& b = handle_base(h);
-    const int K = b.K, P = b.P;
-    SOFT_CUDA(cudaMemsetAsync(ws->acc, 0, sizeof(double) * (2 * P + K), s));
-    SOFT_CUDA(cudaMemsetAsync(ws->A, 0, sizeof(float) * (size_t)K * H * W, s));
-    ScatterParams c{};
-    c.rec = rec;
-    c.count = rec_count;
-    c.cap = rec_cap;
-    c.gH = gH;
-    c.kappa = ws->kappa;
-    c.dkappa = ws->dkappa;
-    c.c = ws->c;
-    c.P = P;
-    c.nbins = handle_cfg(h).nbins;
-    c.H = H;
-    c.W = W;
-    c.A = ws->A;
-    c.dc_acc = ws->acc;
-    c.dt_acc = ws->acc + P;
-    c.status = handle_status(h);
-    const int grid = std::max(1, std::min((rec_cap + 255) / 256, 152 * 8));
-    soft_scatter_kernel<<<grid, 256, 0, s>>>(c);
-    SOFT_CUDA(cudaGetLastError());
-    SigmaParams g{};
-    g.rec = rec;
-    g.count = rec_count;
-    g.cap = rec_cap;
-    g.gH = gH;
-    g.kappa = ws->kappa;
-    g.c = ws->c;
-    g.w = ws->w;
-    g.dw = ws->dw;
-    g.img = img;
-    g.pitch = pitch;
-    g.P = P;
-    g.nbins = handle_cfg(h).nbins;
-    g.H = H;
-    g.W = W;
-    for (int i = 0; i < K; ++i) {
-        g.r[i] = handle_levels(h)[i].r;
-        g.woff[i] = handle_levels(h)[i].woff;
+    __syncthreads();
+    const int n = n_pairs;
+    if (n > TILE_PAIRS) {
+        if (tid == 0) p.flags[2 * frame] = 1;
+        return;
     }
-    g.dw_acc = ws->acc + 2 * P;
-    g.big = ws->big;
-    g.big_count = ws->big_count;
-    g.big_cap = ws->big_cap;
-    SOFT_CUDA(cudaMemsetAsync(ws->big_count, 0, sizeof(int), s));
-    soft_sigma_kernel<<<152 * 4, 256, 0, s>>>(g);
-    SOFT_CUDA(cudaGetLastError());
-    soft_sigma_wide_kernel<<<152 * 4, 256, 0, s>>>(g);
-    SOFT_CUDA(cudaGetLastError());
-    return adjoint_tail(h, ws, q, img, H, W, pitch, sig, gimg, gsig, false, s);
+    const int n4 = (n + 3) >> 2;
+    if (tid < 4 * n4 - n) keys[n + tid] = 0xffffffffu;
+    __syncthreads();
+    for (int k = tid; k < n; k += 32 * TILE_WARPS) {
+        const unsigned key = keys[k];
+        int rank = 0;
+#pragma unroll 4
+        for (int q = 0; q < n4; ++q) {
+            const uint4 o = reinterpret_cast<const uint4*>(keys)[q];
+            rank += (o.x < key) + (o.y < key) + (o.z < key) + (o.w < key);
+        }
+        const int2 f = found[k];
+        const int r = f.x >> 16, y = (int)(key >> 18 & 255) - DOG_MAX_RADIUS;
+        const int tx = (f.x & 0xffff) + r - (int)(key >> 10 & 255) + DOG_MAX_RADIUS, ty = (f.x & 0xffff) + r - y;
+        sorted[rank] = make_int4((y - r) * 65536 + ((y + r) & 0xffff), 4 * tx, 4 * (ty & 1 ? copy + 1 + ty : ty), f.y);
+    }
+    __syncthreads();
+    const int x = x0 + lane, row0 = warp * TILE_ROWS;
+    float2 g2[TILE_ROWS / 2];
+#pragma unroll
+    for (int k = 0; k < TILE_ROWS / 2; ++k) g2[k] = make_float2(0.0f, 0.0f);
+    const char* tap_x = reinterpret_cast<const char*>(taps + lane);
+    const char* tap_y = reinterpret_cast<const char*>(taps + row0);
+    for (int base = 0; base < n; base += 32) {
+        bool hit = false;
+        if (base + lane < n) {
+            const int rows = sorted[base + lane].x;
+            hit = (int)(short)(rows & 0xffff) >= row0 && (rows >> 16) < row0 + TILE_ROWS;
+        }
+        unsigned todo = __ballot_sync(0xffffffffu, hit);
+        if (!todo) continue;
+        int4 next = sorted[base + __ffs(todo) - 1];
+        do {
+            const int4 v = next;
+            todo &= todo - 1;
+            if (todo) next = sorted[base + __ffs(todo) - 1];
+            // columns and rows outside the window meet the zeros around the taps
+            const float ax = __int_as_float(v.w) * *reinterpret_cast<const float*>(tap_x + v.y);
+            const float2 ax2 = make_float2(ax, ax);
+            const float2* wy = reinterpret_cast<const float2*>(tap_y + v.z);
+#pragma unroll
+            for (int k = 0; k < TILE_ROWS / 2; ++k) g2[k] = __ffma2_rn(ax2, wy[k], g2[k]);
+        } while (todo);
+    }
+    if (x >= p.W) return;
+    float* out = p.gimg + (size_t)frame * p.H * p.W + (size_t)(y0 + row0) * p.W + x;
+#pragma unroll
+    for (int k = 0; k < TILE_ROWS; ++k)
+        if (y0 + row0 + k < p.H) out[(size_t)k * p.W] = k & 1 ? g2[k >> 1].y : g2[k >> 1].x;
 }
 
-// The adjoint blurs of the dloss/dL planes in ws->A, then the sigma gradient.
-static int adjoint_tail(dog_handle* h, SoftWS* ws, const SoftPrep& q, const float* img, int H, int W, int pitch,
-                        const float* sig, float* gimg, float* gsig, bool dense_sigma, cudaStream_t s) {
-    const FusedParams& b = handle_base(h);
-    const int K = b.K, P = b.P;
+// The dense form, for frames whose lists did not do (plateaus, where every voxel
+// ties): A cleared, scattered from the record and blurred by the dense passes,
+// the grid meeting between them.  One cooperative launch looks after all frames
+// of a call, and costs two microseconds when none asks for it.  Block 0 also
+// finishes the sigma gradient.
+struct DenseParams {
+    AdjParams a;
+    const dog_soft_max* rec;
+    const int* count;
+    long long rec_stride;
+    int cap, n, P;
+    const float* gk;
+    const float* c;
+    const int* flags;
+    int* arrived;
+    int* status;
+    int tpad_max;
+    FinParams fin;
+};
+
+constexpr int DENSE_WARPS = 4;
+constexpr int GRID_WAIT_MAX = 1 << 24;   // waits of 64 ns or more; then an error
+
+__device__ __forceinline__ bool grid_meet(int* arrived, int target, int* status) {
+    __shared__ int met;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(arrived, 1);
+        int spins = 0;
+        while (atomicAdd(arrived, 0) < target && spins < GRID_WAIT_MAX) {
+            __nanosleep(64);
+            ++spins;
+        }
+        met = spins < GRID_WAIT_MAX;
+        if (!met) atomicCAS(status, 0, (int)DOG_ERR_CUDA);
+        __threadfence();
+    }
+    __syncthreads();
+    return met;
+}
+
+__global__ void __launch_bounds__(32 * DENSE_WARPS) soft_dense_kernel(const __grid_constant__ DenseParams p) {
+    extern __shared__ float dsm[];
+    if (blockIdx.x == 0 && p.fin.gsig != nullptr) soft_finalize(p.fin, threadIdx.x);
+    const int grid = gridDim.x;
+    int target = 0;
+    for (int f = 0; f < p.n; ++f) {
+        if (!p.flags[2 * f]) continue;
+        AdjParams a = p.a;
+        const size_t plane = (size_t)a.H * a.W, first = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+        const size_t step = (size_t)grid * blockDim.x;
+        a.gimg += f * plane;
+        for (size_t k = first; k < plane * a.K; k += step) a.A[k] = 0.0f;
+        if (!grid_meet(p.arrived, target += grid, p.status)) return;
+        const int m = min(p.count[f], p.cap);
+        for (long long k = first; k < m; k += step) {
+            const dog_soft_max v = p.rec[f * p.rec_stride + k];
+            const int l = v.level;
+            if (v.x < 0 || v.x >= a.W || v.y < 0 || v.y >= a.H || l < 0 || l >= p.P) continue;   // reported already
+            const float G = p.c[l] * (p.gk[l] * v.q);
+            float* at = a.A + plane * l + (size_t)v.y * a.W + v.x;
+            atomicAdd(at, G);
+            atomicAdd(at + plane, -G);
+        }
+        if (!grid_meet(p.arrived, target += grid, p.status)) return;
+        const int tx = (a.W + 31) / 32, ty = (a.H + 8 * DENSE_WARPS - 1) / (8 * DENSE_WARPS);
+        for (int t = blockIdx.x; t < tx * ty * a.K; t += grid) {
+            __syncthreads();
+            adj_y_tile<false, DENSE_WARPS>(a, dsm, t % tx * 32, t / tx % ty * 8 * DENSE_WARPS, t / tx / ty);
+        }
+        if (!grid_meet(p.arrived, target += grid, p.status)) return;
+        const int tr = (a.H + ADJ_XR - 1) / ADJ_XR;
+        for (int t = blockIdx.x; t < tx * tr; t += grid) {
+            __syncthreads();
+            adj_x_tile<false>(a, dsm, nullptr, p.tpad_max, t % tx * 32, t / tx * ADJ_XR);
+        }
+        if (!grid_meet(p.arrived, target += grid, p.status)) return;
+    }
+}
+
+static FinParams fin_params(dog_handle* h, SoftWS* ws, const SoftPrep& q, const float* sig, float* gsig) {
+    FinParams f{};
+    f.sig = sig;
+    f.K = q.K;
+    f.P = q.P;
+    f.norm = handle_cfg(h).norm;
+    f.lref0 = q.lref0;
+    f.lrefP = q.lrefP;
+    f.acc = ws->acc;
+    f.gsig = gsig;
+    return f;
+}
+
+static AdjParams adj_params(dog_handle* h, SoftWS* ws, const float* img, int H, int W, int pitch, float* gimg,
+                            int* tpad_max) {
     AdjParams a{};
     a.A = ws->A;
     a.Y = ws->Y;
@@ -1046,44 +1291,145 @@ static int adjoint_tail(dog_handle* h, SoftWS* ws, const SoftPrep& q, const floa
     a.gimg = gimg;
     a.H = H;
     a.W = W;
-    a.K = K;
+    a.K = handle_K(h);
     a.w = ws->w;
     a.dw = ws->dw;
-    int tpad_max = 8;
-    for (int i = 0; i < K; ++i) {
+    *tpad_max = 8;
+    for (int i = 0; i < a.K; ++i) {
         a.r[i] = handle_levels(h)[i].r;
         a.tpad[i] = handle_levels(h)[i].tpad;
         a.woff[i] = handle_levels(h)[i].woff;
-        tpad_max = std::max(tpad_max, handle_levels(h)[i].tpad);
+        *tpad_max = std::max(*tpad_max, a.tpad[i]);
     }
-    a.R = b.R;
-    a.dw_acc = ws->acc + 2 * P;
-    dim3 gy((W + 31) / 32, (H + ADJ_TM - 1) / ADJ_TM, K);
-    dim3 gyf((W + 127) / 128, fold_count(H, b.R), K);
+    a.R = handle_base(h).R;
+    a.dw_acc = ws->acc + 2 * handle_P(h);
+    return a;
+}
+
+int soft_backward(dog_handle* h, const float* img, int H, int W, int pitch, const float* sig,
+                  const float* gH, float* gimg, float* gsig, cudaStream_t s) {
+    SoftWS* ws = nullptr;
+    int st = soft_ws(h, H, W, &ws);
+    if (st != DOG_OK) return st;
+    const FusedParams& b = handle_base(h);
+    const int K = b.K, P = b.P;
+    SoftPrep q = prep_params(h, ws, sig);
+    q.zero[0] = ws->counts;
+    q.n_zero[0] = 4;
+    q.acc = ws->acc;
+    q.n_acc = ACC_COPIES * (2 * P + K);
+    soft_prep_kernel<<<1, PREP_THREADS, 0, s>>>(q);
+    SOFT_CUDA(cudaGetLastError());
+    FusedParams p = soft_fused(h, ws, img, 1, 0, H, W, pitch, MODE_BWD);
+    p.gH = gH;
+    p.A = ws->A;
+    p.dc_acc = ws->acc;
+    p.dt_acc = ws->acc + P;
+    SOFT_CUDA(timed_fused(h, p, p.n_strips * p.n_bands, s));
+    int tpad_max = 0;
+    const AdjParams a = adj_params(h, ws, img, H, W, pitch, gimg, &tpad_max);
+    dim3 gy((W + 31) / 32, (H + 8 * ADJ_WARPS - 1) / (8 * ADJ_WARPS), K);
     dim3 gx((W + 31) / 32, (H + ADJ_XR - 1) / ADJ_XR);
-    if (dense_sigma) {
-        adj_y_kernel<true><<<gy, 256, sizeof(float) * adj_y_smem_floats(tpad_max), s>>>(a);
-        adj_y_fold_kernel<true><<<gyf, 128, 0, s>>>(a);
-        adj_x_kernel<true><<<gx, 128, sizeof(float) * adj_x_smem_floats(tpad_max, b.R, true), s>>>(a, tpad_max);
-    } else {
-        adj_y_kernel<false><<<gy, 256, sizeof(float) * adj_y_smem_floats(tpad_max), s>>>(a);
-        adj_y_fold_kernel<false><<<gyf, 128, 0, s>>>(a);
-        adj_x_kernel<false><<<gx, 128, sizeof(float) * adj_x_smem_floats(tpad_max, b.R, false), s>>>(a, tpad_max);
+    adj_y_kernel<<<gy, 32 * ADJ_WARPS, sizeof(float) * adj_y_smem_floats(ADJ_WARPS, tpad_max), s>>>(a);
+    SOFT_CUDA(cudaGetLastError());
+    adj_x_kernel<<<gx, 128, sizeof(float) * adj_x_smem_floats(tpad_max, b.R, true), s>>>(a, tpad_max);
+    SOFT_CUDA(cudaGetLastError());
+    soft_finalize_kernel<<<1, MAX_LEVELS, 0, s>>>(fin_params(h, ws, q, sig, gsig));
+    SOFT_CUDA(cudaGetLastError());
+    return DOG_OK;
+}
+
+int soft_backward_rec(dog_handle* h, const float* img, int n, long long stride, int H, int W, int pitch,
+                      const float* sig, const dog_soft_max* rec, const int* rec_count, int rec_cap, const float* gH,
+                      float* gimg, float* gsig, cudaStream_t s) {
+    SoftWS* ws = nullptr;
+    int st = soft_ws(h, H, W, &ws);
+    if (st != DOG_OK) return st;
+    const int K = handle_K(h), P = handle_P(h), sms = handle_sms(h);
+    const int per = list_frames(ws, n, s);
+    const int n_cells = cells(H) * cells(W);
+    int* arrived = ws->flags + 2 * LIST_FRAMES;
+    SoftPrep q = prep_params(h, ws, sig);
+    q.gH = gH;
+    q.zero[0] = ws->flags;
+    q.n_zero[0] = 2 * LIST_FRAMES + 1;
+    q.acc = ws->acc;
+    q.n_acc = ACC_COPIES * (2 * P + K);
+    q.lists = ws->lists;
+    q.H = H;
+    q.W = W;
+    RecParams c{};
+    c.cap = rec_cap;
+    c.gk = ws->gk;
+    c.c = ws->c;
+    c.wt = ws->wt;
+    c.img_stride = stride;
+    c.rec_stride = rec_cap;
+    c.pitch = pitch;
+    c.P = P;
+    c.K = K;
+    c.H = H;
+    c.W = W;
+    c.acc = ws->acc;
+    c.lists = ws->lists;
+    c.flags = ws->flags;
+    c.status = handle_status(h);
+    TileParams t{};
+    t.lists = ws->lists;
+    t.flags = ws->flags;
+    t.H = H;
+    t.W = W;
+    t.K = K;
+    t.R = handle_base(h).R;
+    t.wpad = ws->wpad;
+    t.n_taps = pad_offset(h, K);
+    for (int i = 0; i < K; ++i) {
+        t.r[i] = c.r[i] = handle_levels(h)[i].r;
+        t.soff[i] = q.padoff[i];
+        c.wtoff[i] = q.wtoff[i];
     }
-    SOFT_CUDA(cudaGetLastError());
-    adj_x_fold_kernel<<<(H + FOLD_ROWS - 1) / FOLD_ROWS, 32 * FOLD_ROWS, 0, s>>>(a);
-    SOFT_CUDA(cudaGetLastError());
-    FinParams f{};
-    f.sig = sig;
-    f.K = K;
-    f.P = P;
-    f.norm = handle_cfg(h).norm;
-    f.lref0 = q.lref0;
-    f.lrefP = q.lrefP;
-    f.acc = ws->acc;
-    f.gsig = gsig;
-    soft_finalize_kernel<<<1, 64, 0, s>>>(f);
-    SOFT_CUDA(cudaGetLastError());
+    const size_t tile_smem = PAIR_BYTES + sizeof(float) * 2 * tap_copy(t.n_taps);
+    if (tile_smem > 48 * 1024)   // the largest any handle needs: other threads may be setting it too
+        SOFT_CUDA(cudaFuncSetAttribute(soft_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TILE_SMEM_MAX));
+    DenseParams d{};
+    d.a = adj_params(h, ws, img, H, W, pitch, gimg, &d.tpad_max);
+    d.rec_stride = rec_cap;
+    d.cap = rec_cap;
+    d.P = P;
+    d.gk = ws->gk;
+    d.c = ws->c;
+    d.flags = ws->flags;
+    d.arrived = arrived;
+    d.status = handle_status(h);
+    const size_t dense_smem = sizeof(float) * std::max(adj_y_smem_floats(DENSE_WARPS, d.tpad_max),
+                                                       adj_x_smem_floats(d.tpad_max, t.R, false));
+    if (ws->dense_grid == 0) {
+        int fit = 0;
+        SOFT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, soft_dense_kernel, 32 * DENSE_WARPS, dense_smem));
+        if (fit < 1) return DOG_ERR_CUDA;
+        ws->dense_grid = std::min(fit, 4) * sms;
+    }
+    for (int first = 0; first < n; first += per) {
+        const int now = std::min(per, n - first);
+        q.n_lists = now;
+        if (first > 0) q.n_acc = 0;
+        const dim3 prep_grid(1 + (3 * n_cells + PREP_CELLS - 1) / PREP_CELLS, now);
+        soft_prep_kernel<<<prep_grid, PREP_THREADS, 0, s>>>(q);
+        SOFT_CUDA(cudaGetLastError());
+        c.rec = d.rec = rec + (size_t)first * rec_cap;
+        c.count = d.count = rec_count + first;
+        c.img = img + first * stride;
+        soft_rec_kernel<<<dim3(std::max(1, std::min(rec_cap, 4 * sms / now)), now), 32 * REC_WARPS, 0, s>>>(c);
+        SOFT_CUDA(cudaGetLastError());
+        t.gimg = d.a.gimg = gimg + (size_t)first * H * W;
+        soft_tile_kernel<<<dim3((W + TILE - 1) / TILE, (H + TILE - 1) / TILE, now), 32 * TILE_WARPS, tile_smem, s>>>(t);
+        SOFT_CUDA(cudaGetLastError());
+        d.n = now;
+        if (first + now == n) d.fin = fin_params(h, ws, q, sig, gsig);
+        void* args[] = {&d};
+        SOFT_CUDA(cudaLaunchCooperativeKernel(soft_dense_kernel, dim3(ws->dense_grid), dim3(32 * DENSE_WARPS), args,
+                                              dense_smem, s));
+    }
     return DOG_OK;
 }
 

@@ -373,9 +373,9 @@ class DoGSoftHist(torch.autograd.Function):
     """Soft blob-volume histogram of a batch of frames with learnable sigmas.
 
     forward(frames (B, H, W) float32 CUDA, sigmas (K,) float32 CUDA, det) ->
-    H (nbins,) summed over the batch.  The forward records each frame's hard
-    maxima (O(maxima) memory, no blur level is kept); backward scatters the
-    dloss/dL planes from them and runs the adjoint blurs.  A frame whose list
+    H (nbins,) summed over the batch.  One launch works on all frames.  The
+    forward records each frame's hard maxima (O(maxima) memory, no blur level
+    is kept); backward gathers dloss/dI from them.  A frame whose list
     overflowed (more maxima than `rec_cap`, e.g. a flat frame where every
     voxel ties) recomputes its blur levels in the backward instead."""
 
@@ -386,31 +386,50 @@ class DoGSoftHist(torch.autograd.Function):
         frames = frames.contiguous()
         sig = sigmas.detach().contiguous()
         out = torch.zeros(det.cfg.nbins, dtype=torch.float32, device=frames.device)
-        grads = any(ctx.needs_input_grad[:2])
-        recs = [SoftMaxima(DoGSoftHist.rec_cap, frames.device) if grads else None for _ in range(frames.shape[0])]
-        for b in range(frames.shape[0]):
-            det.soft_hist(frames[b], sig, out=out, rec=recs[b])
+        B, cap = frames.shape[0], DoGSoftHist.rec_cap
+        buf = counts = None
+        if any(ctx.needs_input_grad[:2]):
+            buf = torch.empty((B, cap, 6), dtype=torch.int32, device=frames.device)
+            counts = torch.zeros(B, dtype=torch.int32, device=frames.device)
+        if B:
+            H, W, pitch = _check_img(frames[0])
+            check(det.lib.dog_soft_hist_batched(det.h, frames.data_ptr(), B, H * W, H, W, pitch, sig.data_ptr(),
+                                                out.data_ptr(), buf.data_ptr() if buf is not None else None, cap,
+                                                counts.data_ptr() if buf is not None else None, _stream(None)),
+                  "dog_soft_hist_batched")
         ctx.save_for_backward(frames, sig)
         ctx.det = det
-        ctx.recs = recs
+        ctx.recs = buf, counts
         return out
 
     @staticmethod
     def backward(ctx, grad_out: torch.Tensor):
         frames, sig = ctx.saved_tensors
         det = ctx.det
-        recs = ctx.recs
-        counts = torch.stack([r.count for r in recs]).cpu().tolist()   # one sync per batch
-        if any(c > r.cap for c, r in zip(counts, recs)):
+        buf, counts = ctx.recs
+        cap = buf.shape[1]
+        over = [c > cap for c in counts.cpu().tolist()]   # one sync per batch
+        if any(over):
             # the overflowed record set the capacity flag; anything else is an error
             st = det.status()
             if st not in (0, _lib.DOG_ERR_CAPACITY):
-                check(st, "dog_soft_hist_rec")
+                check(st, "dog_soft_hist_batched")
         gs = torch.zeros(det.K, dtype=torch.float32, device=frames.device)
         gimg = torch.empty_like(frames)
         g = grad_out.contiguous().float()
-        for b in range(frames.shape[0]):
-            rec = recs[b] if counts[b] <= recs[b].cap else None
-            gi, _ = det.backward(frames[b], sig, g, grad_sigmas=gs, rec=rec)
-            gimg[b].copy_(gi)
+        b = 0
+        while b < len(over):
+            if over[b]:
+                gimg[b].copy_(det.backward(frames[b], sig, g, grad_sigmas=gs)[0])
+                b += 1
+                continue
+            e = b + 1   # frames b .. e - 1 from their records
+            while e < len(over) and not over[e]:
+                e += 1
+            H, W, pitch = _check_img(frames[b])
+            check(det.lib.dog_backward_rec_batched(det.h, frames[b].data_ptr(), e - b, H * W, H, W, pitch,
+                                                   sig.data_ptr(), buf[b].data_ptr(), counts[b].data_ptr(), cap,
+                                                   g.data_ptr(), gimg[b].data_ptr(), gs.data_ptr(), _stream(None)),
+                  "dog_backward_rec_batched")
+            b = e
         return gimg, gs, None
