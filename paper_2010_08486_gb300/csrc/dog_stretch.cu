@@ -7,10 +7,11 @@
 // map (c - lo) / (hi - lo) is clipped to [0, 1]; counts above 4095 count as
 // 4095.  On the GPU the order statistics come from a 4096-bin histogram per
 // frame (shared-memory counts, one global atomic per nonzero bin and CTA) and
-// a block-wide scan of it; the map itself is applied where the detection
-// kernels ingest the frame (stretch_px) or by stretch_apply_kernel.
+// a scan of it by the frame's last CTA; the map itself is applied where the
+// detection kernels ingest the frame (stretch_px) or by stretch_apply_kernel.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "dog_internal.cuh"
@@ -18,17 +19,29 @@
 
 namespace dogk {
 
-constexpr int HIST_THREADS = 256;
-constexpr int LIM_THREADS = 1024;
-static_assert(STRETCH_BINS == 4 * LIM_THREADS, "four bins per thread in the limits scan");
+constexpr int HIST_THREADS = 512, HIST_WARPS = HIST_THREADS / 32;
+constexpr int BINS_EACH = STRETCH_BINS / HIST_THREADS;   // bins of a thread in the limits scan
 
-// Histogram of frame blockIdx.y; CTAs blockIdx.x take rows blockIdx.x,
-// blockIdx.x + gridDim.x, ...  frames == nullptr: the single frame (img, H, W,
-// pitch).  hist: STRETCH_BINS counts per frame, zeroed by the caller.
-__global__ void __launch_bounds__(HIST_THREADS) stretch_hist_kernel(const dog_frame* frames, const uint16_t* img,
-                                                                    int H, int W, int pitch, int* hist) {
+constexpr int UNIT = 512;   // counts of a row that a warp takes at a time: two loads of eight per lane
+
+// Histogram of frame blockIdx.y by units of its rows, the warps of all its CTAs in
+// turn; then the limits by
+// the CTA that finishes last: the counts at ranks k and n-1-k (k = floor(sat/2 n),
+// at most (n-1)/2) are the bins v with #(c < v) <= rank < #(c <= v).
+// frames == nullptr: the single frame (img, H, W, pitch).  hist: STRETCH_BINS
+// words per frame, zeroed by the caller; the last one counts the finished CTAs
+// (the last bin is what the others leave of the n pixels).  lohi[2f] = lo,
+// lohi[2f+1] = hi.  The additions to the frame's bins bound it (1024 x 1280, with
+// the limits): one CTA of 512 threads per SM takes 7.8 us, two of 256 take 11.6;
+// one count per load in 6 us and the limits as a launch of their own, 3 us and
+// the gap between, came before.
+__global__ void __launch_bounds__(HIST_THREADS) stretch_limits_kernel(const dog_frame* frames, const uint16_t* img,
+                                                                      int H, int W, int pitch, double sat, int* hist,
+                                                                      int* lohi) {
     __shared__ int sh[STRETCH_BINS];
-    const int f = blockIdx.y;
+    __shared__ int wsum[HIST_WARPS];
+    __shared__ bool last;
+    const int f = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (frames) {
         const dog_frame fr = frames[f];
         if (fr.dtype != DOG_DTYPE_U16) return;   // only 12-bit frames are stretched
@@ -37,47 +50,56 @@ __global__ void __launch_bounds__(HIST_THREADS) stretch_hist_kernel(const dog_fr
         W = fr.w;
         pitch = fr.pitch;
     }
-    for (int q = threadIdx.x; q < STRETCH_BINS; q += HIST_THREADS) sh[q] = 0;
+    for (int q = tid; q < STRETCH_BINS; q += HIST_THREADS) sh[q] = 0;
     __syncthreads();
-    for (int y = blockIdx.x; y < H; y += gridDim.x) {
+    auto add = [&](unsigned v) { atomicAdd(&sh[min(v, (unsigned)STRETCH_BINS - 1)], 1); };
+    const int units = max(1, (W + UNIT - 1) / UNIT);   // of a row
+    const long long all = (long long)H * units;
+    for (long long i = blockIdx.x * HIST_WARPS + warp; i < all; i += gridDim.x * HIST_WARPS) {
+        const int y = (int)(i / units), u = (int)(i - (long long)y * units);
         const uint16_t* row = img + (size_t)y * pitch;
-        for (int x = threadIdx.x; x < W; x += HIST_THREADS) {
-            const int v = min((int)__ldg(row + x), STRETCH_BINS - 1);
-            atomicAdd(&sh[v], 1);
+        const int head = min(W, (int)((16 - (reinterpret_cast<size_t>(row) & 15)) & 15) / 2), n8 = (W - head) / 8;
+        const uint4* row8 = reinterpret_cast<const uint4*>(row + head);
+        const int x = u * (UNIT / 8) + lane;
+        uint4 v[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            if (x + 32 * k < n8) v[k] = __ldg(row8 + x + 32 * k);
+        if (u == 0) {
+            if (lane < head) add(__ldg(row + lane));
+            for (int t = head + 8 * n8 + lane; t < W; t += 32) add(__ldg(row + t));
         }
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            if (x + 32 * k < n8) {
+                add(v[k].x & 0xffffu); add(v[k].x >> 16); add(v[k].y & 0xffffu); add(v[k].y >> 16);
+                add(v[k].z & 0xffffu); add(v[k].z >> 16); add(v[k].w & 0xffffu); add(v[k].w >> 16);
+            }
     }
     __syncthreads();
     int* out = hist + (size_t)f * STRETCH_BINS;
-    for (int q = threadIdx.x; q < STRETCH_BINS; q += HIST_THREADS)
+    for (int q = tid; q < STRETCH_BINS - 1; q += HIST_THREADS)
         if (sh[q]) atomicAdd(&out[q], sh[q]);
-}
-
-// Limits of frame blockIdx.x from its histogram: the counts at ranks k and
-// n-1-k (k = floor(sat/2 n), at most (n-1)/2): the bin v with
-// #(c < v) <= rank < #(c <= v).  lohi[2f] = lo, lohi[2f+1] = hi.
-__global__ void __launch_bounds__(LIM_THREADS) stretch_limits_kernel(const dog_frame* frames, int H, int W,
-                                                                     double sat, const int* hist, int* lohi) {
-    __shared__ int wsum[LIM_THREADS / 32];
-    const int f = blockIdx.x;
-    if (frames) {
-        const dog_frame fr = frames[f];
-        if (fr.dtype != DOG_DTYPE_U16) return;
-        H = fr.h;
-        W = fr.w;
-    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last = atomicAdd(&out[STRETCH_BINS - 1], 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
     const long long n = (long long)H * W;
     long long k = (long long)floor(sat * 0.5 * (double)n);
     if (k > (n - 1) / 2) k = (n - 1) / 2;
     const long long r_lo = k, r_hi = n - 1 - k;
-    const int* h = hist + (size_t)f * STRETCH_BINS;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    int c[4];
+    int c[BINS_EACH];
     int tsum = 0;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        c[u] = h[4 * tid + u];
-        tsum += c[u];
+    for (int u = 0; u < BINS_EACH; u += 4) {
+        const int4 b = __ldcg(reinterpret_cast<const int4*>(out + BINS_EACH * tid + u));
+        c[u] = b.x; c[u + 1] = b.y; c[u + 2] = b.z; c[u + 3] = b.w;
     }
+    if (tid == HIST_THREADS - 1) c[BINS_EACH - 1] = 0;
+#pragma unroll
+    for (int u = 0; u < BINS_EACH; ++u) tsum += c[u];
     // block exclusive scan of the per-thread sums
     int incl = tsum;
 #pragma unroll
@@ -87,21 +109,13 @@ __global__ void __launch_bounds__(LIM_THREADS) stretch_limits_kernel(const dog_f
     }
     if (lane == 31) wsum[warp] = incl;
     __syncthreads();
-    if (warp == 0) {
-        int t = wsum[lane];
+    long long below = incl - tsum;   // #(c < BINS_EACH tid)
+    for (int w = 0; w < warp; ++w) below += wsum[w];
+    if (tid == HIST_THREADS - 1) c[BINS_EACH - 1] = (int)(n - below - tsum);
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, t, o);
-            if (lane >= o) t += y;
-        }
-        wsum[lane] = t;
-    }
-    __syncthreads();
-    long long below = (long long)(incl - tsum) + (warp > 0 ? wsum[warp - 1] : 0);   // #(c < 4 tid)
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < BINS_EACH; ++u) {
         const long long upto = below + c[u];   // #(c <= v)
-        const int v = 4 * tid + u;
+        const int v = BINS_EACH * tid + u;
         if (below <= r_lo && r_lo < upto) lohi[2 * f] = v;
         if (below <= r_hi && r_hi < upto) lohi[2 * f + 1] = v;
         below = upto;
@@ -137,15 +151,13 @@ cudaError_t launch_stretch_limits(const dog_frame* frames, int n, const uint16_t
     if (n < 1 || n > 65535) return cudaErrorInvalidValue;   // frames index the grid's y dimension
     cudaError_t e = cudaMemsetAsync(hist, 0, sizeof(int) * STRETCH_BINS * (size_t)n, s);
     if (e != cudaSuccess) return e;
-    // about two CTAs per SM over the whole call; a frame's CTAs split its rows
-    int per = (2 * num_sms + n - 1) / n;
-    if (per < 1) per = 1;
-    if (!frames && per > H) per = H;
-    if (per > 1024) per = 1024;
-    stretch_hist_kernel<<<dim3(per, n), HIST_THREADS, 0, s>>>(frames, img, H, W, pitch, hist);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    stretch_limits_kernel<<<n, LIM_THREADS, 0, s>>>(frames, H, W, sat, hist, lohi);
+    // about one CTA per SM over the whole call; a frame's warps split its rows' units
+    int per = (num_sms + n - 1) / n;
+    if (!frames) {
+        const long long all = (long long)H * ((W + UNIT - 1) / UNIT);
+        per = (int)std::min<long long>(per, (all + HIST_WARPS - 1) / HIST_WARPS);
+    }
+    stretch_limits_kernel<<<dim3(per, n), HIST_THREADS, 0, s>>>(frames, img, H, W, pitch, sat, hist, lohi);
     return cudaGetLastError();
 }
 
