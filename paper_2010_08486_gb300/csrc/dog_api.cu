@@ -318,7 +318,9 @@ void handle_tap_slot(const dog_handle* h, int i, int* base, int* lead) {
 // The form to run for a wish of nw warps (0: no wish): the largest that fits and
 // is not larger than the wish.  More warps hide more latency: on every ladder
 // timed (96 frames of 1024 x 1024) the 12-warp form is the faster one, by 7% to
-// 20%, so it is the default wherever it fits.  What the handle reports without
+// 20%, so it is the default wherever it fits; where it does not, the 10-warp form
+// still beats the 8-warp one (eight 1000 x 1000 frames, sigma 2 to 12.3 in 14
+// levels, which fit 10: 886 us, with 8: 978).  What the handle reports without
 // a wish is the rule that callers know: 12 for ladders of 20 or more levels
 // whose largest level fits an even share of 12 warps, else 8.
 static long long level_cost(const LevelInfo& L) {
@@ -337,7 +339,7 @@ static void use_form(dog_handle* h, int nw) {
     } else {
         h->warps = nw;
     }
-    for (int f : {12, 8, 4, 3})
+    for (int f : {12, 10, 8, 4, 3})
         if ((nw == 0 || f <= nw) && (h->forms >> f & 1)) {
             plan_form(h, f);
             return;
@@ -511,7 +513,7 @@ int dog_create(const dog_config* cfg, dog_t** out) {
     // the fused kernel's shared memory must fit; an FFT-backend handle can do
     // without it (its differentiable and batched calls then report UNSUPPORTED)
     if (b.n_taps4 <= MAX_TAPS4 && direct_limit_bytes(h) + 4096 <= (size_t)optin)
-        for (int f : {12, 8, 4, 3})
+        for (int f : {12, 10, 8, 4, 3})
             if (plan_form(h, f) + 4096 <= optin) h->forms |= 1 << f;
     h->direct_ok = h->forms != 0;
     use_form(h, 0);

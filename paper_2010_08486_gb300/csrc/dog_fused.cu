@@ -9,6 +9,7 @@ DOG_FUSED_FORMS(12)
 cudaError_t launch_fused(const FusedParams& p, int grid, cudaStream_t s) {
     if (p.P < 2 || p.P > MAX_LEVELS - 1) return cudaErrorInvalidValue;
     if (p.nw == 12) return launch_fused_w12(p, grid, s);
+    if (p.nw == 10) return launch_fused_w10(p, grid, s);
     if (p.nw == 8) return launch_fused_w8(p, grid, s);
     if (p.nw == 4) return launch_fused_w4(p, grid, s);
     if (p.nw == 3) return launch_fused_w3(p, grid, s);

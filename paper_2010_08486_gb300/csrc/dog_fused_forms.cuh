@@ -869,6 +869,7 @@ static cudaError_t launch_form(const FusedParams& p, int grid, cudaStream_t s) {
 
 // All forms of one warp count (each translation unit instantiates one).
 cudaError_t launch_fused_w12(const FusedParams& p, int grid, cudaStream_t s);
+cudaError_t launch_fused_w10(const FusedParams& p, int grid, cudaStream_t s);
 cudaError_t launch_fused_w8(const FusedParams& p, int grid, cudaStream_t s);
 cudaError_t launch_fused_w4(const FusedParams& p, int grid, cudaStream_t s);
 cudaError_t launch_fused_w3(const FusedParams& p, int grid, cudaStream_t s);
