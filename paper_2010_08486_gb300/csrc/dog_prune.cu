@@ -176,6 +176,7 @@ struct CellSmem {
     float resp[PRUNE_SMEM_CAND];
     int target[PRUNE_SMEM_CAND];
     unsigned hc[DOG_MAX_NBINS];
+    unsigned short cell[PRUNE_SMEM_CAND];
     unsigned char state[PRUNE_SMEM_CAND], in[PRUNE_SMEM_CAND], und[PRUNE_SMEM_CAND];
     union {   // the edges are gone when the members come
         unsigned edge[PRUNE_THREADS / 32 * EDGE_WARP];
@@ -266,13 +267,14 @@ __device__ __forceinline__ bool prune_cells(const PruneParams& p, PruneSmem& s, 
             r.y[at] = mine[u].y;
             r.level[at] = mine[u].level;
             r.resp[at] = mine[u].response;
+            r.cell[at] = (unsigned short)bk[u];
             r.target[at] = -1;
             r.state[at] = ST_UND;
             r.in[at] = 0;
             r.und[at] = 0;
         }
     __syncthreads();
-    // edges: candidate i and row of cells dy per thread; every warp fills and
+    // edges: candidate i and row of cells dy - 1 per thread; every warp fills and
     // later reads its own part of the list (hits are rare, so they may diverge)
     unsigned* edge = r.edge + (tid >> 5) * EDGE_WARP;
     int* n_edge = &s.wsum[tid >> 5];
@@ -280,12 +282,12 @@ __device__ __forceinline__ bool prune_cells(const PruneParams& p, PruneSmem& s, 
     __syncwarp();
     const int reach = p.cell < 46340 ? p.cell * p.cell : INT_MAX;   // no smaller than any conflict distance squared
     for (int t = tid; t < 3 * n; t += PRUNE_THREADS) {
-        const int i = t / 3, cy0 = t - 3 * i - 1;
+        const int dy = (t >= n) + (t >= 2 * n), i = t - dy * n;
         const int xi = r.x[i], yi = r.y[i];
-        const int cy = (int)((unsigned)(yi - oy) / uc) + cy0, cx = (int)((unsigned)(xi - ox) / uc) + 1;
-        if (cy < 0 || cy >= ny) continue;
-        const int end = s.boff[cy * nx + cx + 2];
-        for (int k = s.boff[cy * nx + cx - 1]; k < end; ++k) {
+        const int c = r.cell[i] + (dy - 1) * nx;
+        if (c < 0 || c >= nx * ny) continue;
+        const int end = s.boff[c + 2];
+        for (int k = s.boff[c - 1]; k < end; ++k) {
             const int ex = r.x[k] - xi, ey = r.y[k] - yi, d = ex * ex + ey * ey;
             if (d >= reach || k == i) continue;
             const int li = min(max(r.level[i], 0), p.P - 1), lk = min(max(r.level[k], 0), p.P - 1);
