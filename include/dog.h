@@ -284,16 +284,19 @@ int dog_detect_batched(dog_t* h, const dog_frame* d_frames, int32_t n, int32_t h
                        void* stream);
 
 /* Row-band height used by detection tiles (a multiple of 8, or 0 for whole
- * frames) and the persistent grid multiplier; set by the autotuner. */
+ * frames) and the persistent grid multiplier; set by the autotuner.  The tiles
+ * of a batch take the height as it is.  A call on one frame evens its bands out
+ * over the frame, in a number next to the asked one; with 0 it takes the number
+ * that fills the GPU.  Results do not depend on it. */
 int dog_set_tiling(dog_t* h, int32_t band_rows, int32_t ctas_per_sm);
 
-/* Producer warps of the detection kernel form: 8 (168 registers each) or 12
- * (128 each), or 0 for the handle's default choice (12 for ladders of 20 or
- * more levels whose largest level fits an even share of 12 warps, else 8).
- * Results do not depend on it: every level is computed by the same
- * operations in either form.  Set by the autotuner; the scale levels are
- * re-balanced over the chosen warps on the host.  Not safe to call while a
- * launch on this handle is being issued from another thread.
+/* Warps of the detection kernel form: at most 8 or at most 12, or 0 for no
+ * bound.  The largest form that fits the ladder's shared memory runs (12, 10, 8,
+ * 4 or 3 warps); the handle reports the asked number, and without one 12 for
+ * ladders of 20 or more levels whose largest level fits an even share of 12
+ * warps, else 8.  Results do not depend on it: every level is computed by the
+ * same operations in every form.  Set by the autotuner.  Not safe to call while
+ * a launch on this handle is being issued from another thread.
  * Errors: INVALID (n not 0, 8 or 12). */
 int dog_set_producer_warps(dog_t* h, int32_t n);
 

@@ -1,6 +1,6 @@
 // Fused DoG detector kernel for sm_103a: the kernel forms, templated on the
-// number of warps, the mode and the source of tiles (dog_fused.cu,
-// dog_fused_soft.cu instantiate them).
+// number of warps, the mode and the source of tiles (dog_fused.cu and
+// dog_fused_w10/w8/w4/w3.cu instantiate them).
 //
 // Method (arXiv 2010.08486): scale space L_i = g(sigma_i) * I (Sec. 3), DoG
 // D_i = c_i (L_i - L_{i+1}) (Eq. 2-3), voxels equal to their 3x3x3 maximum
@@ -35,8 +35,9 @@
 // Measured (96 frames of 1024 x 1024, 12-bit, one batched launch, 12 warps):
 // 25 levels to sigma 7.9 9.87 -> 8.45 ms, 12 levels 1.25^k 9.18 -> 5.8 ms, 6
 // levels to sigma 10.5 6.69 -> 3.6 ms, 14 levels to sigma 12.3 (8 warps) 10.56 ->
-// 9.4 ms, against the form before (levels on fixed producer warps, scalar FMAs,
-// taps and L rows through shared memory).
+// 9.4 ms (another 9% less with the 10 warps that fit), against the form before
+// (levels on fixed producer warps, scalar FMAs, taps and L rows through shared
+// memory).
 //
 // Both passes are register-blocked 1-D correlations: 8 outputs per lane, taps
 // in blocks of 8 against a two-window register file whose halves swap roles
