@@ -799,9 +799,10 @@ __global__ void soft_finalize_kernel(const __grid_constant__ FinParams p) { soft
 // A CTA's records are gridDim apart, which evens out the planes.
 //
 // 16 frames of 1024 x 1024 with 35,000 maxima each, 12 levels, in us: this pass
-// 276 (latency of the small windows' loads and the meetings between A, B and C),
-// where a warp per maximum with all taps formed per pixel took 830, and its
-// scatter into zeroed planes 470.
+// 222 (latency of the small windows' loads and the meetings between A, B and C;
+// with chunks of 64 records, and so four times the meetings, 277), where a warp
+// per maximum with all taps formed per pixel took 830, and its scatter into
+// zeroed planes 470.
 struct RecParams {
     const dog_soft_max* rec;
     const int* count;
@@ -821,7 +822,7 @@ struct RecParams {
     int* status;
 };
 
-constexpr int REC_WARPS = 8, REC_CHUNK = 64;
+constexpr int REC_WARPS = 8, REC_CHUNK = 256;
 
 // Column sums of a plane's window around (x, y) at offset t - R2: rows j0,
 // j0 + j_step, ... of both levels, COLS columns (t, t + 1, ...) at once.  A pixel
