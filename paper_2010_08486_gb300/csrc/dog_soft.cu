@@ -64,7 +64,7 @@ struct SoftWS {
     float* A = nullptr;       // K x H x W
     void* lists = nullptr;    // the record path's lists (see Lists) of n_lists frames
     int n_lists = 0;
-    int* flags = nullptr;     // per listed frame: dense form wanted, entries linked; then the grid barrier's counter
+    int* flags = nullptr;     // per listed frame: FrameFlags; then the grid barrier's counter
     int dense_grid = 0;       // co-resident CTAs of the dense record kernel (0: not asked yet)
     float* Y = nullptr;       // K x H x W
     float* Yd = nullptr;      // K x H x W
@@ -102,6 +102,14 @@ struct Lists {
     int* head;        // cells: first of them, -1 for none
     int n_cells, ent_cap;
     long long ints;   // ints of a frame
+};
+// Words of a listed frame.  The record and the tile kernel each ask for the dense
+// form in a word of its own, so that the tile kernel reads none that its own CTAs
+// write (the warps of one would not see the same value).
+struct FrameFlags {
+    int dense;    // set by the record kernel: the lists do not hold the frame
+    int linked;   // entries linked
+    int tiles;    // set by the tile kernel: a tile is reached by too many pairs
 };
 constexpr int LIST_FRAMES = 64;                      // frames of a batch listed at a time, at most,
 constexpr size_t LIST_BYTES = (size_t)256 << 20;     // and the lists' size (one frame's always fit)
@@ -165,7 +173,7 @@ static int soft_ws(dog_handle* h, int H, int W, SoftWS** out) {
     ok(cudaMalloc(&ws->A, sizeof(float) * plane * K));
     ok(cudaMalloc(&ws->lists, sizeof(int) * frame_lists(nullptr, H, W, 0).ints));
     ws->n_lists = 1;
-    ok(cudaMalloc(&ws->flags, sizeof(int) * (2 * LIST_FRAMES + 1)));
+    ok(cudaMalloc(&ws->flags, sizeof(FrameFlags) * LIST_FRAMES + sizeof(int)));
     ok(cudaMalloc(&ws->Y, sizeof(float) * plane * K));
     ok(cudaMalloc(&ws->Yd, sizeof(float) * plane * K));
     ok(cudaMalloc(&ws->acc, sizeof(double) * ACC_COPIES * (2 * P + K)));
@@ -818,7 +826,7 @@ struct RecParams {
     int wtoff[MAX_LEVELS];
     double* acc;            // dc (P), dt (P), dw (K), ACC_COPIES times
     void* lists;
-    int* flags;             // per frame: the dense form wanted; entries linked
+    FrameFlags* flags;
     int* status;
 };
 
@@ -926,9 +934,9 @@ __global__ void __launch_bounds__(32 * REC_WARPS) soft_rec_kernel(const __grid_c
                     if (at < CELL_SLOTS) {
                         lists.slots[(long long)cell * CELL_SLOTS + at] = e;
                     } else {
-                        const int k = atomicAdd(p.flags + 2 * f + 1, 1);
+                        const int k = atomicAdd(&p.flags[f].linked, 1);
                         if (k >= lists.ent_cap || atomicAdd(lists.linked + cell, 1) >= CHAIN_MAX) {
-                            p.flags[2 * f] = 1;
+                            p.flags[f].dense = 1;
                         } else {
                             e.w = atomicExch(lists.head + cell, k);
                             lists.ent[k] = e;
@@ -1018,7 +1026,7 @@ __global__ void __launch_bounds__(32 * REC_WARPS) soft_rec_kernel(const __grid_c
 // 260 us, where the two dense passes and their edge folds took 2260.
 struct TileParams {
     void* lists;
-    int* flags;
+    FrameFlags* flags;
     int H, W, K, R;
     const float* wpad;      // all levels' taps, TAP_PAD zeros around each
     int r[MAX_LEVELS];
@@ -1049,7 +1057,7 @@ __global__ void __launch_bounds__(32 * TILE_WARPS) soft_tile_kernel(const __grid
     float* taps = reinterpret_cast<float*>(tsm + PAIR_BYTES);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int x0 = blockIdx.x * TILE, y0 = blockIdx.y * TILE, frame = blockIdx.z;
-    if (p.flags[2 * frame]) return;
+    if (p.flags[frame].dense) return;   // (this launch does not write it)
     const Lists lists = frame_lists(p.lists, p.H, p.W, frame);
     const int cells_x = cells(p.W), cells_y = cells(p.H);
     // nearby cells' counts, and the heads of all cells within R: one lane per
@@ -1133,7 +1141,7 @@ __global__ void __launch_bounds__(32 * TILE_WARPS) soft_tile_kernel(const __grid
     __syncthreads();
     const int n = n_pairs;
     if (n > TILE_PAIRS) {
-        if (tid == 0) p.flags[2 * frame] = 1;
+        if (tid == 0) p.flags[frame].tiles = 1;
         return;
     }
     const int n4 = (n + 3) >> 2;
@@ -1200,7 +1208,7 @@ struct DenseParams {
     int cap, n, P;
     const float* gk;
     const float* c;
-    const int* flags;
+    const FrameFlags* flags;
     int* arrived;
     int* status;
     int tpad_max;
@@ -1235,7 +1243,7 @@ __global__ void __launch_bounds__(32 * DENSE_WARPS) soft_dense_kernel(const __gr
     const int grid = gridDim.x;
     int target = 0;
     for (int f = 0; f < p.n; ++f) {
-        if (!p.flags[2 * f]) continue;
+        if (!(p.flags[f].dense | p.flags[f].tiles)) continue;
         AdjParams a = p.a;
         const size_t plane = (size_t)a.H * a.W, first = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
         const size_t step = (size_t)grid * blockDim.x;
@@ -1349,11 +1357,12 @@ int soft_backward_rec(dog_handle* h, const float* img, int n, long long stride, 
     const int K = handle_K(h), P = handle_P(h), sms = handle_sms(h);
     const int per = list_frames(ws, n, s);
     const int n_cells = cells(H) * cells(W);
-    int* arrived = ws->flags + 2 * LIST_FRAMES;
+    FrameFlags* flags = reinterpret_cast<FrameFlags*>(ws->flags);
+    int* arrived = reinterpret_cast<int*>(flags + LIST_FRAMES);
     SoftPrep q = prep_params(h, ws, sig);
     q.gH = gH;
     q.zero[0] = ws->flags;
-    q.n_zero[0] = 2 * LIST_FRAMES + 1;
+    q.n_zero[0] = (int)(sizeof(FrameFlags) / sizeof(int)) * LIST_FRAMES + 1;
     q.acc = ws->acc;
     q.n_acc = ACC_COPIES * (2 * P + K);
     q.lists = ws->lists;
@@ -1373,11 +1382,11 @@ int soft_backward_rec(dog_handle* h, const float* img, int n, long long stride, 
     c.W = W;
     c.acc = ws->acc;
     c.lists = ws->lists;
-    c.flags = ws->flags;
+    c.flags = flags;
     c.status = handle_status(h);
     TileParams t{};
     t.lists = ws->lists;
-    t.flags = ws->flags;
+    t.flags = flags;
     t.H = H;
     t.W = W;
     t.K = K;
@@ -1399,7 +1408,7 @@ int soft_backward_rec(dog_handle* h, const float* img, int n, long long stride, 
     d.P = P;
     d.gk = ws->gk;
     d.c = ws->c;
-    d.flags = ws->flags;
+    d.flags = flags;
     d.arrived = arrived;
     d.status = handle_status(h);
     const size_t dense_smem = sizeof(float) * std::max(adj_y_smem_floats(DENSE_WARPS, d.tpad_max),

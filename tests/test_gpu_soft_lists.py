@@ -106,3 +106,24 @@ def test_batch_replays_in_a_graph():
     _, want_i, want_s, _ = _grads(det, frames, s, gH, 1 << 16)
     assert torch.equal(gi, want_i) and det.status() == 0
     torch.testing.assert_close(gs, want_s, rtol=1e-6, atol=0)
+
+
+def test_tiles_reached_by_too_many_pairs():
+    """A bump on every second pixel of every second row: 16 maxima in a cell of
+    8 x 8, which the lists hold, and up to 790 pairs to a tile, which the tiles
+    do not (those of the right edge do, with 150): some CTAs of a frame ask for
+    the dense form while others are at work, beside frames that need none."""
+    shape, n = (160, 200), 9
+    bumps = np.zeros(shape, np.float32)
+    bumps[::2, ::2] = 0.5
+    imgs = [_frame(*shape, seed=i) + (i % 3 != 1) * bumps for i in range(n)]
+    cfg, det, p, sig0, sig = setup(imgs[0])
+    frames, s = torch.from_numpy(np.stack(imgs)).cuda(), torch.from_numpy(sig).cuda()
+    gH = torch.linspace(-1.0, 2.0, cfg.nbins, device="cuda")
+    _, gi, gs, counts = _grads(det, frames, s, gH, 1 << 14)
+    assert int(counts.max()) <= 1 << 14 and det.status() == 0
+    want_s = torch.zeros_like(gs)
+    for b in range(n):
+        plain, _ = det.backward(frames[b], s, gH, grad_sigmas=want_s)
+        assert torch.linalg.norm(gi[b] - plain) <= 1e-5 * torch.linalg.norm(plain)
+    assert torch.linalg.norm(gs - want_s) <= 1e-4 * torch.linalg.norm(want_s)
