@@ -64,6 +64,8 @@ struct SoftWS {
     float* A = nullptr;       // K x H x W
     void* lists = nullptr;    // the record path's lists (see Lists) of n_lists frames
     int n_lists = 0;
+    void* old_lists[8] = {};  // outgrown (see list_frames)
+    int n_old = 0;
     int* flags = nullptr;     // per listed frame: FrameFlags; then the grid barrier's counter
     int dense_grid = 0;       // co-resident CTAs of the dense record kernel (0: not asked yet)
     float* Y = nullptr;       // K x H x W
@@ -79,6 +81,7 @@ void soft_free(dog_handle* h) {
                     ws->lists, ws->flags, ws->Y, ws->Yd, ws->acc, ws->last_sig};
     for (void* p : ptrs)
         if (p) cudaFree(p);
+    for (int i = 0; i < ws->n_old; ++i) cudaFree(ws->old_lists[i]);
     delete ws;
     handle_soft_ws(h) = nullptr;
 }
@@ -112,6 +115,7 @@ struct FrameFlags {
     int tiles;    // set by the tile kernel: a tile is reached by too many pairs
 };
 constexpr int LIST_FRAMES = 64;                      // frames of a batch listed at a time, at most,
+static_assert(LIST_FRAMES <= 64, "seven growths: SoftWS::old_lists");
 constexpr size_t LIST_BYTES = (size_t)256 << 20;     // and the lists' size (one frame's always fit)
 
 // Frame f's lists (all of a frame's arrays lie together).
@@ -385,16 +389,20 @@ static FusedParams soft_fused(dog_handle* h, SoftWS* ws, const float* img, int n
 }
 
 // Frames of a batch whose lists the workspace holds: grown to the batch unless
-// the stream is being captured (then the batch goes in several passes).
+// the stream is being captured (then the batch goes in several passes).  A graph
+// captured earlier keeps the address of the lists of its time, so outgrown ones
+// are kept with the workspace; each growth but the last at least doubles the
+// frames, so that there are at most seven, together below twice the last.
 static int list_frames(SoftWS* ws, int n, cudaStream_t s) {
     const size_t one = sizeof(int) * (size_t)frame_lists(nullptr, ws->H, ws->W, 0).ints;
-    const int want = (int)std::max<size_t>(1, std::min({(size_t)n, (size_t)LIST_FRAMES, LIST_BYTES / one}));
+    const int most = (int)std::max<size_t>(1, std::min((size_t)LIST_FRAMES, LIST_BYTES / one));
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
-    if (want > ws->n_lists && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+    if (std::min(n, most) > ws->n_lists && cudaStreamIsCapturing(s, &cap) == cudaSuccess &&
+        cap == cudaStreamCaptureStatusNone) {
+        const int want = std::min(most, std::max(n, 2 * ws->n_lists));
         void* more = nullptr;
         if (cudaMalloc(&more, want * one) == cudaSuccess) {
-            cudaDeviceSynchronize();
-            cudaFree(ws->lists);
+            ws->old_lists[ws->n_old++] = ws->lists;
             ws->lists = more;
             ws->n_lists = want;
         } else {

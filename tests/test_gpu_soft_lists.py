@@ -127,3 +127,29 @@ def test_tiles_reached_by_too_many_pairs():
         plain, _ = det.backward(frames[b], s, gH, grad_sigmas=want_s)
         assert torch.linalg.norm(gi[b] - plain) <= 1e-5 * torch.linalg.norm(plain)
     assert torch.linalg.norm(gs - want_s) <= 1e-4 * torch.linalg.norm(want_s)
+
+
+def test_a_graph_outlives_the_growth_of_the_lists():
+    """A graph captured on the lists of its time replays after larger batches of
+    the same frames have replaced them, twice, with other work between; the
+    memory that the graph works on is not handed out again."""
+    imgs = np.stack([_frame(120, 130, seed=i) for i in range(5)])
+    cfg, det, p, sig0, sig = setup(imgs[0])
+    frames, s = torch.from_numpy(imgs).cuda(), torch.from_numpy(sig).cuda()
+    gH = torch.linspace(-1.0, 2.0, cfg.nbins, device="cuda")
+    _grads(det, frames[:1], s, gH, 1 << 16)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        _, gi, gs, _ = _grads(det, frames[:2], s, gH, 1 << 16)
+    g.replay()
+    torch.cuda.synchronize()
+    want_i, want_s = gi.clone(), gs.clone()
+    for n in (2, 5):
+        gi.zero_()
+        _, eager, _, _ = _grads(det, frames[:n], s, gH, 1 << 16)
+        gs.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(gi, want_i) and torch.equal(eager[:2], want_i) and det.status() == 0
+        torch.testing.assert_close(gs, want_s, rtol=1e-6, atol=0)
