@@ -92,10 +92,16 @@ __global__ void __launch_bounds__(HIST_THREADS) stretch_limits_kernel(const dog_
     const long long r_lo = k, r_hi = n - 1 - k;
     int c[BINS_EACH];
     int tsum = 0;
+    const int* mine = out + BINS_EACH * tid;
+    if ((reinterpret_cast<size_t>(out) & 15) == 0) {
 #pragma unroll
-    for (int u = 0; u < BINS_EACH; u += 4) {
-        const int4 b = __ldcg(reinterpret_cast<const int4*>(out + BINS_EACH * tid + u));
-        c[u] = b.x; c[u + 1] = b.y; c[u + 2] = b.z; c[u + 3] = b.w;
+        for (int u = 0; u < BINS_EACH; u += 4) {
+            const int4 b = __ldcg(reinterpret_cast<const int4*>(mine + u));
+            c[u] = b.x; c[u + 1] = b.y; c[u + 2] = b.z; c[u + 3] = b.w;
+        }
+    } else {   // the scratch is the caller's, of any alignment of an int
+#pragma unroll
+        for (int u = 0; u < BINS_EACH; ++u) c[u] = __ldcg(mine + u);
     }
     if (tid == HIST_THREADS - 1) c[BINS_EACH - 1] = 0;
 #pragma unroll
