@@ -252,7 +252,11 @@ static void plan_pairs(dog_handle* h) {
 
 // Largest ladders this build accepts for the direct passes: those whose levels,
 // each with a ring of tpad + 8 rows, 18 response rows and two tap tables, and
-// whose input rows fit the shared memory (some form below fits all of them).
+// whose input rows fit the shared memory.  The smallest form fits all of them: an
+// odd ladder's first level takes a whole pair's ring and the narrower level of a
+// pair the wider one's, so the worst are odd ladders of 11 levels with a wide
+// jump (radii 12 12 45 46 53 53 53 55 61 61 63, the worst found by a search over
+// the ladders at the limit: 221,252 bytes of 228,352; with three warps 232,228).
 static size_t direct_limit_bytes(const dog_handle* h) {
     size_t rings = 0, taps = 0;
     int dmin = 1 << 30, dmax = -(1 << 30);
@@ -339,12 +343,12 @@ static void use_form(dog_handle* h, int nw) {
     } else {
         h->warps = nw;
     }
-    for (int f : {12, 10, 8, 4, 3})
+    for (int f : {12, 10, 8, 4, 3, 2})
         if ((nw == 0 || f <= nw) && (h->forms >> f & 1)) {
             plan_form(h, f);
             return;
         }
-    plan_form(h, 3);   // nothing fits (an FFT-backend handle): never launched
+    plan_form(h, 2);   // nothing fits (an FFT-backend handle): never launched
 }
 
 // Row bands of a single-frame launch (one CTA per strip and band, one CTA per
@@ -513,7 +517,7 @@ int dog_create(const dog_config* cfg, dog_t** out) {
     // the fused kernel's shared memory must fit; an FFT-backend handle can do
     // without it (its differentiable and batched calls then report UNSUPPORTED)
     if (b.n_taps4 <= MAX_TAPS4 && direct_limit_bytes(h) + 4096 <= (size_t)optin)
-        for (int f : {12, 10, 8, 4, 3})
+        for (int f : {12, 10, 8, 4, 3, 2})
             if (plan_form(h, f) + 4096 <= optin) h->forms |= 1 << f;
     h->direct_ok = h->forms != 0;
     use_form(h, 0);

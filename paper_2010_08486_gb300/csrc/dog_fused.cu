@@ -13,6 +13,7 @@ cudaError_t launch_fused(const FusedParams& p, int grid, cudaStream_t s) {
     if (p.nw == 8) return launch_fused_w8(p, grid, s);
     if (p.nw == 4) return launch_fused_w4(p, grid, s);
     if (p.nw == 3) return launch_fused_w3(p, grid, s);
+    if (p.nw == 2) return launch_fused_w2(p, grid, s);
     return cudaErrorInvalidValue;
 }
 

@@ -1,6 +1,6 @@
 // Fused DoG detector kernel for sm_103a: the kernel forms, templated on the
 // number of warps, the mode and the source of tiles (dog_fused.cu and
-// dog_fused_w10/w8/w4/w3.cu instantiate them).
+// dog_fused_w10/w8/w4/w3/w2.cu instantiate them).
 //
 // Method (arXiv 2010.08486): scale space L_i = g(sigma_i) * I (Sec. 3), DoG
 // D_i = c_i (L_i - L_{i+1}) (Eq. 2-3), voxels equal to their 3x3x3 maximum
@@ -885,6 +885,7 @@ cudaError_t launch_fused_w10(const FusedParams& p, int grid, cudaStream_t s);
 cudaError_t launch_fused_w8(const FusedParams& p, int grid, cudaStream_t s);
 cudaError_t launch_fused_w4(const FusedParams& p, int grid, cudaStream_t s);
 cudaError_t launch_fused_w3(const FusedParams& p, int grid, cudaStream_t s);
+cudaError_t launch_fused_w2(const FusedParams& p, int grid, cudaStream_t s);
 #define DOG_FUSED_FORMS(NW)                                                                       \
     cudaError_t launch_fused_w##NW(const FusedParams& p, int grid, cudaStream_t s) {              \
         if (p.frames != nullptr) return launch_form<NW, MODE_CANDIDATES, true>(p, grid, s);       \

@@ -13,7 +13,7 @@ namespace dogk {
 // ---- fused strip kernel geometry --------------------------------------------
 // A CTA owns a strip of TX output columns and walks down a band of rows in
 // blocks of one 8-row chunk per warp, all warps on the same pair of scale
-// levels (dog_fused_forms.cuh).  Forms with 12, 10, 8, 4 and 3 warps; the host
+// levels (dog_fused_forms.cuh).  Forms with 12, 10, 8, 4, 3 and 2 warps; the host
 // runs the largest whose shared memory fits the ladder.
 constexpr int TX = 32;
 constexpr int MB = 8;                          // granularity of row bands
@@ -129,7 +129,7 @@ struct FusedParams {
     int t_off, n_taps4;    // taps (soft modes: copied from w; other modes: the array below)
     int dmin, dmax;        // smallest and largest delta of the pairs
     int smem_bytes;
-    int nw;                // warps of the kernel form (12, 10, 8, 4 or 3)
+    int nw;                // warps of the kernel form (12, 10, 8, 4, 3 or 2)
     int n_pairs;
     int lev_off;           // 1: the first pair's first level is absent
     float cn[MAX_LEVELS];  // P normalisation coefficients (as c)

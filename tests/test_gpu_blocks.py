@@ -63,3 +63,31 @@ def test_non_finite_pixel_reaches_each_level_by_its_own_radius(bad, at):
     blobs, hist, _ = det.detect(dev(img))
     torch.cuda.synchronize()
     assert det.status() == 0 and int(hist.sum()) == blobs.n()
+
+
+# ladders at the limit of the shared memory that three warps no longer hold; the
+# first needs the most of all that were found
+@pytest.mark.parametrize("radii", [[12, 12, 45, 46, 53, 53, 53, 55, 61, 61, 63],
+                                   [12, 13, 42, 42, 54, 54, 57, 58, 61, 61, 63],
+                                   [44, 45, 48, 49, 55, 55, 57, 59, 61, 61, 62],
+                                   [48, 49, 50, 50, 53, 55, 58, 59, 59, 60, 61],
+                                   [44, 45, 50, 50, 51, 56, 57, 58, 62, 62, 62]])
+def test_ladders_of_the_smallest_form(radii):
+    sig = [(r + 0.02 * i) / 4.0 for i, r in enumerate(radii)]
+    cfg = dog.DetectorConfig(sigmas=sig, threshold=0.02, max_h=150, max_w=70, norm=1)
+    det = dog.Detector(cfg)
+    assert det.radii == radii
+    img = synth.plif_frame(synth.PLIF_SEED_BASE + 3, 150, 70)
+    full_check(cfg, img, det=det)
+    # the batched and the differentiable calls hold them too
+    single = det.detect(dev(img))
+    out, counts, hists = det.detect_batched([dev(img)])
+    assert int(counts[0]) == single[0].n() and torch.equal(hists[0], single[1])
+    s = torch.tensor(sig, dtype=torch.float32, device="cuda")
+    rec = dog.SoftMaxima(1 << 16, "cuda")
+    H = det.soft_hist(dev(img), s, rec=rec)
+    gi, gs = det.backward(dev(img), s, torch.ones_like(H), rec=rec)
+    gi2, gs2 = det.backward(dev(img), s, torch.ones_like(H))
+    assert 0 < int(rec.count) <= rec.cap and det.status() == 0
+    assert torch.linalg.norm(gi - gi2) <= 1e-5 * torch.linalg.norm(gi2)
+    assert torch.linalg.norm(gs - gs2) <= 1e-4 * torch.linalg.norm(gs2)
