@@ -290,8 +290,8 @@ int dog_detect_batched(dog_t* h, const dog_frame* d_frames, int32_t n, int32_t h
  * that fills the GPU.  Results do not depend on it. */
 int dog_set_tiling(dog_t* h, int32_t band_rows, int32_t ctas_per_sm);
 
-/* Warps of the detection kernel form: at most 8 or at most 12, or 0 for no
- * bound.  The largest form that fits the ladder's shared memory runs (12, 10, 8,
+/* Warps of the detection kernel form: at most 8 or at most 12, or 0, or the
+ * number that the handle reports before any is set, for no bound.  The largest form that fits the ladder's shared memory runs (12, 10, 8,
  * 4, 3 or 2 warps); the handle reports the asked number, and without one 12 for
  * ladders of 20 or more levels whose largest level fits an even share of 12
  * warps, else 8.  Results do not depend on it: every level is computed by the

@@ -326,23 +326,23 @@ void handle_tap_slot(const dog_handle* h, int i, int* base, int* lead) {
 // still beats the 8-warp one (eight 1000 x 1000 frames, sigma 2 to 12.3 in 14
 // levels, which fit 10: 886 us, with 8: 978).  What the handle reports without
 // a wish is the rule that callers know: 12 for ladders of 20 or more levels
-// whose largest level fits an even share of 12 warps, else 8.
+// whose largest level fits an even share of 12 warps, else 8.  A wish for that
+// number is none: callers read it, time other forms and set it again, and saved
+// tunings hold it.
 static long long level_cost(const LevelInfo& L) {
     const bool tail = ((2 * L.r + 1) & 7) == 1;
     return 10 * (L.tpad / 8) + 17 - (tail ? 8 : 0);
 }
 
 static void use_form(dog_handle* h, int nw) {
-    if (nw == 0) {
-        long long total = 0, biggest = 0;
-        for (const LevelInfo& L : h->lv) {
-            total += level_cost(L);
-            biggest = std::max(biggest, level_cost(L));
-        }
-        h->warps = h->K >= 20 && 12 * biggest <= total ? 12 : 8;
-    } else {
-        h->warps = nw;
+    long long total = 0, biggest = 0;
+    for (const LevelInfo& L : h->lv) {
+        total += level_cost(L);
+        biggest = std::max(biggest, level_cost(L));
     }
+    const int own = h->K >= 20 && 12 * biggest <= total ? 12 : 8;
+    h->warps = nw ? nw : own;
+    if (nw == own) nw = 0;
     for (int f : {12, 10, 8, 4, 3, 2})
         if ((nw == 0 || f <= nw) && (h->forms >> f & 1)) {
             plan_form(h, f);
