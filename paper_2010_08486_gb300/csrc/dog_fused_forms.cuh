@@ -91,7 +91,7 @@ __device__ __forceinline__ unsigned lanemask_lt() {
 
 // Shared scalars of one CTA (static shared memory; the host reserves 4 KB).
 struct SmemSmall {
-    float c[MAX_LEVELS];
+    float c[MAX_LEVELS];      // normalisation (soft modes: its size; sg has the sign)
     float sig[MAX_LEVELS];
     float gk[MAX_LEVELS];     // sum_b gH_b kappa_b(t_l)
     float gdk[MAX_LEVELS];    // sum_b gH_b dkappa_b/dt(t_l)
@@ -102,6 +102,8 @@ struct SmemSmall {
     float dt[MAX_LEVELS];
     PixelSource px;           // the tile in work (load8 reads it here: fewer registers held)
     int tile;
+    float sg[MAX_LEVELS];     // soft modes: the sign of c
+    int flip;                 // soft modes: some c is negative
     int careful;              // a pixel of the tile is not finite (or huge): exact_taps
 };
 static_assert(sizeof(SmemSmall) <= 4096, "reserved next to the dynamic shared memory");
@@ -354,7 +356,7 @@ __device__ __noinline__ void flush(const FusedParams& p, SmemSmall& ss, int x0, 
                     if (idx < p.rec_cap) {
                         const float q = s * (1.0f - s) * p.inv_T;
                         dog_soft_max m;
-                        m.x = x; m.y = y; m.level = l; m.q = q; m.qe = q * e; m.s = s;
+                        m.x = x; m.y = y; m.level = l; m.q = q; m.qe = q * (ss.sg[l] * e); m.s = s;
                         p.rec[(size_t)frame * p.rec_cap + idx] = m;
                     } else {
                         atomicCAS(p.status, 0, (int)DOG_ERR_CAPACITY);
@@ -403,9 +405,9 @@ __device__ __forceinline__ void settle(const FusedParams& p, SmemSmall& ss, cons
                 const float d = __fmul_rn(c, cen[t]);
                 const float s = 1.0f / (1.0f + __expf(-(d - p.thr) * p.inv_T));
                 const float G = ss.gk[l1] * s * (1.0f - s) * p.inv_T;
-                atomicAdd(&ss.dc[l1], G * d / c);
+                atomicAdd(&ss.dc[l1], ss.sg[l1] * (G * d / c));
                 atomicAdd(&ss.dt[l1], s * ss.gdk[l1]);
-                g = c * G;
+                g = ss.sg[l1] * (c * G);
             }
             if (at.own && (at.rows >> t & 1)) {
                 const size_t o = ((size_t)l1 * tc.H + at.y + t) * tc.W + x;
@@ -438,7 +440,8 @@ __device__ __forceinline__ void settle(const FusedParams& p, SmemSmall& ss, cons
 // give the 3x3 maxima of the test rows; then the plane below it in scale, whose
 // centre differences are cen, is settled.  Rows and columns outside the frame
 // hold -inf.  c > 0 and rounding is monotonic, so the maximum of the scaled
-// values is the scaled maximum.  Lanes 0 and 31 receive their own value from
+// values is the scaled maximum.  (In the soft modes the caller's sigmas may
+// cross, which makes c negative: the differences then carry its sign.)  Lanes 0 and 31 receive their own value from
 // the shuffles, which leaves their maximum unchanged: neighbours outside the
 // strip are outside the frame or settled elsewhere.  mprev: maxima of plane
 // l - 1; mout: of plane l; two[t]: the larger of the last two planes' maxima.
@@ -699,6 +702,15 @@ __device__ __forceinline__ void process_tile(const FusedParams& p, float* sm, Sm
                     eB[k] = __fsub_rn(acc[k].x, acc[k].y);
                     Lp[k] = acc[k].y;
                 }
+                if ((MODE == MODE_SOFT || MODE == MODE_BWD) && ss.flip) {
+                    const int l = 2 * q - 1 - off;
+                    const float sa = ss.sg[max(l, 0)], sb = ss.sg[max(l + 1, 0)];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        eA[k] *= sa;
+                        eB[k] *= sb;
+                    }
+                }
                 if (MODE == MODE_DUMP) {
 #pragma unroll
                     for (int s = 0; s < 2; ++s) {
@@ -759,10 +771,14 @@ __global__ void __launch_bounds__(NW * 32, 1) dog_fused_kernel(const __grid_cons
         for (int q = tid; q < p.in_rows * nc; q += NTHREADS) sm[p.in_off + q / nc * p.in_stride + c0 + q % nc] = 0.0f;
     }
     for (int q = tid; q < p.P; q += NTHREADS) {
-        ss.c[q] = p.c[q];
+        ss.c[q] = SOFT ? fabsf(p.c[q]) : p.c[q];
         ss.sig[q] = p.c[p.P + q];
+        if (SOFT) ss.sg[q] = copysignf(1.0f, p.c[q]);
     }
     if (SOFT) {
+        bool neg = false;
+        for (int q = tid; q < p.P; q += NTHREADS) neg |= p.c[q] < 0.0f;
+        ss.flip = __syncthreads_or(neg);
         float4* t4 = reinterpret_cast<float4*>(sm + p.t_off);
         const float4* w4 = reinterpret_cast<const float4*>(p.w);
         for (int q = tid; q < p.n_taps4; q += NTHREADS) t4[q] = w4[q];

@@ -232,3 +232,32 @@ def test_full_frame_gradient_matches_oracle():
                                gH.astype(np.float64), mask)
     assert np.linalg.norm(gi - oi) <= 1e-4 * np.linalg.norm(oi)
     assert np.linalg.norm(gs - osg) <= 1e-4 * np.linalg.norm(osg)
+
+
+@pytest.mark.parametrize("norm", [0, 1])
+@pytest.mark.parametrize("use_rec", [False, True])
+def test_sigmas_that_cross(use_rec, norm):
+    """The ladder is the caller's: a tuning step may move a sigma past its
+    neighbour, which makes that plane's normalisation negative.  Radii stay."""
+    img = crop(synth.GRAD_SEED_BASE + 3, n=96)
+    cfg = dog.grad_config(max_h=96, max_w=96, norm=norm)
+    det = dog.Detector(cfg)
+    p, sig0, rad = parity.oracle_params(cfg), np.asarray(det.sigmas), np.asarray(det.radii)
+    sig = sig0.copy()
+    sig[3], sig[4] = 1.02 * sig0[4], 0.98 * sig0[3]
+    sig[7], sig[8] = 1.02 * sig0[8], 0.98 * sig0[7]
+    sig = sig.astype(np.float32)
+    assert (np.diff(sig) < 0).sum() == 2
+    t, s = torch.from_numpy(img).cuda(), torch.from_numpy(sig).cuda()
+    rec = dog.SoftMaxima(1 << 16, "cuda")
+    H = det.soft_hist(t, s, rec=rec).cpu().numpy().astype(np.float64)
+    mask = check_record_mask(rec, img, sig, rad, p)
+    Ho = oracle.soft_hist(img.astype(np.float64), sig.astype(np.float64), rad, p, sig0, mask)
+    assert np.abs(H - Ho).max() <= 1e-4 * Ho.sum() + 1e-5
+    gH = (2.0 * (Ho - 0.5 * Ho.mean())).astype(np.float32)
+    gi, gs = det.backward(t, s, torch.from_numpy(gH).cuda(), rec=rec if use_rec else None)
+    oi, osg = oracle.soft_grad(img.astype(np.float64), sig.astype(np.float64), rad, p, sig0, gH.astype(np.float64),
+                               mask)
+    assert det.status() == 0
+    assert np.linalg.norm(gi.cpu().numpy() - oi) <= 1e-4 * np.linalg.norm(oi)
+    assert np.linalg.norm(gs.cpu().numpy() - osg) <= 1e-4 * np.linalg.norm(osg)
