@@ -516,9 +516,9 @@ int dog_create(const dog_config* cfg, dog_t** out) {
     }
     // the fused kernel's shared memory must fit; an FFT-backend handle can do
     // without it (its differentiable and batched calls then report UNSUPPORTED)
-    if (b.n_taps4 <= MAX_TAPS4 && direct_limit_bytes(h) + 4096 <= (size_t)optin)
+    if (b.n_taps4 <= MAX_TAPS4 && direct_limit_bytes(h) + SMEM_RESERVE <= (size_t)optin)
         for (int f : {12, 10, 8, 4, 3, 2})
-            if (plan_form(h, f) + 4096 <= optin) h->forms |= 1 << f;
+            if (plan_form(h, f) + SMEM_RESERVE <= optin) h->forms |= 1 << f;
     h->direct_ok = h->forms != 0;
     use_form(h, 0);
     for (int i = 0; i < h->K && h->direct_ok; ++i) {

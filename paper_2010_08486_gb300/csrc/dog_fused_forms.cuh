@@ -89,7 +89,7 @@ __device__ __forceinline__ unsigned lanemask_lt() {
     return m;
 }
 
-// Shared scalars of one CTA (static shared memory; the host reserves 4 KB).
+// Shared scalars of one CTA (static shared memory: SMEM_RESERVE).
 struct SmemSmall {
     float c[MAX_LEVELS];      // normalisation (soft modes: its size; sg has the sign)
     float sig[MAX_LEVELS];
@@ -106,7 +106,7 @@ struct SmemSmall {
     int flip;                 // soft modes: some c is negative
     int careful;              // a pixel of the tile is not finite (or huge): exact_taps
 };
-static_assert(sizeof(SmemSmall) <= 4096, "reserved next to the dynamic shared memory");
+static_assert(sizeof(SmemSmall) <= SMEM_RESERVE, "reserved next to the dynamic shared memory");
 
 // Pixels beyond this magnitude take the careful path (their sums may overflow).
 constexpr float HUGE_PX = 1e37f;
@@ -874,22 +874,22 @@ __global__ void __launch_bounds__(NW * 32, 1) dog_fused_kernel(const __grid_cons
 }
 
 // The dynamic shared-memory limit is raised once per device and kernel form
-// (not on every launch, so launches can be captured into CUDA graphs); atomic
-// because handles on other host threads launch the same forms.
+// (not on every launch, so launches can be captured into CUDA graphs), to the
+// most that any handle asks for: handles of other ladders on other host threads
+// launch the same forms, and setting one size twice is harmless.
 template <int NW, int MODE, bool BATCHED>
 static cudaError_t launch_form(const FusedParams& p, int grid, cudaStream_t s) {
-    static std::atomic<int> limit[64];
-    int dev = 0;
+    static std::atomic<bool> raised[64];
+    int dev = 0, optin = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    std::atomic<int>& lim = limit[dev & 63];
-    if (lim.load(std::memory_order_acquire) < p.smem_bytes) {
-        e = cudaFuncSetAttribute(dog_fused_kernel<NW, MODE, BATCHED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 p.smem_bytes);
+    if (!raised[dev & 63].load(std::memory_order_acquire)) {
+        e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(dog_fused_kernel<NW, MODE, BATCHED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     optin - SMEM_RESERVE);
         if (e != cudaSuccess) return e;
-        int cur = lim.load(std::memory_order_relaxed);
-        while (cur < p.smem_bytes && !lim.compare_exchange_weak(cur, p.smem_bytes)) {
-        }
+        raised[dev & 63].store(true, std::memory_order_release);
     }
     dog_fused_kernel<NW, MODE, BATCHED><<<grid, NW * 32, p.smem_bytes, s>>>(p);
     return cudaGetLastError();

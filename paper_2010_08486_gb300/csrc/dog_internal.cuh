@@ -22,6 +22,7 @@ constexpr int CHUNK = 8 * PAIR_STRIDE;         // 8 rows
 constexpr int MAX_LEVELS = DOG_MAX_LEVELS;
 constexpr int MAX_PAIRS = MAX_LEVELS / 2;
 constexpr int CHUNK_TABLE = 32;                // entries of a pair's table of logical chunks
+constexpr int SMEM_RESERVE = 4096;             // bytes of a CTA's shared memory that no layout takes
 constexpr int QUEUE_CAP = 64;                  // found maxima a warp queues before writing them out
 constexpr int MAX_TAPS4 = 4 * 160;             // float4 of tap blocks (8 taps of two levels each) of all pairs
 

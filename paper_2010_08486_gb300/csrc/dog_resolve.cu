@@ -146,8 +146,9 @@ __global__ void __launch_bounds__(RES_THREADS, 8) dog_resolve_kernel(const __gri
     }
 }
 
-// Raised once per device; atomic because several host threads may launch.
-static std::atomic<int> g_resolve_smem[64];
+// Set once per device, to the largest that any handle needs; atomic because
+// several host threads may launch.
+static std::atomic<bool> g_resolve_attr[64];
 
 cudaError_t launch_resolve(const ResolveParams& p, int max_pending, cudaStream_t s) {
     int R = 0;
@@ -156,13 +157,11 @@ cudaError_t launch_resolve(const ResolveParams& p, int max_pending, cudaStream_t
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    std::atomic<int>& lim = g_resolve_smem[dev & 63];
-    if (smem > 48 * 1024 && lim.load(std::memory_order_acquire) < smem) {
-        e = cudaFuncSetAttribute(dog_resolve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (!g_resolve_attr[dev & 63].load(std::memory_order_acquire)) {
+        e = cudaFuncSetAttribute(dog_resolve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(float) * resolve_smem_floats(DOG_MAX_RADIUS));
         if (e != cudaSuccess) return e;
-        int cur = lim.load(std::memory_order_relaxed);
-        while (cur < smem && !lim.compare_exchange_weak(cur, smem)) {
-        }
+        g_resolve_attr[dev & 63].store(true, std::memory_order_release);
     }
     int grid = max_pending;
     if (grid < 1) grid = 1;

@@ -94,3 +94,38 @@ def test_capacity_overflow_keeps_handle_usable():
     again = det.candidates(img)
     torch.cuda.synchronize()
     assert again.n() == full.n() and det.status() == 0
+
+
+_THREADS = """
+import sys, threading
+import numpy as np, torch
+from paper_2010_08486_gb300 import dog, synth
+img = torch.from_numpy(synth.small_blob_frame(3, 120, 96, n_blobs=9)).cuda()
+cfgs = [dog.plif_config, dog.small_frame_config, dog.grad_config,
+        lambda **k: dog.small_frame_config(sigmas=[1.0, 1.5, 2.0], **k)] * 3
+dets = [c(max_h=120, max_w=96) for c in cfgs]
+dets = [dog.Detector(c) for c in dets]
+start, got = threading.Barrier(len(dets)), [None] * len(dets)
+def work(i):
+    with torch.cuda.stream(torch.cuda.Stream()):
+        start.wait()
+        n = [dets[i].detect(img)[0] for _ in range(3)]
+        torch.cuda.current_stream().synchronize()
+        got[i] = [b.n() for b in n]
+threads = [threading.Thread(target=work, args=(i,)) for i in range(len(dets))]
+torch.cuda.synchronize()
+[t.start() for t in threads]
+[t.join() for t in threads]
+for i, d in enumerate(dets):
+    assert got[i] == [d.detect(img)[0].n()] * 3 and got[i] == got[i % 4] and d.status() == 0, got
+print("threads ok")
+"""
+
+
+def test_first_launches_from_many_threads():
+    """Handles of several ladders whose first launches, of one kernel form with
+    different needs of shared memory, come from many threads at once."""
+    import subprocess
+    import sys
+    r = subprocess.run([sys.executable, "-c", _THREADS], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "threads ok" in r.stdout, r.stdout + r.stderr
