@@ -343,8 +343,8 @@ int dog_soft_hist_rec(dog_t* h, const float* d_img, int32_t img_h, int32_t img_w
  * d_sigmas): dloss/dI is gathered from the maxima whose windows reach a pixel and
  * the sigma gradient is summed over the maxima; no blur level is recomputed (a
  * frame too dense in maxima for that is blurred from its dloss/dL planes, in the
- * same call).  Outputs as in dog_backward.  An incomplete list (*d_count > cap) sets DOG_ERR_CAPACITY and
- * uses the first cap entries. */
+ * same call).  Outputs as in dog_backward.  An incomplete list (*d_count > cap)
+ * sets DOG_ERR_CAPACITY and uses the first cap entries. */
 int dog_backward_rec(dog_t* h, const float* d_img, int32_t img_h, int32_t img_w, int32_t pitch,
                      const float* d_sigmas, const dog_soft_max* d_max, const int32_t* d_count, int32_t cap,
                      const float* d_grad_hist, float* d_grad_img, float* d_grad_sigmas, void* stream);
@@ -416,6 +416,13 @@ int dog_get_status(dog_t* h, int32_t* h_status);
  * again.  -1 switches the injection off.  Process-wide; no counterpart in the
  * paper. */
 int dog_test_fail_alloc(int32_t after);
+
+/* Testing: the rounds (64 ns or more each) that a CTA of this handle's later
+ * launches waits for the others where a kernel's grid meets (the dense form of
+ * dog_backward_rec).  When they run out the status word becomes DOG_ERR_TIMEOUT
+ * and the image gradients in the making NaN.  0: give up at once; -1: the normal
+ * limit of a second or more. */
+int dog_test_wait_limit(dog_t* h, int32_t rounds);
 
 /* Human-readable name of a status code (static string). */
 const char* dog_status_string(int status);

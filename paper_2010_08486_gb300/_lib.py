@@ -35,7 +35,7 @@ EXPORTS = (
     "dog_prune_noalloc", "dog_stretch_limits", "dog_stretch", "dog_render_spheres", "dog_volume_hist", "dog_detect", "dog_detect_batched", "dog_set_tiling", "dog_set_producer_warps", "dog_get_producer_warps", "dog_soft_hist",
     "dog_backward", "dog_soft_hist_rec", "dog_backward_rec", "dog_soft_hist_batched", "dog_backward_rec_batched", "dog_debug_dog", "dog_ring_hist_push", "dog_ring_hist_push_batched",
     "dog_profile_enable", "dog_profile_read", "dog_fma_peak",
-    "dog_get_status", "dog_test_fail_alloc", "dog_status_string",
+    "dog_get_status", "dog_test_fail_alloc", "dog_test_wait_limit", "dog_status_string",
 )
 
 
@@ -142,6 +142,7 @@ def load(path: str | None = None):
         lib.dog_fma_peak.argtypes = [i32, ctypes.c_int64, i32, P(ctypes.c_double), P(ctypes.c_double), vp]
         lib.dog_get_status.argtypes = [vp, P(i32)]
         lib.dog_test_fail_alloc.argtypes = [i32]
+        lib.dog_test_wait_limit.argtypes = [vp, i32]
         lib.dog_status_string.argtypes = [ctypes.c_int]
         lib.dog_status_string.restype = ctypes.c_char_p
         for name in EXPORTS:

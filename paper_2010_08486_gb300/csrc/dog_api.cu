@@ -54,6 +54,7 @@ struct dog_handle {
     int num_sms = 0;
     int band = 0;          // 0: whole frame
     int ctas_per_sm = 1;
+    int wait_limit = -1;   // dog_test_wait_limit
     FusedParams base{};
     std::vector<LevelInfo> lv;
     // device tables
@@ -120,6 +121,7 @@ int handle_band(const dog_handle* h) { return h->band; }
 int handle_w_total(const dog_handle* h) { return h->w_total; }
 const std::vector<LevelInfo>& handle_levels(const dog_handle* h) { return h->lv; }
 int* handle_status(dog_handle* h) { return h->d_status; }
+int handle_wait_limit(const dog_handle* h) { return h->wait_limit; }
 void*& handle_soft_ws(dog_handle* h) { return h->soft_ws; }
 void handle_set_last(dog_handle* h, cudaStream_t s) { h->last = s; }
 
@@ -1112,6 +1114,12 @@ int dog_get_status(dog_t* h, int32_t* h_status) {
     if (cudaMemcpy(&v, h->d_status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return DOG_ERR_CUDA;
     if (cudaMemset(h->d_status, 0, sizeof(int)) != cudaSuccess) return DOG_ERR_CUDA;
     *h_status = v;
+    return DOG_OK;
+}
+
+int dog_test_wait_limit(dog_t* h, int32_t rounds) {
+    if (!h) return DOG_ERR_INVALID;
+    h->wait_limit = rounds;
     return DOG_OK;
 }
 

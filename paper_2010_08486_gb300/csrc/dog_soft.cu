@@ -40,6 +40,7 @@ const dog_config& handle_cfg(const dog_handle* h);
 int handle_band(const dog_handle* h);
 int handle_w_total(const dog_handle* h);
 int handle_sms(const dog_handle* h);
+int handle_wait_limit(const dog_handle* h);
 int pick_band(const FusedParams& b, int num_sms, int H, int n_strips, int asked);
 const std::vector<LevelInfo>& handle_levels(const dog_handle* h);
 void handle_tap_slot(const dog_handle* h, int i, int* base, int* lead);
@@ -1219,30 +1220,40 @@ struct DenseParams {
     const FrameFlags* flags;
     int* arrived;
     int* status;
+    int wait_max;   // rounds of a wait
     int tpad_max;
     FinParams fin;
 };
 
 constexpr int DENSE_WARPS = 4;
-constexpr int GRID_WAIT_MAX = 1 << 24;   // waits of 64 ns or more; then an error
+constexpr int GRID_WAIT_MAX = 1 << 24;   // rounds of a wait, a second or more; then an error
 
-__device__ __forceinline__ bool grid_meet(int* arrived, int target, int* status) {
-    __shared__ int met;
+__device__ __forceinline__ bool grid_meet(const DenseParams& p, int target) {
+    __shared__ bool met;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        atomicAdd(arrived, 1);
-        int spins = 0;
-        while (atomicAdd(arrived, 0) < target && spins < GRID_WAIT_MAX) {
+        atomicAdd(p.arrived, 1);
+        met = atomicAdd(p.arrived, 0) >= target;
+        for (int spins = 0; !met && spins < p.wait_max; ++spins) {
             __nanosleep(64);
-            ++spins;
+            met = atomicAdd(p.arrived, 0) >= target;
         }
-        met = spins < GRID_WAIT_MAX;
-        if (!met) atomicCAS(status, 0, (int)DOG_ERR_CUDA);
+        if (!met) atomicCAS(p.status, 0, (int)DOG_ERR_TIMEOUT);
         __threadfence();
     }
     __syncthreads();
     return met;
+}
+
+// What a CTA whose wait ran out leaves in its share of the frames from f on that
+// wanted the dense form: no half-made gradient.
+__device__ __noinline__ void dense_give_up(const DenseParams& p, int f) {
+    const size_t plane = (size_t)p.a.H * p.a.W;
+    for (; f < p.n; ++f)
+        if (p.flags[f].dense | p.flags[f].tiles)
+            for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < plane; k += (size_t)gridDim.x * blockDim.x)
+                p.a.gimg[f * plane + k] = __int_as_float(0x7fffffff);
 }
 
 __global__ void __launch_bounds__(32 * DENSE_WARPS) soft_dense_kernel(const __grid_constant__ DenseParams p) {
@@ -1257,7 +1268,7 @@ __global__ void __launch_bounds__(32 * DENSE_WARPS) soft_dense_kernel(const __gr
         const size_t step = (size_t)grid * blockDim.x;
         a.gimg += f * plane;
         for (size_t k = first; k < plane * a.K; k += step) a.A[k] = 0.0f;
-        if (!grid_meet(p.arrived, target += grid, p.status)) return;
+        if (!grid_meet(p, target += grid)) return dense_give_up(p, f);
         const int m = min(p.count[f], p.cap);
         for (long long k = first; k < m; k += step) {
             const dog_soft_max v = p.rec[f * p.rec_stride + k];
@@ -1268,19 +1279,19 @@ __global__ void __launch_bounds__(32 * DENSE_WARPS) soft_dense_kernel(const __gr
             atomicAdd(at, G);
             atomicAdd(at + plane, -G);
         }
-        if (!grid_meet(p.arrived, target += grid, p.status)) return;
+        if (!grid_meet(p, target += grid)) return dense_give_up(p, f);
         const int tx = (a.W + 31) / 32, ty = (a.H + 8 * DENSE_WARPS - 1) / (8 * DENSE_WARPS);
         for (int t = blockIdx.x; t < tx * ty * a.K; t += grid) {
             __syncthreads();
             adj_y_tile<false, DENSE_WARPS>(a, dsm, t % tx * 32, t / tx % ty * 8 * DENSE_WARPS, t / tx / ty);
         }
-        if (!grid_meet(p.arrived, target += grid, p.status)) return;
+        if (!grid_meet(p, target += grid)) return dense_give_up(p, f);
         const int tr = (a.H + ADJ_XR - 1) / ADJ_XR;
         for (int t = blockIdx.x; t < tx * tr; t += grid) {
             __syncthreads();
             adj_x_tile<false>(a, dsm, nullptr, p.tpad_max, t % tx * 32, t / tx * ADJ_XR);
         }
-        if (!grid_meet(p.arrived, target += grid, p.status)) return;
+        if (!grid_meet(p, target += grid)) return dense_give_up(p, f);
     }
 }
 
@@ -1419,6 +1430,7 @@ int soft_backward_rec(dog_handle* h, const float* img, int n, long long stride, 
     d.flags = flags;
     d.arrived = arrived;
     d.status = handle_status(h);
+    d.wait_max = handle_wait_limit(h) < 0 ? GRID_WAIT_MAX : handle_wait_limit(h);
     const size_t dense_smem = sizeof(float) * std::max(adj_y_smem_floats(DENSE_WARPS, d.tpad_max),
                                                        adj_x_smem_floats(d.tpad_max, t.R, false));
     if (ws->dense_grid == 0) {

@@ -9,7 +9,7 @@ import torch
 
 import oracle
 from paper_2010_08486_gb300 import build as libbuild
-from paper_2010_08486_gb300 import dog, synth
+from paper_2010_08486_gb300 import _lib, dog, synth
 from tests.test_gpu_soft import check_record_mask, setup
 
 pytestmark = pytest.mark.gpu
@@ -153,3 +153,23 @@ def test_a_graph_outlives_the_growth_of_the_lists():
         torch.cuda.synchronize()
         assert torch.equal(gi, want_i) and torch.equal(eager[:2], want_i) and det.status() == 0
         torch.testing.assert_close(gs, want_s, rtol=1e-6, atol=0)
+
+
+def test_a_wait_that_runs_out_is_reported():
+    """The dense form's CTAs give up at once instead of waiting for one another:
+    the status says so and the frame that wanted the form has no half-made
+    gradient; the frame beside it and the next call are whole."""
+    imgs = [_frame(150, 173), _flat_block(150, 173)]
+    cfg, det, p, sig0, sig = setup(imgs[0])
+    frames, s = torch.from_numpy(np.stack(imgs)).cuda(), torch.from_numpy(sig).cuda()
+    gH = torch.linspace(-1.0, 2.0, cfg.nbins, device="cuda")
+    _, want, _, _ = _grads(det, frames, s, gH, 1 << 18)
+    assert det.status() == 0
+    assert det.lib.dog_test_wait_limit(det.h, 0) == 0
+    _, gi, _, _ = _grads(det, frames, s, gH, 1 << 18)
+    assert det.status() == _lib.DOG_ERR_TIMEOUT
+    assert torch.equal(gi[0], want[0]) and bool(gi[1].isnan().any())
+    assert det.lib.dog_test_wait_limit(det.h, -1) == 0
+    _, gi, _, _ = _grads(det, frames, s, gH, 1 << 18)
+    assert det.status() == 0 and torch.equal(gi[0], want[0])
+    assert torch.linalg.norm(gi[1] - want[1]) <= 1e-5 * torch.linalg.norm(want[1])
