@@ -205,7 +205,8 @@ static_assert(PRUNE_DYN_BYTES + (int)sizeof(PruneSmem) <= 226 * 1024, "shared me
 // the rounds, targets and members run over the edges, and the accepted blobs are
 // binned as they are written.  (Sorting by priority instead, so that it becomes
 // an integer comparison, took 17 us for the sort alone.)  Returns false, having
-// written nothing, when a warp finds more than EDGE_WARP conflicts.
+// written nothing, when a warp finds more than EDGE_WARP conflicts and when the
+// candidates lie too far apart for the grid.
 __device__ __forceinline__ bool prune_cells(const PruneParams& p, PruneSmem& s, CellSmem& r, const dog_blob* cand,
                                             int n, dog_blob* out, int f) {
     const int tid = threadIdx.x, lane = tid & 31;
@@ -248,6 +249,10 @@ __device__ __forceinline__ bool prune_cells(const PruneParams& p, PruneSmem& s, 
     const long long wx = n ? r.box[1] - ox : 0, wy = n ? r.box[3] - oy : 0;
     long long cell = p.cell;
     while ((wx / cell + 3) * (wy / cell + 1) > NBUCKET) cell *= 2;
+    // (candidates of neighbouring cells are less than two cells apart; of cells
+    // this large, in frames of more than 2^24 rows, the squared distance would not
+    // fit an int)
+    if (cell > 16384) return false;
     const int nx = (int)(wx / cell) + 3, ny = (int)(wy / cell) + 1;
     const unsigned uc = (unsigned)cell;   // (at most the extent, below 2^32)
 #pragma unroll

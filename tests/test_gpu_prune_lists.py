@@ -40,3 +40,24 @@ def test_prune_of_a_list(n, size, mode):
     want.sigma = want.sigma.astype(np.float32).astype(np.float64)
     assert parity.same_blob_sets(parity.blobs_to_oracle(*out.to_numpy()), want)
     assert det.status() == 0
+
+
+def test_candidates_far_apart():
+    """A grid that spans the frame has cells of tens of thousands of rows here:
+    candidates 2^16 rows apart, whose squared distance is 0 in 32 bits, do not
+    conflict; close ones at the far end do."""
+    h = 60_000_001
+    cfg = dog.small_frame_config(max_h=64, max_w=64, blob_cap=64)
+    det = dog.Detector(cfg)
+    y = np.array([0, 65536, 131072, 30_000_000, 30_065_536, h - 1, h - 2], np.int32)
+    x = np.array([3, 3, 3, 5, 5, 9, 9], np.int32)
+    level = np.full(7, 2, np.int32)
+    resp = (np.arange(1, 8) / 8.0).astype(np.float32)
+    sig = np.asarray(det.sigmas, np.float32)[level]
+    raw = np.zeros((64, 5), np.int32)
+    raw[:7] = np.stack([x, y, level, sig.view(np.int32), resp.view(np.int32)], 1)
+    cand = dog.BlobList(torch.from_numpy(raw).cuda(), torch.tensor(7, dtype=torch.int32, device="cuda"))
+    out = det.prune(cand, h, 16)
+    torch.cuda.synchronize()
+    got = out.to_numpy()
+    assert sorted(got[1].tolist()) == [0, 65536, 131072, 30_000_000, 30_065_536, h - 2] and det.status() == 0
