@@ -16,7 +16,8 @@
 //
 // A CTA renders a 32 x 32 tile: it first lists, in table order, the spheres
 // whose disc (plus one pixel) meets the tile; spheres left out contribute
-// exactly zero to every sample of the tile, so the sums are unchanged.  A warp
+// exactly zero to every sample of the tile, so the sums are unchanged (see
+// beside).  A warp
 // then takes four blocks of 16 x 2 pixels and skips the listed spheres that miss
 // its block.
 //
@@ -66,6 +67,18 @@ __device__ __forceinline__ uint32_t sum12(unsigned long long pix, uint32_t draw0
     return s;
 }
 
+// The sphere (cx, cy, R, A) contributes exactly zero to every sample of the pixels
+// x0 .. x1, y0 .. y1: its disc and a pixel around it are beside them.  R enters as
+// R^2 only, so its sign does not count.  Of larger spheres the rounding of d^2 /
+// R^2 could let a sample outside the disc through (R = 5e6: 1 - d^2 / R^2 is 4e-7
+// a pixel outside, with an error of up to 3e-7), and an amplitude that is not
+// finite makes even a zero count: those are never left out.
+__device__ __forceinline__ bool beside(const float4& q, float x0, float x1, float y0, float y1) {
+    const float m = fabsf(q.z) + 1.0f;
+    const bool meets = q.x + m >= x0 - 0.5f && q.x - m <= x1 + 0.5f && q.y + m >= y0 - 0.5f && q.y - m <= y1 + 0.5f;
+    return !meets && m < 1.0e6f && fabsf(q.w) < INFINITY;
+}
+
 // The count of one pixel as defined, in double.
 __device__ __noinline__ uint16_t count_exact(double gain, float I, double read_noise, uint32_t s1, uint32_t s2) {
     const double z1 = (double)s1 * (1.0 / 16777216.0) - 6.0, z2 = (double)s2 * (1.0 / 16777216.0) - 6.0;
@@ -85,19 +98,14 @@ __global__ void __launch_bounds__(RTHREADS) render_spheres_kernel(const float4* 
     __shared__ int n_list;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int x0 = blockIdx.x * RT, y0 = blockIdx.y * RT;
-    const float tx0 = (float)x0 - 0.5f, tx1 = (float)(x0 + RT) - 0.5f;
-    const float ty0 = (float)y0 - 0.5f, ty1 = (float)(y0 + RT) - 0.5f;
     if (tid == 0) n_list = 0;
     __syncthreads();
     // spheres meeting the tile, in table order (chunks of RTHREADS, block scan)
     for (int base = 0; base < S; base += RTHREADS) {
         const int s = base + tid;
         bool keep = false;
-        if (s < S) {
-            const float4 q = __ldg(sph + s);
-            const float m = q.z + 1.0f;
-            keep = q.x + m >= tx0 && q.x - m <= tx1 && q.y + m >= ty0 && q.y - m <= ty1;
-        }
+        if (s < S)
+            keep = !beside(__ldg(sph + s), (float)x0, (float)(x0 + RT - 1), (float)y0, (float)(y0 + RT - 1));
         const unsigned mask = __ballot_sync(0xffffffffu, keep);
         if (lane == 0) wsum[warp] = __popc(mask);
         __syncthreads();
@@ -123,10 +131,7 @@ __global__ void __launch_bounds__(RTHREADS) render_spheres_kernel(const float4* 
         float I = bg;
         for (int t = 0; t < n; ++t) {
             const float4 q = __ldg(sph + list[t]);
-            const float m = q.z + 1.0f;
-            if (!(q.x + m >= (float)bx - 0.5f && q.x - m <= (float)bx + 15.5f && q.y + m >= (float)by - 0.5f &&
-                  q.y - m <= (float)by + 1.5f))
-                continue;   // no sample of the block is inside
+            if (beside(q, (float)bx, (float)(bx + 15), (float)by, (float)(by + 1))) continue;
             const float inv_r2 = __fdiv_rn(1.0f, __fmul_rn(q.z, q.z));
             float acc = 0.0f;
             for (int j = 0; j < ss; ++j) {

@@ -31,3 +31,22 @@ def test_counts_at_rounding_edges(h, w, n, bg, gain, rn):
     want_i, want_c = oracle.render_spheres(table, h, w, ss=4, background=bg, gain=gain, read_noise=rn, seed=h + w)
     assert np.array_equal(inten.cpu().numpy().view(np.uint32), want_i.view(np.uint32))
     assert np.array_equal(counts.cpu().numpy().view(np.uint16), want_c)
+
+
+@pytest.mark.parametrize("spheres", [
+    [(20.0, 30.0, -6.0, 0.7), (50.0, 10.0, -2.5, 0.4)],          # the radius enters squared
+    [(3.0e7, 20.0, 3.0e7, 0.5), (40.0, -9.0e6, 9.0e6, 0.3)],     # an edge that single precision blurs over pixels
+    [(20.0, 20.0, 5.0, float("inf"))],                           # inf * 0 outside the disc
+    [(20.0, 20.0, float("nan"), 0.5), (float("nan"), 3.0, 4.0, 0.5), (30.0, 40.0, 0.0, 0.5)],
+])
+def test_spheres_out_of_the_ordinary(spheres):
+    """The sum over all spheres as written, whatever tile or block a pixel is in."""
+    table = np.array(spheres + [(33.0, 33.0, 7.0, 0.25)], np.float32)
+    counts, inten = dog.render_spheres(torch.from_numpy(table).cuda(), 70, 80, ss=2, seed=5, with_intensity=True)
+    torch.cuda.synchronize()
+    want_i, want_c = oracle.render_spheres(table, 70, 80, ss=2, background=0.05, gain=2000.0, read_noise=4.0, seed=5)
+    got_i = inten.cpu().numpy()
+    assert np.array_equal(np.isnan(got_i), np.isnan(want_i))
+    ok = ~np.isnan(want_i)
+    assert np.array_equal(got_i[ok].view(np.uint32), want_i[ok].view(np.uint32))
+    assert np.array_equal(counts.cpu().numpy().view(np.uint16)[ok], want_c[ok])
