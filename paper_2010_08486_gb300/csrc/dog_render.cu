@@ -31,6 +31,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cfloat>
+
 #include "dog.h"
 
 namespace {
@@ -121,7 +123,9 @@ __global__ void __launch_bounds__(RTHREADS) render_spheres_kernel(const float4* 
     }
     const int n = n_list;
     const float inv_n = 1.0f / (float)(ss * ss), half_ss = 0.5f / (float)ss;   // exact: ss is a power of two
-    const float gain_f = (float)gain, rn_f = (float)read_noise;
+    // (a gain below the normal range of single precision has lost digits: NaN, so
+    // that no count is decided in single precision)
+    const float gain_f = fabs(gain) < (double)FLT_MIN && gain != 0.0 ? NAN : (float)gain, rn_f = (float)read_noise;
 #pragma unroll 1
     for (int blk = 0; blk < 4; ++blk) {
         // block of 16 x 2 pixels: warp rows 4 w .. 4 w + 3, two blocks side by side

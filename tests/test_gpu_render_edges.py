@@ -50,3 +50,16 @@ def test_spheres_out_of_the_ordinary(spheres):
     ok = ~np.isnan(want_i)
     assert np.array_equal(got_i[ok].view(np.uint32), want_i[ok].view(np.uint32))
     assert np.array_equal(counts.cpu().numpy().view(np.uint16)[ok], want_c[ok])
+
+
+@pytest.mark.parametrize("gain", [1e-39, 3e-41, 2e-44, 1e-46])
+def test_gains_below_single_precision(gain):
+    """Bright intensities times a gain that single precision holds in a few bits
+    or not at all, with sums of all sizes around a rounding edge."""
+    table = np.zeros((0, 4), np.float32)
+    bg = float(np.float32(min(40.0 / gain, 3.0e38)))   # 40 photons where a float can be that bright
+    counts = dog.render_spheres(torch.from_numpy(table).cuda(), 300, 400, ss=1, background=bg, gain=gain,
+                                read_noise=0.25, seed=3)
+    torch.cuda.synchronize()
+    _, want = oracle.render_spheres(table, 300, 400, ss=1, background=bg, gain=gain, read_noise=0.25, seed=3)
+    assert np.array_equal(counts.cpu().numpy().view(np.uint16), want)
