@@ -38,10 +38,13 @@ def test_equals_eight_warp_form(h, w):
 
 def _form(det, img):
     """The fused kernel's instance (its number of warps first) that a call runs."""
-    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
-        det.candidates(img)
-        torch.cuda.synchronize()
-    names = [e.key for e in prof.key_averages() if "dog_fused_kernel" in e.key]
+    for _ in range(4):   # (a process's first trace may come back empty)
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+            det.candidates(img)
+            torch.cuda.synchronize()
+        names = [e.key for e in prof.key_averages() if "dog_fused_kernel" in e.key]
+        if names:
+            break
     assert len(names) == 1
     return names[0]
 
