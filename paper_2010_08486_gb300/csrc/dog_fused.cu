@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(1024) dog_batch_prep_kernel(const dog_frame* f
             d.dtype = (stretch && fr.dtype == DOG_DTYPE_U16) ? DTYPE_U16_STRETCH : fr.dtype;
             d.blob_off = (long long)f * blob_cap;
             d.n_strips = (fr.w + TX - 1) / TX;
-            d.band = (band > 0 && band < fr.h) ? band : fr.h;
+            d.band = min((band > 0 && band < fr.h) ? band : fr.h, MAX_TILE_ROWS);
             d.n_bands = (fr.h + d.band - 1) / d.band;
             tiles = (long long)d.n_strips * d.n_bands;
             cand_off[f] = (long long)f * blob_cap;

@@ -291,14 +291,18 @@ __device__ __forceinline__ void chunk_table(int* table, const PairInfo& U, int n
 // ---------------------------------------------------------------------------
 // Maxima a warp has found, kept in its own shared-memory queue and written out
 // (or added to the soft histogram) 32 lanes at a time.
-// entry: .x = row (21 bits, counted from the queue's base row) | lane << 21 |
-// plane << 26 | strip edge << 31; .y = L_l - L_{l+1} there.  A tile may have more
-// rows than that (a batched frame of any height in one band): a warp whose next
-// rows are out of range writes its queue out and moves the base to them.
-constexpr int QUEUE_ROWS = 1 << 21;
-__device__ __forceinline__ unsigned q_code(int dy, int lane, int l, bool edge) {
-    return (unsigned)dy | (unsigned)lane << 21 | (unsigned)l << 26 | (unsigned)edge << 31;
+// entry: .x = row (21 bits) | lane << 21 | plane << 26 | strip edge << 31; .y = L_l -
+// L_{l+1} there.  Rows count from the tile's first in detection, whose batched
+// frames may have any number of rows (their tiles have at most MAX_TILE_ROWS; a base
+// that a warp moves along instead cost 11 to 17% of the kernel's time, because the
+// compiler then keeps less in registers), and from the frame's first in the soft
+// modes, whose frames have at most 65,535.
+static_assert(MAX_TILE_ROWS <= 1 << 21, "rows of a queue entry");
+__device__ __forceinline__ unsigned q_code(int y, int lane, int l, bool edge) {
+    return (unsigned)y | (unsigned)lane << 21 | (unsigned)l << 26 | (unsigned)edge << 31;
 }
+template <int MODE>
+__device__ __forceinline__ int q_base(int y0) { return MODE == MODE_CANDIDATES ? y0 : 0; }
 
 template <int MODE>
 __device__ __noinline__ void flush(const FusedParams& p, SmemSmall& ss, int x0, int y_base, int frame,
@@ -308,7 +312,7 @@ __device__ __noinline__ void flush(const FusedParams& p, SmemSmall& ss, int x0, 
     for (int i0 = 0; i0 < n; i0 += 32) {
         const bool have = i0 + lane < n;
         const uint2 v = have ? queue[i0 + lane] : make_uint2(0u, 0u);
-        const int y = y_base + (int)(v.x & (QUEUE_ROWS - 1)), x = x0 + (int)((v.x >> 21) & 31), l = (v.x >> 26) & 31;
+        const int y = y_base + (int)(v.x & ((1 << 21) - 1)), x = x0 + (int)((v.x >> 21) & 31), l = (v.x >> 26) & 31;
         const bool edge = v.x >> 31;
         const float e = __uint_as_float(v.y);
         const float d = __fmul_rn(ss.c[l], e);
@@ -374,7 +378,6 @@ __device__ __noinline__ void flush(const FusedParams& p, SmemSmall& ss, int x0, 
 // Everything a warp's test needs to know about its place.
 struct TestPlace {
     int y;           // image row of test row 0
-    int y_base;      // row that the queue's rows count from
     unsigned rows;   // bit t: test row t belongs to the tile
     bool own, edge;  // this lane settles its column; its neighbours lie in the adjacent strip
 };
@@ -420,7 +423,7 @@ __device__ __forceinline__ void settle(const FusedParams& p, SmemSmall& ss, cons
     }
     while (__any_sync(0xffffffffu, mask != 0u)) {
         if (qn + 32 > QUEUE_CAP) {
-            flush<MODE>(p, ss, tc.x0, at.y_base, tc.frame, tc.blobs, tc.count, queue, qn);
+            flush<MODE>(p, ss, tc.x0, q_base<MODE>(tc.y0), tc.frame, tc.blobs, tc.count, queue, qn);
             qn = 0;
         }
         const unsigned bal = __ballot_sync(0xffffffffu, mask != 0u);
@@ -430,7 +433,7 @@ __device__ __forceinline__ void settle(const FusedParams& p, SmemSmall& ss, cons
             float e = cen[0];
 #pragma unroll
             for (int u = 1; u < 8; ++u) e = t == u ? cen[u] : e;
-            queue[qn + __popc(bal & lanemask_lt())] = make_uint2(q_code(at.y + t - at.y_base, lane, l1, at.edge), __float_as_uint(e));
+            queue[qn + __popc(bal & lanemask_lt())] = make_uint2(q_code(at.y + t - q_base<MODE>(tc.y0), lane, l1, at.edge), __float_as_uint(e));
         }
         qn += __popc(bal);
     }
@@ -600,7 +603,6 @@ __device__ __forceinline__ void process_tile(const FusedParams& p, float* sm, Sm
     int par = 0;     // buffer half of the current interval's pair
     int abs0 = 0;    // chunks before the current block (ring slots are taken modulo e)
     at.rows = 0u;
-    at.y_base = yb0 - 1;
     for (int b = 0;; ++b) {   // block nblk: only the last planes' test
         const int yb = yb0 + MBK * b;
         const bool last = b + 1 == nblk;
@@ -614,11 +616,6 @@ __device__ __forceinline__ void process_tile(const FusedParams& p, float* sm, Sm
             const int lq = q ? q - 1 : n - 1;      // and this was its pair
             if (TEST && q == 1) {   // the planes tested from here on are this block's
                 at.y = yw - 1;
-                if (at.y + 8 - at.y_base > QUEUE_ROWS) {
-                    flush<MODE>(p, ss, tc.x0, at.y_base, tc.frame, tc.blobs, tc.count, queue, qn);
-                    qn = 0;
-                    at.y_base = at.y;
-                }
                 const int lo = max(tc.y0 - at.y, 0), hi = min(tc.y1 - at.y, 8);   // test rows lo .. hi-1
                 at.rows = hi > lo && (MODE != MODE_CANDIDATES || p.thr < INFINITY) ? ((1u << hi) - 1u) & ~((1u << lo) - 1u) : 0u;
             }
@@ -685,7 +682,7 @@ __device__ __forceinline__ void process_tile(const FusedParams& p, float* sm, Sm
                 }
             }
             if (b == nblk) {
-                if (TEST && qn) flush<MODE>(p, ss, tc.x0, at.y_base, tc.frame, tc.blobs, tc.count, queue, qn);
+                if (TEST && qn) flush<MODE>(p, ss, tc.x0, q_base<MODE>(tc.y0), tc.frame, tc.blobs, tc.count, queue, qn);
                 __syncthreads();
                 return;
             }

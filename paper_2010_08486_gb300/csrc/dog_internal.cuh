@@ -21,6 +21,7 @@ constexpr int PAIR_STRIDE = 2 * TX;            // floats per row of a pair's hor
 constexpr int CHUNK = 8 * PAIR_STRIDE;         // 8 rows
 constexpr int MAX_LEVELS = DOG_MAX_LEVELS;
 constexpr int MAX_PAIRS = MAX_LEVELS / 2;
+constexpr int MAX_TILE_ROWS = 1 << 20;         // rows of a tile, at most
 constexpr int CHUNK_TABLE = 32;                // entries of a pair's table of logical chunks
 constexpr int SMEM_RESERVE = 4096;             // bytes of a CTA's shared memory that no layout takes
 constexpr int QUEUE_CAP = 64;                  // found maxima a warp queues before writing them out
