@@ -104,7 +104,7 @@ struct SmemSmall {
     int tile;
     float sg[MAX_LEVELS];     // soft modes: the sign of c
     int flip;                 // soft modes: some c is negative
-    int careful;              // a pixel of the tile is not finite (or huge): exact_taps
+    int careful;              // a pixel of the tile is not finite (or huge): correlate_exact
 };
 static_assert(sizeof(SmemSmall) <= SMEM_RESERVE, "reserved next to the dynamic shared memory");
 
@@ -120,10 +120,6 @@ struct Taps {
     const FusedParams& p;
     const float4* sm;
     __device__ __forceinline__ float4 operator()(int q) const { return CT ? p.taps[q] : sm[q]; }
-    __device__ __forceinline__ float one(int q, int t, int half) const {   // tap t of one level of the pair at q
-        const float4 v = (*this)(q + (t >> 1));
-        return (t & 1) ? (half ? v.w : v.z) : (half ? v.y : v.x);
-    }
 };
 
 // acc[k] += (w_lo[u], w_hi[u]) * X[k + u], u = 0..7: both levels on the same
@@ -182,21 +178,61 @@ __device__ __forceinline__ void correlate(float2 (&acc)[8], Load load, const Tap
     }
 }
 
-// The same sums over one level's real taps only, for tiles with non-finite (or
+// The same sums over each level's real taps only, for tiles with non-finite (or
 // huge) pixels: a zero tap of the padded windows would turn an infinity outside
 // the level's own window into a NaN.  For finite inputs the zero taps add
-// nothing, so both forms give the same bits.  in(k) is input k of the pair's
-// window; the level's own taps are d .. 2 rw - d of its 2 rw + 1.
-template <bool CT, class In>
-__device__ __forceinline__ void exact_taps(float (&acc)[8], In in, const Taps<CT>& tap, int q, int half, int d,
-                                           int rw) {
+// nothing, so both forms give the same bits.  The pair's window has 2 r + 1 taps,
+// of which the first level has those from d to 2 r - d.  Blocks of taps that both
+// levels have are taken as above; the others tap by tap.  (A loop over taps with
+// loads of its own per level made the detection of a 1024 x 1024 frame with one
+// such pixel take 680 us; this 240, and without such pixels 165.)
+__device__ __forceinline__ float second(float x) { return x; }
+__device__ __forceinline__ float second(float2 x) { return x.y; }
+
+template <class T, bool CT>
+__device__ __forceinline__ void exact_block(float2 (&acc)[8], const T (&A)[8], const T (&B)[8], const Taps<CT>& tap,
+                                            int q, int t0, int d, int last) {
+    if (t0 >= d && t0 + 7 <= last - d) {
+        fma_block(acc, A, B, tap, q);
+        return;
+    }
 #pragma unroll
-    for (int k = 0; k < 8; ++k) acc[k] = 0.0f;
+    for (int u = 0; u < 8; ++u) {
+        const float4 w4 = tap(q + (u >> 1));
+        const float2 w = u & 1 ? make_float2(w4.z, w4.w) : make_float2(w4.x, w4.y);
+        if (t0 + u >= d && t0 + u <= last - d) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) acc[k] = __ffma2_rn(w, both((k + u < 8) ? A[k + u] : B[k + u - 8]), acc[k]);
+        } else if (t0 + u <= last) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                acc[k].y = __fmaf_rn(w.y, second((k + u < 8) ? A[k + u] : B[k + u - 8]), acc[k].y);
+        }
+    }
+}
+
+template <class T, bool CT, class Load>
+__device__ __forceinline__ void correlate_exact(float2 (&acc)[8], Load load, const Taps<CT>& tap, int q, int nb,
+                                                bool tail, int d, int last) {
+    T A[8], B[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) acc[k] = make_float2(0.0f, 0.0f);
+    load(A);
 #pragma unroll 1
-    for (int t = d; t <= 2 * rw - d; ++t) {
-        const float w = tap.one(q, t, half);
+    for (int t = 0; t < 8 * nb; t += 8) {
+        load(B);
+        exact_block(acc, A, B, tap, q, t, d, last);
+        q += 4;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) acc[k] = __fmaf_rn(w, in(k + t), acc[k]);
+        for (int k = 0; k < 8; ++k) A[k] = B[k];
+    }
+    if (tail) {   // tap 8 nb, the last one: both levels' if their windows are the same
+        if (d == 0) {
+            fma_tail(acc, A, tap, q);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) acc[k].y = __fmaf_rn(tap(q).y, second(A[k]), acc[k].y);
+        }
     }
 }
 
@@ -211,34 +247,50 @@ __device__ __forceinline__ int chunk_off(int row, int x) {   // float offset of 
     return row * PAIR_STRIDE + 4 * (4 * g + (j ^ chunk_swz(row, g))) + 2 * (x & 1);
 }
 
+// Sums of the horizontal pass into a chunk.
+__device__ __forceinline__ void store_sums(float* dst, int rho, int g, const float2 (&acc)[8]) {
+    float4* d4 = reinterpret_cast<float4*>(dst + rho * PAIR_STRIDE + 16 * g);
+    const int swz = chunk_swz(rho, g);
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        d4[j ^ swz] = make_float4(acc[2 * j].x, acc[2 * j].y, acc[2 * j + 1].x, acc[2 * j + 1].y);
+}
+
+// The horizontal pass over real taps only, src as in hpass.  Out of line: inlined
+// beside the usual path it changes that one's registers (one frame of 1024 x 1024
+// 124 -> 140 us).
+template <bool CT>
+__device__ __noinline__ void hpass_exact(const FusedParams& p, const PairInfo& U, const float* sm, const float* src,
+                                         float* dst) {
+    const Taps<CT> tap{p, reinterpret_cast<const float4*>(sm + p.t_off)};
+    const int lane = threadIdx.x & 31, rho = lane >> 2, g = lane & 3;
+    float2 acc[8];
+    correlate_exact<float>(acc, [&](float (&X)[8]) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) X[k] = src[k];
+        src += 8;
+    }, tap, U.tap, U.nb, U.tail != 0, U.lead, 2 * U.r);
+    store_sums(dst, rho, g, acc);
+}
+
 // Horizontal pass of pair U for 8 rows: lane (rho, g) columns 8g .. 8g+7 of row
 // rho; row: this lane's input row (column 0 is frame column x0 - R).
 template <bool CT>
-__device__ __forceinline__ void hpass(const PairInfo& U, const float* row, int R, float* dst, const Taps<CT>& tap,
-                                      bool careful) {
+__device__ __forceinline__ void hpass(const PairInfo& U, const float* sm, const float* row, int R, float* dst,
+                                      const Taps<CT>& tap, bool careful) {
     const int lane = threadIdx.x & 31, rho = lane >> 2, g = lane & 3;
     const float* src = row + (R - U.r) + 8 * g;
-    if (!careful) {
-        float2 acc[8];
-        correlate<float>(acc, [&](float (&X)[8]) {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) X[k] = src[k];
-            src += 8;
-        }, tap, U.tap, U.nb, U.tail != 0);
-        float4* d4 = reinterpret_cast<float4*>(dst + rho * PAIR_STRIDE + 16 * g);
-        const int swz = chunk_swz(rho, g);
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            d4[j ^ swz] = make_float4(acc[2 * j].x, acc[2 * j].y, acc[2 * j + 1].x, acc[2 * j + 1].y);
-    } else {
-#pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
-            float acc[8];
-            exact_taps(acc, [&](int k) { return src[k]; }, tap, U.tap, h, h ? 0 : U.lead, U.r);
-#pragma unroll
-            for (int k = 0; k < 8; ++k) dst[chunk_off(rho, 8 * g + k) + h] = acc[k];
-        }
+    if (careful) {
+        hpass_exact<CT>(tap.p, U, sm, src, dst);
+        return;
     }
+    float2 acc[8];
+    correlate<float>(acc, [&](float (&X)[8]) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) X[k] = src[k];
+        src += 8;
+    }, tap, U.tap, U.nb, U.tail != 0);
+    store_sums(dst, rho, g, acc);
 }
 
 // Vertical pass of pair U for chunk w of the block: lane = column.  The window
@@ -250,26 +302,17 @@ template <bool CT>
 __device__ __forceinline__ void vpass(const PairInfo& U, const float* sm, const int* at, const Taps<CT>& tap,
                                       bool careful, float2 (&acc)[8]) {
     const int lane = threadIdx.x & 31;
-    if (!careful) {
-        const int off_e = chunk_off(0, lane), off_o = chunk_off(1, lane);
-        correlate<float2>(acc, [&](float2 (&X)[8]) {
-            const float* c = sm + *at++;
+    const int off_e = chunk_off(0, lane), off_o = chunk_off(1, lane);
+    auto load = [&](float2 (&X)[8]) {
+        const float* c = sm + *at++;
 #pragma unroll
-            for (int k = 0; k < 8; k += 2) {
-                X[k] = *reinterpret_cast<const float2*>(c + off_e + k * PAIR_STRIDE);
-                X[k + 1] = *reinterpret_cast<const float2*>(c + off_o + k * PAIR_STRIDE);
-            }
-        }, tap, U.tap, U.nb, U.tail != 0);
-    } else {
-#pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
-            float s[8];
-            exact_taps(s, [&](int k) { return sm[at[k >> 3] + chunk_off(k & 7, lane) + h]; }, tap, U.tap, h,
-                       h ? 0 : U.lead, U.r);
-#pragma unroll
-            for (int k = 0; k < 8; ++k) (h ? acc[k].y : acc[k].x) = s[k];
+        for (int k = 0; k < 8; k += 2) {
+            X[k] = *reinterpret_cast<const float2*>(c + off_e + k * PAIR_STRIDE);
+            X[k + 1] = *reinterpret_cast<const float2*>(c + off_o + k * PAIR_STRIDE);
         }
-    }
+    };
+    if (!careful) correlate<float2>(acc, load, tap, U.tap, U.nb, U.tail != 0);
+    else correlate_exact<float2>(acc, load, tap, U.tap, U.nb, U.tail != 0, U.lead, 2 * U.r);
 }
 
 // n mod e without a division (n < 2^28, e <= 17; rcp = ceil(2^32 / e), 0 for e = 1).
@@ -578,7 +621,7 @@ __device__ __forceinline__ void process_tile(const FusedParams& p, float* sm, Sm
             const PairInfo& U = p.pairs[q];
             const int c = U.e - NW * m + warp;
             if (c >= 0 && c < U.e)
-                hpass(U, row_of(U), R, sm + U.ring_off + c * CHUNK, tap, ss.careful != 0);
+                hpass(U, sm, row_of(U), R, sm + U.ring_off + c * CHUNK, tap, ss.careful != 0);
         }
         __syncthreads();
         int s = base + 8 * warp;   // over the rows no longer read
@@ -586,7 +629,7 @@ __device__ __forceinline__ void process_tile(const FusedParams& p, float* sm, Sm
         base = (base + MBK) % CIN;
         __syncthreads();
     }
-    hpass(p.pairs[0], row_of(p.pairs[0]), R, wbuf + warp * CHUNK, tap, ss.careful != 0);
+    hpass(p.pairs[0], sm, row_of(p.pairs[0]), R, wbuf + warp * CHUNK, tap, ss.careful != 0);
     __syncthreads();
 
     // test state between planes: the scaled 3x3 maxima m1 of the last plane (m2 is
@@ -640,7 +683,7 @@ __device__ __forceinline__ void process_tile(const FusedParams& p, float* sm, Sm
             // it before the test, so that the test's comparisons meet other warps' FMAs
             auto ahead = [&]() {
                 const PairInfo& N = p.pairs[q + 1];
-                hpass(N, row_of(N), R, wbuf + (par ^ 1) * (NW * CHUNK) + warp * CHUNK, tap, careful);
+                hpass(N, sm, row_of(N), R, wbuf + (par ^ 1) * (NW * CHUNK) + warp * CHUNK, tap, careful);
             };
             const bool go = q + 1 < n && act && b < nblk;
             if (go && (warp & 4)) ahead();
@@ -743,7 +786,7 @@ __device__ __forceinline__ void process_tile(const FusedParams& p, float* sm, Sm
                 __syncthreads();
                 base = (base + MBK) % CIN;
                 if (yw + MBK <= ylast)
-                    hpass(p.pairs[0], row_of(p.pairs[0]), R,
+                    hpass(p.pairs[0], sm, row_of(p.pairs[0]), R,
                           wbuf + (par ^ 1) * (NW * CHUNK) + warp * CHUNK, tap, ss.careful != 0);
             }
             __syncthreads();

@@ -91,3 +91,30 @@ def test_ladders_of_the_smallest_form(radii):
     assert 0 < int(rec.count) <= rec.cap and det.status() == 0
     assert torch.linalg.norm(gi - gi2) <= 1e-5 * torch.linalg.norm(gi2)
     assert torch.linalg.norm(gs - gs2) <= 1e-4 * torch.linalg.norm(gs2)
+
+
+@pytest.mark.parametrize("sig", [[1.6 ** i for i in range(6)], [1.0, 5.0, 5.25, 12.0, 12.02], [0.5, 9.0, 15.0]])
+def test_non_finite_pixel_beside_levels_of_very_different_radii(sig):
+    """As above where one level of a pair has many taps fewer than the other, whole
+    blocks of them, and for the differentiable form's maxima away from the pixel."""
+    h, w, at = 190, 100, (97, 33)
+    cfg = dog.DetectorConfig(sigmas=sig, threshold=0.02, max_h=h, max_w=w, norm=1)
+    det = dog.Detector(cfg)
+    clean = synth.plif_frame(synth.PLIF_SEED_BASE + 6, h, w)
+    img = clean.copy()
+    img[at] = np.inf
+    D0, D1 = det.debug_dog(dev(clean)).cpu().numpy(), det.debug_dog(dev(img)).cpu().numpy()
+    dy, dx = np.abs(np.arange(h) - at[0])[:, None], np.abs(np.arange(w) - at[1])[None, :]
+    for l in range(det.P):
+        near = (dy <= det.radii[l + 1]) & (dx <= det.radii[l + 1])
+        assert not np.isfinite(D1[l][near]).any() and np.array_equal(D1[l][~near], D0[l][~near])
+    s = torch.tensor(sig, dtype=torch.float32, device="cuda")
+    sets = []
+    for t in (clean, img):
+        rec = dog.SoftMaxima(1 << 16, "cuda")
+        det.soft_hist(dev(t), s, rec=rec)
+        assert int(rec.count) <= rec.cap
+        r = rec.buf[:int(rec.count)].cpu().numpy()
+        far = np.maximum(np.abs(r[:, 0] - at[1]), np.abs(r[:, 1] - at[0])) > det.radii[-1] + 1
+        sets.append({tuple(v) for v in r[far].tolist()})
+    assert len(sets[0]) > 3 and sets[0] == sets[1]
