@@ -203,10 +203,10 @@ static_assert(PRUNE_DYN_BYTES + (int)sizeof(PruneSmem) <= 226 * 1024, "shared me
 // in the order of a plain grid, the conflicts (few: 2 to 5% of the candidates on
 // PLIF frames) are listed once as edges (candidate, higher-priority neighbour),
 // the rounds, targets and members run over the edges, and the accepted blobs are
-// binned as they are written.  (Sorting by priority instead, so that it becomes
-// an integer comparison, took 17 us for the sort alone.)  Returns false, having
-// written nothing, when a warp finds more than EDGE_WARP conflicts and when the
-// candidates lie too far apart for the grid.
+// binned as they are written.  When a warp finds more conflicts than EDGE_WARP,
+// rounds and targets walk the grid instead.  (Sorting by priority instead, so that
+// it becomes an integer comparison, took 17 us for the sort alone.)  Returns false,
+// having written nothing, when the candidates lie too far apart for the grid.
 __device__ __forceinline__ bool prune_cells(const PruneParams& p, PruneSmem& s, CellSmem& r, const dog_blob* cand,
                                             int n, dog_blob* out, int f) {
     const int tid = threadIdx.x, lane = tid & 31;
@@ -303,37 +303,81 @@ __device__ __forceinline__ bool prune_cells(const PruneParams& p, PruneSmem& s, 
     }
     __syncwarp();
     const int ne = *n_edge;
-    if (__syncthreads_or(ne > EDGE_WARP)) return false;
-    // rounds of the independent-set rule
-    for (;;) {
-        for (int e = lane; e < ne; e += 32) {
-            const int i = edge[e] >> 16;
-            if (r.state[i] != ST_UND) continue;
-            const int st = r.state[edge[e] & 0xffffu];
-            if (st == ST_IN) r.in[i] = 1;
-            else if (st == ST_UND) r.und[i] = 1;
-        }
-        __syncthreads();
-        bool wait = false;
-        for (int i = tid; i < n; i += PRUNE_THREADS) {
-            if (r.state[i] != ST_UND) continue;
-            if (r.in[i] || !r.und[i]) r.state[i] = r.in[i] ? ST_OUT : ST_IN;
-            else wait = true;
-            r.und[i] = 0;
-        }
-        if (!__syncthreads_or(wait)) break;   // (each round settles the first undecided)
-    }
-    // every rejected candidate joins its highest-priority accepted neighbour
     bool any = false;
-    for (int e = lane; e < ne; e += 32) {
-        const int i = edge[e] >> 16, j = edge[e] & 0xffffu;
-        if (r.state[i] != ST_OUT || r.state[j] != ST_IN) continue;
-        any = true;
-        int seen = r.target[i];
-        while (seen < 0 || r.before(j, seen)) {
-            const int now = atomicCAS(&r.target[i], seen, j);
-            if (now == seen) break;
-            seen = now;
+    if (__syncthreads_or(ne > EDGE_WARP)) {
+        // more conflicts than the lists hold: every round and the targets walk the
+        // rows of cells again (a state is settled once, so a round may see others
+        // before or after theirs)
+        auto walk = [&](int i, auto visit) {   // higher-priority neighbours of i
+            const int xi = r.x[i], yi = r.y[i], li = min(max(r.level[i], 0), p.P - 1);
+            for (int dy = -1; dy <= 1; ++dy) {
+                const int c = r.cell[i] + dy * nx;
+                if (c < 0 || c >= nx * ny) continue;
+                const int end = s.boff[c + 2];
+                for (int k = s.boff[c - 1]; k < end; ++k) {
+                    const int ex = r.x[k] - xi, ey = r.y[k] - yi, d = ex * ex + ey * ey;
+                    if (d >= reach || k == i) continue;
+                    if (d < s.d2[li * p.P + min(max(r.level[k], 0), p.P - 1)] && r.before(k, i) && visit(k)) return;
+                }
+            }
+        };
+        volatile unsigned char* state = r.state;
+        for (;;) {
+            bool wait = false;
+            for (int i = tid; i < n; i += PRUNE_THREADS) {
+                if (state[i] != ST_UND) continue;
+                bool in = false, und = false;
+                walk(i, [&](int k) {
+                    const int st = state[k];
+                    und |= st == ST_UND;
+                    return in = st == ST_IN;
+                });
+                if (in || !und) state[i] = in ? ST_OUT : ST_IN;
+                else wait = true;
+            }
+            if (!__syncthreads_or(wait)) break;
+        }
+        for (int i = tid; i < n; i += PRUNE_THREADS) {
+            if (r.state[i] != ST_OUT) continue;
+            int best = -1;
+            walk(i, [&](int k) {
+                if (r.state[k] == ST_IN && (best < 0 || r.before(k, best))) best = k;
+                return false;
+            });
+            r.target[i] = best;
+            any = true;
+        }
+    } else {
+        // rounds of the independent-set rule
+        for (;;) {
+            for (int e = lane; e < ne; e += 32) {
+                const int i = edge[e] >> 16;
+                if (r.state[i] != ST_UND) continue;
+                const int st = r.state[edge[e] & 0xffffu];
+                if (st == ST_IN) r.in[i] = 1;
+                else if (st == ST_UND) r.und[i] = 1;
+            }
+            __syncthreads();
+            bool wait = false;
+            for (int i = tid; i < n; i += PRUNE_THREADS) {
+                if (r.state[i] != ST_UND) continue;
+                if (r.in[i] || !r.und[i]) r.state[i] = r.in[i] ? ST_OUT : ST_IN;
+                else wait = true;
+                r.und[i] = 0;
+            }
+            if (!__syncthreads_or(wait)) break;   // (each round settles the first undecided)
+        }
+        // every rejected candidate joins its highest-priority accepted neighbour
+        for (int e = lane; e < ne; e += 32) {
+            const int i = edge[e] >> 16, j = edge[e] & 0xffffu;
+            if (r.state[i] != ST_OUT || r.state[j] != ST_IN) continue;
+            any = true;
+            int seen = r.target[i];
+            while (seen < 0 || r.before(j, seen)) {
+                const int now = atomicCAS(&r.target[i], seen, j);
+                if (now == seen) break;
+                seen = now;
+            }
         }
     }
     // members of every accepted candidate (the edges are no longer needed)
