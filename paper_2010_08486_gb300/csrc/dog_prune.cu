@@ -161,8 +161,9 @@ __device__ __forceinline__ void scan_buckets(PruneSmem& s) {
     if (tid == PRUNE_THREADS - 1) s.boff[NBUCKET] = e + v;
 }
 
-// Frames with at most PRUNE_SMEM_CAND candidates run in shared memory; larger
-// ones work in global memory.
+// Frames with at most PRUNE_SMEM_CAND candidates take prune_cells; larger ones, and
+// those that it gives back, the hashed cells, with as much of their arrays in
+// shared memory as its size allows.
 constexpr int PRUNE_SMEM_CAND = 4096;
 constexpr int EDGE_WARP = 640;   // conflicts one warp may list
 
@@ -191,8 +192,13 @@ struct CellSmem {
         return x[a] < x[b];
     }
 };
-constexpr int PRUNE_OLD_BYTES = PRUNE_SMEM_CAND * ((int)sizeof(dog_blob) + 3 * (int)sizeof(int));
-constexpr int PRUNE_DYN_BYTES = (int)sizeof(CellSmem) > PRUNE_OLD_BYTES ? (int)sizeof(CellSmem) : PRUNE_OLD_BYTES;
+constexpr int PRUNE_DYN_BYTES = (int)sizeof(CellSmem);
+// hashed cells: the most candidates of which themselves and the three arrays,
+// themselves, two arrays and one array fit
+constexpr int CAND_FIT = PRUNE_DYN_BYTES / (int)sizeof(dog_blob);
+constexpr int PAIR_FIT = PRUNE_DYN_BYTES / 8, ONE_FIT = PRUNE_DYN_BYTES / 4;
+constexpr int ALL_FIT = PRUNE_DYN_BYTES / ((int)sizeof(dog_blob) + 3 * (int)sizeof(int));
+static_assert(ALL_FIT >= PRUNE_SMEM_CAND, "lists that prune_cells gives back");
 static_assert(PRUNE_DYN_BYTES + (int)sizeof(PruneSmem) <= 226 * 1024, "shared memory of one CTA");
 
 // Pruning and histogram of one frame in shared memory.  One thread per
@@ -480,16 +486,33 @@ __global__ void __launch_bounds__(PRUNE_THREADS) dog_prune_kernel(const __grid_c
     int* order = p.order + coff;
     dog_blob* out = p.out + ooff;
     const int n = min(p.cand_count[f], p.cap_in);
-    if (n <= PRUNE_SMEM_CAND && p.mode != DOG_PRUNE_OFF) {
-        if (prune_cells(p, s, *reinterpret_cast<CellSmem*>(prune_dyn), cand, n, out, f)) return;
-        __syncthreads();
-        dog_blob* sc = reinterpret_cast<dog_blob*>(prune_dyn);
-        int* si = reinterpret_cast<int*>(sc + PRUNE_SMEM_CAND);
-        for (int i = tid; i < n; i += PRUNE_THREADS) sc[i] = cand[i];
-        cand = sc;
-        state = si;
-        target = si + PRUNE_SMEM_CAND;
-        order = si + 2 * PRUNE_SMEM_CAND;
+    if (p.mode != DOG_PRUNE_OFF) {
+        if (n <= PRUNE_SMEM_CAND) {
+            if (prune_cells(p, s, *reinterpret_cast<CellSmem*>(prune_dyn), cand, n, out, f)) return;
+            __syncthreads();
+        }
+        // Copies in the shared memory that the launch has anyway, and that leaves the
+        // L1 too small for these arrays in global memory (5000 candidates 820 us, with
+        // 60 KB less of it 706, copied 381): the candidates and all three arrays up to
+        // 5872 of them, the candidates up to 9396; of longer lists the arrays that the
+        // inner loops read most, up to 23490 and 46980 (23,000: 8095, 7740, 5611).
+        int* si = reinterpret_cast<int*>(prune_dyn);
+        if (n <= CAND_FIT) {
+            dog_blob* sc = reinterpret_cast<dog_blob*>(prune_dyn);
+            for (int i = tid; i < n; i += PRUNE_THREADS) sc[i] = cand[i];
+            cand = sc;
+            si = reinterpret_cast<int*>(sc + n);
+        }
+        if (n <= ALL_FIT) {
+            state = si;
+            target = si + n;
+            order = si + 2 * n;
+        } else if (n > CAND_FIT && n <= PAIR_FIT) {
+            state = si;
+            order = si + n;
+        } else if (n > CAND_FIT && n <= ONE_FIT) {
+            state = si;
+        }
         // made visible by the first __syncthreads below
     }
 

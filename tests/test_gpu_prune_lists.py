@@ -61,3 +61,28 @@ def test_candidates_far_apart():
     torch.cuda.synchronize()
     got = out.to_numpy()
     assert sorted(got[1].tolist()) == [0, 65536, 131072, 30_000_000, 30_065_536, h - 2] and det.status() == 0
+
+
+@pytest.mark.parametrize("n", [5872, 5873, 9396, 9397, 23490, 23491, 46981])
+def test_lists_at_the_sizes_of_the_shared_memory(n):
+    """The largest lists of which the candidates and all arrays, the candidates,
+    and two arrays fit the shared memory, and one more; and none of them."""
+    rng = np.random.default_rng(n)
+    size, cap = 1200, 65536
+    cfg = dog.plif_config(max_h=2048, max_w=2048, blob_cap=cap)
+    det = dog.Detector(cfg)
+    cells = rng.choice(size * size * 8, size=n, replace=False)
+    level, pos = cells % 8, cells // 8
+    x, y = pos % size, pos // size
+    resp = (rng.integers(1, 4000, n) / 4096.0).astype(np.float32)
+    sig = np.asarray(det.sigmas, np.float32)[level]
+    raw = np.zeros((cap, 5), np.int32)
+    raw[:n, 0], raw[:n, 1], raw[:n, 2] = x, y, level
+    raw[:n, 3], raw[:n, 4] = sig.view(np.int32), resp.view(np.int32)
+    cand = dog.BlobList(torch.from_numpy(raw).cuda(), torch.tensor(n, dtype=torch.int32, device="cuda"))
+    out = det.prune(cand, 2048, 2048)
+    torch.cuda.synchronize()
+    want = oracle.prune(parity.blobs_to_oracle(x, y, level, sig, resp), parity.oracle_params(cfg))
+    want.sigma = want.sigma.astype(np.float32).astype(np.float64)
+    assert parity.same_blob_sets(parity.blobs_to_oracle(*out.to_numpy()), want)
+    assert det.status() == 0
