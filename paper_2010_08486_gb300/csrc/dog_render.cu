@@ -19,7 +19,8 @@
 // exactly zero to every sample of the tile, so the sums are unchanged (see
 // beside).  A warp
 // then takes four blocks of 16 x 2 pixels and skips the listed spheres that miss
-// its block.
+// its block.  Frames of few tiles give a tile's blocks to two or four CTAs, which
+// list the same spheres each.
 //
 // What bounds it: integer multiplies of the generator (six Philox blocks a
 // pixel).  The double-precision pipe (two lanes a cycle and SM here) was the
@@ -127,7 +128,7 @@ __global__ void __launch_bounds__(RTHREADS) render_spheres_kernel(const float4* 
     // that no count is decided in single precision)
     const float gain_f = fabs(gain) < (double)FLT_MIN && gain != 0.0 ? NAN : (float)gain, rn_f = (float)read_noise;
 #pragma unroll 1
-    for (int blk = 0; blk < 4; ++blk) {
+    for (int blk = blockIdx.z; blk < 4; blk += gridDim.z) {
         // block of 16 x 2 pixels: warp rows 4 w .. 4 w + 3, two blocks side by side
         const int bx = x0 + (blk & 1) * 16, by = y0 + 4 * warp + (blk >> 1) * 2;
         if (bx >= W || by >= H) continue;
@@ -179,8 +180,14 @@ extern "C" int dog_render_spheres(const float* d_spheres, int32_t n_spheres, int
     if (!(ss == 1 || ss == 2 || ss == 4 || ss == 8)) return DOG_ERR_INVALID;
     if (n_spheres > MAX_SPHERES) return DOG_ERR_UNSUPPORTED;
     if ((reinterpret_cast<uintptr_t>(d_spheres) & 15) != 0) return DOG_ERR_INVALID;
-    const dim3 grid((img_w + RT - 1) / RT, (img_h + RT - 1) / RT);
+    dim3 grid((img_w + RT - 1) / RT, (img_h + RT - 1) / RT);
     if (grid.y > 65535) return DOG_ERR_UNSUPPORTED;
+    // CTAs per tile: up to 2560 in all, two and a half times what is resident.  Four
+    // blocks to a CTA leave the SMs idle on fewer tiles (64 x 64 pixels 51 us, with
+    // four CTAs a tile 16; 512 x 512 19.3, 12.1; 1000 x 1000 with two 30.8, 27.2);
+    // on more the lists cost more than that (2000 x 2000 74.9, with two 81.0)
+    const long long tiles = (long long)grid.x * grid.y;
+    grid.z = tiles <= 640 ? 4 : tiles <= 1280 ? 2 : 1;
     render_spheres_kernel<<<grid, RTHREADS, 0, static_cast<cudaStream_t>(stream)>>>(
         reinterpret_cast<const float4*>(d_spheres), n_spheres, img_h, img_w, ss, background, gain, read_noise,
         (uint32_t)seed, (uint32_t)(seed >> 32), d_intensity, d_counts, pitch);

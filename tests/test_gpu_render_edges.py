@@ -63,3 +63,14 @@ def test_gains_below_single_precision(gain):
     torch.cuda.synchronize()
     _, want = oracle.render_spheres(table, 300, 400, ss=1, background=bg, gain=gain, read_noise=0.25, seed=3)
     assert np.array_equal(counts.cpu().numpy().view(np.uint16), want)
+
+
+@pytest.mark.parametrize("h,w", [(639, 1000), (641, 1000), (1279, 1000), (1300, 1025)])
+def test_frames_around_a_change_of_the_grid(h, w):
+    """20, 21, 40 and 41 by 32 or 33 tiles: four, two, two and one CTA to a tile."""
+    table = synth.sphere_table(synth.SPHERE_SEED_BASE + h, n=40, h=h, w=w, r_range=(3.0, 30.0))
+    counts, inten = dog.render_spheres(torch.from_numpy(table).cuda(), h, w, ss=2, seed=h, with_intensity=True)
+    torch.cuda.synchronize()
+    want_i, want_c = oracle.render_spheres(table, h, w, ss=2, background=0.05, gain=2000.0, read_noise=4.0, seed=h)
+    assert np.array_equal(inten.cpu().numpy().view(np.uint32), want_i.view(np.uint32))
+    assert np.array_equal(counts.cpu().numpy().view(np.uint16), want_c)
