@@ -187,12 +187,6 @@ int dogk::conflict_d2(double sa, double sb, double thr) {
     return (int)hi;
 }
 
-static int ceil_pow2(int v) {
-    int p = 1;
-    while (p < v) p <<= 1;
-    return p;
-}
-
 static int status_from(cudaError_t e) {
     if (e == cudaSuccess) return DOG_OK;
     return e == cudaErrorMemoryAllocation ? DOG_ERR_NOMEM : DOG_ERR_CUDA;

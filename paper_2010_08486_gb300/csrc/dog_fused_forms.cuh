@@ -557,7 +557,6 @@ __device__ __forceinline__ void process_tile(const FusedParams& p, float* sm, Sm
     constexpr int MBK = 8 * NW;   // rows of a block
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rho = lane >> 2;
     const int R = p.R, S = p.in_stride, CIN = p.in_rows, n = p.n_pairs, off = p.lev_off;
-    const int ncols = TX + 2 * R;
     float* in = sm + p.in_off;
     float* wbuf = sm + p.w_off;
     float* xch = sm + p.x_off;      // [parity][plane of the pair][warp][2 rows][32]

@@ -59,9 +59,6 @@ struct SoftWS {
     float* gk = nullptr;      // P sums gH . kappa_l, then P sums gH . dkappa_l
     float* wpad = nullptr;    // the taps with TAP_PAD zeros around each level's
     float4* wt = nullptr;     // per plane and window offset: taps and their derivatives of both its levels
-    Pending* pend = nullptr;
-    int pend_cap = 0;
-    int* counts = nullptr;
     float* A = nullptr;       // K x H x W
     void* lists = nullptr;    // the record path's lists (see Lists) of n_lists frames
     int n_lists = 0;
@@ -78,8 +75,7 @@ struct SoftWS {
 void soft_free(dog_handle* h) {
     SoftWS* ws = static_cast<SoftWS*>(handle_soft_ws(h));
     if (!ws) return;
-    void* ptrs[] = {ws->w, ws->dw, ws->wp, ws->c, ws->kappa, ws->dkappa, ws->gk, ws->wpad, ws->wt, ws->pend, ws->counts, ws->A,
-                    ws->lists, ws->flags, ws->Y, ws->Yd, ws->acc, ws->last_sig};
+    void* ptrs[] = {ws->w, ws->dw, ws->wp, ws->c, ws->kappa, ws->dkappa, ws->gk, ws->wpad, ws->wt, ws->A, ws->lists, ws->flags, ws->Y, ws->Yd, ws->acc, ws->last_sig};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (int i = 0; i < ws->n_old; ++i) cudaFree(ws->old_lists[i]);
@@ -156,8 +152,6 @@ static int soft_ws(dog_handle* h, int H, int W, SoftWS** out) {
     const FusedParams& b = handle_base(h);
     const int K = b.K, P = b.P, nb = handle_cfg(h).nbins;
     const size_t plane = (size_t)H * W;
-    const int strips = (W + TX - 1) / TX;
-    ws->pend_cap = (int)std::min<size_t>((size_t)2 * strips * P * H + 1024, (size_t)1 << 28);
     cudaError_t e = cudaSuccess;
     auto ok = [&](cudaError_t x) { if (e == cudaSuccess) e = x; };
     ok(cudaMalloc(&ws->w, sizeof(float) * handle_w_total(h)));
@@ -167,8 +161,6 @@ static int soft_ws(dog_handle* h, int H, int W, SoftWS** out) {
     ok(cudaMalloc(&ws->c, sizeof(float) * 2 * P));
     ok(cudaMalloc(&ws->kappa, sizeof(float) * P * nb));
     ok(cudaMalloc(&ws->dkappa, sizeof(float) * P * nb));
-    ok(cudaMalloc(&ws->pend, sizeof(Pending) * ws->pend_cap));
-    ok(cudaMalloc(&ws->counts, sizeof(int) * 4));
     int n_wt = 0;
     for (int l = 0; l < P; ++l) n_wt += 2 * plane_radius(h, l) + 1;
     ok(cudaMalloc(&ws->wt, sizeof(float4) * n_wt));
@@ -216,8 +208,8 @@ struct SoftPrep {
     int padoff[MAX_LEVELS];
     const float* gH;   // backward: dloss/dH (nullptr in the forward)
     float* gk;
-    int* zero[2];      // counters to clear (nullptr: none), n_zero[k] ints each
-    int n_zero[2];
+    int* zero;         // counters to clear
+    int n_zero;
     double* acc;       // sums to clear
     int n_acc;
     void* lists;       // lists of n_lists frames of H x W to empty
@@ -276,7 +268,8 @@ __device__ void soft_tables(const SoftPrep& p) {
             p.dkappa[l * p.nbins + b] = (a < 1.0 && !clamped) ? (float)(-(double)p.nbins * sg) : 0.0f;
         }
     }
-    for (int i = threadIdx.x; i < p.K; i += blockDim.x) p.last_sig[i] = p.sig[i];    __syncthreads();
+    for (int i = threadIdx.x; i < p.K; i += blockDim.x) p.last_sig[i] = p.sig[i];
+    __syncthreads();
     for (int l = warp; l < p.P; l += PREP_THREADS / 32) {
         const int ra = p.r[l], rb = p.r[l + 1], R2 = max(ra, rb);
         for (int t = lane; t <= 2 * R2; t += 32) {
@@ -304,8 +297,7 @@ __global__ void __launch_bounds__(PREP_THREADS) soft_prep_kernel(const __grid_co
         return;
     }
     if (blockIdx.y > 0) return;
-    for (int k = 0; k < 2; ++k)
-        for (int i = threadIdx.x; i < p.n_zero[k]; i += PREP_THREADS) p.zero[k][i] = 0;
+    for (int i = threadIdx.x; i < p.n_zero; i += PREP_THREADS) p.zero[i] = 0;
     for (int i = threadIdx.x; i < p.n_acc; i += PREP_THREADS) p.acc[i] = 0.0;
     bool changed = false;
     for (int i = threadIdx.x; i < p.K; i += blockDim.x) changed |= !(p.sig[i] == p.last_sig[i]);
@@ -378,9 +370,6 @@ static FusedParams soft_fused(dog_handle* h, SoftWS* ws, const float* img, int n
     p.mode = mode;
     p.w = ws->wp;
     p.c = ws->c;
-    p.pend = ws->pend;
-    p.pend_cap = ws->pend_cap;
-    p.pend_count = ws->counts;
     p.kappa = ws->kappa;
     p.dkappa = ws->dkappa;
     p.nbins = handle_cfg(h).nbins;
@@ -425,11 +414,9 @@ int soft_forward(dog_handle* h, const float* img, int n, long long stride, int H
     int st = soft_ws(h, H, W, &ws);
     if (st != DOG_OK) return st;
     SoftPrep q = prep_params(h, ws, sig);
-    q.zero[0] = ws->counts;
-    q.n_zero[0] = 4;
     if (rec != nullptr) {
-        q.zero[1] = rec_count;
-        q.n_zero[1] = n;
+        q.zero = rec_count;
+        q.n_zero = n;
     }
     soft_prep_kernel<<<1, PREP_THREADS, 0, s>>>(q);
     SOFT_CUDA(cudaGetLastError());
@@ -1342,8 +1329,6 @@ int soft_backward(dog_handle* h, const float* img, int H, int W, int pitch, cons
     const FusedParams& b = handle_base(h);
     const int K = b.K, P = b.P;
     SoftPrep q = prep_params(h, ws, sig);
-    q.zero[0] = ws->counts;
-    q.n_zero[0] = 4;
     q.acc = ws->acc;
     q.n_acc = ACC_COPIES * (2 * P + K);
     soft_prep_kernel<<<1, PREP_THREADS, 0, s>>>(q);
@@ -1380,8 +1365,8 @@ int soft_backward_rec(dog_handle* h, const float* img, int n, long long stride, 
     int* arrived = reinterpret_cast<int*>(flags + LIST_FRAMES);
     SoftPrep q = prep_params(h, ws, sig);
     q.gH = gH;
-    q.zero[0] = ws->flags;
-    q.n_zero[0] = (int)(sizeof(FrameFlags) / sizeof(int)) * LIST_FRAMES + 1;
+    q.zero = ws->flags;
+    q.n_zero = (int)(sizeof(FrameFlags) / sizeof(int)) * LIST_FRAMES + 1;
     q.acc = ws->acc;
     q.n_acc = ACC_COPIES * (2 * P + K);
     q.lists = ws->lists;
