@@ -201,191 +201,32 @@ constexpr int ALL_FIT = PRUNE_DYN_BYTES / ((int)sizeof(dog_blob) + 3 * (int)size
 static_assert(ALL_FIT >= PRUNE_SMEM_CAND, "lists that prune_cells gives back");
 static_assert(PRUNE_DYN_BYTES + (int)sizeof(PruneSmem) <= 226 * 1024, "shared memory of one CTA");
 
-// Pruning and histogram of one frame in shared memory.  One thread per
-// candidate walking its nine hashed cells, once a round and once per group
-// member, is a chain of dependent loads as long as the fullest cell among 32
-// lanes, and the histogram's passes over global memory come on top (69 us for
-// the 1,700 candidates of a 1024 x 1024 frame).  Here the candidates are copied
-// in the order of a plain grid, the conflicts (few: 2 to 5% of the candidates on
-// PLIF frames) are listed once as edges (candidate, higher-priority neighbour),
-// the rounds, targets and members run over the edges, and the accepted blobs are
-// binned as they are written.  When a warp finds more conflicts than EDGE_WARP,
-// rounds and targets walk the grid instead.  (Sorting by priority instead, so that
-// it becomes an integer comparison, took 17 us for the sort alone.)  Returns false,
-// having written nothing, when the candidates lie too far apart for the grid.
-__device__ __forceinline__ bool prune_cells(const PruneParams& p, PruneSmem& s, CellSmem& r, const dog_blob* cand,
-                                            int n, dog_blob* out, int f) {
+// The grid over the candidates' box: cells of at least the largest conflict
+// distance, at most NBUCKET of them with a margin of one column on either side.
+struct CellGrid {
+    long long ox, oy, cell;
+    int nx, ny, reach;   // reach: no smaller than any conflict distance squared
+};
+__device__ __forceinline__ CellGrid cell_grid(const PruneParams& p, const CellSmem& r, int n) {
+    CellGrid g;
+    g.ox = r.box[0];
+    g.oy = r.box[2];
+    const long long wx = n ? r.box[1] - g.ox : 0, wy = n ? r.box[3] - g.oy : 0;
+    g.cell = p.cell;
+    while ((wx / g.cell + 3) * (wy / g.cell + 1) > NBUCKET) g.cell *= 2;
+    g.nx = (int)(wx / g.cell) + 3;
+    g.ny = (int)(wy / g.cell) + 1;
+    g.reach = p.cell < 46340 ? p.cell * p.cell : INT_MAX;
+    return g;
+}
+
+// Members, blobs and histogram of a frame whose states and targets are settled
+// (any: this thread found a target).
+__device__ __forceinline__ void finish_cells(const PruneParams& p, PruneSmem& s, CellSmem& r, int n, bool any,
+                                             dog_blob* out, int f) {
     const int tid = threadIdx.x, lane = tid & 31;
     const HistParams& hp = p.hist;
     const int nbo = hp.hist ? (hp.mode == DOG_HIST_LADDER ? hp.P : hp.nbins) : 0;
-    for (int q = tid; q < NBUCKET; q += PRUNE_THREADS) s.bcount[q] = 0;
-    for (int q = tid; q < p.P * p.P; q += PRUNE_THREADS) s.d2[q] = p.d2thr[q];
-    for (int q = tid; q < p.P; q += PRUNE_THREADS) {
-        r.sig[q] = p.sig[q];
-        r.sig_f[q] = hp.hist ? hp.sig_f[q] : 0.0f;
-        r.level_bin[q] = hp.hist ? hp.level_bin[q] : 0;
-    }
-    for (int q = tid; q < nbo; q += PRUNE_THREADS) { r.hc[q] = 0u; r.hv[q] = 0.0; }
-    if (tid < 4) r.box[tid] = tid & 1 ? INT_MIN : INT_MAX;
-    // this thread's candidates: tid, tid + 1024, ...
-    constexpr int PER = PRUNE_SMEM_CAND / PRUNE_THREADS;
-    dog_blob mine[PER];
-    int bk[PER];
-    int x0 = INT_MAX, x1 = INT_MIN, y0 = INT_MAX, y1 = INT_MIN;
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-        const int i = tid + u * PRUNE_THREADS;
-        if (i < n) {
-            mine[u] = cand[i];
-            x0 = min(x0, mine[u].x); x1 = max(x1, mine[u].x);
-            y0 = min(y0, mine[u].y); y1 = max(y1, mine[u].y);
-        }
-    }
-    x0 = __reduce_min_sync(0xffffffffu, x0); x1 = __reduce_max_sync(0xffffffffu, x1);
-    y0 = __reduce_min_sync(0xffffffffu, y0); y1 = __reduce_max_sync(0xffffffffu, y1);
-    __syncthreads();
-    if (lane == 0) {
-        atomicMin(&r.box[0], x0); atomicMax(&r.box[1], x1);
-        atomicMin(&r.box[2], y0); atomicMax(&r.box[3], y1);
-    }
-    __syncthreads();
-    // the grid: cells of at least the largest conflict distance, at most NBUCKET
-    // of them with a margin of one column on either side
-    const long long ox = r.box[0], oy = r.box[2];
-    const long long wx = n ? r.box[1] - ox : 0, wy = n ? r.box[3] - oy : 0;
-    long long cell = p.cell;
-    while ((wx / cell + 3) * (wy / cell + 1) > NBUCKET) cell *= 2;
-    // (candidates of neighbouring cells are less than two cells apart; of cells
-    // this large, in frames of more than 2^24 rows, the squared distance would not
-    // fit an int)
-    if (cell > 16384) return false;
-    const int nx = (int)(wx / cell) + 3, ny = (int)(wy / cell) + 1;
-    const unsigned uc = (unsigned)cell;   // (at most the extent, below 2^32)
-#pragma unroll
-    for (int u = 0; u < PER; ++u)
-        if (tid + u * PRUNE_THREADS < n) {
-            bk[u] = (int)((unsigned)(mine[u].y - oy) / uc) * nx + (int)((unsigned)(mine[u].x - ox) / uc) + 1;
-            atomicAdd(&s.bcount[bk[u]], 1);
-        }
-    __syncthreads();
-    scan_buckets(s);
-    __syncthreads();
-#pragma unroll
-    for (int u = 0; u < PER; ++u)
-        if (tid + u * PRUNE_THREADS < n) {
-            const int at = s.boff[bk[u]] + atomicSub(&s.bcount[bk[u]], 1) - 1;
-            r.x[at] = mine[u].x;
-            r.y[at] = mine[u].y;
-            r.level[at] = mine[u].level;
-            r.resp[at] = mine[u].response;
-            r.cell[at] = (unsigned short)bk[u];
-            r.target[at] = -1;
-            r.state[at] = ST_UND;
-            r.in[at] = 0;
-            r.und[at] = 0;
-        }
-    __syncthreads();
-    // edges: candidate i and row of cells dy - 1 per thread; every warp fills and
-    // later reads its own part of the list (hits are rare, so they may diverge)
-    unsigned* edge = r.edge + (tid >> 5) * EDGE_WARP;
-    int* n_edge = &s.wsum[tid >> 5];
-    if (lane == 0) *n_edge = 0;
-    __syncwarp();
-    const int reach = p.cell < 46340 ? p.cell * p.cell : INT_MAX;   // no smaller than any conflict distance squared
-    for (int t = tid; t < 3 * n; t += PRUNE_THREADS) {
-        const int dy = (t >= n) + (t >= 2 * n), i = t - dy * n;
-        const int xi = r.x[i], yi = r.y[i];
-        const int c = r.cell[i] + (dy - 1) * nx;
-        if (c < 0 || c >= nx * ny) continue;
-        const int end = s.boff[c + 2];
-        for (int k = s.boff[c - 1]; k < end; ++k) {
-            const int ex = r.x[k] - xi, ey = r.y[k] - yi, d = ex * ex + ey * ey;
-            if (d >= reach || k == i) continue;
-            const int li = min(max(r.level[i], 0), p.P - 1), lk = min(max(r.level[k], 0), p.P - 1);
-            if (d >= s.d2[li * p.P + lk] || !r.before(k, i)) continue;
-            const int e = atomicAdd(n_edge, 1);
-            if (e < EDGE_WARP) edge[e] = (unsigned)i << 16 | (unsigned)k;
-        }
-    }
-    __syncwarp();
-    const int ne = *n_edge;
-    bool any = false;
-    if (__syncthreads_or(ne > EDGE_WARP)) {
-        // more conflicts than the lists hold: every round and the targets walk the
-        // rows of cells again (a state is settled once, so a round may see others
-        // before or after theirs)
-        auto walk = [&](int i, auto visit) {   // higher-priority neighbours of i
-            const int xi = r.x[i], yi = r.y[i], li = min(max(r.level[i], 0), p.P - 1);
-            for (int dy = -1; dy <= 1; ++dy) {
-                const int c = r.cell[i] + dy * nx;
-                if (c < 0 || c >= nx * ny) continue;
-                const int end = s.boff[c + 2];
-                for (int k = s.boff[c - 1]; k < end; ++k) {
-                    const int ex = r.x[k] - xi, ey = r.y[k] - yi, d = ex * ex + ey * ey;
-                    if (d >= reach || k == i) continue;
-                    if (d < s.d2[li * p.P + min(max(r.level[k], 0), p.P - 1)] && r.before(k, i) && visit(k)) return;
-                }
-            }
-        };
-        volatile unsigned char* state = r.state;
-        for (;;) {
-            bool wait = false;
-            for (int i = tid; i < n; i += PRUNE_THREADS) {
-                if (state[i] != ST_UND) continue;
-                bool in = false, und = false;
-                walk(i, [&](int k) {
-                    const int st = state[k];
-                    und |= st == ST_UND;
-                    return in = st == ST_IN;
-                });
-                if (in || !und) state[i] = in ? ST_OUT : ST_IN;
-                else wait = true;
-            }
-            if (!__syncthreads_or(wait)) break;
-        }
-        for (int i = tid; i < n; i += PRUNE_THREADS) {
-            if (r.state[i] != ST_OUT) continue;
-            int best = -1;
-            walk(i, [&](int k) {
-                if (r.state[k] == ST_IN && (best < 0 || r.before(k, best))) best = k;
-                return false;
-            });
-            r.target[i] = best;
-            any = true;
-        }
-    } else {
-        // rounds of the independent-set rule
-        for (;;) {
-            for (int e = lane; e < ne; e += 32) {
-                const int i = edge[e] >> 16;
-                if (r.state[i] != ST_UND) continue;
-                const int st = r.state[edge[e] & 0xffffu];
-                if (st == ST_IN) r.in[i] = 1;
-                else if (st == ST_UND) r.und[i] = 1;
-            }
-            __syncthreads();
-            bool wait = false;
-            for (int i = tid; i < n; i += PRUNE_THREADS) {
-                if (r.state[i] != ST_UND) continue;
-                if (r.in[i] || !r.und[i]) r.state[i] = r.in[i] ? ST_OUT : ST_IN;
-                else wait = true;
-                r.und[i] = 0;
-            }
-            if (!__syncthreads_or(wait)) break;   // (each round settles the first undecided)
-        }
-        // every rejected candidate joins its highest-priority accepted neighbour
-        for (int e = lane; e < ne; e += 32) {
-            const int i = edge[e] >> 16, j = edge[e] & 0xffffu;
-            if (r.state[i] != ST_OUT || r.state[j] != ST_IN) continue;
-            any = true;
-            int seen = r.target[i];
-            while (seen < 0 || r.before(j, seen)) {
-                const int now = atomicCAS(&r.target[i], seen, j);
-                if (now == seen) break;
-                seen = now;
-            }
-        }
-    }
     // members of every accepted candidate (the edges are no longer needed)
     const bool groups = __syncthreads_or(any) && p.mode == DOG_PRUNE_COALESCE;
     if (groups) {
@@ -470,7 +311,200 @@ __device__ __forceinline__ bool prune_cells(const PruneParams& p, PruneSmem& s, 
         hp.hist[(size_t)f * nbo + q] = r.hc[q];
         if (hp.vol) hp.vol[(size_t)f * nbo + q] = r.hv[q];
     }
-    return true;
+}
+
+// Pruning and histogram of one frame in shared memory.  One thread per
+// candidate walking its nine hashed cells, once a round and once per group
+// member, is a chain of dependent loads as long as the fullest cell among 32
+// lanes, and the histogram's passes over global memory come on top (69 us for
+// the 1,700 candidates of a 1024 x 1024 frame).  Here the candidates are copied
+// in the order of a plain grid, the conflicts (few: 2 to 5% of the candidates on
+// PLIF frames) are listed once as edges (candidate, higher-priority neighbour),
+// the rounds, targets and members run over the edges, and the accepted blobs are
+// binned as they are written.  (Sorting by priority instead, so that it becomes
+// an integer comparison, took 17 us for the sort alone.)  Returns CELLS_FULL when a
+// warp finds more than EDGE_WARP conflicts (the candidates are sorted: dense_cells
+// goes on from there), and CELLS_FAR, having written nothing, when the candidates
+// lie too far apart for the grid.
+enum { CELLS_DONE = 0, CELLS_FULL = 1, CELLS_FAR = 2 };
+__device__ __forceinline__ int prune_cells(const PruneParams& p, PruneSmem& s, CellSmem& r, const dog_blob* cand,
+                                            int n, dog_blob* out, int f) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    const HistParams& hp = p.hist;
+    const int nbo = hp.hist ? (hp.mode == DOG_HIST_LADDER ? hp.P : hp.nbins) : 0;
+    for (int q = tid; q < NBUCKET; q += PRUNE_THREADS) s.bcount[q] = 0;
+    for (int q = tid; q < p.P * p.P; q += PRUNE_THREADS) s.d2[q] = p.d2thr[q];
+    for (int q = tid; q < p.P; q += PRUNE_THREADS) {
+        r.sig[q] = p.sig[q];
+        r.sig_f[q] = hp.hist ? hp.sig_f[q] : 0.0f;
+        r.level_bin[q] = hp.hist ? hp.level_bin[q] : 0;
+    }
+    for (int q = tid; q < nbo; q += PRUNE_THREADS) { r.hc[q] = 0u; r.hv[q] = 0.0; }
+    if (tid < 4) r.box[tid] = tid & 1 ? INT_MIN : INT_MAX;
+    // this thread's candidates: tid, tid + 1024, ...
+    constexpr int PER = PRUNE_SMEM_CAND / PRUNE_THREADS;
+    dog_blob mine[PER];
+    int bk[PER];
+    int x0 = INT_MAX, x1 = INT_MIN, y0 = INT_MAX, y1 = INT_MIN;
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        const int i = tid + u * PRUNE_THREADS;
+        if (i < n) {
+            mine[u] = cand[i];
+            x0 = min(x0, mine[u].x); x1 = max(x1, mine[u].x);
+            y0 = min(y0, mine[u].y); y1 = max(y1, mine[u].y);
+        }
+    }
+    x0 = __reduce_min_sync(0xffffffffu, x0); x1 = __reduce_max_sync(0xffffffffu, x1);
+    y0 = __reduce_min_sync(0xffffffffu, y0); y1 = __reduce_max_sync(0xffffffffu, y1);
+    __syncthreads();
+    if (lane == 0) {
+        atomicMin(&r.box[0], x0); atomicMax(&r.box[1], x1);
+        atomicMin(&r.box[2], y0); atomicMax(&r.box[3], y1);
+    }
+    __syncthreads();
+    const CellGrid g = cell_grid(p, r, n);
+    const long long ox = g.ox, oy = g.oy, cell = g.cell;
+    const int nx = g.nx, ny = g.ny;
+    // (candidates of neighbouring cells are less than two cells apart; of cells
+    // this large, in frames of more than 2^24 rows, the squared distance would not
+    // fit an int)
+    if (cell > 16384) return CELLS_FAR;
+    const unsigned uc = (unsigned)cell;   // (at most the extent, below 2^32)
+#pragma unroll
+    for (int u = 0; u < PER; ++u)
+        if (tid + u * PRUNE_THREADS < n) {
+            bk[u] = (int)((unsigned)(mine[u].y - oy) / uc) * nx + (int)((unsigned)(mine[u].x - ox) / uc) + 1;
+            atomicAdd(&s.bcount[bk[u]], 1);
+        }
+    __syncthreads();
+    scan_buckets(s);
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < PER; ++u)
+        if (tid + u * PRUNE_THREADS < n) {
+            const int at = s.boff[bk[u]] + atomicSub(&s.bcount[bk[u]], 1) - 1;
+            r.x[at] = mine[u].x;
+            r.y[at] = mine[u].y;
+            r.level[at] = mine[u].level;
+            r.resp[at] = mine[u].response;
+            r.cell[at] = (unsigned short)bk[u];
+            r.target[at] = -1;
+            r.state[at] = ST_UND;
+            r.in[at] = 0;
+            r.und[at] = 0;
+        }
+    __syncthreads();
+    // edges: candidate i and row of cells dy - 1 per thread; every warp fills and
+    // later reads its own part of the list (hits are rare, so they may diverge)
+    unsigned* edge = r.edge + (tid >> 5) * EDGE_WARP;
+    int* n_edge = &s.wsum[tid >> 5];
+    if (lane == 0) *n_edge = 0;
+    __syncwarp();
+    const int reach = g.reach;
+    for (int t = tid; t < 3 * n; t += PRUNE_THREADS) {
+        const int dy = (t >= n) + (t >= 2 * n), i = t - dy * n;
+        const int xi = r.x[i], yi = r.y[i];
+        const int c = r.cell[i] + (dy - 1) * nx;
+        if (c < 0 || c >= nx * ny) continue;
+        const int end = s.boff[c + 2];
+        for (int k = s.boff[c - 1]; k < end; ++k) {
+            const int ex = r.x[k] - xi, ey = r.y[k] - yi, d = ex * ex + ey * ey;
+            if (d >= reach || k == i) continue;
+            const int li = min(max(r.level[i], 0), p.P - 1), lk = min(max(r.level[k], 0), p.P - 1);
+            if (d >= s.d2[li * p.P + lk] || !r.before(k, i)) continue;
+            const int e = atomicAdd(n_edge, 1);
+            if (e < EDGE_WARP) edge[e] = (unsigned)i << 16 | (unsigned)k;
+        }
+    }
+    __syncwarp();
+    const int ne = *n_edge;
+    if (__syncthreads_or(ne > EDGE_WARP)) return CELLS_FULL;
+    // rounds of the independent-set rule
+    for (;;) {
+        for (int e = lane; e < ne; e += 32) {
+            const int i = edge[e] >> 16;
+            if (r.state[i] != ST_UND) continue;
+            const int st = r.state[edge[e] & 0xffffu];
+            if (st == ST_IN) r.in[i] = 1;
+            else if (st == ST_UND) r.und[i] = 1;
+        }
+        __syncthreads();
+        bool wait = false;
+        for (int i = tid; i < n; i += PRUNE_THREADS) {
+            if (r.state[i] != ST_UND) continue;
+            if (r.in[i] || !r.und[i]) r.state[i] = r.in[i] ? ST_OUT : ST_IN;
+            else wait = true;
+            r.und[i] = 0;
+        }
+        if (!__syncthreads_or(wait)) break;   // (each round settles the first undecided)
+    }
+    // every rejected candidate joins its highest-priority accepted neighbour
+    bool any = false;
+    for (int e = lane; e < ne; e += 32) {
+        const int i = edge[e] >> 16, j = edge[e] & 0xffffu;
+        if (r.state[i] != ST_OUT || r.state[j] != ST_IN) continue;
+        any = true;
+        int seen = r.target[i];
+        while (seen < 0 || r.before(j, seen)) {
+            const int now = atomicCAS(&r.target[i], seen, j);
+            if (now == seen) break;
+            seen = now;
+        }
+    }
+    finish_cells(p, s, r, n, any, out, f);
+    return CELLS_DONE;
+}
+
+// The frame of prune_cells' CELLS_FULL: every round, and then the targets, walk the
+// rows of cells again.  A state is settled once, so a round may see others before
+// or after theirs.  Out of line and apart, so that the frames without need are not
+// compiled for it (with both in prune_cells a frame of the FFT backend took 29.3 us
+// in place of 20.6; apart 21.3).
+__device__ __noinline__ void dense_cells(const PruneParams& p, PruneSmem& s, CellSmem& r, int n, dog_blob* out, int f) {
+    const CellGrid g = cell_grid(p, r, n);
+    const int nx = g.nx, ny = g.ny, reach = g.reach;
+    auto walk = [&](int i, auto visit) {   // i's neighbours of higher priority, until visit() has seen enough
+        const int xi = r.x[i], yi = r.y[i], li = min(max(r.level[i], 0), p.P - 1);
+        for (int dy = -1; dy <= 1; ++dy) {
+            const int c = r.cell[i] + dy * nx;
+            if (c < 0 || c >= nx * ny) continue;
+            const int end = s.boff[c + 2];
+            for (int k = s.boff[c - 1]; k < end; ++k) {
+                const int ex = r.x[k] - xi, ey = r.y[k] - yi, d = ex * ex + ey * ey;
+                if (d >= reach || k == i) continue;
+                if (d < s.d2[li * p.P + min(max(r.level[k], 0), p.P - 1)] && r.before(k, i) && visit(k)) return;
+            }
+        }
+    };
+    volatile unsigned char* state = r.state;
+    for (;;) {
+        bool wait = false;
+        for (int i = threadIdx.x; i < n; i += PRUNE_THREADS) {
+            if (state[i] != ST_UND) continue;
+            bool in = false, und = false;
+            walk(i, [&](int k) {
+                const int st = state[k];
+                und |= st == ST_UND;
+                return in = st == ST_IN;
+            });
+            if (in || !und) state[i] = in ? ST_OUT : ST_IN;
+            else wait = true;
+        }
+        if (!__syncthreads_or(wait)) break;
+    }
+    bool any = false;
+    for (int i = threadIdx.x; i < n; i += PRUNE_THREADS) {
+        if (r.state[i] != ST_OUT) continue;
+        int best = -1;
+        walk(i, [&](int k) {
+            if (r.state[k] == ST_IN && (best < 0 || r.before(k, best))) best = k;
+            return false;
+        });
+        r.target[i] = best;
+        any = true;
+    }
+    finish_cells(p, s, r, n, any, out, f);
 }
 
 __global__ void __launch_bounds__(PRUNE_THREADS) dog_prune_kernel(const __grid_constant__ PruneParams p) {
@@ -488,7 +522,10 @@ __global__ void __launch_bounds__(PRUNE_THREADS) dog_prune_kernel(const __grid_c
     const int n = min(p.cand_count[f], p.cap_in);
     if (p.mode != DOG_PRUNE_OFF) {
         if (n <= PRUNE_SMEM_CAND) {
-            if (prune_cells(p, s, *reinterpret_cast<CellSmem*>(prune_dyn), cand, n, out, f)) return;
+            CellSmem& r = *reinterpret_cast<CellSmem*>(prune_dyn);
+            const int got = prune_cells(p, s, r, cand, n, out, f);
+            if (got == CELLS_FULL) dense_cells(p, s, r, n, out, f);
+            if (got != CELLS_FAR) return;
             __syncthreads();
         }
         // Copies in the shared memory that the launch has anyway, and that leaves the
