@@ -1,6 +1,7 @@
 """Tile-shape autotuner for the fused DoG detection kernel.
 
-A tile of the fused kernel is a strip of 32 output columns by a band of rows.
+A tile of the fused kernel is a strip of 32 output columns by a band of rows,
+walked in blocks of 8 rows per warp of the kernel form (96 rows for 12 warps).
 Before its first output row a tile runs the horizontal passes of the rows its
 vertical blur reaches above the band (the warm-up, about 8 * ceil((2 r_max +
 1) / 8) rows), so a short band pays that halo often; a tall band leaves SMs
@@ -8,11 +9,15 @@ idle in the last wave (few tiles, one CTA per SM).  The best height depends on
 the frame shapes, the ladder and the number of SMs, so it is measured.
 
 The tuner ranks candidate band heights with a cost model (waves x rows walked,
-the halo counted as half a row because only its horizontal pass runs), times
-the best few on the device through the detector's own entry points, and keeps
-the winner per (shapes, ladder) key.  It also times both kernel forms (8 or 12
-producer warps; which is faster depends on the ladder).  The timing function
-is injectable, so the selection logic runs on the CPU in tests.
+the halo counted as half a row because only its horizontal pass runs; blocks
+that a band fills in part are not in it), times the best few on the device
+through the detector's own entry points, and keeps the winner per (shapes,
+ladder) key.  A batch takes the height as it is.  A call on one frame evens its
+bands out over the frame, in a number next to the asked one, so that several of
+the heights timed there are one launch.  The tuner also times both bounds on the
+kernel form (12 and 8 warps); on ladders whose handles report 8, or whose largest
+form has 8 warps, they are the same form.  The timing function is injectable, so
+the selection logic runs on the CPU in tests.
 """
 from __future__ import annotations
 
@@ -22,7 +27,7 @@ import os
 from dataclasses import dataclass, field
 from typing import Callable, Dict, Iterable, List, Optional, Sequence, Tuple
 
-MB = 8          # rows per block of the fused kernel (band heights are multiples of it)
+MB = 8          # band heights are multiples of it
 TX = 32         # columns per strip
 
 
@@ -86,7 +91,7 @@ def candidate_bands(shapes: Sequence[Tuple[int, int]], radii: Sequence[int], n_s
     return out
 
 
-PRODUCER_WARPS = (12, 8)   # kernel forms (0: the handle's default)
+PRODUCER_WARPS = (12, 8)   # bounds on the kernel form's warps (0: none)
 
 
 @dataclass

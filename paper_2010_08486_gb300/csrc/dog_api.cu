@@ -318,7 +318,7 @@ void handle_tap_slot(const dog_handle* h, int i, int* base, int* lead) {
 // The form to run for a wish of nw warps (0: no wish): the largest that fits and
 // is not larger than the wish.  More warps hide more latency: on every ladder
 // timed (96 frames of 1024 x 1024) the 12-warp form is the faster one, by 7% to
-// 20%, so it is the default wherever it fits; where it does not, the 10-warp form
+// 26%, so it is the default wherever it fits; where it does not, the 10-warp form
 // still beats the 8-warp one (eight 1000 x 1000 frames, sigma 2 to 12.3 in 14
 // levels, which fit 10: 886 us, with 8: 978).  What the handle reports without
 // a wish is the rule that callers know: 12 for ladders of 20 or more levels

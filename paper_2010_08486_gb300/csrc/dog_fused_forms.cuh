@@ -32,12 +32,14 @@
 // that fill the windows.  It also gives every warp the same work, so nobody
 // waits at the barrier, and the L rows never go through shared memory.
 //
-// Measured (96 frames of 1024 x 1024, 12-bit, one batched launch, 12 warps):
-// 25 levels to sigma 7.9 9.87 -> 8.45 ms, 12 levels 1.25^k 9.18 -> 5.8 ms, 6
-// levels to sigma 10.5 6.69 -> 3.6 ms, 14 levels to sigma 12.3 (8 warps) 10.56 ->
-// 9.4 ms (another 9% less with the 10 warps that fit), against the form before
-// (levels on fixed producer warps, scalar FMAs, taps and L rows through shared
-// memory).
+// Measured (96 frames of 1024 x 1024, 12-bit, one batched launch): 25 levels to
+// sigma 7.9 9.87 -> 8.24 ms, 12 levels 1.25^k 9.18 -> 5.65 ms, 6 levels to sigma
+// 10.5 6.69 -> 3.52 ms (12 warps), 14 levels to sigma 12.3 10.56 -> 8.25 ms (10
+// warps), against the form before (levels on fixed producer warps, scalar FMAs,
+// taps and L rows through shared memory).  A block is 8 NW rows, so tiles that fill
+// little of one gain least: 25 levels on batched frames of 32 rows or fewer, or of
+// 97, take 5 to 14% longer than the form before (with 8 warps as long as with 12);
+// other ladders are faster there too.
 //
 // Both passes are register-blocked 1-D correlations: 8 outputs per lane, taps
 // in blocks of 8 against a two-window register file whose halves swap roles

@@ -251,7 +251,8 @@ class Detector:
         check(self.lib.dog_set_tiling(self.h, band_rows, ctas_per_sm), "dog_set_tiling")
 
     def set_producer_warps(self, n: int = 0):
-        """Kernel form: 8 or 12 producer warps, 0 for the handle's default."""
+        """Bound on the kernel form's warps: 8 or 12; 0 or the handle's own
+        `producer_warps` for none."""
         check(self.lib.dog_set_producer_warps(self.h, n), "dog_set_producer_warps")
 
     @property
@@ -375,7 +376,9 @@ class DoGSoftHist(torch.autograd.Function):
     forward(frames (B, H, W) float32 CUDA, sigmas (K,) float32 CUDA, det) ->
     H (nbins,) summed over the batch.  One launch works on all frames.  The
     forward records each frame's hard maxima (O(maxima) memory, no blur level
-    is kept); backward gathers dloss/dI from them.  A frame whose list
+    is kept); backward gathers dloss/dI from them (a frame too dense in maxima
+    for that is blurred; should the kernel's wait for its own CTAs run out, that
+    frame's gradient is NaN and the status a timeout).  A frame whose list
     overflowed (more maxima than `rec_cap`, e.g. a flat frame where every
     voxel ties) recomputes its blur levels in the backward instead."""
 
